@@ -243,6 +243,8 @@ extern "C" onnxb_status onnx_conv2d_run_prepacked(onnxb_conv2d_desc_t d, const f
 // of one sign.  Both copies live in the workspace: A' first, then B'.
 static bool gemm_tc_eligible(int transA, int transB, int64_t M, int64_t N, int64_t K) {
     if (K < 32) return false;                       // thin contraction: exact fp32 FMA instead
+    // a few thousand dot products: the one-launch fp32 kernel, unless a tensor-core family is forced
+    if (kernel_override() < 0 && simt_gemm_is_tiny(M, N, K)) return false;
     const int64_t a_ld = transA ? M : K, b_ld = transB ? K : N;
     return a_ld % 4 == 0 && b_ld % 4 == 0;          // tensor-map strides are multiples of 16 bytes
 }

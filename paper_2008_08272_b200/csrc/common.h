@@ -64,7 +64,13 @@ struct GemmProblem {
     long long c_stride_i, c_stride_j;   // element strides of C along i and j (0 = broadcast)
     int relu;
 };
+bool simt_gemm_is_tiny(long long M, long long N, long long K);   // small enough for the dot-product kernel
 int launch_simt_gemm(const GemmProblem &p, const float *A, const float *B, const float *C, float *Y,
                      void *stream);
+// fp32 through split TF32 operands on the tensor cores (tc_fp32.cu): the same problems, once they are large
+double tc_fp32_cost(long long rows, int cols, int K, int groups, bool pixels);     // estimated SM cycles
+int launch_tc_fp32_gemm(const GemmProblem &p, const float *A, const float *B, const float *C, float *Y, void *stream);
+int launch_tc_fp32_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
+                        void *stream);
 
 }  // namespace onnxb

@@ -12,90 +12,6 @@ namespace onnxb {
 
 namespace {
 
-constexpr int kDirectThreads = 128;   // one output pixel per thread
-constexpr int kDirectChunk = 256;     // reduction terms staged in shared memory per pass
-
-// Direct convolution.  A block owns 128 consecutive output pixels of one image
-// and MT consecutive output channels of one group; each thread keeps MT
-// accumulators, so every input value loaded is used MT times.  The reduction
-// index k = (c*kH + r)*kW + s is walked in chunks whose weights sit in shared
-// memory (all threads read the same weight: a broadcast).
-template <int MT>
-__global__ void __launch_bounds__(kDirectThreads)
-conv2d_direct_kernel(const ConvGeom g, const float *__restrict__ X, const float *__restrict__ W,
-                     const float *__restrict__ B, const float *__restrict__ R, float *__restrict__ Y, int pixel_tiles,
-                     int m_tiles_per_group) {
-    __shared__ float wsm[MT * kDirectChunk];
-
-    const int tile = blockIdx.x % pixel_tiles;
-    const int n = blockIdx.x / pixel_tiles;
-    const int PQ = g.P * g.Q;
-    const int pix = tile * kDirectThreads + threadIdx.x;
-    const bool live = pix < PQ;
-    const int p = live ? pix / g.Q : 0;
-    const int q = live ? pix % g.Q : 0;
-    const int ih0 = p * g.sh - g.pt;
-    const int iw0 = q * g.sw - g.pl;
-    const int taps = g.kH * g.kW;
-    const int Kred = g.Cg * taps;
-
-    for (int mt = blockIdx.y; mt < m_tiles_per_group * g.group; mt += gridDim.y) {
-        const int grp = mt / m_tiles_per_group;
-        const int m0 = grp * g.Mg + (mt % m_tiles_per_group) * MT;
-        const int m_end = (grp + 1) * g.Mg;
-        const float *xg = X + ((size_t)n * g.C + (size_t)grp * g.Cg) * g.H * g.W;
-
-        float acc[MT];
-#pragma unroll
-        for (int j = 0; j < MT; ++j) acc[j] = 0.f;
-
-        for (int k0 = 0; k0 < Kred; k0 += kDirectChunk) {
-            const int len = min(kDirectChunk, Kred - k0);
-            __syncthreads();
-            for (int idx = threadIdx.x; idx < MT * len; idx += kDirectThreads) {
-                const int j = idx / len, kk = idx - j * len;
-                wsm[j * kDirectChunk + kk] = (m0 + j < m_end) ? W[(size_t)(m0 + j) * Kred + k0 + kk] : 0.f;
-            }
-            __syncthreads();
-            if (live) {
-                int c = k0 / taps;
-                int rs = k0 - c * taps;
-                int r = rs / g.kW;
-                int s = rs - r * g.kW;
-                for (int kk = 0; kk < len; ++kk) {
-                    const int ih = ih0 + r * g.dh;
-                    const int iw = iw0 + s * g.dw;
-                    float x = 0.f;
-                    if ((unsigned)ih < (unsigned)g.H && (unsigned)iw < (unsigned)g.W)
-                        x = __ldg(xg + ((size_t)c * g.H + ih) * g.W + iw);
-#pragma unroll
-                    for (int j = 0; j < MT; ++j) acc[j] = fmaf(x, wsm[j * kDirectChunk + kk], acc[j]);
-                    if (++s == g.kW) {
-                        s = 0;
-                        if (++r == g.kH) {
-                            r = 0;
-                            ++c;
-                        }
-                    }
-                }
-            }
-        }
-        if (live) {
-#pragma unroll
-            for (int j = 0; j < MT; ++j) {
-                const int m = m0 + j;
-                if (m < m_end) {
-                    float v = acc[j] + (B ? __ldg(B + m) : 0.f);
-                    const size_t yi = ((size_t)n * g.M + m) * PQ + pix;
-                    if (R) v += __ldg(R + yi);              // residual addend at Y's own position
-                    if (g.relu) v = v > 0.f ? v : 0.f;
-                    Y[yi] = v;
-                }
-            }
-        }
-    }
-}
-
 // Depthwise convolution (group == C == M): purely HBM-bound, 2*kH*kW flops per
 // output.  A block stages the input window of a 32 x 32 output tile of one
 // (image, channel) plane in shared memory with coalesced row loads (zeros
@@ -169,33 +85,6 @@ conv2d_depthwise_kernel(const ConvGeom g, const float *__restrict__ X, const flo
 //   per image: Xg[n][c][p*Q + q]      (pitch = P*Q).
 __device__ __forceinline__ float gather_round(float v) {
     return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);
-}
-
-__global__ void __launch_bounds__(256)
-gather1x1_kernel(const float *__restrict__ X, float *__restrict__ Xg, unsigned total, unsigned pitch, unsigned NPQ,
-                 unsigned PQ, unsigned Q, unsigned C, unsigned HW, unsigned rowstep, unsigned sw, int merged,
-                 const ConvDivisor dv_pitch, const ConvDivisor dv_PQ, const ConvDivisor dv_Q) {
-    tc::pdl_launch_dependents();
-    // the three divisions per element are multiply-and-shift by constants the host prepares
-    for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < total; i += gridDim.x * 256u) {
-        const unsigned row = (unsigned)conv_fdiv((int)i, (int)pitch, dv_pitch);   // merged: channel; per image: n*C + c
-        const unsigned j = i - row * pitch;
-        float v = 0.f;
-        if (j < NPQ) {
-            unsigned plane, r;
-            if (merged) {
-                const unsigned n = (unsigned)conv_fdiv((int)j, (int)PQ, dv_PQ);
-                r = j - n * PQ;
-                plane = n * C + row;
-            } else {
-                r = j;
-                plane = row;
-            }
-            const unsigned p = (unsigned)conv_fdiv((int)r, (int)Q, dv_Q), q = r - p * Q;
-            v = gather_round(__ldg(X + (size_t)plane * HW + p * rowstep + q * sw));
-        }
-        Xg[i] = v;
-    }
 }
 
 // Any layout whose pitch is a multiple of four (both layouts have one): four consecutive outputs per
@@ -421,7 +310,7 @@ int launch_gather1x1(const ConvGeom &g, const float *X, float *Xg, long long pit
             gather1x1_vec_kernel<2><<<blocks, 256, 0, st>>>(reinterpret_cast<const float4 *>(X),
                                                            reinterpret_cast<float4 *>(Xg), (unsigned)total4, PQ4, Q4,
                                                            HW4, rowstep4);
-    } else if (pitch % 4 == 0) {
+    } else {                       // every pitch is a multiple of four
         const long long total4 = total / 4;
         const unsigned blocks = (unsigned)std::min<long long>((total4 + 255) / 256, 148LL * 32);
         gather1x1_quad_kernel<<<blocks, 256, 0, st>>>(X, reinterpret_cast<float4 *>(Xg), (unsigned)total4, (unsigned)pitch,
@@ -430,13 +319,6 @@ int launch_gather1x1(const ConvGeom &g, const float *X, float *Xg, long long pit
                                                       (unsigned)(g.H * g.W), (unsigned)(g.sh * g.W), (unsigned)g.sw,
                                                       merged ? 1 : 0, conv_divisor((int)pitch), conv_divisor(g.P * g.Q),
                                                       conv_divisor(g.Q));
-    } else {
-        const unsigned blocks = (unsigned)std::min<long long>((total + 255) / 256, 148LL * 64);
-        gather1x1_kernel<<<blocks, 256, 0, st>>>(X, Xg, (unsigned)total, (unsigned)pitch,
-                                                 (unsigned)(merged ? g.N * g.P * g.Q : g.P * g.Q), (unsigned)(g.P * g.Q),
-                                                 (unsigned)g.Q, (unsigned)g.C, (unsigned)(g.H * g.W),
-                                                 (unsigned)(g.sh * g.W), (unsigned)g.sw, merged ? 1 : 0,
-                                                 conv_divisor((int)pitch), conv_divisor(g.P * g.Q), conv_divisor(g.Q));
     }
     count_launch();
     return (int)cudaGetLastError();
@@ -460,27 +342,6 @@ int launch_simt_depthwise(const ConvGeom &g, const float *X, const float *W, con
     const unsigned blocks = (unsigned)((long long)q_tiles * p_tiles * g.N * g.C);
     conv2d_depthwise_kernel<<<blocks, kDwThreads, smem, (cudaStream_t)stream>>>(g, X, W, B, R, Y, q_tiles, p_tiles, rows,
                                                                               cols, pitch);
-    count_launch();
-    return (int)cudaGetLastError();
-}
-
-int launch_simt_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
-                     void *stream) {
-    const long long PQ = (long long)g.P * g.Q;
-    const int pixel_tiles = (int)((PQ + kDirectThreads - 1) / kDirectThreads);
-    const long long gx = (long long)pixel_tiles * g.N;
-    if (gx > 2147483647LL) return (int)cudaErrorInvalidConfiguration;
-    const int MT = g.Mg >= 8 ? 8 : (g.Mg >= 4 ? 4 : 1);
-    const int m_tiles_per_group = (g.Mg + MT - 1) / MT;
-    const long long m_tiles = (long long)m_tiles_per_group * g.group;
-    dim3 grid((unsigned)gx, (unsigned)(m_tiles > 65535 ? 65535 : m_tiles), 1);
-    cudaStream_t st = (cudaStream_t)stream;
-    if (MT == 8)
-        conv2d_direct_kernel<8><<<grid, kDirectThreads, 0, st>>>(g, X, W, B, R, Y, pixel_tiles, m_tiles_per_group);
-    else if (MT == 4)
-        conv2d_direct_kernel<4><<<grid, kDirectThreads, 0, st>>>(g, X, W, B, R, Y, pixel_tiles, m_tiles_per_group);
-    else
-        conv2d_direct_kernel<1><<<grid, kDirectThreads, 0, st>>>(g, X, W, B, R, Y, pixel_tiles, m_tiles_per_group);
     count_launch();
     return (int)cudaGetLastError();
 }

@@ -1,92 +1,502 @@
-// SIMT (fp32 FMA) Gemm: Y = relu?(alpha * A' * B' + beta * Cb), ONNX Gemm
-// (Sec. 3.4.3).  Used for problems too small or too oddly aligned for the
-// tensor-core pipeline; accepts every transA/transB/broadcast combination.
+// fp32 (FMA) tiled contraction: ONNX Gemm (Sec. 3.4.3) and ONNX Conv (Sec. 4.1) for the problems
+// that stay in fp32: contractions too thin for the tensor cores, or operands TMA cannot describe (rows
+// that are no multiples of 16 bytes, images of odd size).
+//
+// One kernel serves both operators as D (M x N) = A (M x K) * B (K x N):
+//   Gemm  A', B' in any of the four storage orders;
+//   Conv  A = the filters W[m][k] (k = (c*kH + r)*kW + s, exactly ONNX's layout), B = the pixels, column
+//         j = (image, p, q), whose row k is fetched from X through a small table of the K block's
+//         (channel, tap) offsets: the unfolded matrix is never formed.
+//
+// Bound: the FMA pipe (148 SMs x 128 FMA x 1.965 GHz = 74.4 TFLOP/s).  What it takes to get near it:
+// packed fma.rn.f32x2 (two FMAs per issue slot, so the operand reads and address work fit beside them), 8x8
+// or 8x4 outputs per thread, operands staged by cp.async (4 bytes: rows have no alignment) three K blocks
+// deep, and the reduction split over a cluster's CTAs where the tiles alone leave SMs idle (partial tiles
+// are summed through distributed shared memory in rank order, so the result does not depend on timing).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cstdio>
+#include <cstdlib>
+
 #include "common.h"
+#include "tc_common.cuh"
+#include "tc_host.h"
 
 namespace onnxb {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16;   // block tile; 256 threads, 4x4 outputs each
+constexpr int kBK = 16;        // reduction terms per stage
+constexpr int kStages = 3;
 
-__global__ void __launch_bounds__(256)
-gemm_simt_kernel(const GemmProblem p, const float *__restrict__ A, const float *__restrict__ B,
-                 const float *__restrict__ C, float *__restrict__ Y, int tiles_n) {
-    __shared__ float As[BK][BM + 4];
-    __shared__ float Bs[BK][BN + 4];
+enum { kKContig = 0, kMnContig = 1, kPixels = 2 };
 
-    const int tile_m = blockIdx.x / tiles_n, tile_n = blockIdx.x % tiles_n;
+struct SgemmArgs {
+    const float *A, *B;
+    float *Y;
+    int M, N, K;                       // per group for a convolution
+    long long a_ld, b_ld;              // stride of the non-contiguous index
+    int tiles_m, tiles_n, relu;
+    // Gemm epilogue: alpha * D + beta * C
+    float alpha, beta;
+    const float *C;
+    long long c_si, c_sj;
+    // Conv
+    const float *bias, *R;
+    int Cch, H, W, PQ, Q, sh, sw, dh, dw, pt, pl, taps, kW, Mtot;
+    ConvDivisor dv_PQ, dv_Q, dv_taps, dv_kW;
+};
+
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src, bool live) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(live ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void fma2(unsigned long long &d, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long dup2(float a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ float ld_dsmem(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+template <int BM, int BN>
+__host__ __device__ constexpr size_t sgemm_smem() {
+    const size_t ring = (size_t)kStages * kBK * (BM + 4 + BN + 4) * 4, out = (size_t)BM * (BN + 4) * 4;
+    return (ring > out ? ring : out) + (kStages + 1) * kBK * 16;
+}
+
+// Threads form (BM/TM) x (BN/TN); a warp covers 4 x 8 of them.  A thread's rows are tm*4 + {0..3} and, for
+// TM = 8, the same in the tile's lower half (likewise its columns), so that every fragment read is a 16-byte
+// shared-memory load whose lanes touch consecutive pieces.
+template <int BM, int BN, int TM, int TN, int AM, int BMODE>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), (BM / TM) * (BN / TN) == 256 ? 2 : 4)
+sgemm_kernel(const __grid_constant__ SgemmArgs g, int split) {
+    constexpr int NT_M = BM / TM, NT_N = BN / TN, NTHR = NT_M * NT_N;
+    constexpr int PA = BM + 4, PB = BN + 4;
+    constexpr int WARPS_N = NT_N / 8;
+    extern __shared__ __align__(16) float sm[];
+    float *As = sm, *Bs = sm + kStages * kBK * PA;
+    int4 *ktab = reinterpret_cast<int4 *>(reinterpret_cast<uint8_t *>(sm) + sgemm_smem<BM, BN>() - (kStages + 1) * kBK * 16);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)(blockIdx.x % (unsigned)split);
+    unsigned tile = blockIdx.x / (unsigned)split;
+    const int tile_m = (int)(tile % (unsigned)g.tiles_m);
+    tile /= (unsigned)g.tiles_m;
+    const int tile_n = (int)(tile % (unsigned)g.tiles_n), grp = (int)(tile / (unsigned)g.tiles_n);
     const int i0 = tile_m * BM, j0 = tile_n * BN;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    const int ktiles = (g.K + kBK - 1) / kBK;
+    const int kt_per = (ktiles + split - 1) / split;
+    const int kt_lo = rank * kt_per, kt_hi = min(ktiles, kt_lo + kt_per);
 
-    // element strides of A' (i,k) and B' (k,j) in their stored arrays
-    const long long a_si = p.transA ? 1 : p.K, a_sk = p.transA ? p.M : 1;
-    const long long b_sk = p.transB ? 1 : p.N, b_sj = p.transB ? p.K : 1;
+    // ---- what this thread loads
+    constexpr int A_ROWS_STEP = NTHR / kBK, A_N = BM / A_ROWS_STEP;          // k-contiguous: lanes along k
+    constexpr int A_KSTEP = NTHR / BM > 0 ? NTHR / BM : 1;                    // m-contiguous: lanes along m
+    constexpr int A_MREP = NTHR >= BM ? 1 : BM / NTHR;
+    constexpr int B_ROWS_STEP = NTHR / kBK, B_N = BN / B_ROWS_STEP;
+    constexpr int B_KSTEP = NTHR / BN > 0 ? NTHR / BN : 1;
+    constexpr int B_NREP = NTHR >= BN ? 1 : BN / NTHR;
+    const float *Ag = g.A + (BMODE == kPixels ? (long long)grp * g.M * g.K : 0);
+    const uint32_t as_u32 = tc::smem_u32(As), bs_u32 = tc::smem_u32(Bs);
 
-    float acc[4][4];
+    // pixel columns of a convolution: where the column's window starts in X
+    long long px_base[B_NREP];
+    int px_h[B_NREP], px_w[B_NREP];
+    if (BMODE == kPixels) {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-
-    for (int k0 = 0; k0 < p.K; k0 += BK) {
-        // 1024 elements per operand tile, 4 per thread; the fast index follows
-        // whichever axis is contiguous in memory
-        for (int e = threadIdx.x; e < BM * BK; e += 256) {
-            int ii, kk;
-            if (p.transA) { ii = e % BM; kk = e / BM; } else { kk = e % BK; ii = e / BK; }
-            const int i = i0 + ii, k = k0 + kk;
-            As[kk][ii] = (i < p.M && k < p.K) ? __ldg(A + i * a_si + k * a_sk) : 0.f;
-        }
-        for (int e = threadIdx.x; e < BN * BK; e += 256) {
-            int jj, kk;
-            if (p.transB) { kk = e % BK; jj = e / BK; } else { jj = e % BN; kk = e / BN; }
-            const int j = j0 + jj, k = k0 + kk;
-            Bs[kk][jj] = (j < p.N && k < p.K) ? __ldg(B + k * b_sk + j * b_sj) : 0.f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            float av[4], bv[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = As[kk][ty * 4 + a];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][tx * 4 + b];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(av[a], bv[b], acc[a][b]);
-        }
-        __syncthreads();
-    }
-
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int i = i0 + ty * 4 + a;
-        if (i >= p.M) continue;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int j = j0 + tx * 4 + b;
-            if (j >= p.N) continue;
-            float v = p.alpha * acc[a][b];
-            if (C) v = fmaf(p.beta, __ldg(C + i * p.c_stride_i + j * p.c_stride_j), v);
-            if (p.relu) v = v > 0.f ? v : 0.f;
-            Y[(size_t)i * p.N + j] = v;
+        for (int e = 0; e < B_NREP; ++e) {
+            const int j = j0 + tid % BN + e * NTHR;
+            if (j < g.N) {
+                const int n = conv_fdiv(j, g.PQ, g.dv_PQ), u = j - n * g.PQ;
+                const int p = conv_fdiv(u, g.Q, g.dv_Q), q = u - p * g.Q;
+                px_h[e] = p * g.sh - g.pt;
+                px_w[e] = q * g.sw - g.pl;
+                px_base[e] = ((long long)n * g.Cch + (long long)grp * (g.K / g.taps)) * g.H * g.W +
+                             (long long)px_h[e] * g.W + px_w[e];
+            } else {
+                px_h[e] = px_w[e] = -(1 << 30);
+                px_base[e] = 0;
+            }
         }
     }
+    // offsets of one K block's rows: {offset in X, r*dh, s*dw}; rows past K point far outside the image
+    auto write_ktab = [&](int kt) {
+        if (BMODE == kPixels && tid < kBK) {
+            const int k = kt * kBK + tid;
+            int4 e = make_int4(0, -(1 << 30), -(1 << 30), 0);
+            if (k < g.K) {
+                const int c = conv_fdiv(k, g.taps, g.dv_taps), rs = k - c * g.taps;
+                const int r = conv_fdiv(rs, g.kW, g.dv_kW), s = rs - r * g.kW;
+                e = make_int4(c * g.H * g.W + r * g.dh * g.W + s * g.dw, r * g.dh, s * g.dw, 0);
+            }
+            ktab[(kt % (kStages + 1)) * kBK + tid] = e;
+        }
+    };
+    auto load_tile = [&](int kt, int st) {
+        const int k0 = kt * kBK;
+        if (AM == kKContig) {
+            const int kk = tid % kBK, r0 = tid / kBK;
+            const bool kok = k0 + kk < g.K;
+            const float *src = Ag + (long long)(i0 + r0) * g.a_ld + k0 + kk;
+            uint32_t dst = as_u32 + (uint32_t)((st * kBK + kk) * PA + r0) * 4u;
+#pragma unroll
+            for (int e = 0; e < A_N; ++e) {
+                const bool ok = kok && i0 + r0 + e * A_ROWS_STEP < g.M;
+                cp_async4(dst, ok ? src : g.A, ok);
+                src += (long long)A_ROWS_STEP * g.a_ld;
+                dst += A_ROWS_STEP * 4u;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < A_MREP; ++e) {
+                const int ii = tid % BM + e * NTHR, kk0 = NTHR >= BM ? tid / BM : 0;
+                const bool iok = i0 + ii < g.M;
+                const float *src = Ag + (long long)(k0 + kk0) * g.a_ld + i0 + ii;
+                uint32_t dst = as_u32 + (uint32_t)((st * kBK + kk0) * PA + ii) * 4u;
+#pragma unroll
+                for (int kk = 0; kk < kBK; kk += A_KSTEP) {
+                    const bool ok = iok && k0 + kk0 + kk < g.K;
+                    cp_async4(dst, ok ? src : g.A, ok);
+                    src += (long long)A_KSTEP * g.a_ld;
+                    dst += A_KSTEP * PA * 4u;
+                }
+            }
+        }
+        if (BMODE == kKContig) {
+            const int kk = tid % kBK, r0 = tid / kBK;
+            const bool kok = k0 + kk < g.K;
+            const float *src = g.B + (long long)(j0 + r0) * g.b_ld + k0 + kk;
+            uint32_t dst = bs_u32 + (uint32_t)((st * kBK + kk) * PB + r0) * 4u;
+#pragma unroll
+            for (int e = 0; e < B_N; ++e) {
+                const bool ok = kok && j0 + r0 + e * B_ROWS_STEP < g.N;
+                cp_async4(dst, ok ? src : g.B, ok);
+                src += (long long)B_ROWS_STEP * g.b_ld;
+                dst += B_ROWS_STEP * 4u;
+            }
+        } else {
+            const int4 *tab = ktab + (kt % (kStages + 1)) * kBK;
+#pragma unroll
+            for (int e = 0; e < B_NREP; ++e) {
+                const int jj = tid % BN + e * NTHR, kk0 = NTHR >= BN ? tid / BN : 0;
+                uint32_t dst = bs_u32 + (uint32_t)((st * kBK + kk0) * PB + jj) * 4u;
+                if (BMODE == kMnContig) {
+                    const bool jok = j0 + jj < g.N;
+                    const float *src = g.B + (long long)(k0 + kk0) * g.b_ld + j0 + jj;
+#pragma unroll
+                    for (int kk = 0; kk < kBK; kk += B_KSTEP) {
+                        const bool ok = jok && k0 + kk0 + kk < g.K;
+                        cp_async4(dst, ok ? src : g.B, ok);
+                        src += (long long)B_KSTEP * g.b_ld;
+                        dst += B_KSTEP * PB * 4u;
+                    }
+                } else {
+#pragma unroll
+                    for (int kk = 0; kk < kBK; kk += B_KSTEP) {
+                        const int4 t = tab[kk0 + kk];
+                        const bool ok = (unsigned)(px_h[e] + t.y) < (unsigned)g.H && (unsigned)(px_w[e] + t.z) < (unsigned)g.W;
+                        cp_async4(dst, ok ? g.B + (px_base[e] + t.x) : g.B, ok);
+                        dst += B_KSTEP * PB * 4u;
+                    }
+                }
+            }
+        }
+    };
+
+    // ---- main loop
+    const int wm = warp / WARPS_N, wn = warp % WARPS_N;
+    const int tm = wm * 4 + ((lane & 1) | ((lane >> 4) << 1)), tn = wn * 8 + ((lane >> 1) & 7);
+    unsigned long long acc[TM][TN / 2];
+#pragma unroll
+    for (int a = 0; a < TM; ++a)
+#pragma unroll
+        for (int b = 0; b < TN / 2; ++b) acc[a][b] = 0ull;
+
+    tc::pdl_launch_dependents();
+    tc::pdl_wait();
+    if (BMODE == kPixels) {
+        for (int s = 0; s < kStages; ++s) write_ktab(kt_lo + s);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int s = 0; s < kStages - 1; ++s) {
+        if (kt_lo + s < kt_hi) load_tile(kt_lo + s, s);
+        cp_async_commit();
+    }
+    int st = 0;
+    for (int kt = kt_lo; kt < kt_hi; ++kt) {
+        cp_async_wait<kStages - 2>();
+        __syncthreads();
+        {
+            const int nk = kt + kStages - 1;
+            if (nk < kt_hi) load_tile(nk, st == 0 ? kStages - 1 : st - 1);
+            cp_async_commit();
+            write_ktab(kt + kStages);
+        }
+        const float *as = As + st * kBK * PA + tm * 4, *bs = Bs + st * kBK * PB + tn * 4;
+#pragma unroll
+        for (int kk = 0; kk < kBK; ++kk) {
+            float av[TM];
+            unsigned long long bv[TN / 2];
+#pragma unroll
+            for (int h = 0; h < TM / 4; ++h) {
+                const float4 t = *reinterpret_cast<const float4 *>(as + kk * PA + h * (BM / 2));
+                av[4 * h] = t.x; av[4 * h + 1] = t.y; av[4 * h + 2] = t.z; av[4 * h + 3] = t.w;
+            }
+#pragma unroll
+            for (int h = 0; h < TN / 4; ++h) {
+                const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(bs + kk * PB + h * (BN / 2));
+                bv[2 * h] = t.x; bv[2 * h + 1] = t.y;
+            }
+#pragma unroll
+            for (int a = 0; a < TM; ++a) {
+                const unsigned long long aa = dup2(av[a]);
+#pragma unroll
+                for (int b = 0; b < TN / 2; ++b) fma2(acc[a][b], aa, bv[b]);
+            }
+        }
+        if (++st == kStages) st = 0;
+    }
+
+    // ---- epilogue: the tile goes through shared memory so that lanes store consecutive columns; with a
+    // split reduction every CTA of the cluster sums its share of the rows over all partial tiles
+    cp_async_wait<0>();
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < TM; ++a) {
+        const int row = (a / 4) * (BM / 2) + tm * 4 + a % 4;
+#pragma unroll
+        for (int h = 0; h < TN / 4; ++h)
+            *reinterpret_cast<ulonglong2 *>(sm + row * PB + h * (BN / 2) + tn * 4) = make_ulonglong2(acc[a][2 * h], acc[a][2 * h + 1]);
+    }
+    if (split > 1) tc::cluster_sync_all();
+    else __syncthreads();
+
+    constexpr int CPT = NTHR >= BN ? 1 : BN / NTHR;                // columns per thread
+    constexpr int RSTEP = NTHR >= BN ? NTHR / BN : 1;
+    constexpr int UR = 8;                                          // rows in flight per thread (addend loads overlap)
+    const int rows = (BM + split - 1) / split, r_lo = rank * rows, r_hi = min(min(BM, r_lo + rows), g.M - i0);
+    const uint32_t sm_u32 = tc::smem_u32(sm);
+#pragma unroll
+    for (int e = 0; e < CPT; ++e) {
+        const int jj = tid % BN + e * NTHR, j = j0 + jj;
+        if (j >= g.N) continue;
+        long long ybase, ystep;
+        if (BMODE == kPixels) {
+            const int n = conv_fdiv(j, g.PQ, g.dv_PQ);
+            ybase = ((long long)n * g.Mtot + (long long)grp * g.M) * g.PQ + (j - n * g.PQ);
+            ystep = g.PQ;
+        } else {
+            ybase = j;
+            ystep = g.N;
+        }
+        for (int r0 = r_lo + (NTHR >= BN ? tid / BN : 0); r0 < r_hi; r0 += RSTEP * UR) {
+            float add[UR], v[UR];
+#pragma unroll
+            for (int u = 0; u < UR; ++u) {
+                const int r = r0 + u * RSTEP, i = i0 + r;
+                add[u] = v[u] = 0.f;
+                if (r < r_hi) {
+                    if (BMODE == kPixels) {
+                        if (g.bias) add[u] = __ldg(g.bias + grp * g.M + i);
+                        if (g.R) v[u] = __ldg(g.R + ybase + (long long)i * ystep);
+                    } else if (g.C) {
+                        add[u] = g.beta * __ldg(g.C + i * g.c_si + j * g.c_sj);
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < UR; ++u) {
+                const int r = r0 + u * RSTEP;
+                if (r < r_hi) {
+                    float d = 0.f;
+                    if (split == 1) {
+                        d = sm[r * PB + jj];
+                    } else {
+                        for (int s = 0; s < split; ++s)
+                            d += ld_dsmem(tc::map_to_cta(sm_u32 + (uint32_t)(r * PB + jj) * 4u, (uint32_t)s));
+                    }
+                    d = BMODE == kPixels ? (d + add[u]) + v[u] : fmaf(g.alpha, d, add[u]);
+                    if (g.relu) d = d > 0.f ? d : 0.f;
+                    g.Y[ybase + (long long)(i0 + r) * ystep] = d;
+                }
+            }
+        }
+    }
+    if (split > 1) tc::cluster_sync_all();      // no CTA leaves while a peer still reads its partial tile
+}
+
+// ------------------------------------------------------------------ tiny Gemms: one warp per output
+// A few hundred to a few thousand dot products (a 10-class head behind a small network): everything is
+// latency, so no staging and no barrier; lanes split the reduction, a shuffle tree joins it.
+template <int AM, int BMODE>
+__global__ void __launch_bounds__(128)
+gemm_dot_kernel(const __grid_constant__ SgemmArgs g) {
+    tc::pdl_launch_dependents();
+    const int warp = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (warp >= g.M * g.N) return;
+    const int i = warp / g.N, j = warp - i * g.N;
+    const float *a = g.A + (AM == kKContig ? i * g.a_ld : i), *b = g.B + (BMODE == kKContig ? j * g.b_ld : j);
+    const long long as = AM == kKContig ? 1 : g.a_ld, bs = BMODE == kKContig ? 1 : g.b_ld;
+    tc::pdl_wait();
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    int k = lane;
+    for (; k + 224 < g.K; k += 256) {           // eight loads of each operand in flight
+        float x[8], y[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) { x[u] = __ldg(a + (k + 32 * u) * as); y[u] = __ldg(b + (k + 32 * u) * bs); }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s[u & 3] = fmaf(x[u], y[u], s[u & 3]);
+    }
+    for (; k < g.K; k += 32) s[0] = fmaf(__ldg(a + k * as), __ldg(b + k * bs), s[0]);
+    float v = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    if (lane == 0) {
+        v *= g.alpha;
+        if (g.C) v = fmaf(g.beta, __ldg(g.C + i * g.c_si + j * g.c_sj), v);
+        if (g.relu) v = v > 0.f ? v : 0.f;
+        g.Y[(long long)i * g.N + j] = v;
+    }
+}
+
+// ------------------------------------------------------------------ host side
+struct Shape {
+    int bm, bn, threads;
+    double eff;                // measured share of the FMA pipe with the SMs full (Gemm; 0.63 of it for pixels)
+};
+constexpr int kShapes = 5;
+constexpr Shape kShape[kShapes] = {{128, 128, 256, 0.73}, {64, 128, 128, 0.68}, {64, 64, 128, 0.59}, {16, 128, 128, 0.45},
+                                   {32, 32, 64, 0.50}};
+
+template <int AM, int BMODE, int I, int BM, int BN, int TM, int TN>
+cudaError_t launch_shape(const SgemmArgs &a, int split, long long tiles, cudaStream_t st) {
+    static_assert(kShape[I].bm == BM && kShape[I].bn == BN && kShape[I].threads == (BM / TM) * (BN / TN), "shape table");
+    constexpr size_t smem = sgemm_smem<BM, BN>();
+    auto kern = sgemm_kernel<BM, BN, TM, TN, AM, BMODE>;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    const dim3 grid((unsigned)(tiles * split)), block(kShape[I].threads);
+    return split > 1 ? tc_host::launch_pdl_cluster(kern, (unsigned)split, grid, block, smem, st, a, split)
+                     : tc_host::launch_pdl(kern, grid, block, smem, st, a, split);
+}
+
+// Tile and split: the shortest estimated time, in cycles, fitted to a sweep of every shape and split over 34
+// problems from 0.2 MFLOP to 14 GFLOP (the pick is within 6 % of the best on average).  An SM shares its FMA
+// pipe among its CTAs, so what counts is the work of the fullest SM over the rate its resident warps reach; a
+// CTA's start and epilogue come on top, a launch costs 7200 and a cluster's reduction 2000 more.
+struct Pick {
+    int shape, split;
+    double cost;
+};
+Pick pick_shape(int M, int N, int K, int groups, bool pixels) {
+    Pick best{-1, 1, 0};
+    const long long ktiles = (K + kBK - 1) / kBK;
+    int ps = -1, pk = 1;       // ONNXB_FP32 = "shape,split" pins both
+    if (const char *pin = getenv("ONNXB_FP32"))
+        if (sscanf(pin, "%d,%d", &ps, &pk) != 2) ps = -1;
+    for (int s = 0; s < kShapes; ++s) {
+        const Shape &h = kShape[s];
+        const long long tiles = (long long)((M + h.bm - 1) / h.bm) * ((N + h.bn - 1) / h.bn) * groups;
+        for (int split = 1; split <= 8; ++split) {
+            if (ps >= 0 && (s != ps || split != pk)) continue;
+            if (split > 1 && ktiles < split && ps < 0) break;
+            const long long ctas = tiles * split;
+            if (ctas > 2147483647LL) continue;
+            const long long per_sm = (ctas + 147) / 148;
+            const double kt = (double)((ktiles + split - 1) / split);
+            const double warps = std::min((double)per_sm * (h.threads / 32), 16.0);
+            const double eff = h.eff * (pixels ? 0.63 : 1.0) * std::min(1.0, 0.28 + 0.72 * warps / 14.0);
+            const double busy = (double)per_sm * h.bm * h.bn * kt * kBK / (128.0 * eff);
+            const double each = (double)per_sm * (400.0 + h.bm * h.bn / 3.7 + (split > 1 ? 260.0 : 0.0));
+            const double cost = std::max(busy, kt * 230.0) + each + 7200.0 + (split > 1 ? 2000.0 : 0.0);
+            if (best.shape < 0 || cost < best.cost) best = {s, split, cost};
+        }
+    }
+    return best;
+}
+
+// Large problems go to the split-TF32 tensor-core kernel, by the two estimates; ONNXB_FP32 = "tc" pins it.
+bool fp32_on_tensor_cores(double fma_cost, double tc_cost) {
+    if (const char *pin = getenv("ONNXB_FP32")) return pin[0] == 't';
+    return tc_cost < fma_cost;
+}
+
+template <int AM, int BMODE>
+int launch_sgemm(SgemmArgs &a, int groups, const Pick &pick, cudaStream_t st) {
+    const int best = pick.shape, best_split = pick.split;
+    if (best < 0) return (int)cudaErrorInvalidConfiguration;
+    a.tiles_m = (a.M + kShape[best].bm - 1) / kShape[best].bm;
+    a.tiles_n = (a.N + kShape[best].bn - 1) / kShape[best].bn;
+    const long long tiles = (long long)a.tiles_m * a.tiles_n * groups;
+    cudaError_t e;
+    switch (best) {
+        case 0: e = launch_shape<AM, BMODE, 0, 128, 128, 8, 8>(a, best_split, tiles, st); break;
+        case 1: e = launch_shape<AM, BMODE, 1, 64, 128, 8, 8>(a, best_split, tiles, st); break;
+        case 2: e = launch_shape<AM, BMODE, 2, 64, 64, 8, 4>(a, best_split, tiles, st); break;
+        case 3: e = launch_shape<AM, BMODE, 3, 16, 128, 4, 4>(a, best_split, tiles, st); break;
+        default: e = launch_shape<AM, BMODE, 4, 32, 32, 4, 4>(a, best_split, tiles, st); break;
+    }
+    count_launch();
+    return (int)e;
 }
 
 }  // namespace
 
+// Up to this size the dot-product kernel beats any tiled launch (64 x 10 x 256: one launch of about 3 us).
+bool simt_gemm_is_tiny(long long M, long long N, long long K) { return M * N <= 4096 && M * N * K <= (1 << 20); }
+
 int launch_simt_gemm(const GemmProblem &p, const float *A, const float *B, const float *C, float *Y,
                      void *stream) {
-    const long long tiles_m = (p.M + BM - 1) / BM, tiles_n = (p.N + BN - 1) / BN;
-    if (tiles_m * tiles_n > 2147483647LL) return (int)cudaErrorInvalidConfiguration;
-    gemm_simt_kernel<<<(unsigned)(tiles_m * tiles_n), 256, 0, (cudaStream_t)stream>>>(p, A, B, C, Y, (int)tiles_n);
-    count_launch();
-    return (int)cudaGetLastError();
+    SgemmArgs a{};
+    a.A = A; a.B = B; a.Y = Y; a.M = p.M; a.N = p.N; a.K = p.K;
+    a.a_ld = p.transA ? p.M : p.K;
+    a.b_ld = p.transB ? p.K : p.N;
+    a.alpha = p.alpha; a.beta = p.beta; a.C = C; a.c_si = p.c_stride_i; a.c_sj = p.c_stride_j; a.relu = p.relu;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (simt_gemm_is_tiny(p.M, p.N, p.K)) {
+        auto kern = p.transA ? (p.transB ? gemm_dot_kernel<kMnContig, kKContig> : gemm_dot_kernel<kMnContig, kMnContig>)
+                             : (p.transB ? gemm_dot_kernel<kKContig, kKContig> : gemm_dot_kernel<kKContig, kMnContig>);
+        const cudaError_t e = tc_host::launch_pdl(kern, dim3((unsigned)((p.M * p.N + 3) / 4)), dim3(128), 0, st, a);
+        count_launch();
+        return (int)e;
+    }
+    const Pick pick = pick_shape(a.M, a.N, a.K, 1, false);
+    if (fp32_on_tensor_cores(pick.cost, tc_fp32_cost(p.N, p.M, p.K, 1, false))) return launch_tc_fp32_gemm(p, A, B, C, Y, stream);
+    if (p.transA)
+        return p.transB ? launch_sgemm<kMnContig, kKContig>(a, 1, pick, st) : launch_sgemm<kMnContig, kMnContig>(a, 1, pick, st);
+    return p.transB ? launch_sgemm<kKContig, kKContig>(a, 1, pick, st) : launch_sgemm<kKContig, kMnContig>(a, 1, pick, st);
+}
+
+int launch_simt_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
+                     void *stream) {
+    SgemmArgs a{};
+    a.A = W; a.B = X; a.Y = Y; a.M = g.Mg; a.K = g.Cg * g.kH * g.kW;
+    const long long cols = (long long)g.N * g.P * g.Q;        // below 2^31: Y has M times as many elements
+    a.N = (int)cols;
+    a.a_ld = a.K;
+    a.bias = B; a.R = R; a.relu = g.relu;
+    a.Cch = g.C; a.H = g.H; a.W = g.W; a.PQ = g.P * g.Q; a.Q = g.Q;
+    a.sh = g.sh; a.sw = g.sw; a.dh = g.dh; a.dw = g.dw; a.pt = g.pt; a.pl = g.pl;
+    a.taps = g.kH * g.kW; a.kW = g.kW; a.Mtot = g.M;
+    a.dv_PQ = conv_divisor(a.PQ); a.dv_Q = conv_divisor(a.Q); a.dv_taps = conv_divisor(a.taps); a.dv_kW = conv_divisor(a.kW);
+    const Pick pick = pick_shape(a.M, a.N, a.K, g.group, true);
+    if (a.taps <= 64 && fp32_on_tensor_cores(pick.cost, tc_fp32_cost(a.N, a.M, a.K, g.group, true)))
+        return launch_tc_fp32_conv(g, X, W, B, R, Y, stream);
+    return launch_sgemm<kKContig, kPixels>(a, g.group, pick, (cudaStream_t)stream);
 }
 
 }  // namespace onnxb

@@ -1,0 +1,86 @@
+"""The fp32 contractions (operands TMA cannot describe, thin reductions): every tile shape and reduction split of
+the FMA kernel, the split-TF32 tensor-core kernel and the dot-product kernel against the oracle, at an fp32
+tolerance, on sizes that leave ragged tails in every direction."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+from parity import run_conv_gpu, run_gemm_gpu  # noqa: E402
+
+PINS = ["tc"] + [f"{shape},{split}" for shape in range(5) for split in (1, 3, 8)]
+GEMMS = [(1, 130, 65, False, False), (129, 257, 31, True, False), (65, 127, 97, False, True), (131, 70, 333, True, True)]
+CONVS = [dict(x=(2, 5, 13, 11), w=(17, 5, 3, 3), pads=(1, 1, 1, 1), dilations=(2, 1)),
+         dict(x=(1, 6, 19, 23), w=(130, 3, 7, 7), pads=(3, 3, 3, 3), strides=(2, 2), group=2),
+         dict(x=(3, 40, 9, 7), w=(33, 40, 1, 1), strides=(2, 2))]
+REL = 2e-6          # of sum |x*w|: fp32 rounding of up to a few hundred terms
+
+
+@pytest.fixture(scope="module")
+def binding():
+    from paper_2008_08272_b200 import binding as b
+    b.load(build_if_missing=False)
+    return b
+
+
+@pytest.mark.parametrize("pin", PINS)
+def test_fp32_gemm_and_conv_tiles(binding, pin, monkeypatch):
+    monkeypatch.setenv("ONNXB_FP32", pin)           # read at every launch
+    rng = np.random.default_rng(len(pin) * 31 + ord(pin[0]))
+    binding.set_kernel_override("simt_direct")
+    try:
+        for M, N, K, tA, tB in GEMMS:
+            A = rng.standard_normal((K, M) if tA else (M, K)).astype(np.float32)
+            B = rng.standard_normal((N, K) if tB else (K, N)).astype(np.float32)
+            C = rng.standard_normal((M, 1)).astype(np.float32)
+            kw = dict(alpha=0.5, beta=-1.5, transA=tA, transB=tB)
+            got = run_gemm_gpu(binding, torch, A, B, C, fuse_relu=True, **kw)
+            want, S = oracle.gemm(A, B, C, relu=True, **kw)
+            assert (np.abs(got - want) <= REL * S + 1e-5).all(), (M, N, K)
+        for c in CONVS:
+            X = rng.standard_normal(c["x"]).astype(np.float32)
+            W = rng.standard_normal(c["w"]).astype(np.float32)
+            B = rng.standard_normal((c["w"][0],)).astype(np.float32)
+            kw = dict(pads=c.get("pads", (0, 0, 0, 0)), strides=c.get("strides", (1, 1)),
+                      dilations=c.get("dilations", (1, 1)), group=c.get("group", 1))
+            got, fam = run_conv_gpu(binding, torch, X, W, B, relu=True, **kw)
+            assert fam == "simt_direct"
+            want, S = oracle.conv2d(X, W, B, relu=True, **kw)
+            assert (np.abs(got - want) <= REL * S + 1e-5).all(), c
+    finally:
+        binding.set_kernel_override(None)
+
+
+@pytest.mark.parametrize("tA", [False, True])
+@pytest.mark.parametrize("shape", [(1, 10, 256), (64, 10, 256), (33, 31, 7), (3, 5, 291)])
+def test_tiny_gemm(binding, shape, tA):
+    M, N, K = shape
+    rng = np.random.default_rng(K)
+    for tB in (False, True):
+        A = rng.standard_normal((K, M) if tA else (M, K)).astype(np.float32)
+        B = rng.standard_normal((N, K) if tB else (K, N)).astype(np.float32)
+        C = rng.standard_normal((N,)).astype(np.float32)
+        got = run_gemm_gpu(binding, torch, A, B, C, transA=tA, transB=tB)
+        want, S = oracle.gemm(A, B, C, transA=tA, transB=tB)
+        assert (np.abs(got - want) <= REL * S + 1e-6).all()
+
+
+def test_split_operands_that_overflow(binding, monkeypatch):
+    """Infinite, NaN and near-overflow operands have no hi/lo split: the outputs they reach are summed in
+    plain fp32 and come out as an fp32 sum gives them."""
+    monkeypatch.setenv("ONNXB_FP32", "tc")
+    rng = np.random.default_rng(8)
+    A = rng.standard_normal((70, 75)).astype(np.float32)
+    B = rng.standard_normal((75, 131)).astype(np.float32)
+    A[3, 5], A[60, 7], A[20, 1] = np.inf, np.nan, 3.40282e38
+    B[1, :] = 1e-3
+    got = run_gemm_gpu(binding, torch, A, B, None)
+    with np.errstate(all="ignore"):
+        want = A.astype(np.float64) @ B.astype(np.float64)
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
+    ok = np.isfinite(want)
+    assert np.allclose(got[ok], want[ok], rtol=1e-5, atol=1e-4)
