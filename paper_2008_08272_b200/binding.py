@@ -4,6 +4,9 @@ Argument marshalling only: every step of Conv and Gemm runs in the library's
 CUDA kernels.  Tensors are torch CUDA tensors used as device memory; the current
 torch stream is passed through.  There is no CPU fallback: if the compiled
 library is missing, or a tensor is not on a CUDA device, the call raises.
+
+The operator calls go through ``ext/fast_binding.cpp``, which does the marshalling below natively; a call it
+declines (returning None, nothing launched) is repeated here, where every check raises its own error.
 """
 from __future__ import annotations
 
@@ -49,6 +52,24 @@ class ConvAttrs(ctypes.Structure):
 
 
 _lib = None
+_fast_mod = None
+
+
+def _fast():
+    """The native call path, loaded with the first operator call (it needs torch's C++ libraries)."""
+    global _fast_mod
+    if _fast_mod is None:
+        import importlib.util
+        import torch  # noqa: F401  (its libraries must be loaded first)
+        load()
+        if not os.path.exists(_build.EXT_PATH):
+            _build.build_ext()
+        spec = importlib.util.spec_from_file_location("_onnxb_fast", _build.EXT_PATH)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        mod.bind(_build.LIB_PATH)
+        _fast_mod = mod
+    return _fast_mod
 
 
 def library_path() -> str:
@@ -178,9 +199,24 @@ class Conv2dDesc:
         self.pads = tuple(int(v) for v in p)
         self.workspace_bytes = int(ws.value)
         self.kernel_family = KERNEL_FAMILIES[self._lib.onnx_conv2d_desc_query_kernel(self._h)]
+        self._prepacked_needs_ws = bool(
+            (self.kernel_family not in WEIGHT_COPY_FAMILIES or self.kernel_family == "mma_gather_gemm")
+            and self.workspace_bytes)
+        self._plan = None
+
+    def _native(self, X, W, packed, B, R, Y, workspace, stream):
+        """The call through the native path; None when it declined."""
+        if self._plan is None:
+            if not self._h:
+                return None
+            self._plan = _fast().plan(self._h.value, self.y_shape, self.workspace_bytes, self._prepacked_needs_ws)
+        return _fast_mod.conv(self._plan, X, W, packed, B, R, Y, workspace, stream)
 
     def run(self, X, W, B=None, Y=None, workspace=None, stream=None):
         """``onnx_conv2d_run``; allocates Y (and a workspace) with torch when not supplied."""
+        y = self._native(X, W, None, B, None, Y, workspace, stream)
+        if y is not None:
+            return y
         import torch
         if Y is None:
             Y = torch.empty(self.y_shape, dtype=torch.float32, device=X.device)
@@ -195,6 +231,10 @@ class Conv2dDesc:
 
     def run_add(self, X, W, B, R, Y=None, workspace=None, stream=None):
         """``onnx_conv2d_add_run``: Y = relu?(Conv(X, W) + B + R), R shaped like Y (a residual connection)."""
+        if R is not None:
+            y = self._native(X, W, None, B, R, Y, workspace, stream)
+            if y is not None:
+                return y
         import torch
         if Y is None:
             Y = torch.empty(self.y_shape, dtype=torch.float32, device=X.device)
@@ -219,12 +259,14 @@ class Conv2dDesc:
 
     def run_prepacked(self, X, W, packed, B=None, R=None, Y=None, workspace=None, stream=None):
         """``onnx_conv2d_run_prepacked``: run (R None) or run_add (R given) from a packed copy of W."""
+        if packed is not None:
+            y = self._native(X, W, packed, B, R, Y, workspace, stream)
+            if y is not None:
+                return y
         import torch
         if Y is None:
             Y = torch.empty(self.y_shape, dtype=torch.float32, device=X.device)
-        needs_ws = (self.kernel_family not in WEIGHT_COPY_FAMILIES or self.kernel_family == "mma_gather_gemm") \
-            and self.workspace_bytes
-        if workspace is None and needs_ws:
+        if workspace is None and self._prepacked_needs_ws:
             workspace = torch.empty(self.workspace_bytes, dtype=torch.uint8, device=X.device)
         ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
         ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
@@ -248,6 +290,7 @@ class Conv2dDesc:
         return Y
 
     def close(self):
+        self._plan = None
         if self._h:
             self._lib.onnx_conv2d_desc_destroy(self._h)
             self._h = ctypes.c_void_p()
@@ -278,6 +321,9 @@ def gemm_workspace_bytes(transA, transB, M, N, K) -> int:
 def onnx_gemm(A, B, C=None, *, alpha=1.0, beta=1.0, transA=False, transB=False, fuse_relu=False,
               Y=None, workspace=None, stream=None):
     """``onnx_gemm_run``: Y = relu?(alpha * A' @ B' + beta * C)."""
+    y = (_fast_mod or _fast()).gemm(A, B, C, alpha, beta, transA, transB, fuse_relu, Y, workspace, stream)
+    if y is not None:
+        return y
     import torch
     lib = load()
     M, K = (A.shape[1], A.shape[0]) if transA else (A.shape[0], A.shape[1])
@@ -338,6 +384,10 @@ def probe_wait_timeout(limit_cycles: int = 1000000, stream=None) -> None:
 
 def onnx_matmul_add(A, B, C=None, *, fuse_relu=False, Y=None, workspace=None, stream=None):
     """``onnx_matmul_add_run``: Y = relu?(A @ B + C), the MatMul + Add pair as one fused Gemm."""
+    # (exactly onnx_gemm_run with transA = transB = 0 and alpha = beta = 1)
+    y = (_fast_mod or _fast()).gemm(A, B, C, 1.0, 1.0, False, False, fuse_relu, Y, workspace, stream)
+    if y is not None:
+        return y
     import torch
     lib = load()
     M, K = A.shape
@@ -377,6 +427,9 @@ def maxpool2d_shape(x_shape, kernel_shape, pads=None, strides=None):
 
 def onnx_maxpool2d(X, kernel_shape, *, pads=None, strides=None, Y=None, stream=None):
     """``onnx_maxpool2d_run``: ONNX MaxPool (2-D, NCHW, dilation 1, ceil_mode 0)."""
+    y = (_fast_mod or _fast()).maxpool(X, kernel_shape, pads, strides, Y, stream)
+    if y is not None:
+        return y
     import torch
     y_shape = maxpool2d_shape(tuple(X.shape), kernel_shape, pads, strides)
     if Y is None:
@@ -388,6 +441,9 @@ def onnx_maxpool2d(X, kernel_shape, *, pads=None, strides=None, Y=None, stream=N
 
 def onnx_global_average_pool(X, *, Y=None, stream=None):
     """``onnx_global_average_pool_run``: Y[n,c,0,0] = mean of X[n,c,:,:]."""
+    y = (_fast_mod or _fast()).gap(X, Y, stream)
+    if y is not None:
+        return y
     import torch
     if Y is None:
         Y = torch.empty((X.shape[0], X.shape[1], 1, 1), dtype=torch.float32, device=X.device)

@@ -1,4 +1,4 @@
-"""Builds libonnx_b200.so in-tree with nvcc for sm_100a.
+"""Builds libonnx_b200.so in-tree with nvcc for sm_100a, and the binding's native call path with g++.
 
 Usage: ``python -m paper_2008_08272_b200.build [--force] [--verbose]``.
 """
@@ -15,6 +15,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB_DIR = os.path.join(HERE, "_lib")
 LIB_PATH = os.path.join(LIB_DIR, "libonnx_b200.so")
+EXT_SRC = os.path.join(HERE, "ext", "fast_binding.cpp")
+EXT_PATH = os.path.join(LIB_DIR, "_onnxb_fast.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -38,8 +40,35 @@ def is_stale() -> bool:
     return any(os.path.getmtime(f) > t for f in _inputs())
 
 
+def build_ext(force: bool = False, verbose: bool = False) -> str:
+    """Compile the binding's native call path (a CPython extension on torch's C++ tensors)."""
+    import sysconfig
+    deps = [EXT_SRC, os.path.join(ROOT, "include", "onnx_b200.h")]
+    if not force and os.path.exists(EXT_PATH) and all(os.path.getmtime(EXT_PATH) >= os.path.getmtime(f) for f in deps):
+        return EXT_PATH
+    import torch
+    tdir = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    os.makedirs(LIB_DIR, exist_ok=True)
+    tmp = EXT_PATH + ".%d.tmp" % os.getpid()
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-I" + os.path.join(ROOT, "include"), "-I" + os.path.join(tdir, "include"),
+           "-I" + os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
+           "-I" + os.path.join(cuda, "include"), "-I" + sysconfig.get_paths()["include"], EXT_SRC, "-o", tmp,
+           "-L" + os.path.join(tdir, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-ldl"]
+    proc = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    if verbose or proc.returncode != 0:
+        sys.stderr.write(proc.stdout)
+    if proc.returncode != 0:
+        raise RuntimeError("g++ failed building _onnxb_fast.so")
+    os.replace(tmp, EXT_PATH)
+    return EXT_PATH
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every CUDA source of the library into one shared object."""
+    """Compile every CUDA source of the library into one shared object, and the binding's native call path."""
+    build_ext(force, verbose)
     if not force and not is_stale():
         return LIB_PATH
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"

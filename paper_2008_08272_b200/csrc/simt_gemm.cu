@@ -402,7 +402,7 @@ struct Pick {
     int shape, split;
     double cost;
 };
-Pick pick_shape(int M, int N, int K, int groups, bool pixels) {
+Pick search_shape(int M, int N, int K, int groups, bool pixels) {
     Pick best{-1, 1, 0};
     const long long ktiles = (K + kBK - 1) / kBK;
     int ps = -1, pk = 1;       // ONNXB_FP32 = "shape,split" pins both
@@ -427,6 +427,28 @@ Pick pick_shape(int M, int N, int K, int groups, bool pixels) {
         }
     }
     return best;
+}
+
+// What a launch is: a tile shape and split, or the tensor-core kernel.  The search costs about 2 us of host
+// time, as much as the launch itself, so each thread remembers the choices of the last few problems.
+struct Choice {
+    int M, N, K, groups, pixels;
+    Pick pick;
+    bool tc;
+};
+bool fp32_on_tensor_cores(double fma_cost, double tc_cost);
+Choice choose(int M, int N, int K, int groups, bool pixels) {
+    thread_local Choice memo[64] = {};
+    const bool pinned = getenv("ONNXB_FP32") != nullptr;
+    const unsigned h = ((unsigned)M * 2654435761u ^ (unsigned)N * 2246822519u ^ (unsigned)K * 3266489917u ^ (unsigned)groups * 668265263u ^
+                        (unsigned)pixels) >> 7;
+    Choice &c = memo[h % 64];
+    if (!pinned && c.M == M && c.N == N && c.K == K && c.groups == groups && c.pixels == (int)pixels) return c;
+    Choice r{M, N, K, groups, (int)pixels, search_shape(M, N, K, groups, pixels), false};
+    // (rows and columns change places there: its rows are the index contiguous in Y)
+    r.tc = fp32_on_tensor_cores(r.pick.cost, tc_fp32_cost(N, M, K, groups, pixels));
+    if (!pinned) c = r;
+    return r;
 }
 
 // Large problems go to the split-TF32 tensor-core kernel, by the two estimates; ONNXB_FP32 = "tc" pins it.
@@ -474,8 +496,9 @@ int launch_simt_gemm(const GemmProblem &p, const float *A, const float *B, const
         count_launch();
         return (int)e;
     }
-    const Pick pick = pick_shape(a.M, a.N, a.K, 1, false);
-    if (fp32_on_tensor_cores(pick.cost, tc_fp32_cost(p.N, p.M, p.K, 1, false))) return launch_tc_fp32_gemm(p, A, B, C, Y, stream);
+    const Choice ch = choose(a.M, a.N, a.K, 1, false);
+    const Pick pick = ch.pick;
+    if (ch.tc) return launch_tc_fp32_gemm(p, A, B, C, Y, stream);
     if (p.transA)
         return p.transB ? launch_sgemm<kMnContig, kKContig>(a, 1, pick, st) : launch_sgemm<kMnContig, kMnContig>(a, 1, pick, st);
     return p.transB ? launch_sgemm<kKContig, kKContig>(a, 1, pick, st) : launch_sgemm<kKContig, kMnContig>(a, 1, pick, st);
@@ -493,9 +516,9 @@ int launch_simt_conv(const ConvGeom &g, const float *X, const float *W, const fl
     a.sh = g.sh; a.sw = g.sw; a.dh = g.dh; a.dw = g.dw; a.pt = g.pt; a.pl = g.pl;
     a.taps = g.kH * g.kW; a.kW = g.kW; a.Mtot = g.M;
     a.dv_PQ = conv_divisor(a.PQ); a.dv_Q = conv_divisor(a.Q); a.dv_taps = conv_divisor(a.taps); a.dv_kW = conv_divisor(a.kW);
-    const Pick pick = pick_shape(a.M, a.N, a.K, g.group, true);
-    if (a.taps <= 64 && fp32_on_tensor_cores(pick.cost, tc_fp32_cost(a.N, a.M, a.K, g.group, true)))
-        return launch_tc_fp32_conv(g, X, W, B, R, Y, stream);
+    const Choice ch = choose(a.M, a.N, a.K, g.group, true);
+    const Pick pick = ch.pick;
+    if (ch.tc && a.taps <= 64) return launch_tc_fp32_conv(g, X, W, B, R, Y, stream);
     return launch_sgemm<kKContig, kPixels>(a, g.group, pick, (cudaStream_t)stream);
 }
 
