@@ -288,7 +288,7 @@ extern "C" onnxb_status onnx_gemm_run(int transA, int transB, float alpha, float
     t.a_mn_major = p.transA; t.a_ld = p.transA ? p.M : p.K;
     t.b_mn_major = !p.transB; t.b_ld = p.transB ? p.K : p.N;
     t.alpha = alpha; t.beta = beta; t.C = C; t.c_si = p.c_stride_i; t.c_sj = p.c_stride_j; t.c_sb = 0;
-    t.row_bias = nullptr; t.relu = p.relu;
+    t.row_bias = nullptr; t.relu = p.relu; t.round_operands = 1;
     t.Y = Y; t.y_ld = p.N; t.y_bs = 0;
     const int forced = kernel_override();
     const bool forced_tc = forced == ONNXB_KERNEL_MMA_GEMM || forced == ONNXB_KERNEL_MMA_IMPLICIT;
@@ -298,12 +298,12 @@ extern "C" onnxb_status onnx_gemm_run(int transA, int transB, float alpha, float
         const size_t need = onnx_gemm_workspace_bytes(transA, transB, M, N, K);
         if (!workspace || workspace_bytes < need) return ONNXB_ERR_WORKSPACE;
         if (tc_gemm_splitk_fits(t)) {
-            // few tiles and a long reduction: the split-K kernel rounds its operands itself
+            // few tiles: the split-K kernel rounds its operands itself
             err = launch_tc_gemm(t, cuda_stream);
         } else {
             float *Ar = static_cast<float *>(workspace), *Br = Ar + M * K;
             err = launch_round_tf32_copy(A, Ar, M * K, B, Br, K * N, cuda_stream);
-            t.A = Ar; t.B = Br;
+            t.A = Ar; t.B = Br; t.round_operands = 0;
             if (err == 0) err = launch_tc_gemm(t, cuda_stream);
         }
     } else if (forced_tc) {

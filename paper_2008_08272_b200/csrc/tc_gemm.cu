@@ -608,6 +608,26 @@ static int gemm_max_pairs() {
     return n;
 }
 
+// CTA pairs when the rows fill 256-row tiles: each CTA then fetches half of B.  That is what the
+// layers bound by the L2 -> shared-memory stream (small images, many channels) need: measured 7-15 %
+// faster on the 14x14 and strided 1x1 layers of ResNet-50, neutral on the HBM-bound ones.
+static bool gemm_pairs(const TcGemmProblem &g) {
+    if (const char *e = getenv("ONNXB_GEMM_PAIR"))          // "0"/"1": pin the choice for A/B measurements
+        if (e[0] == '0' || e[0] == '1') return e[0] == '1' && g.M > 128 && g.N >= 64;
+    return g.M >= 256 && (g.M % 256 == 0 || g.M % 256 > 128) && g.N >= 64;
+}
+
+// Fitted together with the split-K form's estimate (see there); includes ONNX Gemm's rounding pre-pass.
+double tc_gemm_estimate_ns(const TcGemmProblem &g) {
+    const int ctas = gemm_pairs(g) ? 2 : 1, units = ctas == 2 ? gemm_max_pairs() : tc_host::num_sms();
+    const long long tiles_m = (g.M + kBM * ctas - 1) / (kBM * ctas);
+    const int bn = pick_bn(tiles_m, g.N, g.batch, units, ctas);
+    const long long tiles = tiles_m * ((g.N + bn - 1) / bn) * g.batch;
+    const double waves = (double)((tiles + units - 1) / units);
+    const double t = waves * ((g.K + kBK - 1) / kBK * (189.0 + 1.45 * bn / ctas + (ctas == 2 ? 45.0 : 0.0)) + 11.0 * bn) + 3270.0;
+    return t + (g.round_operands ? 2360.0 + 166e-6 * 4.0 * ((double)g.M * g.K + (double)g.K * g.N) : 0.0);
+}
+
 int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     using namespace tc_host;
     if (tc_gemm_splitk_fits(g)) return launch_tc_gemm_splitk(g, stream);      // few tiles, long reduction
@@ -616,16 +636,7 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     p.a_mn = g.a_mn_major; p.b_mn = g.b_mn_major;
     p.a_batched = g.a_batched && g.batch > 1; p.b_batched = g.b_batched && g.batch > 1;
     const int sms = num_sms();
-    // CTA pairs when the rows fill 256-row tiles: each CTA then fetches half of B.  That is what the
-    // layers bound by the L2 -> shared-memory stream (small images, many channels) need: measured 7-15 %
-    // faster on the 14x14 and strided 1x1 layers of ResNet-50, neutral on the HBM-bound ones.
-    p.ctas = 1;
-    {
-        const char *e = getenv("ONNXB_GEMM_PAIR");          // "0"/"1": pin the choice for A/B measurements
-        bool pair = g.M >= 256 && (g.M % 256 == 0 || g.M % 256 > 128) && g.N >= 64;
-        if (e && (e[0] == '0' || e[0] == '1')) pair = e[0] == '1' && g.M > 128 && g.N >= 64;
-        if (pair) p.ctas = 2;
-    }
+    p.ctas = gemm_pairs(g) ? 2 : 1;
     const int units = p.ctas == 2 ? gemm_max_pairs() : sms;
     p.tiles_m = (g.M + kBM * p.ctas - 1) / (kBM * p.ctas);
     p.BN = pick_bn(p.tiles_m, g.N, g.batch, units, p.ctas);

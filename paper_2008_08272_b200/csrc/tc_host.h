@@ -23,6 +23,7 @@ struct TcGemmProblem {
     const float *row_bias;
     const float *residual;   // optional addend with Y's own layout, added before Relu (ignored when C is given)
     int relu;
+    int round_operands;      // A and B are raw fp32: the split-K form rounds them itself, the other form is given copies
     float *Y;
     long long y_ld, y_bs;
     // When y_split > 0 the N columns are `y_split`-wide groups laid y_group_stride elements apart in Y
@@ -34,7 +35,8 @@ struct TcGemmProblem {
 
 bool tc_gemm_supports(const TcGemmProblem &g);
 int launch_tc_gemm(const TcGemmProblem &g, void *stream);
-// Split-K form for small M and a long reduction (tc_gemm_splitk.cu); launch_tc_gemm uses it where it fits.
+// Split-K form for few output tiles (tc_gemm_splitk.cu); launch_tc_gemm uses it where it fits.
+double tc_gemm_estimate_ns(const TcGemmProblem &g);       // the persistent kernel's estimated time
 bool tc_gemm_splitk_fits(const TcGemmProblem &g);
 int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream);
 
