@@ -110,6 +110,12 @@ __global__ void pack_weights_kernel(const TcConvPlan g, const float *__restrict_
     }
 }
 
+__device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
+
 // Channel blocks are summed in a rotated order that differs from tile to tile: CTAs working at the
 // same time then stream different parts of the (shared) packed weights, instead of all asking the
 // same L2 lines at the same moment.
@@ -119,7 +125,11 @@ __device__ __forceinline__ int cb_rotation(long long tile, int ncb) { return (in
 // kAdd: the epilogue also adds a tensor laid out like Y (a residual connection) before the Relu.  A
 // separate instantiation, so that the plain kernel's register allocation is not disturbed.
 // kEpiWarps: 8 or 4 epilogue warps (see the thread layout above).
-template <int kCtas, bool kAdd, int kEpiWarps>
+// kSplit: the problem has few tiles, so a cluster of g.split CTAs shares one: CTA r reduces the channel blocks
+// [r * cb_per, (r + 1) * cb_per), parks its partial tile in shared memory (over the stages, which are done with),
+// and after a cluster barrier sums one slice of the tile's channels over all partials through distributed
+// shared memory, in rank order.  One 14x14 image, 256 -> 256 channels: 24 -> 8 us.
+template <int kCtas, bool kAdd, int kEpiWarps, bool kSplit>
 __global__ void __launch_bounds__(threads_for(kEpiWarps), 1)
 tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, const float *__restrict__ X,
                const float *__restrict__ Wpk, const float *__restrict__ bias, const float *__restrict__ R,
@@ -139,7 +149,10 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
     const int tile_rows = g.MT * 128;
     // CTA pair: rank within the cluster, and the tiles this CTA (pair) walks
     const uint32_t rank = kCtas == 2 ? cluster_ctarank() : 0u;
-    const long long first_tile = blockIdx.x / kCtas, tile_step = gridDim.x / kCtas;
+    const int per_tile = kSplit ? g.split : kCtas;             // CTAs working on one tile
+    const long long first_tile = blockIdx.x / per_tile, tile_step = gridDim.x / per_tile;
+    const int cb_lo = kSplit ? (int)cluster_ctarank() * g.cb_per : 0;                  // channel blocks of this CTA
+    const int cb_cnt = kSplit ? min(g.ncb - cb_lo, g.cb_per) : g.ncb;
     const int cgt = g.ctiles * g.group;        // channel tiles over all groups
     // accumulator placement in TMEM: two alternating sets when one set fits in 256 columns
     const bool acc_dbl = g.MT == 1 || g.BN <= 128;
@@ -191,7 +204,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             uint32_t rphase = 0, tile_it = 0;
             const long long HW = (long long)g.H * g.W;
             const long long planes_total = (long long)g.N * g.C;
-            const int KB = g.KB, ncb = g.ncb, box_floats = g.KB * g.BOXP;
+            const int KB = g.KB, ncb = cb_cnt, box_floats = g.KB * g.BOXP;
             for (long long t = first_tile; t < g.total_tiles; t += tile_step) {
                 const int ct_all = (int)(t % cgt);
                 const int grp = ct_all / g.ctiles;
@@ -211,12 +224,12 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                 }
                 const int nseg = segs->nseg;
                 const uint32_t tile_bytes = (uint32_t)segs->total_floats * 4u;
-                const int rot = cb_rotation(t, ncb);
+                const int rot = kSplit ? cb_lo : cb_rotation(t, ncb);
                 for (int cb = 0; cb < ncb; ++cb) {
                     mbar_wait(&bars->raw_empty[rs], rphase ^ 1, err, 11);
                     LOG(0, cb);
                     float *dst = reinterpret_cast<float *>(raw_st + (size_t)rs * g.raw_stage_bytes);
-                    const int cbx = cb + rot < ncb ? cb + rot : cb + rot - ncb;
+                    const int cbx = kSplit || cb + rot < ncb ? cb + rot : cb + rot - ncb;
                     const int c0 = grp * g.Cg + cbx * KB;
                     if (g.raw_mode == 0) {
                         mbar_arrive_expect_tx(&bars->raw_full[rs], tile_bytes);
@@ -257,15 +270,15 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             int bs = 0;
             uint32_t bphase = 0;
             const long long per_ct = (long long)g.ncb * g.n_steps * g.b_step_bytes;   // bytes per channel tile and CTA
-            const int nb = g.nb_stages, ncb = g.ncb, b_steps = g.b_steps, spb = g.spb, n_steps = g.n_steps;
+            const int nb = g.nb_stages, ncb = cb_cnt, b_steps = g.b_steps, spb = g.spb, n_steps = g.n_steps;
             const uint32_t stage_bytes = (uint32_t)g.b_stage_bytes, step_bytes = (uint32_t)g.b_step_bytes;
             pdl_wait();             // the packed weights may come from the kernel just before this one
             for (long long t = first_tile; t < g.total_tiles; t += tile_step) {
                 const int ct_all = (int)(t % cgt);
                 const uint8_t *tile_src = reinterpret_cast<const uint8_t *>(Wpk) + (ct_all * kCtas + (int)rank) * per_ct;
-                const int rot = cb_rotation(t, ncb);
+                const int rot = kSplit ? cb_lo : cb_rotation(t, ncb);
                 for (int cb = 0; cb < ncb; ++cb) {
-                    const int cbx = cb + rot < ncb ? cb + rot : cb + rot - ncb;
+                    const int cbx = kSplit || cb + rot < ncb ? cb + rot : cb + rot - ncb;
                     const uint8_t *src = tile_src + (long long)cbx * n_steps * step_bytes;
                     for (int bstep = 0; bstep < b_steps; ++bstep) {
                         const uint32_t bytes = (uint32_t)min(spb, n_steps - bstep * spb) * step_bytes;
@@ -308,7 +321,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             const uint32_t a_stage16 = (uint32_t)g.a_stage_bytes >> 4, b_stage16 = (uint32_t)g.b_stage_bytes >> 4;
             const uint32_t b_step16 = (uint32_t)g.b_step_bytes >> 4;
             const uint32_t idesc = g.idesc;
-            const int n_steps = g.n_steps, ncb = g.ncb, nb = g.nb_stages, spb = g.spb, b_steps = g.b_steps;
+            const int n_steps = g.n_steps, ncb = cb_cnt, nb = g.nb_stages, spb = g.spb, b_steps = g.b_steps;
             const bool two = g.MT == 2;
             int as = 0, bs = 0;
             uint32_t aphase = 0, bphase = 0, it = 0;
@@ -398,7 +411,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
         const int xt = xw * 32 + lane;             // 0..255
         const int cp = g.raw_mode == 1 ? g.H * g.W : g.BOXP;    // channel pitch inside the raw stage
         const int per_stage_slots = g.planes * g.SLOTS;
-        const int nchunks = g.nchunks, KB = g.KB, ncb = g.ncb, box_floats = g.KB * g.BOXP, nr = g.nr_stages;
+        const int nchunks = g.nchunks, KB = g.KB, ncb = cb_cnt, box_floats = g.KB * g.BOXP, nr = g.nr_stages;
         // Work units: one (slot, 4-channel chunk) pair = four raw reads and one 16-byte operand row.
         // Unit u = chunk * slots + slot; this thread owns units xt, xt + 256, ...
         const int units = per_stage_slots * nchunks;
@@ -433,7 +446,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
         for (long long t = first_tile; t < g.total_tiles; t += tile_step) {
             const long long G0 = ((t / cgt) * kCtas + rank) * tile_rows;
             int uoff[kOwned];                      // raw float offset of the unit's first channel, -1 = padding
-            const int rot = cb_rotation(t, ncb);
+            const int rot = kSplit ? cb_lo : cb_rotation(t, ncb);
             {
                 // per-thread offsets of the tile, from its segment table (ready before the data)
                 const uint32_t sp = tile_it & 1u;
@@ -522,7 +535,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                 if (xt == 0) LOG(6, cb);
                 const float *raw = reinterpret_cast<const float *>(raw_st + (size_t)rs * g.raw_stage_bytes);
                 uint8_t *adst = a_st + (size_t)as * g.a_stage_bytes;
-                const int cbx = cb + rot < ncb ? cb + rot : cb + rot - ncb;
+                const int cbx = kSplit || cb + rot < ncb ? cb + rot : cb + rot - ncb;
                 const int c_left = g.Cg - cbx * KB;    // channels of this block that exist
                 // In two batches of five units: all reads of a batch first (independent, so their latencies
                 // overlap), then round and store; channels past the end of the group (last block only)
@@ -590,8 +603,22 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             if (it == 0) pdl_wait();        // long since satisfied: the producers passed theirs before the first load
             if (ew == 0 && lane == 0) LOG(8, 2);
             const int nch = (g.BN + 31) / 32;
+            if (kSplit) {
+                // park the partial tile as [channel][row]: lanes write consecutive rows
+                float *part = reinterpret_cast<float *>(smem);
+                const int pitch = tile_rows + 4, mt = two ? ew >> 2 : 0;
+                const int row = mt * 128 + quarter * 32 + lane;
+                for (int chunk = two ? 0 : ew >> 2; chunk < nch; chunk += two ? 1 : 2) {
+                    uint32_t v[32];
+                    tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + ab * 256u + (uint32_t)mt * mt_cols + (uint32_t)(chunk * 32), v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (chunk * 32 + j < g.BN) part[(chunk * 32 + j) * pitch + row] = __uint_as_float(v[j]);
+                }
+            }
             // eight warps: two per TMEM lane quarter, each taking half of the tile; four: one per quarter, both halves
-            for (int hf = ew >> 2; hf < 2; hf += kEpiWarps / 4) {
+            for (int hf = ew >> 2; hf < 2 && !kSplit; hf += kEpiWarps / 4) {
             int mt, ch_lo, ch_hi;
             if (two) { mt = hf; ch_lo = 0; ch_hi = nch; }
             else { mt = 0; ch_lo = hf ? (nch + 1) / 2 : 0; ch_hi = hf ? nch : (nch + 1) / 2; }
@@ -638,7 +665,40 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
 
     tc_fence_before_sync();
     __syncthreads();
-    if (kCtas == 2) cluster_sync_all();     // no CTA leaves while its peer may still signal it
+    if (kSplit) {
+        cluster_sync_all();                 // every CTA's partial tile is in its shared memory
+        const int rows = tile_rows, pitch = tile_rows + 4, nthr = 512, tid = threadIdx.x;
+        const int cols_per = (g.BN + g.split - 1) / g.split, col_lo = (int)cluster_ctarank() * cols_per;
+        const int ct_all = (int)(first_tile % cgt), grp = ct_all / g.ctiles, ct = ct_all % g.ctiles;
+        const int col_hi = min(min(g.BN, col_lo + cols_per), g.Mg - ct * g.BN);
+        const int row = tid % rows;         // lanes along pixels
+        const uint32_t G = (uint32_t)((first_tile / cgt) * tile_rows) + (uint32_t)row;
+        if (tid < nthr && G < (uint32_t)g.total_slots) {
+            pdl_wait();                     // long since satisfied
+            const int n = conv_fdiv((int)G, g.L, g.dv_L), u = (int)G - n * g.L;
+            const int p = conv_fdiv(u, g.Ws, g.dv_Ws), q = u - p * g.Ws;
+            if (p < g.P && q < g.Q) {
+                const long long PQ = (long long)g.P * g.Q;
+                const uint32_t part_addr = smem_u32(smem);
+                for (int col = col_lo + tid / rows; col < col_hi; col += nthr / rows) {
+                    const int m = grp * g.Mg + ct * g.BN + col;
+                    const long long yi = ((long long)n * g.M + m) * PQ + (long long)p * g.Q + q;
+                    const float b = bias ? __ldg(bias + m) : 0.f, r = kAdd ? __ldg(R + yi) : 0.f;
+                    float x = 0.f;
+                    for (int sp = 0; sp < g.split; sp += 2) {
+                        const uint32_t off = part_addr + (uint32_t)(col * pitch + row) * 4u;
+                        const float x0 = ld_cluster_f32(map_to_cta(off, (uint32_t)sp)), x1 = ld_cluster_f32(map_to_cta(off, (uint32_t)sp + 1u));
+                        x = (x + x0) + x1;
+                    }
+                    x += b;
+                    if (kAdd) x += r;
+                    if (g.relu) x = fmaxf(x, 0.f);
+                    Y[yi] = x;
+                }
+            }
+        }
+    }
+    if (kCtas == 2 || kSplit) cluster_sync_all();     // no CTA leaves while a peer may still signal it or read its partial tile
     if (threadIdx.x == 0) LOG(8, 4);
     if (warp == 2) {
         __syncwarp();
@@ -695,6 +755,8 @@ int pick_conv_bn(int Mg) {
 bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &g) {
     if (ctas == 2 && BN % 16) return false;      // M = 256 instructions take N in multiples of 16
     g.ctas = ctas;
+    g.split = 1;
+    g.cb_per = 0;
     g.BNH = BN / ctas;
     g.N = c.N; g.C = c.C; g.H = c.H; g.W = c.W; g.M = c.M; g.Cg = c.Cg; g.Mg = c.Mg;
     g.kH = c.kH; g.kW = c.kW; g.P = c.P; g.Q = c.Q; g.pt = c.pt; g.pl = c.pl;
@@ -893,6 +955,38 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     return true;
 }
 
+// Cost in SM cycles per CTA, fitted to measured tile sweeps of the ResNet-50 3x3 layers.  Per channel block the
+// slowest of: the tensor pipe (BN/2 cycles per 128 x BN x 8 share of an instruction, or the 128 bytes/cycle of
+// shared memory its operands need, whichever is longer), shared memory as a whole (operand reads plus the
+// stages written and the transform, at about 90 bytes/cycle sustained), the weight stream out of L2 (about 3600
+// bytes/cycle over all SMs, at most 48 per SM) and the transform warps; plus a fixed hand-over cost per block,
+// larger for pairs (their barriers cross the cluster).  split: CTAs sharing a tile's channel blocks.
+double tile_cost(const TcConvPlan &p, int split) {
+    const int sms = 148;
+    const int units = sms / p.ctas / split;                             // tiles in flight
+    const long long waves = (p.total_tiles + units - 1) / units;
+    const double active = (double)std::min<long long>(p.total_tiles, units) * p.ctas * split;
+    const double n_inst = (double)p.n_steps * p.MT;
+    const double op_bytes = 4096.0 + p.BNH * 32.0;
+    const double t_mma = n_inst * (std::max(p.BN / 2.0, op_bytes / 128.0) + (p.ctas == 2 ? 10.0 : 0.0));
+    const double w_bytes = (double)p.n_steps * p.b_step_bytes;
+    const double slots16 = (double)p.planes * p.SLOTS * 16.0 * p.nchunks;
+    const double t_smem = (n_inst * op_bytes + w_bytes + 3.0 * slots16) / 90.0;
+    // the weight ring must also cover the latency of its copies (about 2500 cycles from issue to
+    // landing under load): a ring holding less than that much of the stream paces the block
+    const double ring = (double)p.nb_stages * p.b_stage_bytes;
+    const double t_w = std::max(w_bytes / std::min(48.0, 3600.0 / active), w_bytes * 2500.0 / ring);
+    const double t_x = 300.0 + 100.0 * ((p.planes * p.SLOTS * p.nchunks + 255) / 256);
+    // (three operand stages hide most of the hand-over)
+    const double per_cb = std::max(std::max(t_mma, t_smem), std::max(t_w, t_x)) +
+                          (p.na_stages == 3 ? 300.0 : 400.0 + (p.ctas == 2 ? 700.0 : 0.0));
+    const bool dbl = p.MT == 1 || p.BN <= 128;
+    const double t_epi = 8.0 * p.MT * p.BN;                             // read-back and stores of one tile
+    if (split > 1) return (double)waves * ((p.ncb + split - 1) / split * per_cb + t_epi + 8000.0) + 9000.0;
+    const double per_tile = (dbl ? std::max(p.ncb * per_cb, t_epi) : p.ncb * per_cb + t_epi) + 3000.0;
+    return (double)waves * per_tile + 9000.0 + (dbl ? t_epi : 0.0);
+}
+
 }  // namespace
 
 bool tc_conv_plan(const ConvGeom &c, TcConvPlan &plan, bool forced) {
@@ -933,34 +1027,7 @@ bool tc_conv_plan(const ConvGeom &c, TcConvPlan &plan, bool forced) {
     for (int i = 0; i < ncand; ++i) {
         TcConvPlan p;
         if (!fill_plan(c, cand[i][0], cand[i][1], cand[i][2], cand[i][3], p)) continue;
-        // Cost in SM cycles per CTA, fitted to measured tile sweeps of the ResNet-50 3x3 layers.  Per
-        // channel block the slowest of: the tensor pipe (BN/2 cycles per 128 x BN x 8 share of an
-        // instruction, or the 128 bytes/cycle of shared memory its operands need, whichever is longer),
-        // shared memory as a whole (operand reads plus the stages written and the transform, at about
-        // 90 bytes/cycle sustained), the weight stream out of L2 (about 3600 bytes/cycle over all SMs, at
-        // most 48 per SM) and the transform warps; plus a fixed hand-over cost per block, larger for
-        // pairs (their barriers cross the cluster).
-        const int units = sms / p.ctas;                                     // tiles in flight
-        const long long waves = (p.total_tiles + units - 1) / units;
-        const double active = (double)std::min<long long>(p.total_tiles, units) * p.ctas;
-        const double n_inst = (double)p.n_steps * p.MT;
-        const double op_bytes = 4096.0 + p.BNH * 32.0;
-        const double t_mma = n_inst * (std::max(p.BN / 2.0, op_bytes / 128.0) + (p.ctas == 2 ? 10.0 : 0.0));
-        const double w_bytes = (double)p.n_steps * p.b_step_bytes;
-        const double slots16 = (double)p.planes * p.SLOTS * 16.0 * p.nchunks;
-        const double t_smem = (n_inst * op_bytes + w_bytes + 3.0 * slots16) / 90.0;
-        // the weight ring must also cover the latency of its copies (about 2500 cycles from issue to
-        // landing under load): a ring holding less than that much of the stream paces the block
-        const double ring = (double)p.nb_stages * p.b_stage_bytes;
-        const double t_w = std::max(w_bytes / std::min(48.0, 3600.0 / active), w_bytes * 2500.0 / ring);
-        const double t_x = 300.0 + 100.0 * ((p.planes * p.SLOTS * p.nchunks + 255) / 256);
-        // (three operand stages hide most of the hand-over)
-        const double per_cb = std::max(std::max(t_mma, t_smem), std::max(t_w, t_x)) +
-                              (p.na_stages == 3 ? 300.0 : 400.0 + (p.ctas == 2 ? 700.0 : 0.0));
-        const bool dbl = p.MT == 1 || p.BN <= 128;
-        const double t_epi = 8.0 * p.MT * p.BN;                             // read-back and stores of one tile
-        const double per_tile = (dbl ? std::max(p.ncb * per_cb, t_epi) : p.ncb * per_cb + t_epi) + 3000.0;
-        double cost = (double)waves * per_tile + 9000.0 + (dbl ? t_epi : 0.0);
+        double cost = tile_cost(p, 1);
         // pairs of 64-channel tiles with two accumulators measure 12-15 % slower than this model says
         // (64 -> 64 channels at 56x56: 59 us against 52 us with one CTA per tile)
         if (p.ctas == 2 && p.MT == 2 && p.BN <= 64 && p.KB >= 16) cost *= 1.15;
@@ -971,6 +1038,41 @@ bool tc_conv_plan(const ConvGeom &c, TcConvPlan &plan, bool forced) {
             have = true;
             best_cost = cost;
             plan = p;
+        }
+    }
+    // Few tiles: let a cluster share each one's channel blocks (not for thin layers, which have one block).  A
+    // cluster of 8 does not fit every GPC: 14 of them are resident at once, and 33 of 4.
+    {
+        int pb = 0, pk = 0, ps = 0;         // ONNXB_CONV_SPLIT = "BN,KB,S" pins the shape, "0" rules the split out
+        const char *e = getenv("ONNXB_CONV_SPLIT");
+        const bool pinned = e && sscanf(e, "%d,%d,%d", &pb, &pk, &ps) == 3;
+        const bool ruled_out = (e && !pinned) || getenv("ONNXB_CONV_TILE") || getenv("ONNXB_CONV_STAGES") || getenv("ONNXB_CONV_EPI");
+        if (c.Cg >= 32 && !ruled_out && (pinned || (have && plan.total_tiles * plan.ctas <= 74))) {
+            if (pinned) have = false;
+            for (int kb = 16; kb <= 32; kb *= 2)
+                for (int bn = 16; bn <= 256; bn *= 2) {
+                    const int b = std::min(bn, (c.Mg + 15) / 16 * 16);
+                    if (pinned && (bn != pb || kb != pk)) continue;
+                    if (!pinned && bn > 16 && b <= bn / 2) break;
+                    TcConvPlan p;
+                    if (!fill_plan(c, 1, 1, b, kb, p)) continue;
+                    for (int S = 2; S <= 8; S *= 2) {
+                        if (pinned && S != ps) continue;
+                        p.cb_per = (p.ncb + S - 1) / S;
+                        if (p.cb_per * (S - 1) >= p.ncb) continue;                            // every CTA needs a block
+                        // the partial tile is parked over the stages
+                        if (128 * 4LL * (b + 1) + 16LL * b > (long long)p.na_stages * p.a_stage_bytes + (long long)p.nr_stages * p.raw_stage_bytes +
+                                                                 (long long)p.nb_stages * p.b_stage_bytes) continue;
+                        if (!pinned && p.total_tiles * S > (S == 8 ? 112 : S == 4 ? 132 : 148)) continue;
+                        const double cost = tile_cost(p, S);
+                        if (!have || cost < best_cost * 0.97) {
+                            have = true;
+                            best_cost = cost;
+                            plan = p;
+                            plan.split = S;
+                        }
+                    }
+                }
         }
     }
     if (have) {
@@ -1008,7 +1110,7 @@ static int max_pairs() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_conv_kernel<2, false, 8>, &cfg) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, tc_conv_kernel<2, false, 8, false>, &cfg) != cudaSuccess || n < 1) {
         cudaGetLastError();
         n = tc_host::num_sms() / 2;
     }
@@ -1050,18 +1152,20 @@ int launch_tc_conv(const TcConvPlan &plan, const float *X, const float *W, const
     const bool pair = plan.ctas == 2;
     const bool add = R != nullptr;
     const bool epi4 = plan.epi_warps == 4;
-    auto kern = epi4 ? (pair ? (add ? tc_conv_kernel<2, true, 4> : tc_conv_kernel<2, false, 4>)
-                             : (add ? tc_conv_kernel<1, true, 4> : tc_conv_kernel<1, false, 4>))
-                     : (pair ? (add ? tc_conv_kernel<2, true, 8> : tc_conv_kernel<2, false, 8>)
-                             : (add ? tc_conv_kernel<1, true, 8> : tc_conv_kernel<1, false, 8>));
-    const int threads = threads_for(epi4 ? 4 : 8);
+    const bool split = plan.split > 1;
+    auto kern = split  ? (add ? tc_conv_kernel<1, true, 8, true> : tc_conv_kernel<1, false, 8, true>)
+                : epi4 ? (pair ? (add ? tc_conv_kernel<2, true, 4, false> : tc_conv_kernel<2, false, 4, false>)
+                               : (add ? tc_conv_kernel<1, true, 4, false> : tc_conv_kernel<1, false, 4, false>))
+                       : (pair ? (add ? tc_conv_kernel<2, true, 8, false> : tc_conv_kernel<2, false, 8, false>)
+                               : (add ? tc_conv_kernel<1, true, 8, false> : tc_conv_kernel<1, false, 8, false>));
+    const int threads = threads_for(epi4 && !split ? 4 : 8);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return (int)e;
     const int sms = num_sms();
     // persistent: one CTA per SM; pairs are clusters of two neighbouring SMs
     const int units = pair ? max_pairs() : sms;
     if (units < 1) return (int)cudaErrorLaunchOutOfResources;
-    const int grid = (int)std::min<long long>(plan.total_tiles, units) * plan.ctas;
+    const int grid = split ? (int)plan.total_tiles * plan.split : (int)std::min<long long>(plan.total_tiles, units) * plan.ctas;
 #ifdef ONNXB_PROFILE
     fprintf(stderr, "[plan] ctas %d MT %d BN %d ctiles %d SLOTS %d planes %d Hs %d Ws %d L %d KB %d ncb %d steps %d spb %d tiles %lld grid %d raw_mode %d BOXP %d a_stage %d raw_stage %d b_stage %d nb %d smem %zu\n",
             plan.ctas, plan.MT, plan.BN, plan.ctiles, plan.SLOTS, plan.planes, plan.Hs, plan.Ws, plan.L, plan.KB, plan.ncb,
@@ -1069,7 +1173,7 @@ int launch_tc_conv(const TcConvPlan &plan, const float *X, const float *W, const
             plan.raw_stage_bytes, plan.b_stage_bytes, plan.nb_stages, smem);
 #endif
     const cudaError_t le =
-        pair ? launch_pdl_cluster(kern, 2, dim3(grid), dim3(threads), smem, st, tmX, plan, X,
+        pair || split ? launch_pdl_cluster(kern, split ? (unsigned)plan.split : 2u, dim3(grid), dim3(threads), smem, st, tmX, plan, X,
                                   reinterpret_cast<const float *>(workspace), B, R, Y, err)
              : launch_pdl(kern, dim3(grid), dim3(threads), smem, st, tmX, plan, X,
                           reinterpret_cast<const float *>(workspace), B, R, Y, err);

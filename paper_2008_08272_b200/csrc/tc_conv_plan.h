@@ -68,6 +68,7 @@ struct TcConvPlan {
     // divisors device code needs per slot, as multiply-and-shift constants (see conv_fdiv)
     ConvDivisor dv_L, dv_Ws, dv_Hs, dv_BOXP, dv_SLOTS, dv_pss;
     int boxp_shift;                  // log2(BOXP) when BOXP is a power of two, else -1
+    int split, cb_per;               // CTAs (a cluster) sharing a tile's channel blocks, blocks of each; split = 1: none
     int epi_warps;                   // epilogue warps of the launch: 8, or 4 (then 128 registers per thread)
     int relay;                       // pairs: the odd CTA's "operand stage written" goes through its relay warp
 };
