@@ -44,6 +44,9 @@ int launch_simt_conv(const ConvGeom &g, const float *X, const float *W, const fl
                      void *stream);
 int launch_simt_depthwise(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                           void *stream);
+double small_conv_cost(const ConvGeom &g);           // estimated SM cycles; negative: not for this problem
+int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
+                      void *stream);
 bool simt_depthwise_supports(const ConvGeom &g);
 bool conv_fits_mma_gemm(const ConvGeom &g);
 bool conv_fits_mma_gather_gemm(const ConvGeom &g);   // other unpadded 1x1: gather the pixels read, then the same GEMM

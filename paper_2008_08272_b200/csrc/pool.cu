@@ -7,7 +7,9 @@
 #include <cfloat>
 
 #include "common.h"
+#include "tc_common.cuh"
 #include "tc_conv_plan.h"
+#include "tc_host.h"
 
 namespace onnxb {
 namespace {
@@ -43,6 +45,33 @@ maxpool2d_kernel(const float *__restrict__ X, float *__restrict__ Y, int H, int 
 #pragma unroll
     for (int j = 0; j < 4; ++j)
         if (q0 + j < Q) yp[j] = best[j];
+}
+
+// Small outputs (one image of an MNIST-size network): one output per thread, all K*K loads in flight at once.
+template <int K>
+__global__ void __launch_bounds__(128)
+maxpool_small_kernel(const float *__restrict__ X, float *__restrict__ Y, int H, int W, int P, int Q, int pt, int pl, int sh, int sw,
+                     unsigned total, ConvDivisor dv_Q, ConvDivisor dv_P) {
+    tc::pdl_launch_dependents();
+    const unsigned i = blockIdx.x * 128u + threadIdx.x;
+    const unsigned t = (unsigned)conv_fdiv((int)i, Q, dv_Q), q = i - t * (unsigned)Q;
+    const unsigned plane = (unsigned)conv_fdiv((int)t, P, dv_P), p = t - plane * (unsigned)P;
+    const int h0 = (int)p * sh - pt, w0 = (int)q * sw - pl;
+    const float *xp = X + (size_t)plane * H * W;
+    tc::pdl_wait();
+    if (i >= total) return;
+    float v[K * K];
+#pragma unroll
+    for (int r = 0; r < K; ++r)
+#pragma unroll
+        for (int s = 0; s < K; ++s) {
+            const int h = h0 + r, w = w0 + s;
+            v[r * K + s] = (unsigned)h < (unsigned)H && (unsigned)w < (unsigned)W ? __ldg(xp + (size_t)h * W + w) : -INFINITY;
+        }
+    float m = v[0];
+#pragma unroll
+    for (int k = 1; k < K * K; ++k) m = fmaxf(m, v[k]);
+    Y[i] = m;
 }
 
 // The ResNet-50 pool: 3x3 window, stride 2, one row/column of padding in front (any amount behind),
@@ -158,6 +187,16 @@ extern "C" onnxb_status onnx_maxpool2d_run(const int64_t x_dims[4], const int64_
             conv_divisor((int)P2));
         count_launch();
         return cudaGetLastError() == cudaSuccess ? ONNXB_OK : ONNXB_ERR_CUDA;
+    }
+    // below about 300 000 outputs the launch is too short to fill the SMs with four outputs per thread
+    const int64_t outputs = y[0] * y[1] * P * Q;
+    if (kernel_shape[0] == kernel_shape[1] && (kernel_shape[0] == 2 || kernel_shape[0] == 3) && outputs <= 148 * 2048) {
+        auto kern = kernel_shape[0] == 2 ? maxpool_small_kernel<2> : maxpool_small_kernel<3>;
+        const cudaError_t e = tc_host::launch_pdl(kern, dim3((unsigned)((outputs + 127) / 128)), dim3(128), 0, (cudaStream_t)cuda_stream,
+                                                  X, Y, (int)x_dims[2], (int)x_dims[3], P, Q, (int)pt0, (int)pl0, (int)sh0, (int)sw0,
+                                                  (unsigned)outputs, conv_divisor(Q), conv_divisor(P));
+        count_launch();
+        return e == cudaSuccess ? ONNXB_OK : ONNXB_ERR_CUDA;
     }
     const unsigned Q4 = (unsigned)((Q + 3) / 4);
     const int64_t items = y[0] * y[1] * P * Q4;

@@ -7,10 +7,130 @@
 
 #include "common.h"
 #include "tc_common.cuh"
+#include "tc_host.h"
 
 namespace onnxb {
 
 namespace {
+
+// Convolution of small images (an MNIST-size layer): latency, not throughput.  A block owns 128 output pixels
+// of one image and MB output channels of one group; it brings the group's padded input image and its
+// filters into shared memory in one go (every load in flight at once, zeros for the padding, so the taps need
+// no bounds checks) and each thread then sums its pixel's MB outputs.  Filters lie as [c][tap, padded to 4]
+// (MB = 1: one 16-byte read serves four taps) or [c][tap][MB] (MB > 1: one read serves four channels).
+// K > 0: a K x K filter with unrolled taps; K = 0: any.  One 14x14 image, 8 -> 16 channels, 5x5: 6.8 -> 4 us.
+constexpr int kSmallThreads = 128;
+constexpr int kSmallSmem = 48 * 1024;
+
+template <int MB, int K>
+__global__ void __launch_bounds__(kSmallThreads)
+conv2d_small_kernel(const __grid_constant__ ConvGeom g, const float *__restrict__ X, const float *__restrict__ W,
+                    const float *__restrict__ B, const float *__restrict__ R, float *__restrict__ Y, int Hp, int Wp, int taps4,
+                    const ConvDivisor dv_Wp, const ConvDivisor dv_HpWp, const ConvDivisor dv_Q, const ConvDivisor dv_taps) {
+    extern __shared__ __align__(16) float sm[];
+    const int taps = K > 0 ? K * K : g.kH * g.kW, kW = K > 0 ? K : g.kW;
+    const int ptiles = (g.P * g.Q + kSmallThreads - 1) / kSmallThreads, mtiles = (g.Mg + MB - 1) / MB;
+    int b = blockIdx.x;
+    const int pt = b % ptiles; b /= ptiles;
+    const int mt = b % mtiles; b /= mtiles;
+    const int grp = b % g.group, n = b / g.group;
+    const int m0 = mt * MB, plane = Hp * Wp;
+    float *ws = sm, *xs = sm + g.Cg * (MB == 1 ? taps4 : taps * MB);
+    tc::pdl_launch_dependents();
+    tc::pdl_wait();
+
+    const int kred = g.Cg * taps;
+    // eight loads in flight per thread
+    for (int i0 = threadIdx.x; i0 < kred * MB; i0 += 8 * kSmallThreads) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = i0 + u * kSmallThreads, j = MB == 1 ? 0 : i & (MB - 1), k = i / MB;
+            v[u] = i < kred * MB && m0 + j < g.Mg ? __ldg(W + (size_t)(grp * g.Mg + m0 + j) * kred + k) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = i0 + u * kSmallThreads, c = conv_fdiv(i, taps, dv_taps);
+            if (i < kred * MB) ws[MB == 1 ? c * taps4 + (i - c * taps) : i] = v[u];
+        }
+    }
+    const float *xg = X + ((size_t)n * g.C + (size_t)grp * g.Cg) * g.H * g.W;
+    const int total = g.Cg * plane;
+    for (int i0 = threadIdx.x; i0 < total; i0 += 8 * kSmallThreads) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = i0 + u * kSmallThreads;
+            const int c = conv_fdiv(i, plane, dv_HpWp), r = i - c * plane;
+            const int hp = conv_fdiv(r, Wp, dv_Wp), h = hp - g.pt, w = r - hp * Wp - g.pl;
+            const bool ok = i < total && (unsigned)h < (unsigned)g.H && (unsigned)w < (unsigned)g.W;
+            v[u] = ok ? __ldg(xg + ((size_t)c * g.H + h) * g.W + w) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (i0 + u * kSmallThreads < total) xs[i0 + u * kSmallThreads] = v[u];
+    }
+    __syncthreads();
+
+    const int pix = pt * kSmallThreads + threadIdx.x;
+    if (pix >= g.P * g.Q) return;
+    const int p = conv_fdiv(pix, g.Q, dv_Q), q = pix - p * g.Q;
+    float acc[MB];
+#pragma unroll
+    for (int j = 0; j < MB; ++j) acc[j] = 0.f;
+    const float *xc = xs + p * g.sh * Wp + q * g.sw;
+    for (int c = 0; c < g.Cg; ++c, xc += plane) {
+        if (K > 0) {
+            float x[K > 0 ? K * K : 1];
+#pragma unroll
+            for (int r = 0; r < K; ++r)
+#pragma unroll
+                for (int s = 0; s < K; ++s) x[r * K + s] = xc[r * g.dh * Wp + s * g.dw];
+            if (MB == 1) {
+                const float4 *wc = reinterpret_cast<const float4 *>(ws + c * taps4);
+#pragma unroll
+                for (int t = 0; t < (K * K + 3) / 4; ++t) {
+                    const float4 w = wc[t];
+                    acc[0] = fmaf(x[4 * t], w.x, acc[0]);
+                    if (4 * t + 1 < K * K) acc[0] = fmaf(x[4 * t + 1 < K * K ? 4 * t + 1 : 0], w.y, acc[0]);
+                    if (4 * t + 2 < K * K) acc[0] = fmaf(x[4 * t + 2 < K * K ? 4 * t + 2 : 0], w.z, acc[0]);
+                    if (4 * t + 3 < K * K) acc[0] = fmaf(x[4 * t + 3 < K * K ? 4 * t + 3 : 0], w.w, acc[0]);
+                }
+            } else {
+#pragma unroll
+                for (int t = 0; t < K * K; ++t) {
+#pragma unroll
+                    for (int j = 0; j + 3 < MB; j += 4) {
+                        const float4 w = *reinterpret_cast<const float4 *>(ws + (c * taps + t) * MB + j);
+                        acc[j] = fmaf(x[t], w.x, acc[j]);
+                        acc[j + 1] = fmaf(x[t], w.y, acc[j + 1]);
+                        acc[j + 2] = fmaf(x[t], w.z, acc[j + 2]);
+                        acc[j + 3] = fmaf(x[t], w.w, acc[j + 3]);
+                    }
+                }
+            }
+        } else {
+            int r = 0, s = 0;
+            for (int t = 0; t < taps; ++t) {
+                const float x = xc[r * g.dh * Wp + s * g.dw];
+#pragma unroll
+                for (int j = 0; j < MB; ++j) acc[j] = fmaf(x, ws[MB == 1 ? c * taps4 + t : (c * taps + t) * MB + j], acc[j]);
+                if (++s == kW) { s = 0; ++r; }
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < MB; ++j) {
+        if (m0 + j < g.Mg) {
+            const int m = grp * g.Mg + m0 + j;
+            const size_t yi = ((size_t)n * g.M + m) * g.P * g.Q + pix;
+            float v = acc[j] + (B ? __ldg(B + m) : 0.f);
+            if (R) v += __ldg(R + yi);
+            if (g.relu) v = v > 0.f ? v : 0.f;
+            Y[yi] = v;
+        }
+    }
+}
 
 // Depthwise convolution (group == C == M): purely HBM-bound, 2*kH*kW flops per
 // output.  A block stages the input window of a 32 x 32 output tile of one
@@ -150,18 +270,21 @@ gather1x1_vec_kernel(const float4 *__restrict__ X4, float4 *__restrict__ Xg4, un
 // flop per byte, so the only thing that matters is to move each plane once with few instructions.
 // A thread owns a strip of 4 output columns by ROWS output rows of one (image, channel) plane, reads
 // the KH + ROWS - 1 input rows it needs straight from global memory (neighbouring threads' overlapping
-// reads are served by L1) and keeps the window in registers: with ROWS = 4 and a 3x3 filter, 18 loads
-// and 144 FMAs for 16 outputs, every input row fetched 1.5 times instead of twice with ROWS = 2.  VEC: the row pitch and the left pad allow one aligned 16-byte load per row for the
-// strip's middle columns; otherwise every column is loaded on its own.
+// reads are served by L1) and keeps the window in registers: with ROWS = 4 and a 3x3 filter, 6 row loads
+// and 144 FMAs for 16 outputs, every input row fetched 1.5 times instead of twice with ROWS = 2.  VEC: rows are whole
+// 16-byte pieces and as wide as the output, so a row costs one aligned 16-byte load; the columns to its left and
+// right come from the neighbouring lanes, which hold them (the first and last lane of a warp load theirs), and
+// beyond the row's ends lies padding.  Otherwise every column is loaded on its own.
 template <int KH, int KW, bool VEC, int ROWS>
 __global__ void __launch_bounds__(256)
 conv2d_depthwise_unit_kernel(const ConvGeom g, const float *__restrict__ X, const float *__restrict__ W,
                              const float *__restrict__ B, const float *__restrict__ R, float *__restrict__ Y,
                              unsigned items, unsigned Q4, unsigned P2, double inv_Q4, double inv_P2) {
     constexpr int WIN = KW + 3;                // input columns a strip of 4 outputs touches
-    tc::pdl_launch_dependents();               // (launched plainly itself) lets the next kernel set up early
-    const unsigned i = blockIdx.x * 256u + threadIdx.x;
-    if (i >= items) return;
+    tc::pdl_launch_dependents();
+    const unsigned i_own = blockIdx.x * 256u + threadIdx.x;
+    if (!VEC && i_own >= items) return;
+    const unsigned i = VEC && i_own >= items ? items - 1 : i_own;      // (the neighbours of a live lane must stay)
     // i = (plane * P2 + row group) * Q4 + column quad (P2 = row groups per plane); quotients by reciprocal multiplication in
     // double (right for 31-bit operands up to one unit, which the two comparisons repair)
     unsigned t = __double2uint_rd((double)i * inv_Q4);
@@ -174,6 +297,58 @@ conv2d_depthwise_unit_kernel(const ConvGeom g, const float *__restrict__ X, cons
     const int p0 = (int)(t - plane * P2) * ROWS, q0 = (int)q4 * 4;
     const int c = (int)(plane % (unsigned)g.C);
 
+    const float *xp = X + (size_t)plane * g.H * g.W;
+    const int iw0 = q0 - g.pl;
+    tc::pdl_wait();
+    // Every input row of the window is requested before the first FMA: the kernel is bound by the
+    // latency of these loads, so each thread keeps all of them in flight at once.
+    float v[KH + ROWS - 1][WIN];
+    if (VEC) {
+        constexpr int L = (KW - 1) / 2, RT = KW - 1 - L;       // columns to the left (= the pad) and right of the quad
+        const int lane = threadIdx.x & 31;
+        const bool left_in = q0 > 0, right_in = q0 + 4 < g.W;
+        float e[KH + ROWS - 1][L > RT ? L : RT];               // what the warp's first and last lane load themselves
+#pragma unroll
+        for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
+            const int ih = p0 - g.pt + rr;
+            const bool row_in = (unsigned)ih < (unsigned)g.H;
+            const float *row = xp + (size_t)ih * g.W + q0;
+            float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row_in) m = __ldg(reinterpret_cast<const float4 *>(row));
+            v[rr][L] = m.x; v[rr][L + 1] = m.y; v[rr][L + 2] = m.z; v[rr][L + 3] = m.w;
+#pragma unroll
+            for (int k = 0; k < (L > RT ? L : RT); ++k) {
+                e[rr][k] = 0.f;
+                if (lane == 0 && k < L && row_in && left_in) e[rr][k] = __ldg(row - L + k);
+                if (lane == 31 && k < RT && row_in && right_in) e[rr][k] = __ldg(row + 4 + k);
+            }
+        }
+#pragma unroll
+        for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
+#pragma unroll
+            for (int k = 0; k < L; ++k) {
+                const float x = __shfl_up_sync(0xffffffffu, v[rr][L + 4 - L + k], 1);
+                v[rr][k] = !left_in ? 0.f : lane == 0 ? e[rr][k] : x;
+            }
+#pragma unroll
+            for (int k = 0; k < RT; ++k) {
+                const float x = __shfl_down_sync(0xffffffffu, v[rr][L + k], 1);
+                v[rr][L + 4 + k] = !right_in ? 0.f : lane == 31 ? e[rr][k] : x;
+            }
+        }
+        if (i_own >= items) return;
+    } else {
+#pragma unroll
+        for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
+            const int ih = p0 - g.pt + rr;
+            const float *row = xp + (size_t)ih * g.W;
+#pragma unroll
+            for (int k = 0; k < WIN; ++k) {
+                v[rr][k] = 0.f;
+                if ((unsigned)ih < (unsigned)g.H && (unsigned)(iw0 + k) < (unsigned)g.W) v[rr][k] = __ldg(row + iw0 + k);
+            }
+        }
+    }
     float w[KH * KW];
 #pragma unroll
     for (int k = 0; k < KH * KW; ++k) w[k] = __ldg(W + (size_t)c * (KH * KW) + k);
@@ -183,37 +358,6 @@ conv2d_depthwise_unit_kernel(const ConvGeom g, const float *__restrict__ X, cons
     for (int k = 0; k < ROWS; ++k)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[k][j] = bias;
-
-    const float *xp = X + (size_t)plane * g.H * g.W;
-    const int iw0 = q0 - g.pl;
-    // Every input row of the window is requested before the first FMA: the kernel is bound by the
-    // latency of these loads, so each thread keeps all of them in flight at once.
-    float v[KH + ROWS - 1][WIN];
-#pragma unroll
-    for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
-        const int ih = p0 - g.pt + rr;
-#pragma unroll
-        for (int k = 0; k < WIN; ++k) v[rr][k] = 0.f;
-        if ((unsigned)ih < (unsigned)g.H) {
-            const float *row = xp + (size_t)ih * g.W;
-            if (VEC) {
-                // pl == 1: columns q0-1 .. q0+KW+1; q0 .. q0+3 are one aligned float4
-                if (iw0 >= 0) v[rr][0] = __ldg(row + iw0);
-                if (q0 + 3 < g.W) {
-                    const float4 m = __ldg(reinterpret_cast<const float4 *>(row + q0));
-                    v[rr][1] = m.x; v[rr][2] = m.y; v[rr][3] = m.z; v[rr][4] = m.w;
-                } else {
-#pragma unroll
-                    for (int k = 1; k < 5; ++k) if (iw0 + k < g.W) v[rr][k] = __ldg(row + iw0 + k);
-                }
-#pragma unroll
-                for (int k = 5; k < WIN; ++k) if (iw0 + k < g.W) v[rr][k] = __ldg(row + iw0 + k);
-            } else {
-#pragma unroll
-                for (int k = 0; k < WIN; ++k) if ((unsigned)(iw0 + k) < (unsigned)g.W) v[rr][k] = __ldg(row + iw0 + k);
-            }
-        }
-    }
 #pragma unroll
     for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
         // input row rr is filter row rr - k of output row p0 + k
@@ -261,10 +405,17 @@ int launch_depthwise_unit(const ConvGeom &g, const float *X, const float *W, con
     const long long items = (long long)g.N * g.C * P2 * Q4;
     const unsigned blocks = (unsigned)((items + 255) / 256);
     // aligned 16-byte accesses: every input and output row starts on a 16-byte boundary
-    const bool vec = g.pl == 1 && g.W % 4 == 0 && g.Q % 4 == 0 &&
+    const bool vec = g.pl == (KW - 1) / 2 && g.W % 4 == 0 && g.Q == g.W &&
                      (reinterpret_cast<uintptr_t>(X) & 15) == 0 && (reinterpret_cast<uintptr_t>(Y) & 15) == 0;
     auto kern = vec ? (rows4 ? conv2d_depthwise_unit_kernel<KH, KW, true, 4> : conv2d_depthwise_unit_kernel<KH, KW, true, 2>)
                     : (rows4 ? conv2d_depthwise_unit_kernel<KH, KW, false, 4> : conv2d_depthwise_unit_kernel<KH, KW, false, 2>);
+    // early launch gains 0.5 us behind another kernel where the rows are vectorised, and loses as much where not
+    if (vec) {
+        const cudaError_t e = tc_host::launch_pdl(kern, dim3(blocks), dim3(256), 0, st, g, X, W, B, R, Y, (unsigned)items, Q4, P2,
+                                                  1.0 / (double)Q4, 1.0 / (double)P2);
+        count_launch();
+        return (int)e;
+    }
     kern<<<blocks, 256, 0, st>>>(g, X, W, B, R, Y, (unsigned)items, Q4, P2, 1.0 / (double)Q4, 1.0 / (double)P2);
     count_launch();
     return (int)cudaGetLastError();
@@ -284,6 +435,56 @@ void depthwise_window(const ConvGeom &g, int &rows, int &cols, int &pitch) {
 }
 
 }  // namespace
+
+// Channels per block: as many as still leave every SM two blocks.
+static int small_mb(const ConvGeom &g) {
+    const long long ptiles = ((long long)g.P * g.Q + kSmallThreads - 1) / kSmallThreads;
+    for (int mb = 16; mb >= 4; mb /= 2)
+        if (g.Mg > mb / 2 && (long long)g.N * g.group * ((g.Mg + mb - 1) / mb) * ptiles >= 148 * 2) return mb;
+    return 1;
+}
+static size_t small_smem(const ConvGeom &g, int mb) {
+    const long long Hp = (long long)(g.P - 1) * g.sh + (long long)(g.kH - 1) * g.dh + 1, Wp = (long long)(g.Q - 1) * g.sw + (long long)(g.kW - 1) * g.dw + 1;
+    const long long taps = (long long)g.kH * g.kW;
+    if (Hp * Wp > 16384 || taps > 4096 || g.Cg > 16384) return (size_t)-1;
+    return (size_t)g.Cg * 4 * (Hp * Wp + (mb == 1 ? (taps + 3) / 4 * 4 : taps * mb));
+}
+// Estimated SM cycles, or a negative number where the kernel does not apply.
+double small_conv_cost(const ConvGeom &g) {
+    const int mb = small_mb(g);
+    const size_t smem = small_smem(g, mb);
+    if (smem > (size_t)kSmallSmem || (long long)g.P * g.Q > 4096) return -1;
+    const long long ptiles = ((long long)g.P * g.Q + kSmallThreads - 1) / kSmallThreads;
+    const long long blocks = (long long)g.N * g.group * ((g.Mg + mb - 1) / mb) * ptiles;
+    if (blocks > 1000000) return -1;
+    // One wave of resident blocks: the loads come in batches of eight per thread, each a trip to L2, then the sum;
+    // and no less than what an SM's blocks need in turn (measured: 100 cycles per element a thread brings in).
+    const double kred = (double)g.Cg * g.kH * g.kW, per_sm = (double)((blocks + 147) / 148);
+    const double unrolled = g.kH == g.kW && (g.kH == 3 || g.kH == 5) ? 1.0 : 2.5;
+    const double fill = (double)smem / 4 / kSmallThreads;
+    const double resident = std::min(16.0, 200e3 / (double)(smem + 1024)), waves = std::max(1.0, per_sm / resident);
+    const double latency = waves * (fill / 8 * 700.0 + kred * 9.0 * unrolled);
+    const double issue = per_sm * (fill * 100.0 + kred * unrolled * (mb == 1 ? 3.0 : 1.5 + 2.2 * mb));
+    return 5500.0 + std::max(latency, issue);
+}
+
+int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y, void *stream) {
+    const int mb = small_mb(g), taps = g.kH * g.kW;
+    const int Hp = (g.P - 1) * g.sh + (g.kH - 1) * g.dh + 1, Wp = (g.Q - 1) * g.sw + (g.kW - 1) * g.dw + 1;
+    const long long ptiles = ((long long)g.P * g.Q + kSmallThreads - 1) / kSmallThreads;
+    const long long blocks = (long long)g.N * g.group * ((g.Mg + mb - 1) / mb) * ptiles;
+    const int k = g.kH == g.kW && (g.kH == 3 || g.kH == 5) ? g.kH : 0;
+    auto pick = [k](auto k3, auto k5, auto any) { return k == 3 ? k3 : k == 5 ? k5 : any; };
+    auto kern = mb == 1   ? pick(conv2d_small_kernel<1, 3>, conv2d_small_kernel<1, 5>, conv2d_small_kernel<1, 0>)
+                : mb == 4 ? pick(conv2d_small_kernel<4, 3>, conv2d_small_kernel<4, 5>, conv2d_small_kernel<4, 0>)
+                : mb == 8 ? pick(conv2d_small_kernel<8, 3>, conv2d_small_kernel<8, 5>, conv2d_small_kernel<8, 0>)
+                          : pick(conv2d_small_kernel<16, 3>, conv2d_small_kernel<16, 5>, conv2d_small_kernel<16, 0>);
+    const cudaError_t e = tc_host::launch_pdl(kern, dim3((unsigned)blocks), dim3(kSmallThreads), small_smem(g, mb), (cudaStream_t)stream,
+                                              g, X, W, B, R, Y, Hp, Wp, (taps + 3) / 4 * 4, conv_divisor(Wp),
+                                              conv_divisor(Hp * Wp), conv_divisor(g.Q), conv_divisor(taps));
+    count_launch();
+    return (int)e;
+}
 
 bool simt_depthwise_supports(const ConvGeom &g) {
     if (!(g.Cg == 1 && g.Mg == 1)) return false;

@@ -434,6 +434,7 @@ Pick search_shape(int M, int N, int K, int groups, bool pixels) {
 struct Choice {
     int M, N, K, groups, pixels;
     Pick pick;
+    double tc_cost;
     bool tc;
 };
 bool fp32_on_tensor_cores(double fma_cost, double tc_cost);
@@ -444,9 +445,9 @@ Choice choose(int M, int N, int K, int groups, bool pixels) {
                         (unsigned)pixels) >> 7;
     Choice &c = memo[h % 64];
     if (!pinned && c.M == M && c.N == N && c.K == K && c.groups == groups && c.pixels == (int)pixels) return c;
-    Choice r{M, N, K, groups, (int)pixels, search_shape(M, N, K, groups, pixels), false};
     // (rows and columns change places there: its rows are the index contiguous in Y)
-    r.tc = fp32_on_tensor_cores(r.pick.cost, tc_fp32_cost(N, M, K, groups, pixels));
+    Choice r{M, N, K, groups, (int)pixels, search_shape(M, N, K, groups, pixels), tc_fp32_cost(N, M, K, groups, pixels), false};
+    r.tc = fp32_on_tensor_cores(r.pick.cost, r.tc_cost);
     if (!pinned) c = r;
     return r;
 }
@@ -518,6 +519,10 @@ int launch_simt_conv(const ConvGeom &g, const float *X, const float *W, const fl
     a.dv_PQ = conv_divisor(a.PQ); a.dv_Q = conv_divisor(a.Q); a.dv_taps = conv_divisor(a.taps); a.dv_kW = conv_divisor(a.kW);
     const Choice ch = choose(a.M, a.N, a.K, g.group, true);
     const Pick pick = ch.pick;
+    const double small = small_conv_cost(g);
+    const char *pin = getenv("ONNXB_FP32");              // "small" pins the small-image kernel
+    if (small >= 0 && (pin ? pin[0] == 's' : 0.85 * small < std::min(ch.pick.cost, ch.tc_cost)))      // (the tiled estimates run low here)
+        return launch_small_conv(g, X, W, B, R, Y, stream);
     if (ch.tc && a.taps <= 64) return launch_tc_fp32_conv(g, X, W, B, R, Y, stream);
     return launch_sgemm<kKContig, kPixels>(a, g.group, pick, (cudaStream_t)stream);
 }

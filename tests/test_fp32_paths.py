@@ -55,6 +55,35 @@ def test_fp32_gemm_and_conv_tiles(binding, pin, monkeypatch):
         binding.set_kernel_override(None)
 
 
+SMALL_CONVS = [dict(x=(1, 1, 28, 28), w=(8, 1, 5, 5), pads=(2, 2, 2, 2)), dict(x=(90, 3, 13, 11), w=(7, 3, 3, 3), pads=(1, 0, 2, 1)),
+               dict(x=(100, 4, 9, 9), w=(18, 2, 2, 4), strides=(2, 1), dilations=(1, 2), group=2),
+               dict(x=(70, 2, 17, 19), w=(16, 2, 5, 5), pads=(2, 2, 2, 2), strides=(2, 2))]
+
+
+@pytest.mark.parametrize("c", SMALL_CONVS, ids=lambda c: "x".join(map(str, c["x"] + c["w"])))
+def test_small_image_conv(binding, c, monkeypatch):
+    """The whole-image-in-shared-memory kernel at every channel count per block, ragged channels and pixels."""
+    monkeypatch.setenv("ONNXB_FP32", "small")
+    rng = np.random.default_rng(17)
+    X = rng.standard_normal(c["x"]).astype(np.float32)
+    W = rng.standard_normal(c["w"]).astype(np.float32)
+    B = rng.standard_normal((c["w"][0],)).astype(np.float32)
+    kw = dict(pads=c.get("pads", (0, 0, 0, 0)), strides=c.get("strides", (1, 1)), dilations=c.get("dilations", (1, 1)),
+              group=c.get("group", 1))
+    for images in (1, c["x"][0]):
+        got, fam = run_conv_gpu(binding, torch, X[:images], W, B, relu=True, **kw)
+        assert fam == "simt_direct"
+        want, S = oracle.conv2d(X[:images], W, B, relu=True, **kw)
+        assert (np.abs(got - want) <= REL * S + 1e-5).all()
+
+
+@pytest.mark.parametrize("shape,k,st,pads", [((1, 8, 28, 28), 2, 2, 0), ((1, 16, 14, 14), 3, 3, 0), ((2, 5, 9, 11), 3, 2, 1)])
+def test_small_max_pool(binding, shape, k, st, pads):
+    X = torch.randn(shape, device="cuda")
+    got = binding.onnx_maxpool2d(X, (k, k), pads=(pads,) * 4, strides=(st, st))
+    assert torch.equal(got.cpu(), torch.nn.functional.max_pool2d(X.cpu(), k, st, padding=pads))
+
+
 @pytest.mark.parametrize("tA", [False, True])
 @pytest.mark.parametrize("shape", [(1, 10, 256), (64, 10, 256), (33, 31, 7), (3, 5, 291)])
 def test_tiny_gemm(binding, shape, tA):
