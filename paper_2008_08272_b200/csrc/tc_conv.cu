@@ -158,7 +158,30 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
     const bool acc_dbl = g.MT == 1 || g.BN <= 128;
     const uint32_t mt_cols = acc_dbl ? 128u : 256u;     // column distance between a CTA's two accumulators
 
-    if (threadIdx.x == 0) {
+    if (kSplit && warp == kRelayWarp) {
+        // a barrier of each kind per lane: one thread alone takes a thousand cycles for them (which the other
+        // forms hide behind the previous kernel)
+        if (lane < g.nr_stages) {
+            mbar_init(&bars->raw_full[lane], 1);
+            mbar_init(&bars->raw_empty[lane], kXformWarps);
+        }
+        if (lane < g.na_stages) {
+            mbar_init(&bars->a_full[lane], kXformWarps);
+            mbar_init(&bars->a_empty[lane], 1);
+        }
+        if (lane < g.nb_stages) {
+            mbar_init(&bars->b_full[lane], 1);
+            mbar_init(&bars->b_empty[lane], 1);
+        }
+        if (lane < 2) {
+            mbar_init(&bars->acc_full[lane], 1);
+            mbar_init(&bars->acc_empty[lane], kEpiWarps);
+            mbar_init(&bars->seg_full[lane], 1);
+            mbar_init(&bars->seg_empty[lane], kXformWarps);
+        }
+        mbar_fence_init();
+    }
+    if (!kSplit && threadIdx.x == 0) {
         for (int s = 0; s < g.nr_stages; ++s) {
             mbar_init(&bars->raw_full[s], 1);
             mbar_init(&bars->raw_empty[s], kXformWarps);
@@ -183,6 +206,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
         mbar_fence_init();
         if (g.raw_mode == 0) prefetch_tmap(&tmX);
     }
+    if (kSplit && threadIdx.x == 0 && g.raw_mode == 0) prefetch_tmap(&tmX);
     if (warp == 2) {
         tmem_alloc(&bars->tmem_holder, 512);
         tmem_relinquish();
@@ -680,20 +704,33 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             if (p < g.P && q < g.Q) {
                 const long long PQ = (long long)g.P * g.Q;
                 const uint32_t part_addr = smem_u32(smem);
-                for (int col = col_lo + tid / rows; col < col_hi; col += nthr / rows) {
-                    const int m = grp * g.Mg + ct * g.BN + col;
-                    const long long yi = ((long long)n * g.M + m) * PQ + (long long)p * g.Q + q;
-                    const float b = bias ? __ldg(bias + m) : 0.f, r = kAdd ? __ldg(R + yi) : 0.f;
-                    float x = 0.f;
-                    for (int sp = 0; sp < g.split; sp += 2) {
+                // Two channels at a time, all their partials requested at once: a trip to a peer's shared memory
+                // takes some 600 cycles (one 14x14 image, split over 8: 3.7 -> 1.2 us for the exchange).
+                for (int col0 = col_lo + tid / rows; col0 < col_hi; col0 += 2 * (nthr / rows)) {
+                    float v[2][8], b[2], r[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int col = min(col0 + u * (nthr / rows), col_hi - 1), m = grp * g.Mg + ct * g.BN + col;
                         const uint32_t off = part_addr + (uint32_t)(col * pitch + row) * 4u;
-                        const float x0 = ld_cluster_f32(map_to_cta(off, (uint32_t)sp)), x1 = ld_cluster_f32(map_to_cta(off, (uint32_t)sp + 1u));
-                        x = (x + x0) + x1;
+#pragma unroll
+                        for (int sp = 0; sp < 8; ++sp)
+                            if (sp < g.split) v[u][sp] = ld_cluster_f32(map_to_cta(off, (uint32_t)sp));
+                        b[u] = bias ? __ldg(bias + m) : 0.f;
+                        r[u] = kAdd ? __ldg(R + ((long long)n * g.M + m) * PQ + (long long)p * g.Q + q) : 0.f;
                     }
-                    x += b;
-                    if (kAdd) x += r;
-                    if (g.relu) x = fmaxf(x, 0.f);
-                    Y[yi] = x;
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int col = col0 + u * (nthr / rows);
+                        if (col >= col_hi) break;
+                        float x = 0.f;
+#pragma unroll
+                        for (int sp = 0; sp < 8; ++sp)
+                            if (sp < g.split) x += v[u][sp];
+                        x += b[u];
+                        if (kAdd) x += r[u];
+                        if (g.relu) x = fmaxf(x, 0.f);
+                        Y[((long long)n * g.M + grp * g.Mg + ct * g.BN + col) * PQ + (long long)p * g.Q + q] = x;
+                    }
                 }
             }
         }

@@ -53,6 +53,7 @@ struct Params {
     int M, N, K, batch;
     int a_mn, b_mn;            // operand is MN-major (else K-major)
     int a_batched, b_batched;
+    int a_kbox, b_kbox;        // K-major operand with K a multiple of 32: one copy brings all of a stage's K blocks
     int BN, tiles_m, tiles_n, num_kb, num_stages;
     uint32_t idesc, stage_bytes, tx_bytes;
     // The last tile along N is only as wide as the columns left, rounded up to 16: its MMAs take the
@@ -84,7 +85,12 @@ struct Params {
     unsigned int *err;
 };
 
-template <int kCtas>
+// kKS: K blocks of 32 per stage.  What a stage costs its two single threads bounds thin tiles: the producer and
+// the MMA issuer pay every instruction's full latency.  So a stage is one copy per operand, waits are on barriers
+// of the CTA's own (both CTAs' copies of a pair's stage complete on the issuing CTA's barrier), the MMAs are
+// straight-line code with one add per descriptor, and thin tiles put two K blocks behind one barrier.  Per K block
+// of a 256 x 64 pair tile: 660 -> 390 cycles; Gemm 1024 x 1024 x 4096 48.6 -> 34.3 us, 4096^3 239 -> 223 us.
+template <int kCtas, int kKS>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmBb, const __grid_constant__ CUtensorMap tmY,
@@ -108,8 +114,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.num_stages; ++s) {
-            // issuing CTA of a pair: its own producer plus the peer's "landed" message
-            mbar_init(&full[s], (kCtas == 2 && rank == 0) ? 2 : 1);
+            // a pair's stage counts on the issuing (even) CTA's barrier alone: one arrival, which announces the
+            // bytes of both CTAs' copies
+            mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
         for (int a = 0; a < 2; ++a) {
@@ -149,11 +156,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         {
             int stage = 0;
             uint32_t phase = 0;
-            const int na = p.a_mn ? kBM / 32 : 1;
+            const uint32_t full_issuer = kCtas == 2 ? map_to_cta(smem_u32(&full[0]), 0) : 0u;
+            const int na = p.a_mn ? kBM / 32 : p.a_kbox ? 1 : kKS;       // copies of A per stage
+            const int nb1 = p.b_mn || p.b_kbox ? 1 : kKS;                // copies of B, unless block by block
             const int hb = p.BNH / 32;                 // 32-column blocks of B this CTA stages (MN-major B)
-            // lanes [0, na): A pieces; lane na: B in one copy; lanes [na + 1, na + 1 + hb): B block by block
-            const bool is_a = lane < na;
-            const int jb = lane - na - 1;
+            // lanes [0, na): A pieces; [na, na + nb1): B; [na + nb1, na + nb1 + hb): MN-major B block by block
+            const bool is_a = lane < na, is_b = lane >= na && lane < na + nb1;
+            const int jb = lane - na - nb1;
             int glog_i = 0;
             (void)glog_i;
             for (int t = first_tile; t < total_tiles; t += tile_step) {
@@ -170,45 +179,51 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 // (never negative: a CTA whose first column lies past N fetches no block at all, and what it
                 // expects on the stage's barrier is exactly what it issues)
                 const int hb_t = col_b < p.N ? min((bnh_t + 31) / 32, (p.N - col_b + 31) / 32) : 0;
-                const uint32_t tx_bytes = (p.b_mn && !one_box) ? (uint32_t)(kABytes + hb_t * 4096) : p.tx_bytes;
+                uint32_t tx_bytes = kKS * (uint32_t)(kABytes + (p.b_mn && !one_box ? hb_t * 4096 : p.BNH * 128));
+                if (kCtas == 2) {
+                    // the peer's share of the stage, worked out the same way
+                    const int col_p = tn * p.BN + (rank ^ 1) * bnh_t;
+                    const bool box_p = p.b_mn && p.b_big && (col_p & 31) == 0 && col_p / 32 + hb <= p.b_nblk_full;
+                    const int hb_p = col_p < p.N ? min((bnh_t + 31) / 32, (p.N - col_p + 31) / 32) : 0;
+                    tx_bytes += kKS * (uint32_t)(kABytes + (p.b_mn && !box_p ? hb_p * 4096 : p.BNH * 128));
+                }
                 // This lane's copy.  Every view has four dimensions (the plain ones end in a unit
                 // dimension), so the copies of a stage are ONE instruction executed by several lanes
                 // with their own coordinates; two different copy instructions would run one after the
                 // other and each holds the warp for about 290 cycles.
-                int c0 = 0, c1 = 0, c2 = 0, c3 = 0, d0 = 0, d1 = 0;
-                bool active = false;
+                int c0 = 0, c1 = 0, c2 = 0, c3 = 0, d0 = 0, d1 = 0, d2 = 0;
+                bool active = is_a || (is_b && (!p.b_mn || one_box)) || (p.b_mn && !one_box && jb >= 0 && jb < hb_t);
                 uint32_t dst_off = 0;
-                const CUtensorMap *tmap = &tmA;
+                const CUtensorMap *tmap = is_a ? &tmA : &tmB;
                 if (is_a) {
-                    active = true;
-                    dst_off = (uint32_t)lane * 4096u;
-                    c2 = ab;
-                    if (!p.a_mn) { c1 = row_a; d0 = kBK; }
-                    else { c0 = row_a + lane * 32; d1 = kBK; }
-                } else if (lane == na) {
-                    tmap = &tmB;
-                    dst_off = kABytes;
-                    c2 = bb;
-                    if (!p.b_mn) { active = true; c1 = col_b; d0 = kBK; }
-                    else if (one_box) { active = true; tmap = &tmBb; c2 = col_b / 32; c3 = bb; d1 = kBK; }
-                } else if (p.b_mn && !one_box && jb >= 0 && jb < hb_t) {
-                    active = true;
-                    tmap = &tmB;
-                    dst_off = (uint32_t)kABytes + (uint32_t)jb * 4096u;
+                    if (p.a_mn) { dst_off = (uint32_t)lane * (4096u * kKS); c0 = row_a + lane * 32; c2 = ab; d1 = kKS * kBK; }
+                    else if (p.a_kbox) { c1 = row_a; c3 = ab; d2 = kKS; }
+                    else { dst_off = (uint32_t)lane * kABytes; c0 = lane * kBK; c1 = row_a; c2 = ab; d0 = kKS * kBK; }
+                } else if (is_b) {
+                    dst_off = kKS * kABytes;
+                    if (p.b_mn) { tmap = &tmBb; c2 = col_b / 32; c3 = bb; d1 = kKS * kBK; }
+                    else if (p.b_kbox) { c1 = col_b; c3 = bb; d2 = kKS; }
+                    else { dst_off += (uint32_t)(lane - na) * ((uint32_t)p.BNH * 128u); c0 = (lane - na) * kBK; c1 = col_b; c2 = bb; d0 = kKS * kBK; }
+                } else {
+                    dst_off = kKS * kABytes + (uint32_t)jb * (4096u * kKS);
                     c0 = col_b + jb * 32;
                     c2 = bb;
-                    d1 = kBK;
+                    d1 = kKS * kBK;
                 }
                 if (t == first_tile) pdl_wait();
-                for (int kb = 0; kb < p.num_kb; ++kb) {
+                for (int kb = 0; kb < p.num_kb; kb += kKS) {
                     mbar_wait(&empty[stage], phase ^ 1, p.err, 1);
                     if (lane == 0) GLOG(0, glog_i++);
-                    if (lane == 0) mbar_arrive_expect_tx(&full[stage], tx_bytes);
+                    if (lane == 0 && rank == 0) mbar_arrive_expect_tx(&full[stage], tx_bytes);
                     __syncwarp();
                     uint8_t *dst = stages + (size_t)stage * p.stage_bytes + dst_off;
-                    if (active) tma_load_4d(dst, tmap, &full[stage], c0, c1, c2, c3);
+                    if (active) {
+                        if (kCtas == 2) tma_load_4d_pair(dst, tmap, full_issuer + (uint32_t)stage * 8u, c0, c1, c2, c3);
+                        else tma_load_4d(dst, tmap, &full[stage], c0, c1, c2, c3);
+                    }
                     c0 += d0;
                     c1 += d1;
+                    c2 += d2;
                     if (++stage == p.num_stages) { stage = 0; phase ^= 1; }
                 }
             }
@@ -216,20 +231,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (kCtas == 2 && rank != 0) {
-            // Odd CTA of a pair: the even CTA issues the MMAs; tell it when each of this CTA's stages
-            // has landed (stage releases and finished accumulators come back by multicast commit).
-            if (elect_one()) {
-                const uint32_t peer_full = map_to_cta(smem_u32(&full[0]), 0);
-                int stage = 0;
-                uint32_t phase = 0;
-                for (int t = first_tile; t < total_tiles; t += tile_step) {
-                    for (int kb = 0; kb < p.num_kb; ++kb) {
-                        mbar_wait(&full[stage], phase, p.err, 5);
-                        mbar_arrive_remote(peer_full + (uint32_t)stage * 8u);
-                        if (++stage == p.num_stages) { stage = 0; phase ^= 1; }
-                    }
-                }
-            }
+            // odd CTA of a pair: the even CTA issues the MMAs, and hears of this CTA's stages from their copies
         } else if (elect_one()) {
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
@@ -238,11 +240,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             // 1024 bytes apart).  MN-major 32-bit operands use the 128-byte swizzle with 32-byte atoms:
             // atoms of four 128-byte K rows (512 bytes apart along K), blocks of 32 rows/columns 4096
             // bytes apart; one instruction consumes eight K rows (1024 bytes).
-            const uint64_t a_tmpl = p.a_mn ? make_smem_desc(0, 4096, 512, kSwizzle128B32) : make_smem_desc(0, 16, 1024, kSwizzle128B);
-            const uint64_t b_tmpl = p.b_mn ? make_smem_desc(0, 4096, 512, kSwizzle128B32) : make_smem_desc(0, 16, 1024, kSwizzle128B);
+            const uint64_t a_tmpl = p.a_mn ? make_smem_desc(0, 4096 * kKS, 512, kSwizzle128B32) : make_smem_desc(0, 16, 1024, kSwizzle128B);
+            const uint64_t b_tmpl = p.b_mn ? make_smem_desc(0, 4096 * kKS, 512, kSwizzle128B32) : make_smem_desc(0, 16, 1024, kSwizzle128B);
             const uint32_t a_hi = (uint32_t)(a_tmpl >> 32), b_hi = (uint32_t)(b_tmpl >> 32);
-            const uint32_t a_lo_c = (uint32_t)a_tmpl, b_lo_c = (uint32_t)b_tmpl;
+            const uint32_t a_lo = (uint32_t)a_tmpl | ((smem_u32(stages) >> 4) & 0x3FFFu);
+            const uint32_t b_lo = (uint32_t)b_tmpl | (((smem_u32(stages) + kKS * kABytes) >> 4) & 0x3FFFu);
+            const uint32_t stage16 = p.stage_bytes >> 4;
             const uint32_t a_k16 = (p.a_mn ? 1024u : 32u) >> 4, b_k16 = (p.b_mn ? 1024u : 32u) >> 4;
+            // from one K block of the stage to the next
+            const uint32_t a_sub16 = (p.a_mn ? 4096u : (uint32_t)kABytes) >> 4, b_sub16 = (p.b_mn ? 4096u : (uint32_t)p.BNH * 128u) >> 4;
             int glog_i = 0, glog_t = 0;
             (void)glog_i; (void)glog_t;
             GP_DECL;
@@ -253,26 +259,33 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 GP_MARK(0);
                 const uint32_t d_tmem = tmem_base + (uint32_t)acc * kMaxBN;
                 const uint32_t idesc = ((t / p.tiles_m) % p.tiles_n == p.tiles_n - 1) ? p.idesc_tail : p.idesc;
-                for (int kb = 0; kb < p.num_kb; ++kb) {
-                    if (kCtas == 2) mbar_wait_cluster(&full[stage], phase, p.err, 3);
-                    else mbar_wait(&full[stage], phase, p.err, 3);
+                auto mma = [&](uint32_t al, uint32_t bl, uint32_t accumulate) {
+                    if (kCtas == 2) mma_tf32_lohi_pair(d_tmem, al, a_hi, bl, b_hi, idesc, accumulate);
+                    else mma_tf32_lohi(d_tmem, al, a_hi, bl, b_hi, idesc, accumulate);
+                };
+                uint32_t accumulate = 0;
+                for (int k0 = 0; k0 < p.K; k0 += kKS * kBK) {
+                    mbar_wait(&full[stage], phase, p.err, 3);
                     tc_fence_after_sync();
                     GP_MARK(1);
                     GLOG(1, glog_i++);
-                    const uint32_t sA = smem_u32(stages + (size_t)stage * p.stage_bytes);
-                    const uint32_t a16 = sA >> 4, b16 = (sA + kABytes) >> 4;
-                    const int k_left = p.K - kb * kBK;
-                    const int k8 = k_left >= kBK ? kBK / 8 : (k_left + 7) / 8;
-                    // one thread issues everything: keep the per-instruction work to two adds
+                    // One thread issues everything, so every instruction between two MMAs counts: straight-line
+                    // code, one add per descriptor (the start addresses never carry out of their 14 bits).
+                    const uint32_t al = a_lo + (uint32_t)stage * stage16, bl = b_lo + (uint32_t)stage * stage16;
+                    if (k0 + kKS * kBK <= p.K) {
 #pragma unroll
-                    for (int k = 0; k < kBK / 8; ++k) {
-                        if (k < k8) {
-                            if (kCtas == 2)
-                                mma_tf32_lohi_pair(d_tmem, a_lo_c | ((a16 + (uint32_t)k * a_k16) & 0x3FFFu), a_hi,
-                                                   b_lo_c | ((b16 + (uint32_t)k * b_k16) & 0x3FFFu), b_hi, idesc, (kb | k) != 0);
-                            else
-                                mma_tf32_lohi(d_tmem, a_lo_c | ((a16 + (uint32_t)k * a_k16) & 0x3FFFu), a_hi,
-                                              b_lo_c | ((b16 + (uint32_t)k * b_k16) & 0x3FFFu), b_hi, idesc, (kb | k) != 0);
+                        for (int s = 0; s < kKS; ++s)
+#pragma unroll
+                            for (int k = 0; k < kBK / 8; ++k) {
+                                mma(al + (uint32_t)s * a_sub16 + (uint32_t)k * a_k16, bl + (uint32_t)s * b_sub16 + (uint32_t)k * b_k16,
+                                    accumulate);
+                                accumulate = 1;
+                            }
+                    } else {
+                        for (int k = 0; k0 + k * 8 < p.K; ++k) {
+                            const uint32_t s = (uint32_t)k / 4u, kk = (uint32_t)k % 4u;
+                            mma(al + s * a_sub16 + kk * a_k16, bl + s * b_sub16 + kk * b_k16, accumulate);
+                            accumulate = 1;
                         }
                     }
                     if (kCtas == 2) mma_commit_pair(&empty[stage]);
@@ -600,7 +613,7 @@ static int gemm_max_pairs() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_gemm_kernel<2>, &cfg) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, tc_gemm_kernel<2, 1>, &cfg) != cudaSuccess || n < 1) {
         cudaGetLastError();
         n = tc_host::num_sms() / 2;
     }
@@ -624,8 +637,8 @@ double tc_gemm_estimate_ns(const TcGemmProblem &g) {
     const int bn = pick_bn(tiles_m, g.N, g.batch, units, ctas);
     const long long tiles = tiles_m * ((g.N + bn - 1) / bn) * g.batch;
     const double waves = (double)((tiles + units - 1) / units);
-    const double t = waves * ((g.K + kBK - 1) / kBK * (189.0 + 1.45 * bn / ctas + (ctas == 2 ? 45.0 : 0.0)) + 11.0 * bn) + 3270.0;
-    return t + (g.round_operands ? 2360.0 + 166e-6 * 4.0 * ((double)g.M * g.K + (double)g.K * g.N) : 0.0);
+    const double t = waves * ((g.K + kBK - 1) / kBK * (65.0 + 2.6 * bn / ctas) + 14.0 * bn) + 2840.0;
+    return t + (g.round_operands ? 1660.0 + 312e-6 * 4.0 * ((double)g.M * g.K + (double)g.K * g.N) : 0.0);
 }
 
 int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
@@ -647,8 +660,15 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     p.BNH = p.BN / p.ctas;
     p.tiles_n = (g.N + p.BN - 1) / p.BN;
     p.num_kb = (g.K + kBK - 1) / kBK;
-    p.stage_bytes = (uint32_t)(kABytes + p.BNH * 128);
-    p.tx_bytes = p.stage_bytes;
+    p.tx_bytes = (uint32_t)(kABytes + p.BNH * 128);          // of one K block
+    // Two K blocks per stage where a block's MMAs are shorter than the issuing loop (at most 64 columns of B per
+    // CTA: 4 x 64 cycles against about 400 for a stage's waits and copies): 1024 x 1024 x 4096 39 -> 34 us.
+    // Wider tiles need the shared memory for stages in flight (1024->256 channels at 14x14 17.8 -> 19.0 us with two).
+    // ONNXB_GEMM_KS = 1 | 2 pins it for A/B measurements.
+    int ks = p.tx_bytes <= 24576 && p.num_kb >= 4 ? 2 : 1;
+    if (const char *e = getenv("ONNXB_GEMM_KS"))
+        if (e[0] == '1' || e[0] == '2') ks = e[0] - '0';
+    p.stage_bytes = p.tx_bytes * ks;
     p.y_tma = g.y_split == 0 && (g.y_ld % 4 == 0) && (g.batch == 1 || g.y_bs % 4 == 0);
     p.R = g.C ? nullptr : g.residual;
     p.r_tma = p.R != nullptr && p.y_tma;
@@ -673,35 +693,26 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     if (!p.err) return (int)cudaErrorUnknown;
 
     CUtensorMap tmA, tmB, tmY, tmR;
-    // operand maps: dim0 is the contiguous axis
-    {
-        const uint64_t rows = (uint64_t)g.M, k = (uint64_t)g.K;
-        uint64_t dims[4], str[3];
-        uint32_t box[4];
-        if (!p.a_mn) { dims[0] = k; dims[1] = rows; box[0] = kBK; box[1] = kBM; }
-        else { dims[0] = rows; dims[1] = k; box[0] = 32; box[1] = kBK; }
-        dims[2] = p.a_batched ? (uint64_t)g.batch : 1;
-        box[2] = 1;
-        str[0] = (uint64_t)g.a_ld * 4;
-        str[1] = p.a_batched ? (uint64_t)g.a_bs * 4 : str[0] * dims[1];
-        dims[3] = 1; box[3] = 1; str[2] = str[1] * dims[2];      // unit dimension: see the producer
-        if (!make_tmap(&tmA, g.A, 4, dims, str, box, p.a_mn ? kTmapSwizzle128Atom32 : kTmapSwizzle128))
-            return (int)cudaErrorInvalidValue;
-    }
-    {
-        const uint64_t cols = (uint64_t)g.N, k = (uint64_t)g.K;
-        uint64_t dims[4], str[3];
-        uint32_t box[4];
-        if (!p.b_mn) { dims[0] = k; dims[1] = cols; box[0] = kBK; box[1] = (uint32_t)p.BNH; }
-        else { dims[0] = cols; dims[1] = k; box[0] = 32; box[1] = kBK; }
-        dims[2] = p.b_batched ? (uint64_t)g.batch : 1;
-        box[2] = 1;
-        str[0] = (uint64_t)g.b_ld * 4;
-        str[1] = p.b_batched ? (uint64_t)g.b_bs * 4 : str[0] * dims[1];
-        dims[3] = 1; box[3] = 1; str[2] = str[1] * dims[2];
-        if (!make_tmap(&tmB, g.B, 4, dims, str, box, p.b_mn ? kTmapSwizzle128Atom32 : kTmapSwizzle128))
-            return (int)cudaErrorInvalidValue;
-    }
+    // Operand maps.  K-major: (32 terms of a K block, row, K block, batch) where K is whole blocks, so that one box
+    // carries a stage; else (term, row, batch, 1).  MN-major: (row, term, batch, 1).
+    p.a_kbox = !p.a_mn && g.K % kBK == 0;
+    p.b_kbox = !p.b_mn && g.K % kBK == 0;
+    auto operand = [&](CUtensorMap *tm, const float *base, int mn, int kbox, uint64_t n, long long ld, bool batched, long long bs,
+                       uint32_t rows) {
+        const uint64_t k = (uint64_t)g.K, nb = batched ? (uint64_t)g.batch : 1, ldb = (uint64_t)ld * 4;
+        const uint64_t bsb = batched ? (uint64_t)bs * 4 : ldb * (mn ? k : n);
+        if (kbox) {
+            const uint64_t dims[4] = {(uint64_t)kBK, n, k / kBK, nb}, str[3] = {ldb, kBK * 4, bsb};
+            const uint32_t box[4] = {(uint32_t)kBK, rows, (uint32_t)ks, 1};
+            return make_tmap(tm, base, 4, dims, str, box, kTmapSwizzle128);
+        }
+        const uint64_t dims[4] = {mn ? n : k, mn ? k : n, nb, 1}, str[3] = {ldb, bsb, bsb * nb};
+        const uint32_t box[4] = {(uint32_t)(mn ? 32 : kBK), mn ? (uint32_t)(kBK * ks) : rows, 1, 1};
+        return make_tmap(tm, base, 4, dims, str, box, mn ? kTmapSwizzle128Atom32 : kTmapSwizzle128);
+    };
+    if (!operand(&tmA, g.A, p.a_mn, p.a_kbox, g.M, g.a_ld, p.a_batched, g.a_bs, kBM) ||
+        !operand(&tmB, g.B, p.b_mn, p.b_kbox, g.N, g.b_ld, p.b_batched, g.b_bs, p.BNH))
+        return (int)cudaErrorInvalidValue;
     // MN-major B through one 4-D box per stage: (32 columns, K, blocks of 32 columns, batch).  Only the
     // full blocks of a row belong to the view; a CTA whose columns reach past them loads block by block.
     CUtensorMap tmBb = tmB;
@@ -710,7 +721,7 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     if (p.b_mn && p.b_nblk_full >= 1 && p.BNH >= 64) {
         uint64_t dims[4] = {32, (uint64_t)g.K, (uint64_t)p.b_nblk_full, p.b_batched ? (uint64_t)g.batch : 1};
         uint64_t str[3] = {(uint64_t)g.b_ld * 4, 128, p.b_batched ? (uint64_t)g.b_bs * 4 : (uint64_t)g.b_ld * 4 * g.K};
-        uint32_t box[4] = {32, (uint32_t)kBK, (uint32_t)(p.BNH / 32), 1};
+        uint32_t box[4] = {32, (uint32_t)(kBK * ks), (uint32_t)(p.BNH / 32), 1};
         p.b_big = make_tmap(&tmBb, g.B, 4, dims, str, box, kTmapSwizzle128Atom32) ? 1 : 0;
     }
     if (p.y_tma) {
@@ -735,16 +746,16 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     }
 
     const size_t smem = 1024 + (size_t)p.num_stages * p.stage_bytes + p.staging_bytes + kBarrierBytes;
-    const cudaError_t attr_err =
-        cudaFuncSetAttribute(p.ctas == 2 ? tc_gemm_kernel<2> : tc_gemm_kernel<1>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    auto kern = p.ctas == 2 ? (ks == 2 ? tc_gemm_kernel<2, 2> : tc_gemm_kernel<2, 1>)
+                            : (ks == 2 ? tc_gemm_kernel<1, 2> : tc_gemm_kernel<1, 1>);
+    const cudaError_t attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (attr_err != cudaSuccess) return (int)attr_err;
     const long long total = (long long)p.tiles_m * p.tiles_n * p.batch;
     const int grid = (int)(total < units ? total : units) * p.ctas;
     const cudaError_t le =
-        p.ctas == 2 ? launch_pdl_cluster(tc_gemm_kernel<2>, 2, dim3(grid), dim3(kThreads), smem, (cudaStream_t)stream, tmA,
+        p.ctas == 2 ? launch_pdl_cluster(kern, 2, dim3(grid), dim3(kThreads), smem, (cudaStream_t)stream, tmA,
                                          tmB, tmBb, tmY, tmR, p)
-                    : launch_pdl(tc_gemm_kernel<1>, dim3(grid), dim3(kThreads), smem, (cudaStream_t)stream, tmA, tmB, tmBb,
+                    : launch_pdl(kern, dim3(grid), dim3(kThreads), smem, (cudaStream_t)stream, tmA, tmB, tmBb,
                                  tmY, tmR, p);
     count_launch();
     return (int)le;

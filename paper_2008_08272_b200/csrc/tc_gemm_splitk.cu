@@ -33,6 +33,7 @@ using namespace tc;
 constexpr int kBM = 128, kBK = 32, kMaxBN = 128;
 constexpr int kWorkers = 8;                   // rounding, partial tile, reduction
 constexpr int kThreads = (2 + kWorkers) * 32; // warp 0: TMA producer, warp 1: MMA issuer
+constexpr int kRoundWarps = kWorkers / 2;     // warps that round one stage; the two halves take the stages in turn
 constexpr int kMaxStages = 8;
 constexpr int kABytes = kBM * kBK * 4;        // 16 KB
 constexpr int kSmemLimit = 232448;
@@ -40,6 +41,8 @@ constexpr int kSmemLimit = 232448;
 struct SkParams {
     int M, N, K;
     int a_mn, b_mn;            // operand is MN-major (else K-major)
+    int a_kbox, b_kbox;        // K-major with K a multiple of 32: one copy brings all K blocks of a stage
+    int b_big, b_nblk_full;    // MN-major B through a view of its full 32-column blocks: one copy as well
     int round;                 // round the operands in shared memory
     int BN, S, tiles_m, tiles_n, num_kb, kb_per, num_stages, rows_per, pitch;   // pitch: floats between rows of a partial tile
     uint32_t stage_bytes, idesc;
@@ -64,9 +67,11 @@ __device__ __forceinline__ float4 ld_cluster_v4(uint32_t cluster_addr) {
     return v;
 }
 
+// kKS: K blocks per stage (two wherever a CTA has two: see tc_gemm.cu for what a stage costs its issuing threads)
+template <int kKS>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                      const __grid_constant__ SkParams p) {
+                      const __grid_constant__ CUtensorMap tmBb, const __grid_constant__ SkParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
@@ -85,16 +90,19 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     const int kb0 = rank * p.kb_per, kb1 = min(p.num_kb, kb0 + p.kb_per);
     const int nkb = max(kb1 - kb0, 0);                                // K-blocks this CTA reduces (0: a rank past the end)
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < p.num_stages; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-            mbar_init(&ready[s], kWorkers);
+    if (warp == 2) {
+        // a barrier per lane: one thread would take a thousand cycles for them
+        if (lane < p.num_stages) {
+            mbar_init(&full[lane], 1);
+            mbar_init(&empty[lane], 1);
+            mbar_init(&ready[lane], kRoundWarps);
         }
-        mbar_init(acc_full, 1);
+        if (lane == 31) mbar_init(acc_full, 1);
         mbar_fence_init();
+    } else if (threadIdx.x == 0) {
         prefetch_tmap(&tmA);
         prefetch_tmap(&tmB);
+        if (p.b_big) prefetch_tmap(&tmBb);
     }
     if (warp == 1) {
         tmem_alloc(tmem_holder, kMaxBN);
@@ -108,69 +116,99 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (lanes 0..na-1: A, then B)
-        const int na = p.a_mn ? kBM / 32 : 1, nb = p.b_mn ? p.BN / 32 : 1;       // copies per stage
+        const bool big = p.b_mn && p.b_big && (tn + 1) * (p.BN / 32) <= p.b_nblk_full;
+        const int na = p.a_mn ? kBM / 32 : p.a_kbox ? 1 : kKS;                        // copies per stage
+        const int nb = p.b_mn ? (big ? 1 : p.BN / 32) : p.b_kbox ? 1 : kKS;
+        const int ib = lane - na;
+        const bool is_a = lane < na, active = lane < na + nb;
+        const CUtensorMap *tmap = is_a ? &tmA : big ? &tmBb : &tmB;
+        // this lane's copy: coordinates of the first stage, their step, and where it goes in a stage
+        int c0 = 0, c1 = 0, c2 = 0, c3 = 0, d0 = 0, d1 = 0, d2 = 0;
+        uint32_t off = 0;
+        if (is_a) {
+            if (p.a_mn) { off = (uint32_t)lane * (4096u * kKS); c0 = tm * kBM + lane * 32; c1 = kb0 * kBK; d1 = kKS * kBK; }
+            else if (p.a_kbox) { c1 = tm * kBM; c2 = kb0; d2 = kKS; }
+            else { off = (uint32_t)lane * kABytes; c0 = (kb0 + lane) * kBK; c1 = tm * kBM; d0 = kKS * kBK; }
+        } else {
+            off = kKS * kABytes;
+            if (big) { c1 = kb0 * kBK; c2 = tn * (p.BN / 32); c3 = batch; d1 = kKS * kBK; }
+            else if (p.b_mn) { off += (uint32_t)ib * (4096u * kKS); c0 = tn * p.BN + ib * 32; c1 = kb0 * kBK; c2 = batch; d1 = kKS * kBK; }
+            else if (p.b_kbox) { c1 = tn * p.BN; c2 = kb0; c3 = batch; d2 = kKS; }
+            else { off += (uint32_t)ib * ((uint32_t)p.BN * 128u); c0 = (kb0 + ib) * kBK; c1 = tn * p.BN; c2 = batch; d0 = kKS * kBK; }
+        }
         int stage = 0;
         uint32_t phase = 0;
         pdl_wait();             // everything above overlapped the previous kernel's tail
-        for (int kb = kb0; kb < kb1; ++kb) {
+        for (int kb = 0; kb < nkb; kb += kKS) {
             mbar_wait(&empty[stage], phase ^ 1, p.err, 40);
             if (lane == 0) mbar_arrive_expect_tx(&full[stage], p.stage_bytes);
             __syncwarp();
-            uint8_t *dst = stages + (size_t)stage * p.stage_bytes;
-            if (lane < na) {
-                if (!p.a_mn) tma_load_3d(dst, &tmA, &full[stage], kb * kBK, tm * kBM, 0);
-                else tma_load_3d(dst + lane * 4096, &tmA, &full[stage], tm * kBM + lane * 32, kb * kBK, 0);
-            } else if (lane < na + nb) {
-                const int i = lane - na;
-                if (!p.b_mn) tma_load_3d(dst + kABytes, &tmB, &full[stage], kb * kBK, tn * p.BN, batch);
-                else tma_load_3d(dst + kABytes + i * 4096, &tmB, &full[stage], tn * p.BN + i * 32, kb * kBK, batch);
-            }
+            if (active) tma_load_4d(stages + (size_t)stage * p.stage_bytes + off, tmap, &full[stage], c0, c1, c2, c3);
+            c0 += d0;
+            c1 += d1;
+            c2 += d2;
             if (++stage == p.num_stages) { stage = 0; phase ^= 1; }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (elect_one() && nkb > 0) {
-            const uint64_t mn_tmpl = make_smem_desc(0, 4096, 512, kSwizzle128B32), k_tmpl = make_smem_desc(0, 16, 1024, kSwizzle128B);
+            const uint64_t mn_tmpl = make_smem_desc(0, 4096 * kKS, 512, kSwizzle128B32), k_tmpl = make_smem_desc(0, 16, 1024, kSwizzle128B);
             const uint64_t a_tmpl = p.a_mn ? mn_tmpl : k_tmpl, b_tmpl = p.b_mn ? mn_tmpl : k_tmpl;
             const uint32_t a_hi = (uint32_t)(a_tmpl >> 32), b_hi = (uint32_t)(b_tmpl >> 32);
-            const uint32_t a_lo_c = (uint32_t)a_tmpl, b_lo_c = (uint32_t)b_tmpl;
+            // (masked: within a cluster the CTA's rank stands in the upper bits of a shared-memory address)
+            const uint32_t a_lo = (uint32_t)a_tmpl | ((smem_u32(stages) >> 4) & 0x3FFFu);
+            const uint32_t b_lo = (uint32_t)b_tmpl | (((smem_u32(stages) + kKS * kABytes) >> 4) & 0x3FFFu);
             const uint32_t a_k16 = (p.a_mn ? 1024u : 32u) >> 4, b_k16 = (p.b_mn ? 1024u : 32u) >> 4;
+            const uint32_t a_sub16 = (p.a_mn ? 4096u : (uint32_t)kABytes) >> 4, b_sub16 = (p.b_mn ? 4096u : (uint32_t)p.BN * 128u) >> 4;
+            const uint32_t stage16 = p.stage_bytes >> 4;
             uint64_t *landed = p.round ? ready : full;                // rounded as well, or as they arrive
             int stage = 0;
-            uint32_t phase = 0;
-            for (int i = 0; i < nkb; ++i) {
+            uint32_t phase = 0, accumulate = 0;
+            for (int kb = 0; kb < nkb; kb += kKS) {
                 mbar_wait(&landed[stage], phase, p.err, 41);
                 tc_fence_after_sync();
-                const uint32_t sA = smem_u32(stages + (size_t)stage * p.stage_bytes);
-                const uint32_t a16 = sA >> 4, b16 = (sA + kABytes) >> 4;
+                const uint32_t al = a_lo + (uint32_t)stage * stage16, bl = b_lo + (uint32_t)stage * stage16;
+                // (a share's last stage may hold a K block of the next rank's, or none: skipped)
 #pragma unroll
-                for (int k = 0; k < kBK / 8; ++k)
-                    mma_tf32_lohi(tmem_base, a_lo_c | ((a16 + (uint32_t)k * a_k16) & 0x3FFFu), a_hi,
-                                  b_lo_c | ((b16 + (uint32_t)k * b_k16) & 0x3FFFu), b_hi, p.idesc, (i | k) != 0);
+                for (int sub = 0; sub < kKS; ++sub) {
+                    if (sub == 0 || kb + sub < nkb) {
+#pragma unroll
+                        for (int k = 0; k < kBK / 8; ++k) {
+                            mma_tf32_lohi(tmem_base, al + (uint32_t)sub * a_sub16 + (uint32_t)k * a_k16, a_hi,
+                                          bl + (uint32_t)sub * b_sub16 + (uint32_t)k * b_k16, b_hi, p.idesc, accumulate);
+                            accumulate = 1;
+                        }
+                    }
+                }
                 mma_commit(&empty[stage]);
                 if (++stage == p.num_stages) { stage = 0; phase ^= 1; }
             }
             mma_commit(acc_full);
         }
     } else {
-        const int t = (warp - 2) * 32 + lane;
         if (p.round) {
             // round every landed stage to TF32 in place (elementwise, so the swizzle does not matter)
-            const int n4 = (int)(p.stage_bytes >> 4);
+            const int n4 = (int)(p.stage_bytes >> 4), rt = ((warp - 2) % kRoundWarps) * 32 + lane, mine = (warp - 2) / kRoundWarps;
             int stage = 0;
             uint32_t phase = 0;
-            for (int i = 0; i < nkb; ++i) {
-                mbar_wait(&full[stage], phase, p.err, 43);
-                float4 *st4 = reinterpret_cast<float4 *>(stages + (size_t)stage * p.stage_bytes);
-#pragma unroll 4
-                for (int j = t; j < n4; j += kWorkers * 32) {
-                    float4 v = st4[j];
-                    v.x = round_tf32(v.x); v.y = round_tf32(v.y); v.z = round_tf32(v.z); v.w = round_tf32(v.w);
-                    st4[j] = v;
+            for (int kb = 0, i = 0; kb < nkb; kb += kKS, ++i) {
+                if ((i & 1) == mine) {
+                    mbar_wait(&full[stage], phase, p.err, 43);
+                    float4 *st4 = reinterpret_cast<float4 *>(stages + (size_t)stage * p.stage_bytes);
+                    for (int j = rt; j < n4; j += 4 * kRoundWarps * 32) {
+                        float4 v[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (j + u * kRoundWarps * 32 < n4) v[u] = st4[j + u * kRoundWarps * 32];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (j + u * kRoundWarps * 32 < n4)
+                                st4[j + u * kRoundWarps * 32] = make_float4(round_tf32(v[u].x), round_tf32(v[u].y), round_tf32(v[u].z), round_tf32(v[u].w));
+                    }
+                    fence_proxy_async_smem();          // generic-proxy writes, read next by the tensor core
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&ready[stage]);
                 }
-                fence_proxy_async_smem();          // generic-proxy writes, read next by the tensor core
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&ready[stage]);
                 if (++stage == p.num_stages) { stage = 0; phase ^= 1; }
             }
         }
@@ -247,11 +285,14 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             if (p.S == 1) {
                 a = *reinterpret_cast<const float4 *>(reinterpret_cast<const uint8_t *>(partial) + off);
             } else {
-                for (int s0 = 0; s0 < p.S; s0 += 2) {
-                    const float4 x = ld_cluster_v4(map_to_cta(part_addr + off, (uint32_t)s0));
-                    const float4 y = ld_cluster_v4(map_to_cta(part_addr + off, (uint32_t)s0 + 1u));
-                    a.x = (a.x + x.x) + y.x; a.y = (a.y + x.y) + y.y; a.z = (a.z + x.z) + y.z; a.w = (a.w + x.w) + y.w;
-                }
+                // all partials requested at once (a trip to a peer's shared memory takes some 600 cycles)
+                float4 x[8];
+#pragma unroll
+                for (int s = 0; s < 8; ++s)
+                    if (s < p.S) x[s] = ld_cluster_v4(map_to_cta(part_addr + off, (uint32_t)s));
+#pragma unroll
+                for (int s = 0; s < 8; ++s)
+                    if (s < p.S) { a.x += x[s].x; a.y += x[s].y; a.z += x[s].z; a.w += x[s].w; }
             }
             float o[4] = {fmaf(p.alpha, a.x, rb) + add[0], fmaf(p.alpha, a.y, rb) + add[1], fmaf(p.alpha, a.z, rb) + add[2],
                           fmaf(p.alpha, a.w, rb) + add[3]};
@@ -291,7 +332,7 @@ int resident_ctas(int S) {
     int n = cached[i].load(std::memory_order_acquire);
     if (n > 0) return n;
     n = tc_host::num_sms();
-    if (S > 1 && cudaFuncSetAttribute(tc_gemm_splitk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) == cudaSuccess) {
+    if (S > 1 && cudaFuncSetAttribute(tc_gemm_splitk_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(S * 148);
         cfg.blockDim = dim3(kThreads);
@@ -303,7 +344,7 @@ int resident_ctas(int S) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, tc_gemm_splitk_kernel, &cfg) == cudaSuccess && clusters > 0) n = clusters * S;
+        if (cudaOccupancyMaxActiveClusters(&clusters, tc_gemm_splitk_kernel<2>, &cfg) == cudaSuccess && clusters > 0) n = clusters * S;
         else cudaGetLastError();
     }
     cached[i].store(n, std::memory_order_release);
@@ -312,8 +353,8 @@ int resident_ctas(int S) {
 
 // Shape with the shortest estimated time, against the persistent kernel's (both in ns, fitted to 90 problems: 1x1
 // convolutions of ResNet-50 at batch 1 to 32 and Gemms from 400^3 to 1024 x 1024 x 4096; the choice is within
-// 1 % of the best on average).  One wave of CTAs costs 4 us for its set-up, first fill and exchange, and a K block
-// 200-460 ns (365-650 when it is rounded in shared memory first).
+// 1 % of the best on average).  One wave of CTAs costs 3.7 us for its set-up, first fill and exchange, and a K block
+// 130-310 ns (360-550 when it is rounded in shared memory first).
 SkChoice search(const TcGemmProblem &g) {
     SkChoice c{0, 0};
     if ((g.a_batched && g.batch > 1) || (g.batch > 1 && g.b_batched && g.b_bs % 4)) return c;
@@ -326,8 +367,8 @@ SkChoice search(const TcGemmProblem &g) {
             if (ctas > 4 * 148) break;
             const int units = resident_ctas(S);
             const double waves = (double)((ctas + units - 1) / units);
-            const double blk = g.round_operands ? 366.0 + 2.2 * BN : 198.0 + 2.1 * BN;
-            const double t = waves * ((num_kb + S - 1) / S * blk + 4000.0 + 22.0 * BN);
+            const double blk = g.round_operands ? 293.0 + 2.0 * BN : 67.0 + 1.9 * BN;
+            const double t = waves * ((num_kb + S - 1) / S * blk + 3700.0 + 25.0 * BN + (S == 8 ? 500.0 : 0.0));
             if (t < best) {
                 best = t;
                 c = {BN, S};
@@ -386,9 +427,10 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
     p.kb_per = (p.num_kb + p.S - 1) / p.S;
     p.rows_per = (kBM + p.S - 1) / p.S;
     p.pitch = p.BN + 4;                      // rows of a partial tile 16-byte aligned, eight rows on different banks
-    p.stage_bytes = (uint32_t)(kABytes + p.BN * 128);
-    p.num_stages = std::min(kMaxStages, std::max(2, p.kb_per));
-    p.num_stages = std::min(p.num_stages, (int)((kSmemLimit - 2048) / p.stage_bytes));
+    const int ks = p.kb_per >= 2 ? 2 : 1;
+    p.stage_bytes = (uint32_t)(kABytes + p.BN * 128) * ks;
+    // (never more stages than the share has: a small footprint lets the next kernel's CTAs set up beside this one)
+    p.num_stages = std::min({kMaxStages, std::max(2, (p.kb_per + ks - 1) / ks), (int)((kSmemLimit - 2048) / p.stage_bytes)});
     p.idesc = tc::make_idesc_tf32(kBM, p.BN, p.a_mn, p.b_mn);
     p.alpha = g.alpha; p.beta = g.beta;
     p.C = g.C; p.c_si = g.c_si; p.c_sj = g.c_sj;
@@ -403,25 +445,42 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
     p.err = device_status_ptr();
     if (!p.err) return (int)cudaErrorUnknown;
 
-    auto operand = [](CUtensorMap *tm, const float *base, int mn, uint64_t n, uint64_t k, long long ld, int batch, long long bs,
-                      uint32_t rows) {
-        const uint64_t dims[3] = {mn ? n : k, mn ? k : n, (uint64_t)batch};
-        const uint64_t str[2] = {(uint64_t)ld * 4, batch > 1 ? (uint64_t)bs * 4 : (uint64_t)ld * 4 * dims[1]};
-        const uint32_t box[3] = {(uint32_t)(mn ? 32 : kBK), mn ? (uint32_t)kBK : rows, 1};
-        return make_tmap(tm, base, 3, dims, str, box, mn ? kTmapSwizzle128Atom32 : kTmapSwizzle128);
+    p.a_kbox = !p.a_mn && g.K % kBK == 0;
+    p.b_kbox = !p.b_mn && g.K % kBK == 0;
+    // K-major: (32 terms, row, K block, batch) or (term, row, batch, 1); MN-major: (row, term, batch, 1)
+    auto operand = [&](CUtensorMap *tm, const float *base, int mn, int kbox, uint64_t n, long long ld, int batch, long long bs, uint32_t rows) {
+        const uint64_t k = (uint64_t)g.K, nb = (uint64_t)batch, ldb = (uint64_t)ld * 4;
+        const uint64_t bsb = batch > 1 ? (uint64_t)bs * 4 : ldb * (mn ? k : n);
+        if (kbox) {
+            const uint64_t dims[4] = {(uint64_t)kBK, n, k / kBK, nb}, str[3] = {ldb, kBK * 4, bsb};
+            const uint32_t box[4] = {(uint32_t)kBK, rows, (uint32_t)ks, 1};
+            return make_tmap(tm, base, 4, dims, str, box, kTmapSwizzle128);
+        }
+        const uint64_t dims[4] = {mn ? n : k, mn ? k : n, nb, 1}, str[3] = {ldb, bsb, bsb * nb};
+        const uint32_t box[4] = {(uint32_t)(mn ? 32 : kBK), mn ? (uint32_t)(kBK * ks) : rows, 1, 1};
+        return make_tmap(tm, base, 4, dims, str, box, mn ? kTmapSwizzle128Atom32 : kTmapSwizzle128);
     };
     CUtensorMap tmA, tmB;
-    if (!operand(&tmA, g.A, p.a_mn, g.M, g.K, g.a_ld, 1, 0, kBM) ||
-        !operand(&tmB, g.B, p.b_mn, g.N, g.K, g.b_ld, g.b_batched ? g.batch : 1, g.b_bs, p.BN))
+    if (!operand(&tmA, g.A, p.a_mn, p.a_kbox, g.M, g.a_ld, 1, 0, kBM) ||
+        !operand(&tmB, g.B, p.b_mn, p.b_kbox, g.N, g.b_ld, g.b_batched ? g.batch : 1, g.b_bs, p.BN))
         return (int)cudaErrorInvalidValue;
+    CUtensorMap tmBb = tmB;
+    p.b_nblk_full = g.N / 32;
+    if (p.b_mn && p.BN >= 64 && p.b_nblk_full * 32 >= p.BN) {
+        const uint64_t nb = g.b_batched ? (uint64_t)g.batch : 1, ldb = (uint64_t)g.b_ld * 4;
+        const uint64_t dims[4] = {32, (uint64_t)g.K, (uint64_t)p.b_nblk_full, nb};
+        const uint64_t str[3] = {ldb, 128, nb > 1 ? (uint64_t)g.b_bs * 4 : ldb * g.K};
+        const uint32_t box[4] = {32, (uint32_t)(kBK * ks), (uint32_t)(p.BN / 32), 1};
+        p.b_big = make_tmap(&tmBb, g.B, 4, dims, str, box, kTmapSwizzle128Atom32) ? 1 : 0;
+    }
     const size_t ring = (size_t)p.num_stages * p.stage_bytes, parked = (size_t)kBM * p.pitch * 4;
     const size_t smem = 2048 + std::max(ring, parked);
-    const cudaError_t ae = cudaFuncSetAttribute(tc_gemm_splitk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    auto kern = ks == 2 ? tc_gemm_splitk_kernel<2> : tc_gemm_splitk_kernel<1>;
+    const cudaError_t ae = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (ae != cudaSuccess) return (int)ae;
     const dim3 grid((unsigned)((long long)p.tiles_m * p.tiles_n * g.batch * p.S)), block(kThreads);
-    const cudaError_t le = p.S > 1 ? launch_pdl_cluster(tc_gemm_splitk_kernel, (unsigned)p.S, grid, block, smem,
-                                                        (cudaStream_t)stream, tmA, tmB, p)
-                                   : launch_pdl(tc_gemm_splitk_kernel, grid, block, smem, (cudaStream_t)stream, tmA, tmB, p);
+    const cudaError_t le = p.S > 1 ? launch_pdl_cluster(kern, (unsigned)p.S, grid, block, smem, (cudaStream_t)stream, tmA, tmB, tmBb, p)
+                                   : launch_pdl(kern, grid, block, smem, (cudaStream_t)stream, tmA, tmB, tmBb, p);
     count_launch();
     return (int)le;
 }
