@@ -6,12 +6,12 @@
 // formed; per block of KB input channels
 //   warp 0      stages the raw NCHW rows the tile touches into shared memory by TMA
 //               (zero fill outside the tensor);
-//   warps 4-11  re-lay them into the K-major "4 channels x slot" operand layout of the MMA,
+//   warps 4-15  re-lay them into the K-major "4 channels x slot" operand layout of the MMA,
 //               rounding fp32 to TF32 (nearest) and writing zeros for padding;
 //   warp 1      streams the pre-packed, pre-rounded weights by bulk copy;
 //   warp 2      issues, for every tap, tcgen05.mma on the SAME activation tile at a start address
 //               shifted by the tap's slot offset, accumulating in TMEM;
-//   warps 12-19 read finished accumulators back (tcgen05.ld), add bias, apply Relu and store NCHW
+//   warps 16-23 read finished accumulators back (tcgen05.ld), add bias, apply Relu and store NCHW
 //               with lanes along consecutive pixels (coalesced); when a tile's accumulators fill at
 //               most half of TMEM it holds two sets, so this overlaps the next tile's MMAs.
 // CTA pairs (kCtas = 2): two CTAs of a cluster share one tile of 2 x MT x 128 pixels.  Each stages
@@ -44,24 +44,25 @@ namespace {
 
 using namespace tc;
 
-// Warps: raw producer, weight producer, MMA issuer, relay, 8 transform warps, then kEpi (8 or 4) epilogue
-// warps.  With 8 epilogue warps the block has 640 threads and 96 registers per thread; with 4 it has 512
-// and 128, which the transform warps (ten independent address chains, twenty values in flight) turn into
-// speed: layers bound by the transform and with several tiles per CTA (so that the slower epilogue
-// hides behind the next tile) take the 4-warp form.
-constexpr int kXformWarps = 8;
-constexpr int kXformThreads = kXformWarps * 32;
+// Warps: raw producer, weight producer, MMA issuer, relay, then 12 transform warps and 8 epilogue warps: 768 threads,
+// 80 registers each.  Both kernels below stay within them without a spill, on purpose: with 227 KB of shared memory
+// per CTA next to no L1 is left, and a value spilled in a transform loop is a trip to L2 (the same kernel with 40 to 90
+// bytes of spills took 51.6 us on the 64-channel 56x56 layer at batch 64, without them 44.3; the stem 101 -> 78).
+constexpr int kXformWarps = 12, kXformThreads = kXformWarps * 32, kEpiWarps = 8;
 constexpr int kRelayWarp = 3;               // odd CTA of a pair: passes "operand stage written" on to the issuing CTA
 constexpr int kFirstXformWarp = 4, kFirstEpiWarp = kFirstXformWarp + kXformWarps;
-constexpr int threads_for(int epi_warps) { return (kFirstEpiWarp + epi_warps) * 32; }
-constexpr int kOwned = 10;                 // (slot, chunk) units of an A stage one transform thread may own
+constexpr int kThreads = (kFirstEpiWarp + kEpiWarps) * 32;
+constexpr int kMaxUnits = 2560;             // (slot, chunk) pairs of an A stage at most
+// units of an A stage one transform thread may own (see there): blocks of one chunk, or of several
+constexpr int kOwnedThin = (kMaxUnits + kXformThreads - 1) / kXformThreads, kOwnedThick = 2;
 constexpr int kMaxRawStages = 4;
 constexpr int kMaxAStages = 3;
-constexpr int kMaxSpb = 8;                 // K-steps per weight stage (the MMA issue loop is unrolled over them)
+constexpr int kMaxSpb = 9;                 // K-steps per weight stage (the MMA issue loop is unrolled over them)
 constexpr int kMaxBStages = 12;
 constexpr int kSmemLimit = 232448;
 constexpr int kBarBytes = 512;
 constexpr int kSegBytes = 256;             // >= sizeof(TcConvSegs)
+constexpr int kBiasBytes = 8 * 128;        // 32 biases per epilogue warp
 static_assert(sizeof(TcConvSegs) <= kSegBytes, "segment table does not fit its slot");
 
 struct Bars {
@@ -129,11 +130,13 @@ __device__ __forceinline__ int cb_rotation(long long tile, int ncb) { return (in
 // [r * cb_per, (r + 1) * cb_per), parks its partial tile in shared memory (over the stages, which are done with),
 // and after a cluster barrier sums one slice of the tile's channels over all partials through distributed
 // shared memory, in rank order.  One 14x14 image, 256 -> 256 channels: 24 -> 8 us.
-template <int kCtas, bool kAdd, int kEpiWarps, bool kSplit>
-__global__ void __launch_bounds__(threads_for(kEpiWarps), 1)
+// kThin: blocks of one 4-channel chunk (tap pairs).
+template <int kCtas, bool kAdd, bool kThin, bool kSplit>
+__global__ void __launch_bounds__(kThreads, 1)
 tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, const float *__restrict__ X,
                const float *__restrict__ Wpk, const float *__restrict__ bias, const float *__restrict__ R,
                float *__restrict__ Y, unsigned int *err) {
+    constexpr int kOwned = kThin ? kOwnedThin : kOwnedThick;
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment by pointer arithmetic on the shared array itself, so that the compiler
     // keeps treating everything derived from it as shared memory (LDS/STS, not generic accesses)
@@ -142,7 +145,8 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
     uint8_t *raw_st = a_st + (size_t)g.na_stages * g.a_stage_bytes;
     uint8_t *b_st = raw_st + (size_t)g.nr_stages * g.raw_stage_bytes;
     uint8_t *seg_st = b_st + (size_t)g.nb_stages * g.b_stage_bytes;
-    Bars *bars = reinterpret_cast<Bars *>(seg_st + kMaxRawStages * kSegBytes);
+    uint8_t *bias_st = seg_st + kMaxRawStages * kSegBytes;
+    Bars *bars = reinterpret_cast<Bars *>(bias_st + kBiasBytes);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) LOG(8, 0);
@@ -228,7 +232,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             uint32_t rphase = 0, tile_it = 0;
             const long long HW = (long long)g.H * g.W;
             const long long planes_total = (long long)g.N * g.C;
-            const int KB = g.KB, ncb = cb_cnt, box_floats = g.KB * g.BOXP;
+            const int KB = g.KB, ncb = cb_cnt, box_floats = g.KBR * g.BOXP;
             for (long long t = first_tile; t < g.total_tiles; t += tile_step) {
                 const int ct_all = (int)(t % cgt);
                 const int grp = ct_all / g.ctiles;
@@ -270,7 +274,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                         for (int i = 0; i < nseg; ++i) {
                             if (!segs->nbox[i]) continue;
                             long long nch = planes_total - ((long long)(segs->n_first + i) * g.C + c0);
-                            if (nch > KB) nch = KB;
+                            if (nch > g.KBR) nch = g.KBR;
                             if (nch > 0) total += (uint32_t)(nch * HW * 4);
                         }
                         mbar_arrive_expect_tx(&bars->raw_full[rs], total);
@@ -278,7 +282,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                             if (!segs->nbox[i]) continue;
                             const long long plane0 = (long long)(segs->n_first + i) * g.C + c0;
                             long long nch = planes_total - plane0;
-                            if (nch > KB) nch = KB;
+                            if (nch > g.KBR) nch = g.KBR;
                             if (nch > 0)
                                 bulk_load_1d(dst + segs->base[i], X + plane0 * HW, (uint32_t)(nch * HW * 4),
                                              &bars->raw_full[rs]);
@@ -297,7 +301,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             const int nb = g.nb_stages, ncb = cb_cnt, b_steps = g.b_steps, spb = g.spb, n_steps = g.n_steps;
             const uint32_t stage_bytes = (uint32_t)g.b_stage_bytes, step_bytes = (uint32_t)g.b_step_bytes;
             pdl_wait();             // the packed weights may come from the kernel just before this one
-            for (long long t = first_tile; t < g.total_tiles; t += tile_step) {
+            for (long long t = first_tile; t < g.total_tiles; t += g.b_resident ? g.total_tiles : tile_step) {
                 const int ct_all = (int)(t % cgt);
                 const uint8_t *tile_src = reinterpret_cast<const uint8_t *>(Wpk) + (ct_all * kCtas + (int)rank) * per_ct;
                 const int rot = kSplit ? cb_lo : cb_rotation(t, ncb);
@@ -330,7 +334,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                 const int ncb = g.ncb, nb = g.nb_stages, b_steps = g.b_steps;
                 int bs = 0;
                 uint32_t bphase = 0;
-                for (long long t = first_tile; t < g.total_tiles; t += tile_step) {
+                for (long long t = first_tile; t < g.total_tiles; t += g.b_resident ? g.total_tiles : tile_step) {
                     for (int i = 0; i < ncb * b_steps; ++i) {
                         mbar_wait(&bars->b_full[bs], bphase, err, 19);
                         mbar_arrive_remote(peer_b_full + (uint32_t)bs * 8u);
@@ -346,7 +350,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             const uint32_t b_step16 = (uint32_t)g.b_step_bytes >> 4;
             const uint32_t idesc = g.idesc;
             const int n_steps = g.n_steps, ncb = cb_cnt, nb = g.nb_stages, spb = g.spb, b_steps = g.b_steps;
-            const bool two = g.MT == 2;
+            const bool two = g.MT == 2, resident = g.b_resident != 0;
             int as = 0, bs = 0;
             uint32_t aphase = 0, bphase = 0, it = 0;
             PROF_DECL;
@@ -365,36 +369,43 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                     LOG(2, cb);
                     const uint32_t a_lo = a_base16 + (uint32_t)as * a_stage16;
                     for (int bstep = 0; bstep < b_steps; ++bstep) {
-                        if (kCtas == 2) mbar_wait_cluster(&bars->b_full[bs], bphase, err, 15);
-                        else mbar_wait(&bars->b_full[bs], bphase, err, 15);
+                        if (!resident || it == 0) {
+                            if (kCtas == 2) mbar_wait_cluster(&bars->b_full[bs], bphase, err, 15);
+                            else mbar_wait(&bars->b_full[bs], bphase, err, 15);
+                        }
                         tc_fence_after_sync();
                         PROF_MARK(2);
                         LOG(3, cb * b_steps + bstep);
-                        // One thread issues everything, so every dependent instruction here costs
-                        // its full latency: fetch the stage's table entries together, then issue
-                        // the MMAs back to back with nothing but adds in between.
+                        // One thread issues everything, so every instruction here costs its full latency: fetch
+                        // the stage's table entries together, then issue the MMAs back to back with nothing
+                        // but adds in between (a full stage as straight-line code).
                         const int s0 = bstep * spb, cnt = min(n_steps - s0, spb);
-                        const uint32_t bl = b_lo0 + (uint32_t)bs * b_stage16;
-                        uint32_t sa[kMaxSpb];
+                        uint32_t bl = b_lo0 + (uint32_t)bs * b_stage16;
+                        auto mma = [&](uint32_t d, uint32_t al) {
+                            if (kCtas == 2) mma_tf32_lohi_pair(d, al, desc_hi, bl, desc_hi, idesc, accumulate);
+                            else mma_tf32_lohi(d, al, desc_hi, bl, desc_hi, idesc, accumulate);
+                        };
+                        auto step = [&](uint32_t sa_j) {
+                            mma(d0, a_lo + sa_j);
+                            if (two) mma(d1, a_lo + sa_j + 128u);
+                            accumulate = 1;
+                            bl += b_step16;
+                        };
+                        if (cnt == kMaxSpb) {
+                            uint32_t sa[kMaxSpb];
 #pragma unroll
-                        for (int j = 0; j < kMaxSpb; ++j) sa[j] = j < cnt ? g.step_a[s0 + j] : 0u;
+                            for (int j = 0; j < kMaxSpb; ++j) sa[j] = g.step_a[s0 + j];
 #pragma unroll
-                        for (int j = 0; j < kMaxSpb; ++j) {
-                            if (j < cnt) {
-                                const uint32_t al = a_lo + sa[j], blj = bl + (uint32_t)j * b_step16;
-                                if (kCtas == 2) {
-                                    mma_tf32_lohi_pair(d0, al, desc_hi, blj, desc_hi, idesc, accumulate);
-                                    if (two) mma_tf32_lohi_pair(d1, al + 128u, desc_hi, blj, desc_hi, idesc, accumulate);
-                                } else {
-                                    mma_tf32_lohi(d0, al, desc_hi, blj, desc_hi, idesc, accumulate);
-                                    if (two) mma_tf32_lohi(d1, al + 128u, desc_hi, blj, desc_hi, idesc, accumulate);
-                                }
-                                accumulate = 1;
-                            }
+                            for (int j = 0; j < kMaxSpb; ++j) step(sa[j]);
+                        } else {
+#pragma unroll 4
+                            for (int j = 0; j < cnt; ++j) step(g.step_a[s0 + j]);
                         }
-                        if (kCtas == 2) mma_commit_pair(&bars->b_empty[bs]);
-                        else mma_commit(&bars->b_empty[bs]);
-                        if (++bs == nb) { bs = 0; bphase ^= 1; }
+                        if (!resident) {
+                            if (kCtas == 2) mma_commit_pair(&bars->b_empty[bs]);
+                            else mma_commit(&bars->b_empty[bs]);
+                        }
+                        if (++bs == nb || (resident && bstep == b_steps - 1)) { bs = 0; bphase ^= 1; }
                         PROF_MARK(3);
                     }
                     if (kCtas == 2) mma_commit_pair(&bars->a_empty[as]);
@@ -431,14 +442,15 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
         }
     } else if (warp < kFirstEpiWarp) {
         // ------------------------------------------------------------ transform warps
-        const int xw = warp - kFirstXformWarp;     // 0..7
-        const int xt = xw * 32 + lane;             // 0..255
+        const int xt = (warp - kFirstXformWarp) * 32 + lane;
         const int cp = g.raw_mode == 1 ? g.H * g.W : g.BOXP;    // channel pitch inside the raw stage
         const int per_stage_slots = g.planes * g.SLOTS;
-        const int nchunks = g.nchunks, KB = g.KB, ncb = cb_cnt, box_floats = g.KB * g.BOXP, nr = g.nr_stages;
-        // Work units: one (slot, 4-channel chunk) pair = four raw reads and one 16-byte operand row.
-        // Unit u = chunk * slots + slot; this thread owns units xt, xt + 256, ...
-        const int units = per_stage_slots * nchunks;
+        const int KB = g.KB, ncb = cb_cnt, box_floats = g.KBR * g.BOXP, nr = g.nr_stages;
+        // Work units: one slot and `cpu` of its 4-channel chunks (each four raw reads and one 16-byte operand row);
+        // unit u = chunk group * slots + slot, and this thread owns units xt, xt + kXformThreads, ...  The offset
+        // arithmetic is per unit, not per chunk, and few units keep everything in registers: a spilled value
+        // costs a trip to L2 here (shared memory leaves next to no L1).
+        const int cpu = kThin ? 1 : g.chunks_per_unit, units = per_stage_slots * (kThin ? 1 : g.chunk_groups);
         const int nu = (units - xt + kXformThreads - 1) / kXformThreads;
         int rs = 0, as = 0;
         uint32_t rphase = 0, aphase = 0, tile_it = 0;
@@ -446,29 +458,32 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
         const uint32_t a_full_addr = kCtas == 2 ? map_to_cta(smem_u32(&bars->a_full[0]), 0) : 0u;
         // What does not depend on the tile is worked out once: where a unit's operand row goes, and
         // which slot of which parity plane it reads.
-        uint32_t udst[kOwned];                     // byte offset of the unit's operand row inside an A stage | chunk index
-        // plane << 28 | the slot's place in the stage: as slot rows << 12 | slot columns from the tile's first
-        // slot (4 epilogue warps), or as the plain slot index (8)
-        uint32_t ujp[kOwned];
+        uint32_t udst[kOwned];                     // byte offset of the unit's operand row inside an A stage | chunk group
+        uint32_t ujp[kOwned];                      // slot rows << 12 | slot columns from the tile's first slot
+        uint32_t upix[kOwned];                     // the same distance in pixels, the plane's and the padding's share added: rows << 16 | columns (signed)
 #pragma unroll
         for (int i = 0; i < kOwned; ++i) {
             udst[i] = 0;
             ujp[i] = 0;
+            upix[i] = 0;
             if (i < nu) {
                 const int u = xt + i * kXformThreads;
-                const int ch = conv_fdiv(u, g.planes * g.SLOTS, g.dv_pss), idx = u - ch * per_stage_slots;
-                // operand rows are 16 bytes apart: the low four bits carry the unit's chunk index
-                udst[i] = ((uint32_t)ch * (uint32_t)g.chunk_pitch + (uint32_t)idx * 16u) | (uint32_t)ch;
+                const int cg = kThin ? 0 : conv_fdiv(u, g.planes * g.SLOTS, g.dv_pss), idx = u - cg * per_stage_slots;
+                // operand rows are 16 bytes apart: the low four bits carry the unit's chunk group
+                udst[i] = ((uint32_t)(cg * cpu) * (uint32_t)g.chunk_pitch + (uint32_t)idx * 16u) | (uint32_t)cg;
                 const int pl = conv_fdiv(idx, g.SLOTS, g.dv_SLOTS), j = idx - pl * g.SLOTS;
                 // the slot's distance from the tile's first slot, as whole slot rows and columns
-                // (both below 2^12: a stage holds at most kOwned * 256 slots)
+                // (both below 2^12: a stage holds at most 2560 slots)
                 const int dh = conv_fdiv(j, g.Ws, g.dv_Ws), dw = j - dh * g.Ws;
-                ujp[i] = kEpiWarps == 8 ? (uint32_t)j | ((uint32_t)pl << 28)
-                                        : (uint32_t)dw | ((uint32_t)dh << 12) | ((uint32_t)pl << 28);
+                ujp[i] = (uint32_t)dw | ((uint32_t)dh << 12);
+                // fixed-index reads of the parity tables (a dynamic index into kernel parameters costs an indexed
+                // constant load per use)
+                const int pa = pl == 0 ? g.pa[0] : pl == 1 ? g.pa[1] : pl == 2 ? g.pa[2] : g.pa[3];
+                const int pb = pl == 0 ? g.pb[0] : pl == 1 ? g.pb[1] : pl == 2 ? g.pb[2] : g.pb[3];
+                upix[i] = ((uint32_t)(dh * g.sh + pa - g.pt) << 16) | ((uint32_t)(dw * g.sw + pb - g.pl) & 0xFFFFu);
             }
         }
         for (long long t = first_tile; t < g.total_tiles; t += tile_step) {
-            const long long G0 = ((t / cgt) * kCtas + rank) * tile_rows;
             int uoff[kOwned];                      // raw float offset of the unit's first channel, -1 = padding
             const int rot = kSplit ? cb_lo : cb_rotation(t, ncb);
             {
@@ -479,69 +494,40 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                 ++tile_it;
                 const TcConvSegs *segs = reinterpret_cast<const TcConvSegs *>(seg_st + sp * kSegBytes);
                 const int n0 = segs->n_first, hq0 = segs->hq0, wq0 = segs->wq0;
-                if (kEpiWarps == 8) {
-                    // 96 registers per thread: one unit after the other, each leaving early where it can
+                // Straight-line code, no branches on a lane's own data: the units' chains of dependent integer
+                // operations then overlap instead of running one after the other (this loop, not the data movement,
+                // was the larger part of the thin first layer's time).  Slot -> (image, slot row, slot column) without
+                // dividing the slot number: the tile's first slot was decomposed once (by the producer, in the
+                // segment table), and this unit lies a fixed number of slot rows and columns further on.
+                {
+                    const int nseg = segs->nseg, hbase = hq0 * g.sh, wbase = wq0 * g.sw, Wssw = g.Ws * g.sw, Hssh = g.Hs * g.sh;
+                    // the table's first two entries in registers: a tile of a large image touches no more than two
+                    const int f0a = segs->f0[0], f0b = segs->f0[1], ba = segs->base[0], bb = segs->base[1];
+                    const int images = min(nseg, g.N - n0);
 #pragma unroll
                     for (int i = 0; i < kOwned; ++i) {
-                        uoff[i] = -1;
-                        if (i < nu) {
-                            const int ch = (int)(udst[i] & 15u), pl = (int)(ujp[i] >> 28);
-                            const uint32_t Gs = (uint32_t)G0 + (ujp[i] & 0x0FFFFFFFu);     // the planner keeps slots below 2^31
-                            if (Gs < (uint32_t)g.total_slots) {
-                                const int n = conv_fdiv((int)Gs, g.L, g.dv_L);
-                                const int uu = (int)Gs - n * g.L;
-                                const int hq = conv_fdiv(uu, g.Ws, g.dv_Ws), wq = uu - hq * g.Ws;
-                                // fixed-index reads of the parity tables (a dynamic index into kernel
-                                // parameters costs an indexed constant load per use)
-                                const int pa = pl == 0 ? g.pa[0] : pl == 1 ? g.pa[1] : pl == 2 ? g.pa[2] : g.pa[3];
-                                const int pb = pl == 0 ? g.pb[0] : pl == 1 ? g.pb[1] : pl == 2 ? g.pb[2] : g.pb[3];
-                                const int h = hq * g.sh + pa - g.pt;
-                                const int w = wq * g.sw + pb - g.pl;
-                                const int sg = n - segs->n_first;
-                                if ((unsigned)h < (unsigned)g.H && (unsigned)w < (unsigned)g.W && (unsigned)sg < (unsigned)segs->nseg) {
-                                    const int f = h * g.W + w - segs->f0[sg];
-                                    int o;
-                                    if (g.raw_mode == 1) o = segs->base[sg] + f;
-                                    else {
-                                        const int bx = conv_fdiv(f, g.BOXP, g.dv_BOXP);
-                                        o = segs->base[sg] + bx * box_floats + (f - bx * g.BOXP);
-                                    }
-                                    uoff[i] = o + ch * 4 * cp;
-                                }
-                            }
+                        const int ch = kThin ? 0 : (int)(udst[i] & 15u) * cpu;
+                        const int carry = wq0 + (int)(ujp[i] & 0xFFFu) >= g.Ws ? 1 : 0;
+                        const int hq = hq0 + (int)(ujp[i] >> 12) + carry;
+                        int k = hq >= g.Hs ? 1 : 0, f0 = k ? f0b : f0a, base = k ? bb : ba;        // images crossed
+                        if (nseg > 2) {                                                            // (small images: several)
+                            k = conv_fdiv(hq, g.Hs, g.dv_Hs);
+                            const int sg = k < nseg ? k : 0;                                       // an entry that exists, whatever k is
+                            f0 = segs->f0[sg];
+                            base = segs->base[sg];
                         }
-                    }
-                } else {
-                    // Straight-line code, no branches: the units' chains of dependent integer operations then
-                    // overlap instead of running one after the other (this loop, not the data movement, was
-                    // the larger part of the thin first layer's time when every unit took its own branches).
-                    const int nseg = segs->nseg;
-    #pragma unroll
-                    for (int i = 0; i < kOwned; ++i) {
-                        const int ch = (int)(udst[i] & 15u), pl = (int)(ujp[i] >> 28);
-                        // Slot -> (image, slot row, slot column) without dividing the slot number: the tile's
-                        // first slot was decomposed once (by the producer, in the segment table); this unit
-                        // lies a fixed number of slot rows and columns further on.
-                        int wq = wq0 + (int)(ujp[i] & 0xFFFu);
-                        const int carry = wq >= g.Ws ? 1 : 0;
-                        wq -= carry ? g.Ws : 0;
-                        int hq = hq0 + (int)((ujp[i] >> 12) & 0xFFFu) + carry;
-                        const int k = conv_fdiv(hq, g.Hs, g.dv_Hs);           // images crossed (small images: several)
-                        hq -= k * g.Hs;
-                        // fixed-index reads of the parity tables (a dynamic index into kernel parameters
-                        // costs an indexed constant load per use)
-                        const int pa = pl == 0 ? g.pa[0] : pl == 1 ? g.pa[1] : pl == 2 ? g.pa[2] : g.pa[3];
-                        const int pb = pl == 0 ? g.pb[0] : pl == 1 ? g.pb[1] : pl == 2 ? g.pb[2] : g.pb[3];
-                        const int h = hq * g.sh + pa - g.pt;
-                        const int w = wq * g.sw + pb - g.pl;
-                        const bool ok = i < nu && n0 + k < g.N && (unsigned)h < (unsigned)g.H && (unsigned)w < (unsigned)g.W &&
-                                        k < nseg;
-                        const int sg = k < nseg ? k : 0;                      // a table entry that exists, whatever k is
-                        const int f = h * g.W + w - segs->f0[sg];
-                        int o = segs->base[sg] + f;                           // whole-image slabs
+                        const int h = hbase + ((int)upix[i] >> 16) + carry * g.sh - k * Hssh;
+                        const int w = wbase + (int)(short)upix[i] - carry * Wssw;
+                        const bool ok = i < nu && k < images && (unsigned)h < (unsigned)g.H && (unsigned)w < (unsigned)g.W;
+                        const int f = h * g.W + w - f0;
+                        int o = base + f;                                                          // whole-image slabs
                         if (g.raw_mode != 1) {
-                            const int bx = g.boxp_shift >= 0 ? (f >> g.boxp_shift) : conv_fdiv(ok ? f : 0, g.BOXP, g.dv_BOXP);
-                            o = segs->base[sg] + bx * box_floats + (f - bx * g.BOXP);
+                            if (g.boxp_shift >= 0) {
+                                o = base + (f >> g.boxp_shift) * box_floats + (f & (g.BOXP - 1));
+                            } else {
+                                const int bx = conv_fdiv(ok ? f : 0, g.BOXP, g.dv_BOXP);
+                                o = base + bx * box_floats + (f - bx * g.BOXP);
+                            }
                         }
                         uoff[i] = ok ? o + ch * 4 * cp : -1;
                     }
@@ -561,32 +547,57 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                 uint8_t *adst = a_st + (size_t)as * g.a_stage_bytes;
                 const int cbx = kSplit || cb + rot < ncb ? cb + rot : cb + rot - ncb;
                 const int c_left = g.Cg - cbx * KB;    // channels of this block that exist
-                // In two batches of five units: all reads of a batch first (independent, so their latencies
-                // overlap), then round and store; channels past the end of the group (last block only)
-                // read as zero.
+                if (kThin) {
+                    constexpr int kBatch = (kOwned + 1) / 2;
+                    // In two batches of units: all reads of a batch first (independent, so their latencies
+                    // overlap), then round and store; channels past the end of the group read as zero.
 #pragma unroll
-                for (int h0 = 0; h0 < kOwned; h0 += kOwned / 2) {
-                    float v[kOwned / 2][4];
+                    for (int h0 = 0; h0 < kOwned; h0 += kBatch) {
+                        float v[kBatch][4];
 #pragma unroll
-                    for (int k = 0; k < kOwned / 2; ++k) {
-                        const int i = h0 + k;
-                        v[k][0] = v[k][1] = v[k][2] = v[k][3] = 0.f;
-                        if (i < nu && uoff[i] >= 0) {
-                            const float *r = raw + uoff[i];
-                            const int left = c_left - (int)(udst[i] & 15u) * 4;
-                            if (left > 0) v[k][0] = r[0];
-                            if (left > 1) v[k][1] = r[cp];
-                            if (left > 2) v[k][2] = r[2 * cp];
-                            if (left > 3) v[k][3] = r[3 * cp];
+                        for (int k = 0; k < kBatch; ++k) {
+                            const int i = h0 + k;
+                            if (i >= kOwned) break;
+                            v[k][0] = v[k][1] = v[k][2] = v[k][3] = 0.f;
+                            if (i < nu && uoff[i] >= 0) {
+                                const float *r = raw + uoff[i];
+                                if (c_left > 0) v[k][0] = r[0];
+                                if (c_left > 1) v[k][1] = r[cp];
+                                if (c_left > 2) v[k][2] = r[2 * cp];
+                                if (c_left > 3) v[k][3] = r[3 * cp];
+                            }
+                        }
+#pragma unroll
+                        for (int k = 0; k < kBatch; ++k) {
+                            const int i = h0 + k;
+                            if (i >= kOwned) break;
+                            if (i < nu)
+                                *reinterpret_cast<float4 *>(adst + (udst[i] & ~15u)) =
+                                    make_float4(round_tf32(v[k][0]), round_tf32(v[k][1]), round_tf32(v[k][2]),
+                                                round_tf32(v[k][3]));
                         }
                     }
+                } else {
+                    // Two chunks at a time: their reads first (independent, so their latencies overlap), then round and
+                    // store.  Padding units read word 0 and mask it.
 #pragma unroll
-                    for (int k = 0; k < kOwned / 2; ++k) {
-                        const int i = h0 + k;
-                        if (i < nu)
-                            *reinterpret_cast<float4 *>(adst + (udst[i] & ~15u)) =
-                                make_float4(round_tf32(v[k][0]), round_tf32(v[k][1]), round_tf32(v[k][2]),
-                                            round_tf32(v[k][3]));
+                    for (int i = 0; i < kOwned; ++i) {
+                        if (i < nu) {
+                            const bool ok = uoff[i] >= 0;
+                            const float *r = raw + (ok ? uoff[i] : 0);
+                            uint8_t *d = adst + (udst[i] & ~15u);
+                            int left = ok ? c_left - (int)(udst[i] & 15u) * cpu * 4 : 0;     // channels that exist from here on
+                            for (int c = 0; c < cpu; c += 2) {
+                                float v[8];
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) v[e] = left > e ? r[e * cp] : 0.f;
+                                *reinterpret_cast<float4 *>(d) = make_float4(round_tf32(v[0]), round_tf32(v[1]), round_tf32(v[2]), round_tf32(v[3]));
+                                *reinterpret_cast<float4 *>(d + g.chunk_pitch) = make_float4(round_tf32(v[4]), round_tf32(v[5]), round_tf32(v[6]), round_tf32(v[7]));
+                                r += 8 * cp;
+                                d += 2 * g.chunk_pitch;
+                                left -= 8;
+                            }
+                        }
                     }
                 }
                 PROF_MARK(2);
@@ -612,8 +623,8 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
     } else {
         // ------------------------------------------------------------ epilogue warps
         const int ew = warp - kFirstEpiWarp;       // 0..7
+        float *bias_w = reinterpret_cast<float *>(bias_st) + ew * 32;
         const int quarter = warp & 3;              // TMEM lane quarter this warp may read
-        const long long PQ = (long long)g.P * g.Q;
         const bool two = g.MT == 2;
         const uint32_t acc_empty_addr = kCtas == 2 ? map_to_cta(smem_u32(&bars->acc_empty[0]), 0) : 0u;
         uint32_t it = 0;
@@ -641,41 +652,57 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                         if (chunk * 32 + j < g.BN) part[(chunk * 32 + j) * pitch + row] = __uint_as_float(v[j]);
                 }
             }
-            // eight warps: two per TMEM lane quarter, each taking half of the tile; four: one per quarter, both halves
-            for (int hf = ew >> 2; hf < 2 && !kSplit; hf += kEpiWarps / 4) {
-            int mt, ch_lo, ch_hi;
-            if (two) { mt = hf; ch_lo = 0; ch_hi = nch; }
-            else { mt = 0; ch_lo = hf ? (nch + 1) / 2 : 0; ch_hi = hf ? nch : (nch + 1) / 2; }
-            const uint32_t acc_col = ab * 256u + (uint32_t)mt * mt_cols;
-            const uint32_t G = (uint32_t)G0 + (uint32_t)(mt * 128 + quarter * 32 + lane);
-            bool valid = G < (uint32_t)g.total_slots;
-            float *yrow = Y;
-            if (valid) {
-                const int n = (int)(G / (uint32_t)g.L);
-                const int u = (int)(G - (uint32_t)n * (uint32_t)g.L);
-                const int p = u / g.Ws, q = u - p * g.Ws;
-                valid = p < g.P && q < g.Q;
-                yrow = Y + ((long long)n * g.M * g.P + p) * g.Q + q;
-            }
-            const int m_lim = min(g.Mg, (ct + 1) * g.BN);          // channels of this tile that exist
-            for (int chunk = ch_lo; chunk < ch_hi; ++chunk) {
-                uint32_t v[32];
-                tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc_col + (uint32_t)(chunk * 32), v);
-                const int mg0 = ct * g.BN + chunk * 32;            // first channel (within the group) of the chunk
-                // lane j fetches the bias of column j once; columns then take it by shuffle
-                const float bl = (bias && mg0 + lane < m_lim) ? __ldg(bias + grp * g.Mg + mg0 + lane) : 0.f;
-                float *yp = yrow + (long long)(grp * g.Mg + mg0) * PQ;
-                tmem_ld_wait();
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    float x = __uint_as_float(v[j]) + __shfl_sync(0xffffffffu, bl, j);
-                    const bool live = valid && mg0 + j < m_lim;
-                    if (kAdd && live) x += __ldg(R + (yp - Y));             // residual addend at Y's own position
-                    if (g.relu) x = fmaxf(x, 0.f);
-                    if (live) *yp = x;
-                    yp += PQ;
+            if (!kSplit) {
+                // eight warps: two per TMEM lane quarter, each taking half of the tile
+                const int hf = ew >> 2, mt = two ? hf : 0;
+                const int ch_lo = two ? 0 : hf ? (nch + 1) / 2 : 0, ch_hi = two || hf ? nch : (nch + 1) / 2;
+                const uint32_t acc_col = ab * 256u + (uint32_t)mt * mt_cols;
+                const uint32_t G = (uint32_t)G0 + (uint32_t)(mt * 128 + quarter * 32 + lane);
+                const uint32_t PQ4 = (uint32_t)g.P * (uint32_t)g.Q * 4u;
+                bool valid = G < (uint32_t)g.total_slots;
+                uint32_t off = 0;                      // bytes from Y (and R): the launch keeps them below 2^32
+                if (valid) {
+                    const int n = conv_fdiv((int)G, g.L, g.dv_L), u = (int)G - n * g.L;
+                    const int p = conv_fdiv(u, g.Ws, g.dv_Ws), q = u - p * g.Ws;
+                    valid = p < g.P && q < g.Q;
+                    off = (uint32_t)(n * g.M + grp * g.Mg + ct * g.BN + ch_lo * 32) * PQ4 + (uint32_t)(p * g.Q + q) * 4u;
                 }
-            }
+                char *yb = reinterpret_cast<char *>(Y);
+                const char *rb = reinterpret_cast<const char *>(R);
+                const float lowest = g.relu ? 0.f : -INFINITY;
+                for (int chunk = ch_lo; chunk < ch_hi; ++chunk) {
+                    uint32_t v[32];
+                    tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc_col + (uint32_t)(chunk * 32), v);
+                    const int mg0 = ct * g.BN + chunk * 32;                // first channel (within the group) of the chunk
+                    const int cnt = min(g.Mg, (ct + 1) * g.BN) - mg0;      // channels of the chunk that exist (above 32: all)
+                    // the chunk's biases through shared memory: eight 16-byte broadcasts instead of 32 shuffles
+                    __syncwarp();
+                    bias_w[lane] = bias && lane < cnt ? __ldg(bias + grp * g.Mg + mg0 + lane) : 0.f;
+                    __syncwarp();
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int j0 = 0; j0 < 32; j0 += 8) {
+                        float r[8];
+                        if (kAdd) {                                        // residual addend at Y's own position
+#pragma unroll
+                            for (int j = 0; j < 8; ++j)
+                                r[j] = valid && j0 + j < cnt ? __ldg(reinterpret_cast<const float *>(rb + (off + (uint32_t)j * PQ4))) : 0.f;
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; j += 4) {
+                            const float4 b4 = *reinterpret_cast<const float4 *>(bias_w + j0 + j);
+                            const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                float x = __uint_as_float(v[j0 + j + e]) + b[e];
+                                if (kAdd) x += r[j + e];
+                                x = fmaxf(x, lowest);
+                                if (valid && j0 + j + e < cnt) *reinterpret_cast<float *>(yb + off) = x;
+                                off += PQ4;
+                            }
+                        }
+                    }
+                }
             }
             tc_fence_before_sync();
             __syncwarp();
@@ -810,6 +837,7 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     g.L = (int)L;
     g.total_slots = (long long)c.N * L;
     if (g.total_slots + 4096 >= (1LL << 31)) return false;        // device code indexes slots in 32 bits
+    if ((long long)c.M * c.P * c.Q >= (1LL << 30)) return false;  // and an image's outputs in 32 bits of bytes
     g.planes = 0;
     for (int i = 0; i < ah.npar; ++i)
         for (int j = 0; j < aw.npar; ++j) { g.pa[g.planes] = ah.par[i]; g.pb[g.planes] = aw.par[j]; ++g.planes; }
@@ -819,8 +847,10 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     g.ctiles = (c.Mg + BN - 1) / BN;
     const long long slots = (long long)MT * 128 + maxshift;
     if (c.Cg < 16) KB = 4;
-    if (slots * g.planes * (KB / 4) > kOwned * kXformThreads) return false;
+    if (slots * g.planes * (KB / 4) > kMaxUnits) return false;
     g.SLOTS = (int)slots;
+    // a slot's distance from the tile's first, in pixels, fits 16 signed bits
+    if (slots * std::max(c.sh, c.sw) + std::max(c.pt, c.pl) > 32000) return false;
     if ((g.SLOTS + L - 2) / L + 1 > kConvMaxSeg) return false;
     g.plane_pitch = g.SLOTS * 16;
     g.chunk_pitch = g.planes * g.plane_pitch;
@@ -882,6 +912,22 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
         g.src_c0[s][0] = g.src_c0[s][1] = 0;
     }
     g.nchunks = g.KB / 4;
+    // Chunk groups: the split that gives the busiest transform thread the least work, pairs of chunks at least.
+    g.chunk_groups = 1;
+    g.chunks_per_unit = g.nchunks;
+    if (g.KB > 4) {
+        int best = 1 << 30;
+        for (int groups = 1; groups * 2 <= g.nchunks; groups *= 2) {
+            const long long owned = ((long long)g.planes * g.SLOTS * groups + kXformThreads - 1) / kXformThreads;
+            const int work = (int)owned * (g.nchunks / groups) * 4 + (int)owned;        // chunks, and a little per unit
+            if (owned <= kOwnedThick && work < best) {
+                best = work;
+                g.chunk_groups = groups;
+                g.chunks_per_unit = g.nchunks / groups;
+            }
+        }
+        if (best == 1 << 30) return false;
+    }
     g.ncb = (c.Cg + g.KB - 1) / g.KB;
     const long long ptiles = (g.total_slots + MT * 128 - 1) / (MT * 128);      // per-CTA pixel tiles
     if (ptiles > 0x7fffffffLL) return false;
@@ -899,51 +945,58 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     g.a_stage_bytes = g.nchunks * g.chunk_pitch;
     g.a_stage_bytes = (g.a_stage_bytes + 127) / 128 * 128;
     g.b_step_bytes = g.BNH * 32;
-    g.spb = std::max(1, std::min(std::min(g.n_steps, kMaxSpb), 32768 / g.b_step_bytes));   // several K-steps per weight stage
     g.idesc = tc::make_idesc_tf32(128 * ctas, BN, 0, 0);
     g.packed_floats = (long long)c.group * g.ctiles * g.ncb * g.n_steps * BN * 8;     // both CTAs' parts
     if (g.packed_floats >= (1LL << 32)) return false;                                  // 32-bit indexing in the packing kernel
-    // raw stage size: widest flat pixel range any tile needs, found by walking the tiles
-    g.BOXP = 256;
-    const long long walk = std::min<long long>(ptiles, L + 2);
-    if (g.raw_mode == 0) {
-        int widest = 4;
-        for (long long i = 0; i <= walk; ++i) {
-            const long long pt = i < walk ? i : ptiles - 1;
-            const long long G0 = pt * MT * 128;
-            const long long Gend = std::min<long long>(G0 + g.SLOTS, g.total_slots);
-            const int n_first = (int)(G0 / L), n_last = (int)((Gend - 1) / L);
-            for (int n = n_first; n <= n_last; ++n) {
-                const long long lo = std::max<long long>(G0, (long long)n * L), hi = std::min<long long>(Gend, (long long)(n + 1) * L);
-                const int hq_lo = (int)((lo - (long long)n * L) / g.Ws), hq_hi = (int)((hi - 1 - (long long)n * L) / g.Ws);
-                const int h_min = std::max(0, hq_lo * c.sh + g.a_min - c.pt);
-                const int h_max = std::min(c.H - 1, hq_hi * c.sh + g.a_max - c.pt);
-                if (h_min > h_max) continue;
-                const int f0 = (h_min * c.W) & ~3;
-                widest = std::max(widest, (h_max + 1) * c.W - f0);
-            }
-        }
-        // boxes of <= 256 pixels, split evenly; every box must start on a 128-byte boundary of
-        // shared memory (TMA destination alignment), i.e. KB * BOXP * 4 bytes is a multiple of 128
-        const int align = std::max(4, 32 / g.KB);
-        widest = (widest + 3) / 4 * 4;
-        const int nbox = (widest + 255) / 256;
-        g.BOXP = std::min(256, ((widest + nbox - 1) / nbox + align - 1) / align * align);
-        // Blocks of 4 channels (the thin first layer of a network) stage so little per pixel that whole
-        // 256-pixel boxes cost nothing, and a power of two spares the transform a division per unit.
-        if (g.KB == 4 && widest > 128) g.BOXP = 256;
-    }
-    {
+    // Raw stage size.  What a tile stages depends on where its first slot lies in an image; of the starts in one
+    // slot row the last reaches furthest, and the first image has the most slots after it, so one start per slot
+    // row covers all tiles.
+    g.KBR = std::min(g.KB, c.Cg);
+    auto for_each_start = [&](auto &&f) {
+        for (int r = 0; r < g.Hs; ++r) f(std::min<long long>((long long)r * g.Ws + g.Ws - 1, g.total_slots - 1));
+    };
+    auto stage_floats = [&](int boxp, int &boxes) {
+        g.BOXP = boxp;
         int worst = 0;
-        TcConvSegs segs;
-        for (long long i = 0; i <= walk; ++i) {
-            const long long pt = i < walk ? i : ptiles - 1;
-            tc_conv_segments(g, pt * MT * 128, segs);
+        boxes = 0;
+        for_each_start([&](long long G0) {
+            TcConvSegs segs;
+            tc_conv_segments(g, G0, segs);
             worst = std::max(worst, segs.total_floats);
-        }
-        g.raw_stage_bytes = (worst * 4 + 127) / 128 * 128;
-        if (g.raw_stage_bytes == 0) g.raw_stage_bytes = 128;
+            int n = 0;
+            for (int i = 0; i < segs.nseg; ++i) n += segs.nbox[i];
+            boxes = std::max(boxes, n);
+        });
+        return worst;
+    };
+    int worst, boxes;
+    if (g.raw_mode == 1) {
+        worst = stage_floats(256, boxes);
+    } else if (g.KB == 4) {
+        // Blocks of 4 channels (the thin first layer of a network) stage little per pixel: 256-pixel boxes, and
+        // a power of two spares the transform a division per unit.
+        worst = stage_floats(256, boxes);
+    } else {
+        // Boxes of at most 256 pixels, splitting the widest flat range of an image that a tile needs evenly; every box
+        // starts on a 128-byte boundary of shared memory (TMA destination alignment): KB * BOXP * 4 bytes is a
+        // multiple of 128.  (Smaller boxes stage less beyond what a tile needs, but cost more than that gains:
+        // 64 -> 64 channels at 56x56 44.3 -> 46 us.)
+        int widest = 4;
+        for_each_start([&](long long G0) {
+            const long long Gend = std::min<long long>(G0 + g.SLOTS, g.total_slots);
+            for (long long n = 0; n * L < Gend; ++n) {
+                const long long lo = std::max<long long>(G0, n * L), hi = std::min<long long>(Gend, (n + 1) * L);
+                if (lo >= hi) continue;
+                const int h_min = std::max(0, (int)((lo - n * L) / g.Ws) * c.sh + g.a_min - c.pt);
+                const int h_max = std::min(c.H - 1, (int)((hi - 1 - n * L) / g.Ws) * c.sh + g.a_max - c.pt);
+                if (h_min <= h_max) widest = std::max(widest, (h_max + 1) * c.W - ((h_min * c.W) & ~3));
+            }
+        });
+        const int align = std::max(4, 32 / g.KB), nbox = (widest + 255) / 256;
+        const int boxp = std::min(256, ((widest + nbox - 1) / nbox + align - 1) / align * align);
+        worst = stage_floats(boxp, boxes);
     }
+    g.raw_stage_bytes = std::max(128, (worst * 4 + 127) / 128 * 128);
     // Raw stages: a third one (the raw tiles come from L2/HBM with a microsecond of latency) when that
     // still leaves 64 KB for the weight ring.
     g.na_stages = 2;
@@ -957,7 +1010,7 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
             g.na_stages = fa;
             g.nr_stages = fr;
         } else if (MT == 2 && g.KB >= 16 &&
-                   kSmemLimit - (1024 + 3LL * g.a_stage_bytes + kMaxRawStages * kSegBytes + kBarBytes) -
+                   kSmemLimit - (1024 + 3LL * g.a_stage_bytes + kMaxRawStages * kSegBytes + kBiasBytes + kBarBytes) -
                            2LL * g.raw_stage_bytes >= 65536) {
             // Two accumulators per CTA: a third operand stage instead of a third raw stage (64 -> 64
             // channels at 56x56: 55.5 -> 52.3 us), and in a CTA pair the odd CTA's "stage written" message
@@ -967,18 +1020,33 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
             g.na_stages = 3;
             g.relay = ctas == 2 ? 1 : 0;
         } else {
-            const long long bf = 1024 + 2LL * g.a_stage_bytes + kMaxRawStages * kSegBytes + kBarBytes;
+            const long long bf = 1024 + 2LL * g.a_stage_bytes + kMaxRawStages * kSegBytes + kBiasBytes + kBarBytes;
             for (int nr = 3; nr <= kMaxRawStages - 1; ++nr)
                 if (kSmemLimit - bf - (long long)nr * g.raw_stage_bytes >= 65536) g.nr_stages = nr;
         }
     }
-    const long long base_fixed = 1024 + (long long)g.na_stages * g.a_stage_bytes + kMaxRawStages * kSegBytes + kBarBytes;
+    const long long base_fixed = 1024 + (long long)g.na_stages * g.a_stage_bytes + kMaxRawStages * kSegBytes + kBiasBytes + kBarBytes;
     const long long fixed = base_fixed + (long long)g.nr_stages * g.raw_stage_bytes;
     const long long room = kSmemLimit - fixed;
-    while (room < 3LL * g.spb * g.b_step_bytes && g.spb > 1) g.spb = (g.spb + 1) / 2;   // keep three stages in flight
+    // K-steps per weight stage: as many as leave three stages in flight, the block's steps spread evenly.
+    g.spb = std::min(g.n_steps, kMaxSpb);
+    while (g.spb > 1 && ((long long)g.spb * g.b_step_bytes > 36864 || room < 3LL * g.spb * g.b_step_bytes)) --g.spb;
     g.b_steps = (g.n_steps + g.spb - 1) / g.spb;
+    g.spb = (g.n_steps + g.b_steps - 1) / g.b_steps;
     g.b_stage_bytes = g.spb * g.b_step_bytes;
-    if (room < 2LL * g.b_stage_bytes) return false;
+    // One channel block and one channel tile: every tile uses the same weights.  Kept, where they fit.
+    g.b_resident = 0;
+    if (g.ncb == 1 && g.ctiles * c.group == 1) {
+        const int spb = std::min(g.n_steps, kMaxSpb), steps = (g.n_steps + spb - 1) / spb;
+        const long long even = (g.n_steps + steps - 1) / steps;
+        if (steps <= kMaxBStages && steps * even * g.b_step_bytes <= room) {
+            g.b_resident = 1;
+            g.spb = (int)even;
+            g.b_steps = steps;
+            g.b_stage_bytes = g.spb * g.b_step_bytes;
+        }
+    }
+    if (room < 2LL * g.b_stage_bytes && !g.b_resident) return false;
     g.nb_stages = (int)std::min<long long>(kMaxBStages, room / g.b_stage_bytes);
     g.dv_L = conv_divisor(g.L);
     g.dv_Ws = conv_divisor(g.Ws);
@@ -992,36 +1060,31 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     return true;
 }
 
-// Cost in SM cycles per CTA, fitted to measured tile sweeps of the ResNet-50 3x3 layers.  Per channel block the
-// slowest of: the tensor pipe (BN/2 cycles per 128 x BN x 8 share of an instruction, or the 128 bytes/cycle of
-// shared memory its operands need, whichever is longer), shared memory as a whole (operand reads plus the
-// stages written and the transform, at about 90 bytes/cycle sustained), the weight stream out of L2 (about 3600
-// bytes/cycle over all SMs, at most 48 per SM) and the transform warps; plus a fixed hand-over cost per block,
-// larger for pairs (their barriers cross the cluster).  split: CTAs sharing a tile's channel blocks.
+// Estimated SM cycles of a plan, fitted to 703 measured (shape, tile) pairs: 40 shapes from ResNet-50's 3x3 layers at
+// batch 8 to 64 to random ones of 16-320 channels, 3x3 and 5x5, stride 1 and 2; the pick is within 0.2 % of the
+// best tile on average.  Per channel block the slowest of: the tensor pipe (BN/2 cycles per 128 x BN x 8 share of an
+// instruction, or its operands out of shared memory at 160 bytes/cycle) with 380 cycles per weight stage; shared
+// memory as a whole (operand reads, stages written, re-lay) at 126 bytes/cycle; the weight stream out of L2 (18
+// bytes/cycle and SM, 2800 over all SMs) or, where the ring is short, its latency of 1900 cycles; and the re-lay, 75
+// cycles per chunk of the busiest thread.  split: CTAs sharing a tile's channel blocks.
 double tile_cost(const TcConvPlan &p, int split) {
     const int sms = 148;
     const int units = sms / p.ctas / split;                             // tiles in flight
     const long long waves = (p.total_tiles + units - 1) / units;
     const double active = (double)std::min<long long>(p.total_tiles, units) * p.ctas * split;
-    const double n_inst = (double)p.n_steps * p.MT;
-    const double op_bytes = 4096.0 + p.BNH * 32.0;
-    const double t_mma = n_inst * (std::max(p.BN / 2.0, op_bytes / 128.0) + (p.ctas == 2 ? 10.0 : 0.0));
-    const double w_bytes = (double)p.n_steps * p.b_step_bytes;
+    const bool pair = p.ctas == 2;
+    const double n_inst = (double)p.n_steps * p.MT, op_bytes = 4096.0 + p.BNH * 32.0;
+    const double t_mma = n_inst * std::max(p.BN * 0.485, op_bytes / 160.0) + (p.n_steps + p.spb - 1) / p.spb * 380.0;
+    const double w_bytes = p.b_resident ? 0.0 : (double)p.n_steps * p.b_step_bytes;
     const double slots16 = (double)p.planes * p.SLOTS * 16.0 * p.nchunks;
-    const double t_smem = (n_inst * op_bytes + w_bytes + 3.0 * slots16) / 90.0;
-    // the weight ring must also cover the latency of its copies (about 2500 cycles from issue to
-    // landing under load): a ring holding less than that much of the stream paces the block
+    const double t_smem = (n_inst * op_bytes + w_bytes + 3.0 * slots16) / 126.0;
     const double ring = (double)p.nb_stages * p.b_stage_bytes;
-    const double t_w = std::max(w_bytes / std::min(48.0, 3600.0 / active), w_bytes * 2500.0 / ring);
-    const double t_x = 300.0 + 100.0 * ((p.planes * p.SLOTS * p.nchunks + 255) / 256);
-    // (three operand stages hide most of the hand-over)
-    const double per_cb = std::max(std::max(t_mma, t_smem), std::max(t_w, t_x)) +
-                          (p.na_stages == 3 ? 300.0 : 400.0 + (p.ctas == 2 ? 700.0 : 0.0));
-    const bool dbl = p.MT == 1 || p.BN <= 128;
-    const double t_epi = 8.0 * p.MT * p.BN;                             // read-back and stores of one tile
-    if (split > 1) return (double)waves * ((p.ncb + split - 1) / split * per_cb + t_epi + 8000.0) + 9000.0;
-    const double per_tile = (dbl ? std::max(p.ncb * per_cb, t_epi) : p.ncb * per_cb + t_epi) + 3000.0;
-    return (double)waves * per_tile + 9000.0 + (dbl ? t_epi : 0.0);
+    const double t_w = std::max(w_bytes / std::min(17.6, 2800.0 / active), w_bytes * 1930.0 / ring);
+    const double owned = (p.planes * p.SLOTS * p.chunk_groups + kXformThreads - 1) / kXformThreads;
+    const double t_x = 740.0 + 75.0 * owned * p.chunks_per_unit + (pair ? 1080.0 : 0.0);
+    const double per_cb = std::max(std::max(t_mma, t_smem), std::max(t_w, t_x)) + (p.na_stages == 3 ? 0.0 : 210.0);
+    if (split > 1) return (double)waves * ((p.ncb + split - 1) / split * per_cb + 8.0 * p.MT * p.BN + 8000.0) + 9000.0;
+    return (double)waves * (p.ncb * per_cb + 100.0 * owned + 2500.0) + 9840.0 + (pair ? 1220.0 : 0.0);
 }
 
 }  // namespace
@@ -1034,10 +1097,9 @@ bool tc_conv_plan(const ConvGeom &c, TcConvPlan &plan, bool forced) {
         const double flops = 2.0 * c.N * c.M * c.P * c.Q * c.Cg * (double)taps;
         if (taps < 2 || c.Cg * taps < 32 || (flops < 5e7 && !forced)) return false;
     }
-    const int sms = 148;
     const int bn0 = pick_conv_bn(c.Mg);
     // candidate tiles (CTAs per tile, accumulators per CTA, channels per tile)
-    int cand[48][4];
+    int cand[96][4];
     int ncand = 0;
     auto add = [&](int ctas, int mt, int bn, int kb) {
         for (int i = 0; i < ncand; ++i)
@@ -1053,10 +1115,11 @@ bool tc_conv_plan(const ConvGeom &c, TcConvPlan &plan, bool forced) {
     if (ncand == 0) {
         for (int kb = 16; kb <= 64 && (kb == 16 || kb <= c.Cg); kb *= 2)
             for (int ctas = 2; ctas >= 1; --ctas) {
-                add(ctas, 2, bn0, kb);
-                add(ctas, 1, bn0, kb);
-                if (bn0 > 128) { add(ctas, 2, 128, kb); add(ctas, 1, 128, kb); }
-                if (bn0 > 64) add(ctas, 1, 64, kb);
+                for (int bn : {bn0, 128, 96, 64})
+                    if (bn <= bn0) {
+                        add(ctas, 2, bn, kb);
+                        add(ctas, 1, bn, kb);
+                    }
             }
     }
     bool have = false;
@@ -1064,13 +1127,7 @@ bool tc_conv_plan(const ConvGeom &c, TcConvPlan &plan, bool forced) {
     for (int i = 0; i < ncand; ++i) {
         TcConvPlan p;
         if (!fill_plan(c, cand[i][0], cand[i][1], cand[i][2], cand[i][3], p)) continue;
-        double cost = tile_cost(p, 1);
-        // pairs of 64-channel tiles with two accumulators measure 12-15 % slower than this model says
-        // (64 -> 64 channels at 56x56: 59 us against 52 us with one CTA per tile)
-        if (p.ctas == 2 && p.MT == 2 && p.BN <= 64 && p.KB >= 16) cost *= 1.15;
-        // tap-pair mode (thin first layers) streams hardly any weights, so a pair shares nothing worth its
-        // hand-over (ResNet-50 stem: 106.8 us as pairs, 101.8 us with one CTA per tile)
-        if (p.ctas == 2 && p.KB == 4) cost *= 1.15;
+        const double cost = tile_cost(p, 1);
         if (!have || cost < best_cost * 0.999) {
             have = true;
             best_cost = cost;
@@ -1083,7 +1140,7 @@ bool tc_conv_plan(const ConvGeom &c, TcConvPlan &plan, bool forced) {
         int pb = 0, pk = 0, ps = 0;         // ONNXB_CONV_SPLIT = "BN,KB,S" pins the shape, "0" rules the split out
         const char *e = getenv("ONNXB_CONV_SPLIT");
         const bool pinned = e && sscanf(e, "%d,%d,%d", &pb, &pk, &ps) == 3;
-        const bool ruled_out = (e && !pinned) || getenv("ONNXB_CONV_TILE") || getenv("ONNXB_CONV_STAGES") || getenv("ONNXB_CONV_EPI");
+        const bool ruled_out = (e && !pinned) || getenv("ONNXB_CONV_TILE") || getenv("ONNXB_CONV_STAGES");
         if (c.Cg >= 32 && !ruled_out && (pinned || (have && plan.total_tiles * plan.ctas <= 74))) {
             if (pinned) have = false;
             for (int kb = 16; kb <= 32; kb *= 2)
@@ -1113,14 +1170,6 @@ bool tc_conv_plan(const ConvGeom &c, TcConvPlan &plan, bool forced) {
         }
     }
     if (have) {
-        // Four epilogue warps (and 128 registers per thread) where the transform paces the kernel and a
-        // CTA walks several tiles: the tap-pair mode of thin first layers (measured: 116 -> 104 us on the
-        // ResNet-50 stem; 16-channel blocks gain nothing).  Pinned by
-        // ONNXB_CONV_EPI = 4 | 8 for A/B measurements.
-        const int units = sms / plan.ctas;
-        plan.epi_warps = (plan.KB == 4 && plan.total_tiles >= 3LL * units) ? 4 : 8;
-        if (const char *e = getenv("ONNXB_CONV_EPI"))
-            if (e[0] == '4' || e[0] == '8') plan.epi_warps = e[0] - '0';
         // Thin first layers in tap-pair mode are paced by the transform warps: take their fence off them too
         // (ResNet-50 stem: 109.3 -> 106.6 us).  ONNXB_CONV_RELAY = 0 | 1 pins the choice for A/B measurements.
         if (plan.ctas == 2 && plan.KB == 4) plan.relay = 1;
@@ -1137,7 +1186,7 @@ static int max_pairs() {
     if (n >= 0) return n;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * 148);
-    cfg.blockDim = dim3(threads_for(8));
+    cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmemLimit;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1147,7 +1196,7 @@ static int max_pairs() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_conv_kernel<2, false, 8, false>, &cfg) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, tc_conv_kernel<2, false, false, false>, &cfg) != cudaSuccess || n < 1) {
         cudaGetLastError();
         n = tc_host::num_sms() / 2;
     }
@@ -1156,6 +1205,9 @@ static int max_pairs() {
 }
 
 size_t tc_conv_workspace_bytes(const TcConvPlan &plan) { return (size_t)plan.packed_floats * 4; }
+
+static int launch_images(const TcConvPlan &plan, const float *X, const float *B, const float *R, float *Y, const void *workspace,
+                         unsigned int *err, cudaStream_t st);
 
 int launch_tc_conv(const TcConvPlan &plan, const float *X, const float *W, const float *B, const float *R, float *Y,
                    void *workspace, void *stream, int phase) {
@@ -1174,28 +1226,46 @@ int launch_tc_conv(const TcConvPlan &plan, const float *X, const float *W, const
         if (e != cudaSuccess) return (int)e;
     }
     if (phase == kTcConvPackOnly) return 0;
-    // 2. the convolution
+    // 2. the convolution; the kernel reaches outputs by 32-bit byte offsets, so an output of 4 GB and more is computed
+    // in several launches, some images each
+    const long long image = (long long)plan.M * plan.P * plan.Q;
+    const int most = (int)std::min<long long>(plan.N, ((1LL << 30) - 1) / image);
+    for (int n0 = 0; n0 < plan.N; n0 += most) {
+        TcConvPlan part = plan;
+        part.N = std::min(most, plan.N - n0);
+        part.total_slots = (long long)part.N * part.L;
+        part.pix_tiles = (int)((part.total_slots + part.ctas * part.MT * 128 - 1) / (part.ctas * part.MT * 128));
+        part.total_tiles = (long long)part.pix_tiles * part.ctiles * part.group;
+        const int e = launch_images(part, X + (long long)n0 * plan.C * plan.H * plan.W, B, R ? R + n0 * image : nullptr, Y + n0 * image,
+                                    workspace, err, st);
+        if (e != 0) return e;
+    }
+    return 0;
+}
+
+static int launch_images(const TcConvPlan &plan, const float *X, const float *B, const float *R, float *Y, const void *workspace,
+                         unsigned int *err, cudaStream_t st) {
+    using namespace tc_host;
     CUtensorMap tmX;
     if (plan.raw_mode == 0) {
         const uint64_t dims[2] = {(uint64_t)plan.H * plan.W, (uint64_t)plan.N * plan.C};
         const uint64_t str[1] = {(uint64_t)plan.H * plan.W * 4};
-        const uint32_t box[2] = {(uint32_t)plan.BOXP, (uint32_t)plan.KB};
+        const uint32_t box[2] = {(uint32_t)plan.BOXP, (uint32_t)plan.KBR};
         if (!make_tmap(&tmX, X, 2, dims, str, box, kTmapSwizzleNone)) return (int)cudaErrorInvalidValue;
     } else {
         memset(&tmX, 0, sizeof tmX);
     }
     const size_t smem = 1024 + (size_t)plan.na_stages * plan.a_stage_bytes + (size_t)plan.nr_stages * plan.raw_stage_bytes +
-                        (size_t)plan.nb_stages * plan.b_stage_bytes + kMaxRawStages * kSegBytes + kBarBytes;
+                        (size_t)plan.nb_stages * plan.b_stage_bytes + kMaxRawStages * kSegBytes + kBiasBytes + kBarBytes;
     const bool pair = plan.ctas == 2;
     const bool add = R != nullptr;
-    const bool epi4 = plan.epi_warps == 4;
     const bool split = plan.split > 1;
-    auto kern = split  ? (add ? tc_conv_kernel<1, true, 8, true> : tc_conv_kernel<1, false, 8, true>)
-                : epi4 ? (pair ? (add ? tc_conv_kernel<2, true, 4, false> : tc_conv_kernel<2, false, 4, false>)
-                               : (add ? tc_conv_kernel<1, true, 4, false> : tc_conv_kernel<1, false, 4, false>))
-                       : (pair ? (add ? tc_conv_kernel<2, true, 8, false> : tc_conv_kernel<2, false, 8, false>)
-                               : (add ? tc_conv_kernel<1, true, 8, false> : tc_conv_kernel<1, false, 8, false>));
-    const int threads = threads_for(epi4 && !split ? 4 : 8);
+    const bool thin = plan.KB == 4;
+    auto kern = split  ? (add ? tc_conv_kernel<1, true, false, true> : tc_conv_kernel<1, false, false, true>)
+                : thin ? (pair ? (add ? tc_conv_kernel<2, true, true, false> : tc_conv_kernel<2, false, true, false>)
+                               : (add ? tc_conv_kernel<1, true, true, false> : tc_conv_kernel<1, false, true, false>))
+                       : (pair ? (add ? tc_conv_kernel<2, true, false, false> : tc_conv_kernel<2, false, false, false>)
+                               : (add ? tc_conv_kernel<1, true, false, false> : tc_conv_kernel<1, false, false, false>));
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return (int)e;
     const int sms = num_sms();
@@ -1210,9 +1280,9 @@ int launch_tc_conv(const TcConvPlan &plan, const float *X, const float *W, const
             plan.raw_stage_bytes, plan.b_stage_bytes, plan.nb_stages, smem);
 #endif
     const cudaError_t le =
-        pair || split ? launch_pdl_cluster(kern, split ? (unsigned)plan.split : 2u, dim3(grid), dim3(threads), smem, st, tmX, plan, X,
+        pair || split ? launch_pdl_cluster(kern, split ? (unsigned)plan.split : 2u, dim3(grid), dim3(kThreads), smem, st, tmX, plan, X,
                                   reinterpret_cast<const float *>(workspace), B, R, Y, err)
-             : launch_pdl(kern, dim3(grid), dim3(threads), smem, st, tmX, plan, X,
+             : launch_pdl(kern, dim3(grid), dim3(kThreads), smem, st, tmX, plan, X,
                           reinterpret_cast<const float *>(workspace), B, R, Y, err);
     count_launch();
     return (int)le;

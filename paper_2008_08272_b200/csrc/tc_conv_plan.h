@@ -44,6 +44,7 @@ struct TcConvPlan {
     //   KB = 16 ("channel pairs"): chunks 2j, 2j+1 of the same tap, two steps per tap;
     //   KB = 4  ("tap pairs", for C/group < 16): the single chunk read at two taps of the same plane.
     int KB, nchunks, n_steps;
+    int chunk_groups, chunks_per_unit;   // how the re-lay splits a slot's chunks over threads: nchunks = groups x per unit
     uint32_t step_a[kConvMaxSteps];      // A descriptor low word relative to the stage: offset/16 | (LBO/16) << 16
     short src_tap[kConvMaxSteps][2];     // which filter tap feeds chunk 0 / 1 of the step's weights (-1: zeros)
     short src_c0[kConvMaxSteps][2];      // and from which channel offset inside the block
@@ -59,6 +60,7 @@ struct TcConvPlan {
     // raw staging
     int raw_mode;                    // 0: tensor-map boxes [KB][BOXP] over X seen as (H*W, N*C); 1: whole-image slabs
     int BOXP;
+    int KBR;                         // channels staged per block: KB, or all of a group's if it has fewer
     // shared memory carve-up (bytes)
     int a_stage_bytes, raw_stage_bytes, b_stage_bytes, nb_stages, nr_stages, na_stages;
     int spb, b_step_bytes, b_steps;  // K-steps per weight stage, bytes of one step's weights, weight stages per block
@@ -69,7 +71,7 @@ struct TcConvPlan {
     ConvDivisor dv_L, dv_Ws, dv_Hs, dv_BOXP, dv_SLOTS, dv_pss;
     int boxp_shift;                  // log2(BOXP) when BOXP is a power of two, else -1
     int split, cb_per;               // CTAs (a cluster) sharing a tile's channel blocks, blocks of each; split = 1: none
-    int epi_warps;                   // epilogue warps of the launch: 8, or 4 (then 128 registers per thread)
+    int b_resident;                  // all tiles use the same few weights: fetched once per CTA
     int relay;                       // pairs: the odd CTA's "operand stage written" goes through its relay warp
 };
 
@@ -146,13 +148,13 @@ ONNXB_HD inline void tc_conv_segments(const TcConvPlan &g, long long G0, TcConvS
         } else if (g.raw_mode == 1) {
             t.f0[i] = 0;
             t.nbox[i] = 1;
-            base += g.KB * g.H * g.W;
+            base += g.KBR * g.H * g.W;
         } else {
             const int f0 = (h_min * g.W) & ~3;
             const int len = (h_max + 1) * g.W - f0;
             t.f0[i] = f0;
             t.nbox[i] = conv_fdiv(len + g.BOXP - 1, g.BOXP, g.dv_BOXP);
-            base += t.nbox[i] * g.BOXP * g.KB;
+            base += t.nbox[i] * g.BOXP * g.KBR;
         }
     }
     t.total_floats = base;
