@@ -3,11 +3,13 @@
 // The persistent kernel of tc_gemm.cu gives such a problem one serial K loop per tile on a fraction of the
 // SMs.  Here a cluster of S CTAs shares one 128 x BN output tile: CTA r of the cluster reduces K-blocks
 // [r * kb_per, (r + 1) * kb_per) into its own TMEM accumulator (TMA -> shared memory -> tcgen05.mma, as in
-// tc_gemm.cu), parks the partial tile in its shared memory (over the operand ring, which is done with), and after
-// a cluster barrier every CTA sums one slice of the tile's rows over all S partials through distributed
-// shared memory, applies the epilogue and stores it.  The S partials of an element are always added in
-// rank order, so the result does not depend on timing.
-// Bound: latency (launch, first fill, K loop, exchange); the split shortens the one part that grows with K.
+// tc_gemm.cu).  Every CTA finishes one slice of the tile's rows: the others write their partial sums of it straight
+// from registers into a buffer of that CTA's shared memory (st.async, counted on an mbarrier there), and it adds them
+// in rank order, so the result does not depend on timing, applies the epilogue and stores the slice.
+// Bound: latency (launch, first fill, K loop, exchange); the split shortens the one part that grows with K.  Partial
+// tiles parked in the own shared memory, a cluster barrier, reads of the peers' and a second cluster barrier took
+// some 1.1 us longer (ResNet-50 at batch 1, with 37 such layers: 489 -> 447 us): a read waits for a trip to the peer
+// and back, a write is sent and done with.
 // ONNX Gemm's operands are rounded to TF32 (nearest) inside the kernel: while a stage waits for its MMAs, the
 // eight epilogue warps, otherwise idle during the main loop, round it in place in shared memory, so callers
 // pass A and B as they are and need no rounding pass in front (the tensor core would truncate them).  A
@@ -44,8 +46,9 @@ struct SkParams {
     int a_kbox, b_kbox;        // K-major with K a multiple of 32: one copy brings all K blocks of a stage
     int b_big, b_nblk_full;    // MN-major B through a view of its full 32-column blocks: one copy as well
     int round;                 // round the operands in shared memory
-    int BN, S, tiles_m, tiles_n, num_kb, kb_per, num_stages, rows_per, pitch;   // pitch: floats between rows of a partial tile
-    uint32_t stage_bytes, idesc;
+    int BN, S, tiles_m, tiles_n, num_kb, kb_per, num_stages;
+    int rows_per, pitch;       // rows of a slice; slots of 16 bytes between a slice's column groups (odd: see the exchange)
+    uint32_t stage_bytes, recv_off, idesc;     // recv_off: from the first stage to the partial sums
     float alpha, beta;
     const float *C, *row_bias, *R;
     long long c_si, c_sj;
@@ -58,13 +61,19 @@ struct SkParams {
     unsigned int *err;
 };
 
-__device__ __forceinline__ float4 ld_cluster_v4(uint32_t cluster_addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(cluster_addr)
-                 : "memory");
-    return v;
+// n4 16-byte pieces of a stage to TF32 in place, by kRoundWarps warps
+__device__ __forceinline__ void round_tile(uint8_t *tile, int n4, int rt) {
+    float4 *t4 = reinterpret_cast<float4 *>(tile);
+    for (int j = rt; j < n4; j += 4 * kRoundWarps * 32) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (j + u * kRoundWarps * 32 < n4) v[u] = t4[j + u * kRoundWarps * 32];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (j + u * kRoundWarps * 32 < n4)
+                t4[j + u * kRoundWarps * 32] = make_float4(round_tf32(v[u].x), round_tf32(v[u].y), round_tf32(v[u].z), round_tf32(v[u].w));
+    }
 }
 
 // kKS: K blocks per stage (two wherever a CTA has two: see tc_gemm.cu for what a stage costs its issuing threads)
@@ -76,9 +85,9 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
     uint8_t *stages = smem + 1024;
-    float *partial = reinterpret_cast<float *>(stages);               // [row][pitch], once the ring is done with
-    uint64_t *full = bars, *empty = bars + kMaxStages, *ready = bars + 2 * kMaxStages, *acc_full = bars + 3 * kMaxStages;
-    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bars + 3 * kMaxStages + 1);
+    uint8_t *recv = stages + p.recv_off;
+    uint64_t *full = bars, *empty = bars + kMaxStages, *ready = bars + 2 * kMaxStages, *acc_full = bars + 3 * kMaxStages, *recv_full = acc_full + 1;
+    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bars + 3 * kMaxStages + 2);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = p.S > 1 ? (int)cluster_ctarank() : 0;
@@ -89,6 +98,9 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     const int tn = tile % p.tiles_n, batch = tile / p.tiles_n;
     const int kb0 = rank * p.kb_per, kb1 = min(p.num_kb, kb0 + p.kb_per);
     const int nkb = max(kb1 - kb0, 0);                                // K-blocks this CTA reduces (0: a rank past the end)
+    const int nsrc = min(p.S, (p.num_kb + p.kb_per - 1) / p.kb_per);  // ranks that have any
+    const int row_lo = rank * p.rows_per;                             // the slice of rows this CTA finishes
+    const int row_hi = min(min(kBM, row_lo + p.rows_per), p.M - tm * kBM);
 
     if (warp == 2) {
         // a barrier per lane: one thread would take a thousand cycles for them
@@ -98,6 +110,10 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             mbar_init(&ready[lane], kRoundWarps);
         }
         if (lane == 31) mbar_init(acc_full, 1);
+        if (lane == 30 && p.S > 1) {
+            mbar_init(recv_full, 1);
+            mbar_arrive_expect_tx(recv_full, (uint32_t)(max(row_hi - row_lo, 0) * p.BN * 4 * nsrc));
+        }
         mbar_fence_init();
     } else if (threadIdx.x == 0) {
         prefetch_tmap(&tmA);
@@ -111,6 +127,7 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    if (p.S > 1) cluster_arrive();                                    // this CTA's barriers exist
     const uint32_t tmem_base = *tmem_holder;
     pdl_launch_dependents();
 
@@ -188,22 +205,21 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     } else {
         if (p.round) {
             // round every landed stage to TF32 in place (elementwise, so the swizzle does not matter)
-            const int n4 = (int)(p.stage_bytes >> 4), rt = ((warp - 2) % kRoundWarps) * 32 + lane, mine = (warp - 2) / kRoundWarps;
+            // (of a K-major A only the rows that exist: a classifier head at batch 1 has one of the 128)
+            const int rt = ((warp - 2) % kRoundWarps) * 32 + lane, mine = (warp - 2) / kRoundWarps;
+            const int a_rows = p.a_mn ? kBM : min(kBM, p.M - tm * kBM);
             int stage = 0;
             uint32_t phase = 0;
             for (int kb = 0, i = 0; kb < nkb; kb += kKS, ++i) {
                 if ((i & 1) == mine) {
                     mbar_wait(&full[stage], phase, p.err, 43);
-                    float4 *st4 = reinterpret_cast<float4 *>(stages + (size_t)stage * p.stage_bytes);
-                    for (int j = rt; j < n4; j += 4 * kRoundWarps * 32) {
-                        float4 v[4];
+                    uint8_t *st = stages + (size_t)stage * p.stage_bytes;
+                    if (a_rows == kBM) {
+                        round_tile(st, (int)(p.stage_bytes >> 4), rt);
+                    } else {
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (j + u * kRoundWarps * 32 < n4) v[u] = st4[j + u * kRoundWarps * 32];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (j + u * kRoundWarps * 32 < n4)
-                                st4[j + u * kRoundWarps * 32] = make_float4(round_tf32(v[u].x), round_tf32(v[u].y), round_tf32(v[u].z), round_tf32(v[u].w));
+                        for (int sub = 0; sub < kKS; ++sub) round_tile(st + sub * kABytes, a_rows * (kBK / 4), rt);
+                        round_tile(st + kKS * kABytes, p.BN * (kBK / 4) * kKS, rt);
                     }
                     fence_proxy_async_smem();          // generic-proxy writes, read next by the tensor core
                     __syncwarp();
@@ -212,42 +228,45 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                 if (++stage == p.num_stages) { stage = 0; phase ^= 1; }
             }
         }
-        // ------------------------------------------------------------ park this CTA's partial tile: partial[row][col]
+        // ------------------------------------------------------------ hand every slice of the partial tile to the CTA that finishes it
         const int q = warp & 3, half = (warp - 2) >> 2;               // TMEM lane quarter; two warps share one
         const int row = q * 32 + lane;
+        if (p.S > 1) cluster_wait();                                  // (the peers set up long ago)
         if (nkb > 0) {
+            const int dst = row / p.rows_per, n4 = p.BN / 4;
+            const bool wanted = row < p.M - tm * kBM;
+            uint32_t to = smem_u32(recv) + (uint32_t)((rank * n4 + half * 8) * p.pitch + row - dst * p.rows_per) * 16u, bar = smem_u32(recv_full);
+            if (p.S > 1) {
+                to = map_to_cta(to, (uint32_t)dst);
+                bar = map_to_cta(bar, (uint32_t)dst);
+            }
             mbar_wait(acc_full, 0, p.err, 42);
             tc_fence_after_sync();
-        }
-        for (int c0 = half * 32; c0 < p.BN; c0 += 64) {
-            uint32_t v[32];
-            if (nkb > 0) {
+            for (int c0 = half * 32; c0 < p.BN; c0 += 64, to += 256u * (uint32_t)p.pitch) {
+                uint32_t v[32];
                 tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
                 tmem_ld_wait();
-            } else {
+                if (wanted && p.S == 1) {
+                    float4 *own = reinterpret_cast<float4 *>(recv) + (c0 / 4) * p.pitch + row;
 #pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = 0u;
+                    for (int j = 0; j < 8; ++j)
+                        own[j * p.pitch] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                                                       __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+                } else if (wanted) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        st_async_v4(to + (uint32_t)(j * p.pitch) * 16u, v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3], bar);
+                }
             }
-            float4 *d = reinterpret_cast<float4 *>(partial + row * p.pitch + c0);
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                d[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]), __uint_as_float(v[4 * j + 2]),
-                                   __uint_as_float(v[4 * j + 3]));
         }
         tc_fence_before_sync();
-    }
+        if (p.S == 1) asm volatile("bar.sync 1, %0;" ::"n"(kWorkers * 32) : "memory");
+        else cluster_arrive();                                        // sent; waited for on the way out only
 
-    // every CTA's partial tile is in its shared memory
-    if (p.S > 1) cluster_sync_all();
-    else __syncthreads();
-
-    if (warp >= 2) {
-        // ------------------------------------------------------------ reduce this CTA's slice of rows over the cluster
+        // ------------------------------------------------------------ sum this CTA's slice of rows and store it
         pdl_wait();                                // long since satisfied: the producer passed its own before the first load
         const int t = (warp - 2) * 32 + lane;
-        const int n4 = p.BN / 4, row_lo = rank * p.rows_per;
-        const int row_hi = min(min(kBM, row_lo + p.rows_per), p.M - tm * kBM);
-        const uint32_t part_addr = smem_u32(partial);
+        const int n4 = p.BN / 4;
         const int col4 = t % n4, gcol = tn * p.BN + col4 * 4;
         for (int rr = row_lo + t / n4; rr < row_hi; rr += kWorkers * 32 / n4) {
             if (gcol >= p.N) break;
@@ -280,20 +299,16 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                 }
             }
             const float rb = p.row_bias ? __ldg(p.row_bias + grow) : 0.f;
+            // lanes along columns: an odd pitch puts eight neighbours on different banks
+            if (p.S > 1) mbar_wait_cluster(recv_full, 0, p.err, 44);
+            const float4 *x = reinterpret_cast<const float4 *>(recv) + col4 * p.pitch + rr - row_lo;
             float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-            const uint32_t off = (uint32_t)(rr * p.pitch + col4 * 4) * 4u;
-            if (p.S == 1) {
-                a = *reinterpret_cast<const float4 *>(reinterpret_cast<const uint8_t *>(partial) + off);
-            } else {
-                // all partials requested at once (a trip to a peer's shared memory takes some 600 cycles)
-                float4 x[8];
 #pragma unroll
-                for (int s = 0; s < 8; ++s)
-                    if (s < p.S) x[s] = ld_cluster_v4(map_to_cta(part_addr + off, (uint32_t)s));
-#pragma unroll
-                for (int s = 0; s < 8; ++s)
-                    if (s < p.S) { a.x += x[s].x; a.y += x[s].y; a.z += x[s].z; a.w += x[s].w; }
-            }
+            for (int s = 0; s < 8; ++s)
+                if (s < nsrc) {
+                    const float4 v = x[s * n4 * p.pitch];
+                    a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+                }
             float o[4] = {fmaf(p.alpha, a.x, rb) + add[0], fmaf(p.alpha, a.y, rb) + add[1], fmaf(p.alpha, a.z, rb) + add[2],
                           fmaf(p.alpha, a.w, rb) + add[3]};
             if (p.relu) {
@@ -310,10 +325,17 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         }
     }
 
-    // no CTA leaves while a peer may still read its partial tile
+    // no CTA leaves before its peers have sent their shares (they have, unless a wait above gave up)
+    if (p.S > 1) {
+        if (warp < 2) {
+            __syncwarp();
+            cluster_wait();
+            cluster_arrive();
+        }
+        cluster_wait();
+    }
     tc_fence_before_sync();
-    if (p.S > 1) cluster_sync_all();
-    else __syncthreads();
+    __syncthreads();
     if (warp == 1) {
         __syncwarp();
         tc_fence_after_sync();
@@ -351,10 +373,10 @@ int resident_ctas(int S) {
     return n;
 }
 
-// Shape with the shortest estimated time, against the persistent kernel's (both in ns, fitted to 90 problems: 1x1
-// convolutions of ResNet-50 at batch 1 to 32 and Gemms from 400^3 to 1024 x 1024 x 4096; the choice is within
-// 1 % of the best on average).  One wave of CTAs costs 3.7 us for its set-up, first fill and exchange, and a K block
-// 130-310 ns (360-550 when it is rounded in shared memory first).
+// Shape with the shortest estimated time, against the persistent kernel's (both in ns, fitted to 95 problems: 1x1
+// convolutions of ResNet-50 at batch 1 to 32 and Gemms from 1 x 1000 x 2048 to 1024 x 1024 x 4096; the choice is
+// within 1 % of the best on average).  One wave of CTAs costs 2.1 us for its set-up, first fill and exchange, and a
+// K block 160-400 ns (rounded in shared memory first: 180-570, with the rows of A there are).
 SkChoice search(const TcGemmProblem &g) {
     SkChoice c{0, 0};
     if ((g.a_batched && g.batch > 1) || (g.batch > 1 && g.b_batched && g.b_bs % 4)) return c;
@@ -367,8 +389,8 @@ SkChoice search(const TcGemmProblem &g) {
             if (ctas > 4 * 148) break;
             const int units = resident_ctas(S);
             const double waves = (double)((ctas + units - 1) / units);
-            const double blk = g.round_operands ? 293.0 + 2.0 * BN : 67.0 + 1.9 * BN;
-            const double t = waves * ((num_kb + S - 1) / S * blk + 3700.0 + 25.0 * BN + (S == 8 ? 500.0 : 0.0));
+            const double blk = g.round_operands ? 137.0 + 1.4 * BN + 2.0 * std::min(g.M, kBM) : 79.0 + 2.54 * BN;
+            const double t = waves * ((num_kb + S - 1) / S * blk + 2090.0 + 29.6 * BN) + 1040.0;
             if (t < best) {
                 best = t;
                 c = {BN, S};
@@ -426,11 +448,13 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
     p.num_kb = (g.K + kBK - 1) / kBK;
     p.kb_per = (p.num_kb + p.S - 1) / p.S;
     p.rows_per = (kBM + p.S - 1) / p.S;
-    p.pitch = p.BN + 4;                      // rows of a partial tile 16-byte aligned, eight rows on different banks
+    p.pitch = p.rows_per | 1;
+    const size_t recv_bytes = (size_t)p.S * (p.BN / 4) * p.pitch * 16;
+    // two K blocks per stage, where that leaves two stages beside the partial sums
     const int ks = p.kb_per >= 2 ? 2 : 1;
     p.stage_bytes = (uint32_t)(kABytes + p.BN * 128) * ks;
     // (never more stages than the share has: a small footprint lets the next kernel's CTAs set up beside this one)
-    p.num_stages = std::min({kMaxStages, std::max(2, (p.kb_per + ks - 1) / ks), (int)((kSmemLimit - 2048) / p.stage_bytes)});
+    p.num_stages = std::min({kMaxStages, std::max(2, (p.kb_per + ks - 1) / ks), (int)((kSmemLimit - 2048 - recv_bytes) / p.stage_bytes)});
     p.idesc = tc::make_idesc_tf32(kBM, p.BN, p.a_mn, p.b_mn);
     p.alpha = g.alpha; p.beta = g.beta;
     p.C = g.C; p.c_si = g.c_si; p.c_sj = g.c_sj;
@@ -473,8 +497,8 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
         const uint32_t box[4] = {32, (uint32_t)(kBK * ks), (uint32_t)(p.BN / 32), 1};
         p.b_big = make_tmap(&tmBb, g.B, 4, dims, str, box, kTmapSwizzle128Atom32) ? 1 : 0;
     }
-    const size_t ring = (size_t)p.num_stages * p.stage_bytes, parked = (size_t)kBM * p.pitch * 4;
-    const size_t smem = 2048 + std::max(ring, parked);
+    p.recv_off = (uint32_t)p.num_stages * p.stage_bytes;
+    const size_t smem = 2048 + p.recv_off + recv_bytes;
     auto kern = ks == 2 ? tc_gemm_splitk_kernel<2> : tc_gemm_splitk_kernel<1>;
     const cudaError_t ae = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (ae != cudaSuccess) return (int)ae;
