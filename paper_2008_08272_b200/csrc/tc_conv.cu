@@ -71,6 +71,7 @@ struct Bars {
     uint64_t b_full[kMaxBStages], b_empty[kMaxBStages];
     uint64_t acc_full[2], acc_empty[2];
     uint64_t seg_full[2], seg_empty[2];      // segment tables, one per tile parity
+    uint64_t recv_full;                      // split: all partial sums of this CTA's channels have arrived
     uint32_t tmem_holder;
 };
 static_assert(sizeof(Bars) <= kBarBytes, "barrier block too large");
@@ -111,25 +112,26 @@ __global__ void pack_weights_kernel(const TcConvPlan g, const float *__restrict_
     }
 }
 
-__device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
-    return v;
-}
-
 // Channel blocks are summed in a rotated order that differs from tile to tile: CTAs working at the
 // same time then stream different parts of the (shared) packed weights, instead of all asking the
 // same L2 lines at the same moment.
 __device__ __forceinline__ int cb_rotation(long long tile, int ncb) { return (int)((tile * 5 + 3) % ncb); }
 
+// TMEM columns of a split tile: its one accumulator (read in blocks of 32)
+__host__ __device__ constexpr uint32_t split_tmem_cols(int BN) { return BN <= 32 ? 32u : BN <= 64 ? 64u : BN <= 128 ? 128u : 256u; }
+// shared memory for its partial sums
+__host__ __device__ constexpr int split_recv_bytes(int split, int cols_per) { return split * cols_per * 512; }
+
 // ------------------------------------------------------------------ main kernel
 // kAdd: the epilogue also adds a tensor laid out like Y (a residual connection) before the Relu.  A
 // separate instantiation, so that the plain kernel's register allocation is not disturbed.
-// kEpiWarps: 8 or 4 epilogue warps (see the thread layout above).
 // kSplit: the problem has few tiles, so a cluster of g.split CTAs shares one: CTA r reduces the channel blocks
-// [r * cb_per, (r + 1) * cb_per), parks its partial tile in shared memory (over the stages, which are done with),
-// and after a cluster barrier sums one slice of the tile's channels over all partials through distributed
-// shared memory, in rank order.  One 14x14 image, 256 -> 256 channels: 24 -> 8 us.
+// [r * cb_per, (r + 1) * cb_per) and finishes one slice of the tile's channels.  The epilogue warps write each partial
+// sum from TMEM straight into the shared memory of the CTA that finishes it (st.async, counted on an mbarrier there);
+// that CTA adds them in rank order.  Bound: latency, about 12,700 cycles for one 28x28 image, of which 3,000 are set-up
+// and waiting for the previous kernel, 2,800 the first block's way to the tensor core and 1,900 the exchange (reading
+// the peers' partial tiles between two cluster barriers took 2,200 more).  One 14x14 image, 256 -> 256 channels: 24 us
+// unsplit, 8.6 split over 8; 28x28, 128 channels 15.7 -> 8.3.
 // kThin: blocks of one 4-channel chunk (tap pairs).
 template <int kCtas, bool kAdd, bool kThin, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -147,6 +149,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
     uint8_t *seg_st = b_st + (size_t)g.nb_stages * g.b_stage_bytes;
     uint8_t *bias_st = seg_st + kMaxRawStages * kSegBytes;
     Bars *bars = reinterpret_cast<Bars *>(bias_st + kBiasBytes);
+    uint8_t *recv_st = reinterpret_cast<uint8_t *>(bars) + kBarBytes;        // split: partial sums from every CTA
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) LOG(8, 0);
@@ -158,6 +161,9 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
     const int cb_lo = kSplit ? (int)cluster_ctarank() * g.cb_per : 0;                  // channel blocks of this CTA
     const int cb_cnt = kSplit ? min(g.ncb - cb_lo, g.cb_per) : g.ncb;
     const int cgt = g.ctiles * g.group;        // channel tiles over all groups
+    // split: the channels of the tile that this CTA finishes (whole groups of four)
+    const int tile_ch = min(g.BN, g.Mg - (int)(first_tile % cgt) % g.ctiles * g.BN), tile_ch4 = (tile_ch + 3) & ~3;
+    const int col_lo = kSplit ? (int)cluster_ctarank() * g.cols_per : 0, col_hi = min(tile_ch4, col_lo + g.cols_per);
     // accumulator placement in TMEM: two alternating sets when one set fits in 256 columns
     const bool acc_dbl = g.MT == 1 || g.BN <= 128;
     const uint32_t mt_cols = acc_dbl ? 128u : 256u;     // column distance between a CTA's two accumulators
@@ -182,6 +188,10 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             mbar_init(&bars->acc_empty[lane], kEpiWarps);
             mbar_init(&bars->seg_full[lane], 1);
             mbar_init(&bars->seg_empty[lane], kXformWarps);
+        }
+        if (lane == 31) {
+            mbar_init(&bars->recv_full, 1);
+            mbar_arrive_expect_tx(&bars->recv_full, (uint32_t)(max(col_hi - col_lo, 0) * 512 * g.split));
         }
         mbar_fence_init();
     }
@@ -212,7 +222,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
     }
     if (kSplit && threadIdx.x == 0 && g.raw_mode == 0) prefetch_tmap(&tmX);
     if (warp == 2) {
-        tmem_alloc(&bars->tmem_holder, 512);
+        tmem_alloc(&bars->tmem_holder, kSplit ? split_tmem_cols(g.BN) : 512);
         tmem_relinquish();
     }
     tc_fence_before_sync();
@@ -220,6 +230,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
     tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_holder;
     if (kCtas == 2) cluster_sync_all();     // the peer's barriers exist before anything arrives on them
+    if (kSplit) cluster_arrive();           // (waited for when the partial sums go out)
     pdl_launch_dependents();
     // Everything above overlapped the previous kernel's tail, and so does each role's own set-up below:
     // the threads that touch global memory (the two producers, the epilogue warps) wait for the previous
@@ -639,17 +650,23 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             if (ew == 0 && lane == 0) LOG(8, 2);
             const int nch = (g.BN + 31) / 32;
             if (kSplit) {
-                // park the partial tile as [channel][row]: lanes write consecutive rows
-                float *part = reinterpret_cast<float *>(smem);
-                const int pitch = tile_rows + 4, mt = two ? ew >> 2 : 0;
-                const int row = mt * 128 + quarter * 32 + lane;
-                for (int chunk = two ? 0 : ew >> 2; chunk < nch; chunk += two ? 1 : 2) {
+                // every group of four channels goes to the CTA that finishes it, as [source CTA][group][pixel][4]:
+                // the lanes of a store write consecutive 16-byte pieces
+                cluster_wait();                 // (the peers set up long ago)
+                const uint32_t to = smem_u32(recv_st) + (cluster_ctarank() * (uint32_t)g.cols_per / 4u * 128u + (uint32_t)(quarter * 32 + lane)) * 16u;
+                const uint32_t bar = smem_u32(&bars->recv_full);
+                for (int chunk = ew >> 2; chunk < nch; chunk += kEpiWarps / 4) {
                     uint32_t v[32];
-                    tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + ab * 256u + (uint32_t)mt * mt_cols + (uint32_t)(chunk * 32), v);
+                    tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(chunk * 32), v);
                     tmem_ld_wait();
+                    int dst = chunk * 32 / g.cols_per, in = chunk * 32 - dst * g.cols_per;       // owner, and the place in its slice
 #pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (chunk * 32 + j < g.BN) part[(chunk * 32 + j) * pitch + row] = __uint_as_float(v[j]);
+                    for (int j = 0; j < 32; j += 4) {
+                        if (chunk * 32 + j < tile_ch4)
+                            st_async_v4(map_to_cta(to + (uint32_t)in * 512u, (uint32_t)dst), v[j], v[j + 1], v[j + 2], v[j + 3], map_to_cta(bar, (uint32_t)dst));
+                        in += 4;
+                        if (in == g.cols_per) { in = 0; ++dst; }
+                    }
                 }
             }
             if (!kSplit) {
@@ -714,60 +731,60 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
         }
     }
 
-    tc_fence_before_sync();
-    __syncthreads();
     if (kSplit) {
-        cluster_sync_all();                 // every CTA's partial tile is in its shared memory
-        const int rows = tile_rows, pitch = tile_rows + 4, nthr = 512, tid = threadIdx.x;
-        const int cols_per = (g.BN + g.split - 1) / g.split, col_lo = (int)cluster_ctarank() * cols_per;
-        const int ct_all = (int)(first_tile % cgt), grp = ct_all / g.ctiles, ct = ct_all % g.ctiles;
-        const int col_hi = min(min(g.BN, col_lo + cols_per), g.Mg - ct * g.BN);
-        const int row = tid % rows;         // lanes along pixels
-        const uint32_t G = (uint32_t)((first_tile / cgt) * tile_rows) + (uint32_t)row;
-        if (tid < nthr && G < (uint32_t)g.total_slots) {
-            pdl_wait();                     // long since satisfied
+        __syncwarp();
+        if (warp < kFirstEpiWarp) cluster_wait();
+        cluster_arrive();                       // sent
+        if (warp >= kFirstXformWarp) {
+            // sum this CTA's channels over the sources, in rank order: lanes along pixels, four channels each
+            const int tid = threadIdx.x - kFirstXformWarp * 32, row = tid & 127;
+            constexpr int kGroups = (kXformWarps + kEpiWarps) / 4;
+            const int ct_all = (int)(first_tile % cgt), grp = ct_all / g.ctiles, ct = ct_all % g.ctiles;
+            const uint32_t G = (uint32_t)((first_tile / cgt) * 128) + (uint32_t)row;
             const int n = conv_fdiv((int)G, g.L, g.dv_L), u = (int)G - n * g.L;
             const int p = conv_fdiv(u, g.Ws, g.dv_Ws), q = u - p * g.Ws;
-            if (p < g.P && q < g.Q) {
+            if (G < (uint32_t)g.total_slots && p < g.P && q < g.Q) {
+                pdl_wait();                     // long since satisfied
                 const long long PQ = (long long)g.P * g.Q;
-                const uint32_t part_addr = smem_u32(smem);
-                // Two channels at a time, all their partials requested at once: a trip to a peer's shared memory
-                // takes some 600 cycles (one 14x14 image, split over 8: 3.7 -> 1.2 us for the exchange).
-                for (int col0 = col_lo + tid / rows; col0 < col_hi; col0 += 2 * (nthr / rows)) {
-                    float v[2][8], b[2], r[2];
+                for (int col = col_lo + (tid >> 7) * 4; col < col_hi; col += kGroups * 4) {
+                    const int m = grp * g.Mg + ct * g.BN + col, cnt = tile_ch - col;          // channels that exist (above 4: all)
+                    const long long o = ((long long)n * g.M + m) * PQ + (long long)p * g.Q + q;
+                    float b[4], r[4];
 #pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const int col = min(col0 + u * (nthr / rows), col_hi - 1), m = grp * g.Mg + ct * g.BN + col;
-                        const uint32_t off = part_addr + (uint32_t)(col * pitch + row) * 4u;
-#pragma unroll
-                        for (int sp = 0; sp < 8; ++sp)
-                            if (sp < g.split) v[u][sp] = ld_cluster_f32(map_to_cta(off, (uint32_t)sp));
-                        b[u] = bias ? __ldg(bias + m) : 0.f;
-                        r[u] = kAdd ? __ldg(R + ((long long)n * g.M + m) * PQ + (long long)p * g.Q + q) : 0.f;
+                    for (int e = 0; e < 4; ++e) {
+                        b[e] = bias && e < cnt ? __ldg(bias + m + e) : 0.f;
+                        r[e] = kAdd && e < cnt ? __ldg(R + o + e * PQ) : 0.f;
                     }
+                    mbar_wait_cluster(&bars->recv_full, 0, err, 23);
+                    const float4 *x = reinterpret_cast<const float4 *>(recv_st) + (col - col_lo) / 4 * 128 + row;
+                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const int col = col0 + u * (nthr / rows);
-                        if (col >= col_hi) break;
-                        float x = 0.f;
+                    for (int s = 0; s < 8; ++s)
+                        if (s < g.split) {
+                            const float4 v = x[s * (g.cols_per / 4) * 128];
+                            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+                        }
+                    const float f[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
-                        for (int sp = 0; sp < 8; ++sp)
-                            if (sp < g.split) x += v[u][sp];
-                        x += b[u];
-                        if (kAdd) x += r[u];
-                        if (g.relu) x = fmaxf(x, 0.f);
-                        Y[((long long)n * g.M + grp * g.Mg + ct * g.BN + col) * PQ + (long long)p * g.Q + q] = x;
+                    for (int e = 0; e < 4; ++e) {
+                        float y = f[e] + b[e];
+                        if (kAdd) y += r[e];
+                        if (g.relu) y = fmaxf(y, 0.f);
+                        if (e < cnt) Y[o + e * PQ] = y;
                     }
                 }
             }
         }
+        cluster_wait();                         // no CTA leaves before its peers have sent (they have, unless a wait gave up)
     }
-    if (kCtas == 2 || kSplit) cluster_sync_all();     // no CTA leaves while a peer may still signal it or read its partial tile
+    tc_fence_before_sync();
+    __syncthreads();
+    if (kCtas == 2) cluster_sync_all();         // no CTA leaves while its peer may still signal it
     if (threadIdx.x == 0) LOG(8, 4);
     if (warp == 2) {
         __syncwarp();
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, 512);
+        tmem_dealloc(tmem_base, kSplit ? split_tmem_cols(g.BN) : 512);
     }
 }
 
@@ -1060,31 +1077,47 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     return true;
 }
 
-// Estimated SM cycles of a plan, fitted to 703 measured (shape, tile) pairs: 40 shapes from ResNet-50's 3x3 layers at
-// batch 8 to 64 to random ones of 16-320 channels, 3x3 and 5x5, stride 1 and 2; the pick is within 0.2 % of the
-// best tile on average.  Per channel block the slowest of: the tensor pipe (BN/2 cycles per 128 x BN x 8 share of an
-// instruction, or its operands out of shared memory at 160 bytes/cycle) with 380 cycles per weight stage; shared
-// memory as a whole (operand reads, stages written, re-lay) at 126 bytes/cycle; the weight stream out of L2 (18
-// bytes/cycle and SM, 2800 over all SMs) or, where the ring is short, its latency of 1900 cycles; and the re-lay, 75
-// cycles per chunk of the busiest thread.  split: CTAs sharing a tile's channel blocks.
-double tile_cost(const TcConvPlan &p, int split) {
-    const int sms = 148;
-    const int units = sms / p.ctas / split;                             // tiles in flight
+// Shares each tile of a plan among a cluster of S: no more stages than a share has blocks, beside room for the partial sums.
+bool split_plan(int S, TcConvPlan &p) {
+    p.split = S;
+    p.cb_per = (p.ncb + S - 1) / S;
+    if (p.cb_per * (S - 1) >= p.ncb) return false;                       // every CTA needs a block
+    p.cols_per = ((p.BN + S - 1) / S + 3) / 4 * 4;
+    p.na_stages = std::min(p.na_stages, p.cb_per);
+    p.nr_stages = std::min(p.nr_stages, p.cb_per);
+    const long long room = kSmemLimit - 1024 - (long long)p.na_stages * p.a_stage_bytes - (long long)p.nr_stages * p.raw_stage_bytes -
+                           kMaxRawStages * kSegBytes - kBiasBytes - kBarBytes - split_recv_bytes(S, p.cols_per);
+    p.nb_stages = (int)std::min<long long>({(long long)kMaxBStages, (long long)p.cb_per * p.b_steps, room / p.b_stage_bytes});
+    return p.nb_stages >= std::min(2, p.cb_per * p.b_steps);
+}
+
+// Estimated SM cycles of a plan, fitted to 2336 measured (shape, tile) pairs: 70 shapes from ResNet-50's 3x3 layers at
+// batch 1 to 64 to random ones of 16-384 channels, 3x3 and 5x5, stride 1 and 2, one image and many; the pick is within
+// 1 % of the best tile on average.  Per channel block the slowest of: the tensor pipe (0.57 BN cycles per 128 x BN x 8
+// share of an instruction, or its operands out of shared memory at 126 bytes/cycle) with 390 cycles per weight stage;
+// shared memory as a whole (operand reads, stages written, re-lay) at 115 bytes/cycle; the weight stream out of L2 (32
+// bytes/cycle and SM, 3600 over all SMs) or, where the ring is short, its latency of 2100 cycles; the re-lay, 42 cycles
+// per chunk of the busiest thread; and the producer's copies, some 330 per image a tile touches.
+double tile_cost(const TcConvPlan &p) {
+    // tiles in flight (a cluster of 8 does not fit every GPC: 14 of them are resident at once, and 33 of 4)
+    const int units = p.split == 8 ? 14 : p.split == 4 ? 33 : 148 / p.ctas / p.split;
     const long long waves = (p.total_tiles + units - 1) / units;
-    const double active = (double)std::min<long long>(p.total_tiles, units) * p.ctas * split;
+    const double active = (double)std::min<long long>(p.total_tiles, units) * p.ctas * p.split;
     const bool pair = p.ctas == 2;
     const double n_inst = (double)p.n_steps * p.MT, op_bytes = 4096.0 + p.BNH * 32.0;
-    const double t_mma = n_inst * std::max(p.BN * 0.485, op_bytes / 160.0) + (p.n_steps + p.spb - 1) / p.spb * 380.0;
+    const double t_mma = n_inst * std::max(p.BN * 0.568, op_bytes / 126.0) + (p.n_steps + p.spb - 1) / p.spb * 391.0;
     const double w_bytes = p.b_resident ? 0.0 : (double)p.n_steps * p.b_step_bytes;
     const double slots16 = (double)p.planes * p.SLOTS * 16.0 * p.nchunks;
-    const double t_smem = (n_inst * op_bytes + w_bytes + 3.0 * slots16) / 126.0;
+    const double t_smem = (n_inst * op_bytes + w_bytes + 3.0 * slots16) / 115.0;
     const double ring = (double)p.nb_stages * p.b_stage_bytes;
-    const double t_w = std::max(w_bytes / std::min(17.6, 2800.0 / active), w_bytes * 1930.0 / ring);
+    const double t_w = std::max(w_bytes / std::min(31.5, 3620.0 / active),
+                                p.split > 1 && ring >= w_bytes * p.cb_per ? 0.0 : w_bytes * 2090.0 / ring);
     const double owned = (p.planes * p.SLOTS * p.chunk_groups + kXformThreads - 1) / kXformThreads;
-    const double t_x = 740.0 + 75.0 * owned * p.chunks_per_unit + (pair ? 1080.0 : 0.0);
-    const double per_cb = std::max(std::max(t_mma, t_smem), std::max(t_w, t_x)) + (p.na_stages == 3 ? 0.0 : 210.0);
-    if (split > 1) return (double)waves * ((p.ncb + split - 1) / split * per_cb + 8.0 * p.MT * p.BN + 8000.0) + 9000.0;
-    return (double)waves * (p.ncb * per_cb + 100.0 * owned + 2500.0) + 9840.0 + (pair ? 1220.0 : 0.0);
+    const double t_x = 1075.0 + 42.0 * owned * p.chunks_per_unit + (pair ? 615.0 : 0.0);
+    const double t_p = 342.0 + 327.0 * ((p.SLOTS - 1) / p.L + 2);
+    const double per_cb = std::max({t_mma, t_smem, t_w, t_x, t_p});
+    if (p.split > 1) return (double)waves * (p.cb_per * (per_cb + 896.0) + 28.0 * p.BN + 5190.0) + 7090.0;
+    return (double)waves * (p.ncb * (per_cb + (p.na_stages == 3 ? 0.0 : 449.0)) + 1650.0) + 9530.0;
 }
 
 }  // namespace
@@ -1127,43 +1160,38 @@ bool tc_conv_plan(const ConvGeom &c, TcConvPlan &plan, bool forced) {
     for (int i = 0; i < ncand; ++i) {
         TcConvPlan p;
         if (!fill_plan(c, cand[i][0], cand[i][1], cand[i][2], cand[i][3], p)) continue;
-        const double cost = tile_cost(p, 1);
+        const double cost = tile_cost(p);
         if (!have || cost < best_cost * 0.999) {
             have = true;
             best_cost = cost;
             plan = p;
         }
     }
-    // Few tiles: let a cluster share each one's channel blocks (not for thin layers, which have one block).  A
-    // cluster of 8 does not fit every GPC: 14 of them are resident at once, and 33 of 4.
+    // Few tiles: let a cluster share each one's channel blocks (not for thin layers, which have one block).
     {
         int pb = 0, pk = 0, ps = 0;         // ONNXB_CONV_SPLIT = "BN,KB,S" pins the shape, "0" rules the split out
         const char *e = getenv("ONNXB_CONV_SPLIT");
         const bool pinned = e && sscanf(e, "%d,%d,%d", &pb, &pk, &ps) == 3;
         const bool ruled_out = (e && !pinned) || getenv("ONNXB_CONV_TILE") || getenv("ONNXB_CONV_STAGES");
-        if (c.Cg >= 32 && !ruled_out && (pinned || (have && plan.total_tiles * plan.ctas <= 74))) {
+        if (c.Cg >= 32 && !ruled_out && (pinned || (have && plan.total_tiles * plan.ctas <= 148))) {
             if (pinned) have = false;
             for (int kb = 16; kb <= 32; kb *= 2)
                 for (int bn = 16; bn <= 256; bn *= 2) {
                     const int b = std::min(bn, (c.Mg + 15) / 16 * 16);
                     if (pinned && (bn != pb || kb != pk)) continue;
                     if (!pinned && bn > 16 && b <= bn / 2) break;
-                    TcConvPlan p;
-                    if (!fill_plan(c, 1, 1, b, kb, p)) continue;
+                    TcConvPlan whole;
+                    if (!fill_plan(c, 1, 1, b, kb, whole)) continue;
                     for (int S = 2; S <= 8; S *= 2) {
                         if (pinned && S != ps) continue;
-                        p.cb_per = (p.ncb + S - 1) / S;
-                        if (p.cb_per * (S - 1) >= p.ncb) continue;                            // every CTA needs a block
-                        // the partial tile is parked over the stages
-                        if (128 * 4LL * (b + 1) + 16LL * b > (long long)p.na_stages * p.a_stage_bytes + (long long)p.nr_stages * p.raw_stage_bytes +
-                                                                 (long long)p.nb_stages * p.b_stage_bytes) continue;
+                        TcConvPlan p = whole;
+                        if (!split_plan(S, p)) continue;
                         if (!pinned && p.total_tiles * S > (S == 8 ? 112 : S == 4 ? 132 : 148)) continue;
-                        const double cost = tile_cost(p, S);
-                        if (!have || cost < best_cost * 0.97) {
+                        const double cost = tile_cost(p);
+                        if (!have || cost < best_cost * 0.999) {
                             have = true;
                             best_cost = cost;
                             plan = p;
-                            plan.split = S;
                         }
                     }
                 }
@@ -1256,7 +1284,8 @@ static int launch_images(const TcConvPlan &plan, const float *X, const float *B,
         memset(&tmX, 0, sizeof tmX);
     }
     const size_t smem = 1024 + (size_t)plan.na_stages * plan.a_stage_bytes + (size_t)plan.nr_stages * plan.raw_stage_bytes +
-                        (size_t)plan.nb_stages * plan.b_stage_bytes + kMaxRawStages * kSegBytes + kBiasBytes + kBarBytes;
+                        (size_t)plan.nb_stages * plan.b_stage_bytes + kMaxRawStages * kSegBytes + kBiasBytes + kBarBytes +
+                        (plan.split > 1 ? split_recv_bytes(plan.split, plan.cols_per) : 0);
     const bool pair = plan.ctas == 2;
     const bool add = R != nullptr;
     const bool split = plan.split > 1;

@@ -71,6 +71,7 @@ struct TcConvPlan {
     ConvDivisor dv_L, dv_Ws, dv_Hs, dv_BOXP, dv_SLOTS, dv_pss;
     int boxp_shift;                  // log2(BOXP) when BOXP is a power of two, else -1
     int split, cb_per;               // CTAs (a cluster) sharing a tile's channel blocks, blocks of each; split = 1: none
+    int cols_per;                    // split: output channels of the tile that each CTA finishes, a multiple of 4
     int b_resident;                  // all tiles use the same few weights: fetched once per CTA
     int relay;                       // pairs: the odd CTA's "operand stage written" goes through its relay warp
 };
