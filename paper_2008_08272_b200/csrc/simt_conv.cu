@@ -207,6 +207,9 @@ __device__ __forceinline__ float gather_round(float v) {
     return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);
 }
 
+// Both kernels below are bound by HBM (the pixels read once, the copy written once): one wave of eight blocks per SM, indices
+// by multiplication (256 channels 56x56 -> 28x28 at batch 32: some 20 -> 15 us).
+
 // Any layout whose pitch is a multiple of four (both layouts have one): four consecutive outputs per
 // thread, indices divided once and then stepped, four independent scalar loads, one 16-byte store.
 __global__ void __launch_bounds__(256)
@@ -214,6 +217,7 @@ gather1x1_quad_kernel(const float *__restrict__ X, float4 *__restrict__ Xg4, uns
                       unsigned NPQ, unsigned PQ, unsigned Q, unsigned C, unsigned HW, unsigned rowstep, unsigned sw,
                       int merged, const ConvDivisor dv_pitch, const ConvDivisor dv_PQ, const ConvDivisor dv_Q) {
     tc::pdl_launch_dependents();
+    tc::pdl_wait();
     for (unsigned i4 = blockIdx.x * 256u + threadIdx.x; i4 < total4; i4 += gridDim.x * 256u) {
         const unsigned i = i4 * 4u;
         const unsigned row = (unsigned)conv_fdiv((int)i, (int)pitch, dv_pitch);   // merged: channel; per image: n*C + c
@@ -224,21 +228,16 @@ gather1x1_quad_kernel(const float *__restrict__ X, float4 *__restrict__ Xg4, uns
             r = j - n * PQ;
         }
         unsigned pp = (unsigned)conv_fdiv((int)r, (int)Q, dv_Q), q = r - pp * Q;
-        const float *src[4];
-        bool ok[4];
+        float v[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const unsigned plane = merged ? n * C + row : row;
-            ok[e] = j + e < NPQ;
-            src[e] = X + (size_t)plane * HW + pp * rowstep + q * sw;
+            v[e] = j + e < NPQ ? gather_round(__ldg(X + (size_t)plane * HW + pp * rowstep + q * sw)) : 0.f;
             // step to the next output pixel: along the row, then to the next row, then to the next image
             ++r;
             if (++q == Q) { q = 0; ++pp; }
             if (r == PQ) { r = 0; pp = 0; q = 0; ++n; }
         }
-        float v[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = ok[e] ? gather_round(__ldg(src[e])) : 0.f;
         Xg4[i4] = make_float4(v[0], v[1], v[2], v[3]);
     }
 }
@@ -248,11 +247,12 @@ gather1x1_quad_kernel(const float *__restrict__ X, float4 *__restrict__ Xg4, uns
 template <int SW>
 __global__ void __launch_bounds__(256)
 gather1x1_vec_kernel(const float4 *__restrict__ X4, float4 *__restrict__ Xg4, unsigned total4, unsigned PQ4,
-                     unsigned Q4, unsigned HW4, unsigned rowstep4) {
+                     unsigned Q4, unsigned HW4, unsigned rowstep4, const ConvDivisor dv_PQ4, const ConvDivisor dv_Q4) {
     tc::pdl_launch_dependents();
+    tc::pdl_wait();
     for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < total4; i += gridDim.x * 256u) {
-        const unsigned plane = i / PQ4, r = i - plane * PQ4;
-        const unsigned p = r / Q4, q4 = r - p * Q4;
+        const unsigned plane = (unsigned)conv_fdiv((int)i, (int)PQ4, dv_PQ4), r = i - plane * PQ4;
+        const unsigned p = (unsigned)conv_fdiv((int)r, (int)Q4, dv_Q4), q4 = r - p * Q4;
         const float4 *src = X4 + (size_t)plane * HW4 + p * rowstep4 + q4 * SW;
         float4 o;
         if (SW == 1) {
@@ -261,8 +261,7 @@ gather1x1_vec_kernel(const float4 *__restrict__ X4, float4 *__restrict__ Xg4, un
             const float4 a = __ldg(src), b = __ldg(src + 1);
             o = make_float4(a.x, a.z, b.x, b.z);
         }
-        o.x = gather_round(o.x); o.y = gather_round(o.y); o.z = gather_round(o.z); o.w = gather_round(o.w);
-        Xg4[i] = o;
+        Xg4[i] = make_float4(gather_round(o.x), gather_round(o.y), gather_round(o.z), gather_round(o.w));
     }
 }
 
@@ -499,30 +498,28 @@ bool simt_depthwise_supports(const ConvGeom &g) {
 int launch_gather1x1(const ConvGeom &g, const float *X, float *Xg, long long pitch, bool merged, void *stream) {
     const long long total = merged ? (long long)g.C * pitch : (long long)g.N * g.C * pitch;
     cudaStream_t st = (cudaStream_t)stream;
+    const long long total4 = total / 4;                       // every pitch is a multiple of four
+    const unsigned blocks = (unsigned)std::min<long long>((total4 + 255) / 256, 148LL * 8);
+    // A small copy is set up beside the previous kernel's tail (one image, 7x7 to 28x28: 1.0-1.3 us less).  The blocks of a
+    // large one, placed while that kernel still holds its SMs, would crowd on some of them (batch 32: 15 -> 22 us).
+    auto launch = [&](auto kernel, auto... args) {
+        if (blocks <= 2 * 148) return tc_host::launch_pdl(kernel, dim3(blocks), dim3(256), 0, st, args...);
+        kernel<<<blocks, 256, 0, st>>>(args...);
+        return cudaGetLastError();
+    };
+    cudaError_t e;
     if (!merged && g.Q % 4 == 0 && g.W % 4 == 0 && (g.sw == 1 || g.sw == 2) && g.Q * g.sw <= g.W) {
-        const long long total4 = total / 4;
-        const unsigned blocks = (unsigned)std::min<long long>((total4 + 255) / 256, 148LL * 16);
         const unsigned PQ4 = g.P * g.Q / 4, Q4 = g.Q / 4, HW4 = g.H * g.W / 4, rowstep4 = g.sh * g.W / 4;
-        if (g.sw == 1)
-            gather1x1_vec_kernel<1><<<blocks, 256, 0, st>>>(reinterpret_cast<const float4 *>(X),
-                                                           reinterpret_cast<float4 *>(Xg), (unsigned)total4, PQ4, Q4,
-                                                           HW4, rowstep4);
-        else
-            gather1x1_vec_kernel<2><<<blocks, 256, 0, st>>>(reinterpret_cast<const float4 *>(X),
-                                                           reinterpret_cast<float4 *>(Xg), (unsigned)total4, PQ4, Q4,
-                                                           HW4, rowstep4);
-    } else {                       // every pitch is a multiple of four
-        const long long total4 = total / 4;
-        const unsigned blocks = (unsigned)std::min<long long>((total4 + 255) / 256, 148LL * 32);
-        gather1x1_quad_kernel<<<blocks, 256, 0, st>>>(X, reinterpret_cast<float4 *>(Xg), (unsigned)total4, (unsigned)pitch,
-                                                      (unsigned)(merged ? g.N * g.P * g.Q : g.P * g.Q),
-                                                      (unsigned)(g.P * g.Q), (unsigned)g.Q, (unsigned)g.C,
-                                                      (unsigned)(g.H * g.W), (unsigned)(g.sh * g.W), (unsigned)g.sw,
-                                                      merged ? 1 : 0, conv_divisor((int)pitch), conv_divisor(g.P * g.Q),
-                                                      conv_divisor(g.Q));
+        e = launch(g.sw == 1 ? gather1x1_vec_kernel<1> : gather1x1_vec_kernel<2>, reinterpret_cast<const float4 *>(X),
+                   reinterpret_cast<float4 *>(Xg), (unsigned)total4, PQ4, Q4, HW4, rowstep4, conv_divisor((int)PQ4), conv_divisor((int)Q4));
+    } else {
+        e = launch(gather1x1_quad_kernel, X, reinterpret_cast<float4 *>(Xg), (unsigned)total4, (unsigned)pitch,
+                   (unsigned)(merged ? g.N * g.P * g.Q : g.P * g.Q), (unsigned)(g.P * g.Q), (unsigned)g.Q, (unsigned)g.C,
+                   (unsigned)(g.H * g.W), (unsigned)(g.sh * g.W), (unsigned)g.sw, merged ? 1 : 0, conv_divisor((int)pitch),
+                   conv_divisor(g.P * g.Q), conv_divisor(g.Q));
     }
     count_launch();
-    return (int)cudaGetLastError();
+    return (int)e;
 }
 
 int launch_simt_depthwise(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
