@@ -637,8 +637,8 @@ double tc_gemm_estimate_ns(const TcGemmProblem &g) {
     const int bn = pick_bn(tiles_m, g.N, g.batch, units, ctas);
     const long long tiles = tiles_m * ((g.N + bn - 1) / bn) * g.batch;
     const double waves = (double)((tiles + units - 1) / units);
-    const double t = waves * ((g.K + kBK - 1) / kBK * (61.0 + 2.87 * bn / ctas + (ctas == 2 ? 15.0 : 0.0)) + 13.8 * bn) + 2630.0;
-    return t + (g.round_operands ? 2010.0 + 254e-6 * 4.0 * ((double)g.M * g.K + (double)g.K * g.N) : 0.0);
+    const double t = waves * ((g.K + kBK - 1) / kBK * (52.0 + 3.06 * bn / ctas + (ctas == 2 ? 8.0 : 0.0)) + 14.9 * bn) + 2470.0;
+    return t + (g.round_operands ? 2030.0 + 283e-6 * 4.0 * ((double)g.M * g.K + (double)g.K * g.N) : 0.0);
 }
 
 int launch_tc_gemm(const TcGemmProblem &g, void *stream) {

@@ -48,7 +48,7 @@ struct SkParams {
     int round;                 // round the operands in shared memory
     int BN, S, tiles_m, tiles_n, num_kb, kb_per, num_stages;
     int rows_per, pitch;       // rows of a slice; slots of 16 bytes between a slice's column groups (odd: see the exchange)
-    uint32_t stage_bytes, recv_off, idesc;     // recv_off: from the first stage to the partial sums
+    uint32_t stage_bytes, a_bytes, recv_off, idesc;     // a_bytes: of one K block; recv_off: from the first stage to the partial sums
     float alpha, beta;
     const float *C, *row_bias, *R;
     long long c_si, c_sj;
@@ -60,21 +60,6 @@ struct SkParams {
     ConvDivisor dv_split;
     unsigned int *err;
 };
-
-// n4 16-byte pieces of a stage to TF32 in place, by kRoundWarps warps
-__device__ __forceinline__ void round_tile(uint8_t *tile, int n4, int rt) {
-    float4 *t4 = reinterpret_cast<float4 *>(tile);
-    for (int j = rt; j < n4; j += 4 * kRoundWarps * 32) {
-        float4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (j + u * kRoundWarps * 32 < n4) v[u] = t4[j + u * kRoundWarps * 32];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (j + u * kRoundWarps * 32 < n4)
-                t4[j + u * kRoundWarps * 32] = make_float4(round_tf32(v[u].x), round_tf32(v[u].y), round_tf32(v[u].z), round_tf32(v[u].w));
-    }
-}
 
 // kKS: K blocks per stage (two wherever a CTA has two: see tc_gemm.cu for what a stage costs its issuing threads)
 template <int kKS>
@@ -145,9 +130,9 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         if (is_a) {
             if (p.a_mn) { off = (uint32_t)lane * (4096u * kKS); c0 = tm * kBM + lane * 32; c1 = kb0 * kBK; d1 = kKS * kBK; }
             else if (p.a_kbox) { c1 = tm * kBM; c2 = kb0; d2 = kKS; }
-            else { off = (uint32_t)lane * kABytes; c0 = (kb0 + lane) * kBK; c1 = tm * kBM; d0 = kKS * kBK; }
+            else { off = (uint32_t)lane * p.a_bytes; c0 = (kb0 + lane) * kBK; c1 = tm * kBM; d0 = kKS * kBK; }
         } else {
-            off = kKS * kABytes;
+            off = kKS * p.a_bytes;
             if (big) { c1 = kb0 * kBK; c2 = tn * (p.BN / 32); c3 = batch; d1 = kKS * kBK; }
             else if (p.b_mn) { off += (uint32_t)ib * (4096u * kKS); c0 = tn * p.BN + ib * 32; c1 = kb0 * kBK; c2 = batch; d1 = kKS * kBK; }
             else if (p.b_kbox) { c1 = tn * p.BN; c2 = kb0; c3 = batch; d2 = kKS; }
@@ -174,9 +159,9 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             const uint32_t a_hi = (uint32_t)(a_tmpl >> 32), b_hi = (uint32_t)(b_tmpl >> 32);
             // (masked: within a cluster the CTA's rank stands in the upper bits of a shared-memory address)
             const uint32_t a_lo = (uint32_t)a_tmpl | ((smem_u32(stages) >> 4) & 0x3FFFu);
-            const uint32_t b_lo = (uint32_t)b_tmpl | (((smem_u32(stages) + kKS * kABytes) >> 4) & 0x3FFFu);
+            const uint32_t b_lo = (uint32_t)b_tmpl | (((smem_u32(stages) + kKS * p.a_bytes) >> 4) & 0x3FFFu);
             const uint32_t a_k16 = (p.a_mn ? 1024u : 32u) >> 4, b_k16 = (p.b_mn ? 1024u : 32u) >> 4;
-            const uint32_t a_sub16 = (p.a_mn ? 4096u : (uint32_t)kABytes) >> 4, b_sub16 = (p.b_mn ? 4096u : (uint32_t)p.BN * 128u) >> 4;
+            const uint32_t a_sub16 = (p.a_mn ? 4096u : p.a_bytes) >> 4, b_sub16 = (p.b_mn ? 4096u : (uint32_t)p.BN * 128u) >> 4;
             const uint32_t stage16 = p.stage_bytes >> 4;
             uint64_t *landed = p.round ? ready : full;                // rounded as well, or as they arrive
             int stage = 0;
@@ -205,21 +190,23 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     } else {
         if (p.round) {
             // round every landed stage to TF32 in place (elementwise, so the swizzle does not matter)
-            // (of a K-major A only the rows that exist: a classifier head at batch 1 has one of the 128)
             const int rt = ((warp - 2) % kRoundWarps) * 32 + lane, mine = (warp - 2) / kRoundWarps;
-            const int a_rows = p.a_mn ? kBM : min(kBM, p.M - tm * kBM);
+            const int n4 = (int)(p.stage_bytes >> 4);
             int stage = 0;
             uint32_t phase = 0;
             for (int kb = 0, i = 0; kb < nkb; kb += kKS, ++i) {
                 if ((i & 1) == mine) {
                     mbar_wait(&full[stage], phase, p.err, 43);
-                    uint8_t *st = stages + (size_t)stage * p.stage_bytes;
-                    if (a_rows == kBM) {
-                        round_tile(st, (int)(p.stage_bytes >> 4), rt);
-                    } else {
+                    float4 *st4 = reinterpret_cast<float4 *>(stages + (size_t)stage * p.stage_bytes);
+                    for (int j = rt; j < n4; j += 4 * kRoundWarps * 32) {
+                        float4 v[4];
 #pragma unroll
-                        for (int sub = 0; sub < kKS; ++sub) round_tile(st + sub * kABytes, a_rows * (kBK / 4), rt);
-                        round_tile(st + kKS * kABytes, p.BN * (kBK / 4) * kKS, rt);
+                        for (int u = 0; u < 4; ++u)
+                            if (j + u * kRoundWarps * 32 < n4) v[u] = st4[j + u * kRoundWarps * 32];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (j + u * kRoundWarps * 32 < n4)
+                                st4[j + u * kRoundWarps * 32] = make_float4(round_tf32(v[u].x), round_tf32(v[u].y), round_tf32(v[u].z), round_tf32(v[u].w));
                     }
                     fence_proxy_async_smem();          // generic-proxy writes, read next by the tensor core
                     __syncwarp();
@@ -233,7 +220,7 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         const int row = q * 32 + lane;
         if (p.S > 1) cluster_wait();                                  // (the peers set up long ago)
         if (nkb > 0) {
-            const int dst = row / p.rows_per, n4 = p.BN / 4;
+            const int dst = min(row / p.rows_per, p.S - 1), n4 = p.BN / 4;
             const bool wanted = row < p.M - tm * kBM;
             uint32_t to = smem_u32(recv) + (uint32_t)((rank * n4 + half * 8) * p.pitch + row - dst * p.rows_per) * 16u, bar = smem_u32(recv_full);
             if (p.S > 1) {
@@ -375,8 +362,8 @@ int resident_ctas(int S) {
 
 // Shape with the shortest estimated time, against the persistent kernel's (both in ns, fitted to 95 problems: 1x1
 // convolutions of ResNet-50 at batch 1 to 32 and Gemms from 1 x 1000 x 2048 to 1024 x 1024 x 4096; the choice is
-// within 1 % of the best on average).  One wave of CTAs costs 2.1 us for its set-up, first fill and exchange, and a
-// K block 160-400 ns (rounded in shared memory first: 180-570, with the rows of A there are).
+// within 1 % of the best on average).  A wave of CTAs costs 1.4 us and more for its first fill and exchange, and a
+// K block 160-420 ns (rounded in shared memory first: 130-620, with the rows of A there are).
 SkChoice search(const TcGemmProblem &g) {
     SkChoice c{0, 0};
     if ((g.a_batched && g.batch > 1) || (g.batch > 1 && g.b_batched && g.b_bs % 4)) return c;
@@ -389,8 +376,8 @@ SkChoice search(const TcGemmProblem &g) {
             if (ctas > 4 * 148) break;
             const int units = resident_ctas(S);
             const double waves = (double)((ctas + units - 1) / units);
-            const double blk = g.round_operands ? 137.0 + 1.4 * BN + 2.0 * std::min(g.M, kBM) : 79.0 + 2.54 * BN;
-            const double t = waves * ((num_kb + S - 1) / S * blk + 2090.0 + 29.6 * BN) + 1040.0;
+            const double blk = g.round_operands ? 64.0 + 1.94 * BN + 2.38 * std::min(g.M, kBM) : 72.0 + 2.71 * BN;
+            const double t = waves * ((num_kb + S - 1) / S * blk + 1390.0 + 23.0 * BN) + 1790.0;
             if (t < best) {
                 best = t;
                 c = {BN, S};
@@ -447,14 +434,18 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
     p.tiles_n = (g.N + p.BN - 1) / p.BN;
     p.num_kb = (g.K + kBK - 1) / kBK;
     p.kb_per = (p.num_kb + p.S - 1) / p.S;
-    p.rows_per = (kBM + p.S - 1) / p.S;
+    // A K-major A of fewer than 128 rows is staged without the rows it has not (a classifier head at batch 1 has one):
+    // the tensor core then reads whatever follows in shared memory for them, and no one reads those rows of the result.
+    const int a_rows = p.a_mn ? kBM : std::min(kBM, (g.M + 7) / 8 * 8);
+    p.a_bytes = (uint32_t)a_rows * kBK * 4;
+    p.rows_per = (std::min(kBM, g.M) + p.S - 1) / p.S;
     p.pitch = p.rows_per | 1;
     const size_t recv_bytes = (size_t)p.S * (p.BN / 4) * p.pitch * 16;
     // two K blocks per stage, where that leaves two stages beside the partial sums
     const int ks = p.kb_per >= 2 ? 2 : 1;
-    p.stage_bytes = (uint32_t)(kABytes + p.BN * 128) * ks;
+    p.stage_bytes = (p.a_bytes + p.BN * 128) * ks;
     // (never more stages than the share has: a small footprint lets the next kernel's CTAs set up beside this one)
-    p.num_stages = std::min({kMaxStages, std::max(2, (p.kb_per + ks - 1) / ks), (int)((kSmemLimit - 2048 - recv_bytes) / p.stage_bytes)});
+    p.num_stages = std::min({kMaxStages, std::max(2, (p.kb_per + ks - 1) / ks), (int)((kSmemLimit - 2048 - std::max(recv_bytes, (size_t)kABytes)) / p.stage_bytes)});
     p.idesc = tc::make_idesc_tf32(kBM, p.BN, p.a_mn, p.b_mn);
     p.alpha = g.alpha; p.beta = g.beta;
     p.C = g.C; p.c_si = g.c_si; p.c_sj = g.c_sj;
@@ -485,7 +476,7 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
         return make_tmap(tm, base, 4, dims, str, box, mn ? kTmapSwizzle128Atom32 : kTmapSwizzle128);
     };
     CUtensorMap tmA, tmB;
-    if (!operand(&tmA, g.A, p.a_mn, p.a_kbox, g.M, g.a_ld, 1, 0, kBM) ||
+    if (!operand(&tmA, g.A, p.a_mn, p.a_kbox, g.M, g.a_ld, 1, 0, a_rows) ||
         !operand(&tmB, g.B, p.b_mn, p.b_kbox, g.N, g.b_ld, g.b_batched ? g.batch : 1, g.b_bs, p.BN))
         return (int)cudaErrorInvalidValue;
     CUtensorMap tmBb = tmB;
@@ -498,7 +489,7 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
         p.b_big = make_tmap(&tmBb, g.B, 4, dims, str, box, kTmapSwizzle128Atom32) ? 1 : 0;
     }
     p.recv_off = (uint32_t)p.num_stages * p.stage_bytes;
-    const size_t smem = 2048 + p.recv_off + recv_bytes;
+    const size_t smem = 2048 + p.recv_off + std::max(recv_bytes, (size_t)kABytes);      // (at least what an MMA of the last stage reads)
     auto kern = ks == 2 ? tc_gemm_splitk_kernel<2> : tc_gemm_splitk_kernel<1>;
     const cudaError_t ae = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (ae != cudaSuccess) return (int)ae;
