@@ -274,84 +274,49 @@ gather1x1_vec_kernel(const float4 *__restrict__ X4, float4 *__restrict__ Xg4, un
 // 16-byte pieces and as wide as the output, so a row costs one aligned 16-byte load; the columns to its left and
 // right come from the neighbouring lanes, which hold them (the first and last lane of a warp load theirs), and
 // beyond the row's ends lies padding.  Otherwise every column is loaded on its own.
-template <int KH, int KW, bool VEC, int ROWS>
-__global__ void __launch_bounds__(256)
-conv2d_depthwise_unit_kernel(const ConvGeom g, const float *__restrict__ X, const float *__restrict__ W,
-                             const float *__restrict__ B, const float *__restrict__ R, float *__restrict__ Y,
-                             unsigned items, unsigned Q4, unsigned P2, double inv_Q4, double inv_P2) {
-    constexpr int WIN = KW + 3;                // input columns a strip of 4 outputs touches
-    tc::pdl_launch_dependents();
-    const unsigned i_own = blockIdx.x * 256u + threadIdx.x;
-    if (!VEC && i_own >= items) return;
-    const unsigned i = VEC && i_own >= items ? items - 1 : i_own;      // (the neighbours of a live lane must stay)
-    // i = (plane * P2 + row group) * Q4 + column quad (P2 = row groups per plane); quotients by reciprocal multiplication in
-    // double (right for 31-bit operands up to one unit, which the two comparisons repair)
-    unsigned t = __double2uint_rd((double)i * inv_Q4);
-    if (t * Q4 > i) --t;
-    if ((t + 1) * Q4 <= i) ++t;
-    const unsigned q4 = i - t * Q4;
-    unsigned plane = __double2uint_rd((double)t * inv_P2);
-    if (plane * P2 > t) --plane;
-    if ((plane + 1) * P2 <= t) ++plane;
-    const int p0 = (int)(t - plane * P2) * ROWS, q0 = (int)q4 * 4;
-    const int c = (int)(plane % (unsigned)g.C);
-
-    const float *xp = X + (size_t)plane * g.H * g.W;
-    const int iw0 = q0 - g.pl;
-    tc::pdl_wait();
-    // Every input row of the window is requested before the first FMA: the kernel is bound by the
-    // latency of these loads, so each thread keeps all of them in flight at once.
-    float v[KH + ROWS - 1][WIN];
-    if (VEC) {
-        constexpr int L = (KW - 1) / 2, RT = KW - 1 - L;       // columns to the left (= the pad) and right of the quad
-        const int lane = threadIdx.x & 31;
-        const bool left_in = q0 > 0, right_in = q0 + 4 < g.W;
-        float e[KH + ROWS - 1][L > RT ? L : RT];               // what the warp's first and last lane load themselves
+// The window of a strip whose rows are whole 16-byte pieces (plane: in global or in shared memory).  Every input row is
+// requested before the first use; all lanes of the warp take part.
+template <int KH, int KW, int ROWS, bool SHARED>
+__device__ __forceinline__ void depthwise_window_vec(const float *plane, int H, int W, int h0, int q0, float (&v)[KH + ROWS - 1][KW + 3]) {
+    constexpr int L = (KW - 1) / 2, RT = KW - 1 - L;       // columns to the left (= the pad) and right of the quad
+    const int lane = threadIdx.x & 31;
+    const bool left_in = q0 > 0, right_in = q0 + 4 < W;
+    float e[KH + ROWS - 1][L > RT ? L : RT];               // what the warp's first and last lane load themselves
+    auto get = [](const float *q) { return SHARED ? *q : __ldg(q); };
 #pragma unroll
-        for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
-            const int ih = p0 - g.pt + rr;
-            const bool row_in = (unsigned)ih < (unsigned)g.H;
-            const float *row = xp + (size_t)ih * g.W + q0;
-            float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (row_in) m = __ldg(reinterpret_cast<const float4 *>(row));
-            v[rr][L] = m.x; v[rr][L + 1] = m.y; v[rr][L + 2] = m.z; v[rr][L + 3] = m.w;
+    for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
+        const int ih = h0 + rr;
+        const bool row_in = (unsigned)ih < (unsigned)H;
+        const float *row = plane + (ptrdiff_t)ih * W + q0;
+        float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row_in) m = SHARED ? *reinterpret_cast<const float4 *>(row) : __ldg(reinterpret_cast<const float4 *>(row));
+        v[rr][L] = m.x; v[rr][L + 1] = m.y; v[rr][L + 2] = m.z; v[rr][L + 3] = m.w;
 #pragma unroll
-            for (int k = 0; k < (L > RT ? L : RT); ++k) {
-                e[rr][k] = 0.f;
-                if (lane == 0 && k < L && row_in && left_in) e[rr][k] = __ldg(row - L + k);
-                if (lane == 31 && k < RT && row_in && right_in) e[rr][k] = __ldg(row + 4 + k);
-            }
-        }
-#pragma unroll
-        for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
-#pragma unroll
-            for (int k = 0; k < L; ++k) {
-                const float x = __shfl_up_sync(0xffffffffu, v[rr][L + 4 - L + k], 1);
-                v[rr][k] = !left_in ? 0.f : lane == 0 ? e[rr][k] : x;
-            }
-#pragma unroll
-            for (int k = 0; k < RT; ++k) {
-                const float x = __shfl_down_sync(0xffffffffu, v[rr][L + k], 1);
-                v[rr][L + 4 + k] = !right_in ? 0.f : lane == 31 ? e[rr][k] : x;
-            }
-        }
-        if (i_own >= items) return;
-    } else {
-#pragma unroll
-        for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
-            const int ih = p0 - g.pt + rr;
-            const float *row = xp + (size_t)ih * g.W;
-#pragma unroll
-            for (int k = 0; k < WIN; ++k) {
-                v[rr][k] = 0.f;
-                if ((unsigned)ih < (unsigned)g.H && (unsigned)(iw0 + k) < (unsigned)g.W) v[rr][k] = __ldg(row + iw0 + k);
-            }
+        for (int k = 0; k < (L > RT ? L : RT); ++k) {
+            e[rr][k] = 0.f;
+            if (lane == 0 && k < L && row_in && left_in) e[rr][k] = get(row - L + k);
+            if (lane == 31 && k < RT && row_in && right_in) e[rr][k] = get(row + 4 + k);
         }
     }
-    float w[KH * KW];
 #pragma unroll
-    for (int k = 0; k < KH * KW; ++k) w[k] = __ldg(W + (size_t)c * (KH * KW) + k);
-    const float bias = B ? __ldg(B + c) : 0.f;
+    for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
+#pragma unroll
+        for (int k = 0; k < L; ++k) {
+            const float x = __shfl_up_sync(0xffffffffu, v[rr][L + 4 - L + k], 1);
+            v[rr][k] = !left_in ? 0.f : lane == 0 ? e[rr][k] : x;
+        }
+#pragma unroll
+        for (int k = 0; k < RT; ++k) {
+            const float x = __shfl_down_sync(0xffffffffu, v[rr][L + k], 1);
+            v[rr][L + 4 + k] = !right_in ? 0.f : lane == 31 ? e[rr][k] : x;
+        }
+    }
+}
+
+// Filter, addend, Relu and store of a strip: 4 output columns from q0, ROWS output rows from p0 of one plane.
+template <int KH, int KW, int ROWS, bool VEC>
+__device__ __forceinline__ void depthwise_strip(const ConvGeom &g, const float (&v)[KH + ROWS - 1][KW + 3], const float (&w)[KH * KW],
+                                                float bias, const float *__restrict__ R, float *__restrict__ Y, size_t plane, int p0, int q0) {
     float acc[ROWS][4];
 #pragma unroll
     for (int k = 0; k < ROWS; ++k)
@@ -370,7 +335,7 @@ conv2d_depthwise_unit_kernel(const ConvGeom g, const float *__restrict__ X, cons
             }
         }
     }
-    float *yp = Y + ((size_t)plane * g.P + p0) * g.Q + q0;
+    float *yp = Y + (plane * g.P + p0) * g.Q + q0;
 #pragma unroll
     for (int k = 0; k < ROWS; ++k) {
         float *a = acc[k];
@@ -394,6 +359,113 @@ conv2d_depthwise_unit_kernel(const ConvGeom g, const float *__restrict__ X, cons
     }
 }
 
+template <int KH, int KW, bool VEC, int ROWS>
+__global__ void __launch_bounds__(256)
+conv2d_depthwise_unit_kernel(const ConvGeom g, const float *__restrict__ X, const float *__restrict__ W,
+                             const float *__restrict__ B, const float *__restrict__ R, float *__restrict__ Y,
+                             unsigned items, unsigned Q4, unsigned P2, double inv_Q4, double inv_P2) {
+    constexpr int WIN = KW + 3;                // input columns a strip of 4 outputs touches
+    tc::pdl_launch_dependents();
+    const unsigned i_own = blockIdx.x * 256u + threadIdx.x;
+    if (!VEC && i_own >= items) return;
+    const unsigned i = VEC && i_own >= items ? items - 1 : i_own;      // (the neighbours of a live lane must stay)
+    // i = (plane * P2 + row group) * Q4 + column quad (P2 = row groups per plane); quotients by reciprocal multiplication in
+    // double (right for 31-bit operands up to one unit, which the two comparisons repair)
+    unsigned t = __double2uint_rd((double)i * inv_Q4);
+    if (t * Q4 > i) --t;
+    if ((t + 1) * Q4 <= i) ++t;
+    const unsigned q4 = i - t * Q4;
+    unsigned plane = __double2uint_rd((double)t * inv_P2);
+    if (plane * P2 > t) --plane;
+    if ((plane + 1) * P2 <= t) ++plane;
+    const int p0 = (int)(t - plane * P2) * ROWS, q0 = (int)q4 * 4;
+    const int c = (int)(plane % (unsigned)g.C);
+
+    const float *xp = X + (size_t)plane * g.H * g.W;
+    tc::pdl_wait();
+    // Every input row of the window is requested before the first FMA: the kernel is bound by the
+    // latency of these loads, so each thread keeps all of them in flight at once.
+    float v[KH + ROWS - 1][WIN];
+    if (VEC) {
+        depthwise_window_vec<KH, KW, ROWS, false>(xp, g.H, g.W, p0 - g.pt, q0, v);
+        if (i_own >= items) return;
+    } else {
+        const int iw0 = q0 - g.pl;
+#pragma unroll
+        for (int rr = 0; rr < KH + ROWS - 1; ++rr) {
+            const int ih = p0 - g.pt + rr;
+            const float *row = xp + (size_t)ih * g.W;
+#pragma unroll
+            for (int k = 0; k < WIN; ++k) {
+                v[rr][k] = 0.f;
+                if ((unsigned)ih < (unsigned)g.H && (unsigned)(iw0 + k) < (unsigned)g.W) v[rr][k] = __ldg(row + iw0 + k);
+            }
+        }
+    }
+    float w[KH * KW];
+#pragma unroll
+    for (int k = 0; k < KH * KW; ++k) w[k] = __ldg(W + (size_t)c * (KH * KW) + k);
+    depthwise_strip<KH, KW, ROWS, VEC>(g, v, w, B ? __ldg(B + c) : 0.f, R, Y, plane, p0, q0);
+}
+
+// The same strips, the input streamed through shared memory: planes are contiguous, so a bulk copy brings a block's next
+// `per` of them while it works on the last ones, and the loads that the kernel above waits for on every strip are
+// never out of flight.  One wave of CTAs (as many as fit an SM), each with its own ring of kRingStages copies; more
+// or larger ones were slower (256 channels 28x28, batch 64: 22.4 us by the kernel above, 20.3 with two stages and four
+// CTAs per SM, 20.9 with three and three, 22.4 with five and two).  Bound by HBM, at 5.1 TB/s there.
+constexpr int kRingStages = 2, kRingCtas = 4, kRingStageMax = 24576;
+
+template <int KH, int KW, int ROWS>
+__global__ void __launch_bounds__(256, kRingCtas)
+conv2d_depthwise_ring_kernel(const ConvGeom g, const float *__restrict__ X, const float *__restrict__ W, const float *__restrict__ B,
+                             const float *__restrict__ R, float *__restrict__ Y, unsigned planes, unsigned per, unsigned Q4, unsigned P2,
+                             const ConvDivisor dv_Q4, const ConvDivisor dv_P2, const ConvDivisor dv_C, unsigned int *err) {
+    extern __shared__ __align__(128) float ring[];
+    __shared__ uint64_t full[kRingStages];
+    const unsigned units = (planes + per - 1) / per, plane_floats = (unsigned)(g.H * g.W);
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < kRingStages; ++k) tc::mbar_init(&full[k], 1);
+        tc::mbar_fence_init();
+    }
+    __syncthreads();
+    tc::pdl_launch_dependents();
+    tc::pdl_wait();
+    auto fetch = [&](unsigned u, int stage) {
+        const unsigned cnt = min(per, planes - u * per);
+        tc::mbar_arrive_expect_tx(&full[stage], cnt * plane_floats * 4u);
+        tc::bulk_load_1d(ring + (size_t)stage * per * plane_floats, X + (size_t)u * per * plane_floats, cnt * plane_floats * 4u, &full[stage]);
+    };
+    if (threadIdx.x == 0)
+        for (int k = 0; k < kRingStages; ++k)
+            if (blockIdx.x + k * gridDim.x < units) fetch(blockIdx.x + k * gridDim.x, k);
+    int stage = 0;
+    uint32_t phase = 0;
+    for (unsigned u = blockIdx.x; u < units; u += gridDim.x) {
+        const unsigned items = min(per, planes - u * per) * P2 * Q4;
+        const float *base = ring + (size_t)stage * per * plane_floats;
+        bool landed = false;
+        for (unsigned i0 = 0; i0 < items; i0 += 256u) {
+            const unsigned i_own = i0 + threadIdx.x, i = min(i_own, items - 1);        // (the neighbours of a live lane must stay)
+            const unsigned t = (unsigned)conv_fdiv((int)i, (int)Q4, dv_Q4), pl = (unsigned)conv_fdiv((int)t, (int)P2, dv_P2);
+            const int q0 = (int)(i - t * Q4) * 4, p0 = (int)(t - pl * P2) * ROWS;
+            const unsigned plane = u * per + pl;
+            const unsigned c = plane - (unsigned)conv_fdiv((int)plane, g.C, dv_C) * (unsigned)g.C;
+            float w[KH * KW];
+#pragma unroll
+            for (int k = 0; k < KH * KW; ++k) w[k] = __ldg(W + (size_t)c * (KH * KW) + k);
+            const float bias = B ? __ldg(B + c) : 0.f;
+            if (!landed) tc::mbar_wait(&full[stage], phase, err, 60);
+            landed = true;
+            float v[KH + ROWS - 1][KW + 3];
+            depthwise_window_vec<KH, KW, ROWS, true>(base + pl * plane_floats, g.H, g.W, p0 - g.pt, q0, v);
+            if (i_own < items) depthwise_strip<KH, KW, ROWS, true>(g, v, w, bias, R, Y, plane, p0, q0);
+        }
+        __syncthreads();                                       // every thread has read the stage
+        if (threadIdx.x == 0 && u + kRingStages * gridDim.x < units) fetch(u + kRingStages * gridDim.x, stage);
+        if (++stage == kRingStages) { stage = 0; phase ^= 1; }
+    }
+}
+
 template <int KH, int KW>
 int launch_depthwise_unit(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                           cudaStream_t st) {
@@ -406,6 +478,24 @@ int launch_depthwise_unit(const ConvGeom &g, const float *X, const float *W, con
     // aligned 16-byte accesses: every input and output row starts on a 16-byte boundary
     const bool vec = g.pl == (KW - 1) / 2 && g.W % 4 == 0 && g.Q == g.W &&
                      (reinterpret_cast<uintptr_t>(X) & 15) == 0 && (reinterpret_cast<uintptr_t>(Y) & 15) == 0;
+    // Planes per copy: a strip for every thread, and not many threads without one (56x56 has 196: 38.7 -> 39.4 us); several
+    // units for every CTA, or the ring has nothing to run ahead of.  A 5x5 window does not leave room for four CTAs.
+    const long long planes = (long long)g.N * g.C, plane_bytes = (long long)g.H * g.W * 4;
+    const long long per = std::max(1LL, std::min(256LL / (P2 * Q4), kRingStageMax / plane_bytes)), strips = per * P2 * Q4;
+    if (KH == 3 && vec && rows4 && plane_bytes <= kRingStageMax && strips >= 224 && strips <= 256 &&
+        planes >= per * 148 * kRingCtas * 2) {
+        unsigned int *err = device_status_ptr();
+        if (!err) return (int)cudaErrorUnknown;
+        auto ring = conv2d_depthwise_ring_kernel<3, 3, 4>;
+        const cudaError_t ae = cudaFuncSetAttribute(ring, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingStages * kRingStageMax);
+        if (ae != cudaSuccess) return (int)ae;
+        const unsigned units = (unsigned)((planes + per - 1) / per);
+        const cudaError_t e = tc_host::launch_pdl(ring, dim3(std::min(units, 148u * kRingCtas)), dim3(256), (size_t)(kRingStages * per * plane_bytes), st,
+                                                  g, X, W, B, R, Y, (unsigned)planes, (unsigned)per, Q4, P2, conv_divisor((int)Q4),
+                                                  conv_divisor((int)P2), conv_divisor(g.C), err);
+        count_launch();
+        return (int)e;
+    }
     auto kern = vec ? (rows4 ? conv2d_depthwise_unit_kernel<KH, KW, true, 4> : conv2d_depthwise_unit_kernel<KH, KW, true, 2>)
                     : (rows4 ? conv2d_depthwise_unit_kernel<KH, KW, false, 4> : conv2d_depthwise_unit_kernel<KH, KW, false, 2>);
     // early launch gains 0.5 us behind another kernel where the rows are vectorised, and loses as much where not
