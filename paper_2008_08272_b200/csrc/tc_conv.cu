@@ -1106,13 +1106,22 @@ double tile_cost(const TcConvPlan &p) {
     const bool pair = p.ctas == 2;
     const double n_inst = (double)p.n_steps * p.MT, op_bytes = 4096.0 + p.BNH * 32.0;
     const double t_mma = n_inst * std::max(p.BN * 0.568, op_bytes / 126.0) + (p.n_steps + p.spb - 1) / p.spb * 391.0;
+    const double owned = (p.planes * p.SLOTS * p.chunk_groups + kXformThreads - 1) / kXformThreads;
+    if (p.KB == 4) {
+        // Thin layers, fitted to 108 pairs of their own (14 shapes, pick within 1 %): few steps per tile, so the tile's own
+        // costs count, the epilogue (17 cycles per channel and accumulator, behind the next tile where the accumulators
+        // alternate) and what a pair's CTAs wait for one another (7x7/2 first layer at batch 32: a pair 43.8 us, single CTAs 41.6).
+        const double body = p.ncb * (std::max(t_mma, 1000.0) + 800.0 + (pair ? 390.0 : 0.0)) + 1380.0 + 80.0 * owned;
+        const double epi = 17.0 * p.MT * p.BN;
+        const bool overlapped = p.MT == 1 || p.BN <= 128;
+        return waves * (overlapped ? std::max(body, epi) : body + epi) + (overlapped ? epi : 0.0) + 9580.0 + (pair ? 910.0 : 0.0);
+    }
     const double w_bytes = p.b_resident ? 0.0 : (double)p.n_steps * p.b_step_bytes;
     const double slots16 = (double)p.planes * p.SLOTS * 16.0 * p.nchunks;
     const double t_smem = (n_inst * op_bytes + w_bytes + 3.0 * slots16) / 115.0;
     const double ring = (double)p.nb_stages * p.b_stage_bytes;
     const double t_w = std::max(w_bytes / std::min(31.5, 3620.0 / active),
                                 p.split > 1 && ring >= w_bytes * p.cb_per ? 0.0 : w_bytes * 2090.0 / ring);
-    const double owned = (p.planes * p.SLOTS * p.chunk_groups + kXformThreads - 1) / kXformThreads;
     const double t_x = 1075.0 + 42.0 * owned * p.chunks_per_unit + (pair ? 615.0 : 0.0);
     const double t_p = 342.0 + 327.0 * ((p.SLOTS - 1) / p.L + 2);
     const double per_cb = std::max({t_mma, t_smem, t_w, t_x, t_p});
