@@ -1,0 +1,67 @@
+"""NaN operands: without Relu, an output is NaN exactly where its sum has a NaN term, on every path an operand can take to the
+tensor core, whatever the NaN's bit pattern; every other output is what it is without them."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+from parity import ABS, REL, run_conv_gpu  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def binding():
+    from paper_2008_08272_b200 import binding as b
+    b.load(build_if_missing=False)
+    return b
+
+
+def _same_nans(got, reached, want, S):
+    assert np.array_equal(np.isnan(got), reached), "NaN outputs are not the ones a NaN reaches"
+    ok = ~reached
+    assert ok.any() and (np.abs(got - want)[ok] <= (REL * S + ABS)[ok]).all()
+
+
+def _conv(binding, xs, ws, pattern, family, **kw):
+    rng = np.random.default_rng(xs[1] * 5 + ws[0])
+    X = rng.standard_normal(xs).astype(np.float32)
+    W = (rng.standard_normal(ws) * np.sqrt(2.0 / np.prod(ws[1:]))).astype(np.float32)
+    B = rng.standard_normal((ws[0],)).astype(np.float32)
+    want, S = oracle.conv2d(X, W, B, **kw)
+    spot = tuple(np.asarray(xs) // 2)
+    nan = np.array([pattern], dtype=np.uint32).view(np.float32)[0]
+    for bad, at in ((X.copy(), "X"), (W.copy(), "W")):
+        mx, mw = np.zeros_like(X), np.zeros_like(W)
+        if at == "X":
+            bad[spot] = nan
+            mx[spot], mw[:] = 1, 1
+        else:
+            tap = (ws[0] // 2, ws[1] // 2, ws[2] // 2, ws[3] // 2)        # the middle one: never on padding
+            bad[tap] = nan
+            mw[tap], mx[:] = 1, 1
+        reached = oracle.conv2d(mx, mw, None, **kw)[0] > 0
+        got, fam = run_conv_gpu(binding, torch, bad if at == "X" else X, bad if at == "W" else W, B, **kw)
+        assert fam == family
+        _same_nans(got, reached, want, S)
+
+
+IMPLICIT = [("whole tiles", dict(ONNXB_CONV_SPLIT="0"), (4, 64, 20, 20), (48, 64, 3, 3), dict(pads=(1, 1, 1, 1))),
+            ("tile pairs", dict(ONNXB_CONV_TILE="2,2,64"), (4, 64, 20, 20), (96, 64, 3, 3), dict(pads=(1, 1, 1, 1))),
+            ("split", dict(ONNXB_CONV_SPLIT="64,16,4"), (2, 128, 12, 12), (48, 128, 3, 3), dict(pads=(1, 1, 1, 1))),
+            ("thin", {}, (6, 3, 64, 64), (64, 3, 7, 7), dict(pads=(3, 3, 3, 3), strides=(2, 2)))]
+
+
+@pytest.mark.parametrize("pattern", [0x7FC00000], ids=hex)
+@pytest.mark.parametrize("case", IMPLICIT, ids=lambda c: c[0])
+def test_implicit_conv_without_relu_keeps_nan(binding, case, pattern, monkeypatch):
+    _, env, xs, ws, kw = case
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)                        # read when the descriptor is created
+    binding.set_kernel_override("mma_implicit")
+    try:
+        _conv(binding, xs, ws, pattern, "mma_implicit", **kw)
+    finally:
+        binding.set_kernel_override(None)
