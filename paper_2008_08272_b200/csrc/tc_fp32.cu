@@ -79,11 +79,16 @@ __device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&v)[16])
 }
 
 // hi to nearest; lo's rounding is completed by the tensor core, which ignores the low 13 bits.  A value that is
-// not finite, or rounds to infinity, leaves lo = NaN or -inf, and every output it takes part in NaN: the
-// epilogue then sums that output from the operands themselves.
+// not finite leaves lo = NaN, one that rounds to infinity lo = the opposite infinity, and either way every output it
+// takes part in is NaN: the epilogue then sums that output from the operands themselves.  (Whatever a NaN x becomes in
+// hi: x - hi is the NaN of GPU arithmetic, 0x7FFFFFFF, which half an ulp more would turn into a zero.  The larger of
+// the two as signed integers keeps it, and is the sum for every other value; all 2^32 compared.  It costs 0.2 us of
+// 86 on the dilated grouped 75x61 layer, a comparison and a selection for hi 2.1.)
 __device__ __forceinline__ void split_tf32(float x, float &hi, float &lo) {
-    hi = round_tf32(x);
-    lo = __uint_as_float(__float_as_uint(x - hi) + 0x1000u);
+    hi = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
+    int r;
+    asm("{\n.reg .s32 t;\nadd.s32 t, %1, 0x1000;\nmax.s32 %0, t, %1;\n}" : "=r"(r) : "r"(__float_as_int(x - hi)));
+    lo = __int_as_float(r);
 }
 
 // Where one tile's operands lie, for one producer thread.

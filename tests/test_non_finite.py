@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-from parity import ABS, REL, run_conv_gpu  # noqa: E402
+from parity import ABS, REL, run_conv_gpu, run_gemm_gpu  # noqa: E402
 
 
 @pytest.fixture(scope="module")
@@ -65,3 +65,31 @@ def test_implicit_conv_without_relu_keeps_nan(binding, case, pattern, monkeypatc
         _conv(binding, xs, ws, pattern, "mma_implicit", **kw)
     finally:
         binding.set_kernel_override(None)
+
+
+@pytest.mark.parametrize("pattern", [0x7FC00000, 0x7FFFFFFF, 0xFFFFFFFF], ids=hex)
+def test_split_fp32_keeps_nan(binding, pattern, monkeypatch):
+    """fp32 on the tensor cores, by two TF32 parts of every operand: Gemm and Conv."""
+    monkeypatch.setenv("ONNXB_FP32", "tc")
+    binding.set_kernel_override("simt_direct")
+    try:
+        _gemm(binding, 70, 131, 75, pattern)
+        _conv(binding, (2, 6, 19, 23), (130, 3, 3, 3), pattern, "simt_direct", pads=(1, 1, 1, 1), group=2)
+    finally:
+        binding.set_kernel_override(None)
+
+
+def _gemm(binding, M, N, K, pattern):
+    rng = np.random.default_rng(M + N)
+    A = rng.standard_normal((M, K)).astype(np.float32)
+    B = rng.standard_normal((K, N)).astype(np.float32)
+    want, S = oracle.gemm(A, B, None)
+    nan = np.array([pattern], dtype=np.uint32).view(np.float32)[0]
+    a, b = A.copy(), B.copy()
+    a[M // 2, K - 1] = b[3, N - 2] = nan
+    reached = np.zeros((M, N), bool)
+    reached[M // 2] = True
+    _same_nans(run_gemm_gpu(binding, torch, a, B, None), reached, want, S)
+    reached = np.zeros((M, N), bool)
+    reached[:, N - 2] = True
+    _same_nans(run_gemm_gpu(binding, torch, A, b, None), reached, want, S)
