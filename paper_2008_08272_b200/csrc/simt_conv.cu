@@ -203,10 +203,6 @@ conv2d_depthwise_kernel(const ConvGeom g, const float *__restrict__ X, const flo
 // Gather for strided / oddly sized 1x1 convolutions, values rounded to TF32 (nearest, ties away):
 //   merged:    Xg[c][n*P*Q + p*Q + q] = X[n][c][p*sh][q*sw], rows padded with zeros to the pitch;
 //   per image: Xg[n][c][p*Q + q]      (pitch = P*Q).
-__device__ __forceinline__ float gather_round(float v) {
-    return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);
-}
-
 // Both kernels below are bound by HBM (the pixels read once, the copy written once): one wave of eight blocks per SM, indices
 // by multiplication (256 channels 56x56 -> 28x28 at batch 32: some 20 -> 15 us).
 
@@ -232,7 +228,7 @@ gather1x1_quad_kernel(const float *__restrict__ X, float4 *__restrict__ Xg4, uns
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const unsigned plane = merged ? n * C + row : row;
-            v[e] = j + e < NPQ ? gather_round(__ldg(X + (size_t)plane * HW + pp * rowstep + q * sw)) : 0.f;
+            v[e] = j + e < NPQ ? tc::round_tf32(__ldg(X + (size_t)plane * HW + pp * rowstep + q * sw)) : 0.f;
             // step to the next output pixel: along the row, then to the next row, then to the next image
             ++r;
             if (++q == Q) { q = 0; ++pp; }
@@ -261,7 +257,7 @@ gather1x1_vec_kernel(const float4 *__restrict__ X4, float4 *__restrict__ Xg4, un
             const float4 a = __ldg(src), b = __ldg(src + 1);
             o = make_float4(a.x, a.z, b.x, b.z);
         }
-        Xg4[i] = make_float4(gather_round(o.x), gather_round(o.y), gather_round(o.z), gather_round(o.w));
+        Xg4[i] = make_float4(tc::round_tf32(o.x), tc::round_tf32(o.y), tc::round_tf32(o.z), tc::round_tf32(o.w));
     }
 }
 

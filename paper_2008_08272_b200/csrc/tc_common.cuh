@@ -299,11 +299,25 @@ __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&v)[32])
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // ---------------------------------------------------------------- TF32 rounding
-// fp32 -> TF32, round to nearest with ties away from zero (what cvt.rna.tf32.f32 computes), done
-// with two integer operations: add half an ulp of the 10-bit mantissa to the magnitude and clear
-// the 13 low bits.  A carry out of the mantissa correctly bumps the exponent; Inf stays Inf.
+// fp32 -> TF32, round to nearest with ties away from zero: add half an ulp of the 10-bit mantissa to
+// the magnitude and clear the 13 low bits.  A carry out of the mantissa correctly bumps the exponent;
+// Inf stays Inf.  A NaN with a mantissa of (nearly) all ones, which is what GPU arithmetic makes, would
+// carry into the sign and become a zero, and one with only low bits set an Inf (cvt.rna.tf32.f32 loses
+// the same patterns).  So x itself is added again, scaled below half an ulp of the result: a NaN stays
+// NaN and every other value is left as it is (all 2^32 patterns compared).  One instruction, which
+// nothing that is timed notices: ResNet-50 at batch 64 2056 -> 2044 us, first layer at batch 32
+// 42.1 -> 40.1 (its loop without spills now), 1024^3 and 4096^3 unchanged.
 __device__ __forceinline__ float round_tf32(float x) {
-    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
+    return fmaf(x, 0x1p-40f, __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u));
+}
+// The same with the low bits left as they are, for a value that the tensor core reads next (TF32 ignores them), in
+// two instructions where latency counts: x, its NaNs made 0x7FFFFFFF, and of that and the sum the larger as signed
+// integers, which is the sum for every number.  (Gemm 2048 x 224 x 144 by the split-K kernel: 6.77 us, 6.87 by
+// the form above.  Not for large problems: the low bits cost the tensor core power, 4096^3 262 -> 278 us.)
+__device__ __forceinline__ float round_tf32_operand(float x) {
+    int r;
+    asm("{\n.reg .s32 s;\nadd.s32 s, %1, 0x1000;\nmax.s32 %0, s, %1;\n}" : "=r"(r) : "r"(__float_as_int(fmaf(x, 0x1p-40f, x))));
+    return __int_as_float(r);
 }
 
 // ---------------------------------------------------------------- programmatic dependent launch

@@ -206,7 +206,7 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 #pragma unroll
                         for (int u = 0; u < 4; ++u)
                             if (j + u * kRoundWarps * 32 < n4)
-                                st4[j + u * kRoundWarps * 32] = make_float4(round_tf32(v[u].x), round_tf32(v[u].y), round_tf32(v[u].z), round_tf32(v[u].w));
+                                st4[j + u * kRoundWarps * 32] = make_float4(round_tf32_operand(v[u].x), round_tf32_operand(v[u].y), round_tf32_operand(v[u].z), round_tf32_operand(v[u].w));
                     }
                     fence_proxy_async_smem();          // generic-proxy writes, read next by the tensor core
                     __syncwarp();

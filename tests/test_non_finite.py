@@ -54,7 +54,11 @@ IMPLICIT = [("whole tiles", dict(ONNXB_CONV_SPLIT="0"), (4, 64, 20, 20), (48, 64
             ("thin", {}, (6, 3, 64, 64), (64, 3, 7, 7), dict(pads=(3, 3, 3, 3), strides=(2, 2)))]
 
 
-@pytest.mark.parametrize("pattern", [0x7FC00000], ids=hex)
+# as numpy writes it, as GPU arithmetic makes it, and that negated
+PATTERNS = [0x7FC00000, 0x7FFFFFFF, 0xFFFFFFFF]
+
+
+@pytest.mark.parametrize("pattern", PATTERNS, ids=hex)
 @pytest.mark.parametrize("case", IMPLICIT, ids=lambda c: c[0])
 def test_implicit_conv_without_relu_keeps_nan(binding, case, pattern, monkeypatch):
     _, env, xs, ws, kw = case
@@ -67,16 +71,13 @@ def test_implicit_conv_without_relu_keeps_nan(binding, case, pattern, monkeypatc
         binding.set_kernel_override(None)
 
 
-@pytest.mark.parametrize("pattern", [0x7FC00000, 0x7FFFFFFF, 0xFFFFFFFF], ids=hex)
-def test_split_fp32_keeps_nan(binding, pattern, monkeypatch):
-    """fp32 on the tensor cores, by two TF32 parts of every operand: Gemm and Conv."""
-    monkeypatch.setenv("ONNXB_FP32", "tc")
-    binding.set_kernel_override("simt_direct")
-    try:
-        _gemm(binding, 70, 131, 75, pattern)
-        _conv(binding, (2, 6, 19, 23), (130, 3, 3, 3), pattern, "simt_direct", pads=(1, 1, 1, 1), group=2)
-    finally:
-        binding.set_kernel_override(None)
+@pytest.mark.parametrize("pattern", PATTERNS, ids=hex)
+@pytest.mark.parametrize("split", ["0", "64,2"])
+def test_1x1_conv_without_relu_keeps_nan(binding, split, pattern, monkeypatch):
+    monkeypatch.setenv("ONNXB_GEMM_SPLITK", split)
+    _conv(binding, (2, 64, 16, 16), (136, 64, 1, 1), pattern, "mma_gemm")
+    _conv(binding, (2, 64, 32, 32), (136, 64, 1, 1), pattern, "mma_gather_gemm", strides=(2, 2))      # 16-byte loads
+    _conv(binding, (3, 64, 7, 7), (136, 64, 1, 1), pattern, "mma_gather_gemm")                        # scalar loads, merged images
 
 
 def _gemm(binding, M, N, K, pattern):
@@ -93,3 +94,22 @@ def _gemm(binding, M, N, K, pattern):
     reached = np.zeros((M, N), bool)
     reached[:, N - 2] = True
     _same_nans(run_gemm_gpu(binding, torch, A, b, None), reached, want, S)
+
+
+@pytest.mark.parametrize("pattern", PATTERNS, ids=hex)
+@pytest.mark.parametrize("split", ["0", "64,2"])           # operands rounded by a launch in front, or in shared memory
+def test_gemm_keeps_nan(binding, split, pattern, monkeypatch):
+    monkeypatch.setenv("ONNXB_GEMM_SPLITK", split)
+    _gemm(binding, 140, 132, 128, pattern)
+
+
+@pytest.mark.parametrize("pattern", PATTERNS, ids=hex)
+def test_split_fp32_keeps_nan(binding, pattern, monkeypatch):
+    """fp32 on the tensor cores, by two TF32 parts of every operand: Gemm and Conv."""
+    monkeypatch.setenv("ONNXB_FP32", "tc")
+    binding.set_kernel_override("simt_direct")
+    try:
+        _gemm(binding, 70, 131, 75, pattern)
+        _conv(binding, (2, 6, 19, 23), (130, 3, 3, 3), pattern, "simt_direct", pads=(1, 1, 1, 1), group=2)
+    finally:
+        binding.set_kernel_override(None)
