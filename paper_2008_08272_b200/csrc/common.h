@@ -73,6 +73,7 @@ int launch_simt_gemm(const GemmProblem &p, const float *A, const float *B, const
 // fp32 through split TF32 operands on the tensor cores (tc_fp32.cu): the same problems, once they are large
 double tc_fp32_cost(long long rows, int cols, int K, int groups, bool pixels);     // estimated SM cycles
 int launch_tc_fp32_gemm(const GemmProblem &p, const float *A, const float *B, const float *C, float *Y, void *stream);
+bool tc_fp32_conv_fits(const ConvGeom &g);
 int launch_tc_fp32_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                         void *stream);
 

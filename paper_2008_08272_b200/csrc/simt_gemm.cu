@@ -110,8 +110,10 @@ sgemm_kernel(const __grid_constant__ SgemmArgs g, int split) {
     const float *Ag = g.A + (BMODE == kPixels ? (long long)grp * g.M * g.K : 0);
     const uint32_t as_u32 = tc::smem_u32(As), bs_u32 = tc::smem_u32(Bs);
 
-    // pixel columns of a convolution: where the column's window starts in X
-    long long px_base[B_NREP];
+    // pixel columns of a convolution: where the column's window starts in X.  This offset and those of the table below
+    // are summed modulo 2^32: under a dilation of 2^19 either may lie billions of elements outside X, but the sum, used
+    // only for taps inside the image, is an element of X, and X has fewer than 2^31.
+    unsigned px_base[B_NREP];
     int px_h[B_NREP], px_w[B_NREP];
     if (BMODE == kPixels) {
 #pragma unroll
@@ -122,8 +124,8 @@ sgemm_kernel(const __grid_constant__ SgemmArgs g, int split) {
                 const int p = conv_fdiv(u, g.Q, g.dv_Q), q = u - p * g.Q;
                 px_h[e] = p * g.sh - g.pt;
                 px_w[e] = q * g.sw - g.pl;
-                px_base[e] = ((long long)n * g.Cch + (long long)grp * (g.K / g.taps)) * g.H * g.W +
-                             (long long)px_h[e] * g.W + px_w[e];
+                px_base[e] = (unsigned)(n * g.Cch + grp * (g.K / g.taps)) * (unsigned)(g.H * g.W) + (unsigned)px_h[e] * (unsigned)g.W +
+                             (unsigned)px_w[e];
             } else {
                 px_h[e] = px_w[e] = -(1 << 30);
                 px_base[e] = 0;
@@ -138,7 +140,8 @@ sgemm_kernel(const __grid_constant__ SgemmArgs g, int split) {
             if (k < g.K) {
                 const int c = conv_fdiv(k, g.taps, g.dv_taps), rs = k - c * g.taps;
                 const int r = conv_fdiv(rs, g.kW, g.dv_kW), s = rs - r * g.kW;
-                e = make_int4(c * g.H * g.W + r * g.dh * g.W + s * g.dw, r * g.dh, s * g.dw, 0);
+                const unsigned rh = (unsigned)(r * g.dh), sw = (unsigned)(s * g.dw);
+                e = make_int4((int)((unsigned)(c * g.H * g.W) + rh * (unsigned)g.W + sw), (int)rh, (int)sw, 0);
             }
             ktab[(kt % (kStages + 1)) * kBK + tid] = e;
         }
@@ -206,7 +209,7 @@ sgemm_kernel(const __grid_constant__ SgemmArgs g, int split) {
                     for (int kk = 0; kk < kBK; kk += B_KSTEP) {
                         const int4 t = tab[kk0 + kk];
                         const bool ok = (unsigned)(px_h[e] + t.y) < (unsigned)g.H && (unsigned)(px_w[e] + t.z) < (unsigned)g.W;
-                        cp_async4(dst, ok ? g.B + (px_base[e] + t.x) : g.B, ok);
+                        cp_async4(dst, ok ? g.B + (px_base[e] + (unsigned)t.x) : g.B, ok);
                         dst += B_KSTEP * PB * 4u;
                     }
                 }
@@ -523,7 +526,7 @@ int launch_simt_conv(const ConvGeom &g, const float *X, const float *W, const fl
     const char *pin = getenv("ONNXB_FP32");              // "small" pins the small-image kernel
     if (small >= 0 && (pin ? pin[0] == 's' : 0.85 * small < std::min(ch.pick.cost, ch.tc_cost)))      // (the tiled estimates run low here)
         return launch_small_conv(g, X, W, B, R, Y, stream);
-    if (ch.tc && a.taps <= 64) return launch_tc_fp32_conv(g, X, W, B, R, Y, stream);
+    if (ch.tc && tc_fp32_conv_fits(g)) return launch_tc_fp32_conv(g, X, W, B, R, Y, stream);
     return launch_sgemm<kKContig, kPixels>(a, g.group, pick, (cudaStream_t)stream);
 }
 

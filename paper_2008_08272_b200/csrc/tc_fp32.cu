@@ -154,7 +154,7 @@ __device__ __forceinline__ void src_load(const Args &g, bool rowop, const Src &s
             p += ld;
         }
     } else {
-        // the warp's 16 terms: offset in X and the tap's bit (lanes 0-15 work them out)
+        // the warp's 16 terms: offset in X and the tap's bit (lanes 0-15 work them out; tc_fp32_conv_fits: 31 bits hold it)
         const int k = k0 + (tid >> 7) * 16 + (lane & 15);
         int4 t = make_int4(0, 0, 0, 0);
         if (k < g.K) {
@@ -488,6 +488,14 @@ int launch_tc_fp32_gemm(const GemmProblem &p, const float *A, const float *B, co
     cudaStream_t st = (cudaStream_t)stream;
     if (p.transB) return p.transA ? launch<kKContig, kMnContig>(a, 1, st) : launch<kKContig, kKContig>(a, 1, st);
     return p.transA ? launch<kMnContig, kMnContig>(a, 1, st) : launch<kMnContig, kKContig>(a, 1, st);
+}
+
+// At most 64 taps (a bit each), and offsets of a window's terms from its start that are 32-bit integers: beyond, and only where
+// the image is mostly padding, a dilated row of taps lies 2^31 elements and more further on.  (Sums modulo 2^32 as in
+// the FMA kernel take an addition more per load: 86.3 -> 87.3 us on the dilated grouped 75x61 layer.)
+bool tc_fp32_conv_fits(const ConvGeom &g) {
+    const long long last = (g.Cg - 1LL) * g.H * g.W + (g.kH - 1LL) * g.dh * g.W + (g.kW - 1LL) * g.dw;
+    return g.kH * g.kW <= 64 && last <= 2147483647LL;
 }
 
 int launch_tc_fp32_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,

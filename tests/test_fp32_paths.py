@@ -113,3 +113,20 @@ def test_split_operands_that_overflow(binding, monkeypatch):
     assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
     ok = np.isfinite(want)
     assert np.allclose(got[ok], want[ok], rtol=1e-5, atol=1e-4)
+
+
+@pytest.mark.parametrize("pin", ["tc", "0,1", "2,3", "3,1", "4,8"])
+def test_conv_offsets_beyond_32_bits(binding, pin, monkeypatch):
+    """A dilation and a pad of 2^19 rows of 4096 and more columns: filter taps inside the image whose offset from the
+    window's start is 2^31 elements and more, and (700 rows fewer) just below that."""
+    monkeypatch.setenv("ONNXB_FP32", pin)
+    rng = np.random.default_rng(11)
+    far, near = 1 << 19, (1 << 19) - 700
+    for xs, ws, kw in (((2, 6, 4, 4096), (6, 3, 2, 1), dict(pads=(far, 0, 0, 0), dilations=(far, 1), group=2)),
+                       ((2, 6, 4, 4096), (6, 3, 2, 1), dict(pads=(near, 0, 0, 0), dilations=(near, 1), group=2)),
+                       ((1, 3, 3, 5000), (40, 3, 2, 3), dict(pads=(far, 1, 0, 1), dilations=(far, 1)))):
+        X, W, B = (rng.standard_normal(s).astype(np.float32) for s in (xs, ws, ws[:1]))
+        got, fam = run_conv_gpu(binding, torch, X, W, B, **kw)
+        assert fam == "simt_direct"
+        want, S = oracle.conv2d(X, W, B, **kw)
+        assert (np.abs(got - want) <= REL * S + 1e-5).all()
