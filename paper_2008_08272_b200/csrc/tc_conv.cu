@@ -1293,9 +1293,10 @@ static int launch_images(const TcConvPlan &plan, const float *X, const float *B,
     } else {
         memset(&tmX, 0, sizeof tmX);
     }
-    const size_t smem = 1024 + (size_t)plan.na_stages * plan.a_stage_bytes + (size_t)plan.nr_stages * plan.raw_stage_bytes +
-                        (size_t)plan.nb_stages * plan.b_stage_bytes + kMaxRawStages * kSegBytes + kBiasBytes + kBarBytes +
-                        (plan.split > 1 ? split_recv_bytes(plan.split, plan.cols_per) : 0);
+    const size_t smem = smem_with_tmem(1024 + (size_t)plan.na_stages * plan.a_stage_bytes + (size_t)plan.nr_stages * plan.raw_stage_bytes +
+                                           (size_t)plan.nb_stages * plan.b_stage_bytes + kMaxRawStages * kSegBytes + kBiasBytes + kBarBytes +
+                                           (plan.split > 1 ? split_recv_bytes(plan.split, plan.cols_per) : 0),
+                                       plan.split > 1 ? split_tmem_cols(plan.BN) : 512);
     const bool pair = plan.ctas == 2;
     const bool add = R != nullptr;
     const bool split = plan.split > 1;

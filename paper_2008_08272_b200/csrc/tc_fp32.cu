@@ -41,7 +41,9 @@ constexpr uint32_t kChunkPitch = 128 * 16 + 16;             // one 4-term chunk 
 constexpr uint32_t kPart = (kBK / 4) * kChunkPitch;         // one operand's hi or lo block
 constexpr uint32_t kStageBytes = 4 * kPart;                 // row hi, row lo, column hi, column lo
 constexpr int kTabBytes = kProducerWarps * 16 * 16;         // per producer warp: 16 reduction terms' offsets
+constexpr uint32_t kTmemCols = 256;                         // two accumulators
 constexpr size_t kSmem = 128 + (size_t)kStages * kStageBytes + kTabBytes + 256;
+static_assert(kSmem >= kTmemCols * kSmemPerTmemColumn, "see smem_with_tmem");
 
 struct Bars {
     uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2];
@@ -252,7 +254,7 @@ tc_fp32_kernel(const __grid_constant__ Args g, unsigned int *err) {
         mbar_fence_init();
     }
     if (warp == kMmaWarp) {
-        tmem_alloc(&bars->tmem_holder, 256);
+        tmem_alloc(&bars->tmem_holder, kTmemCols);
         tmem_relinquish();
     }
     tc_fence_before_sync();
@@ -432,7 +434,7 @@ tc_fp32_kernel(const __grid_constant__ Args g, unsigned int *err) {
     if (warp == kMmaWarp) {
         __syncwarp();
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, 256);
+        tmem_dealloc(tmem_base, kTmemCols);
     }
 }
 

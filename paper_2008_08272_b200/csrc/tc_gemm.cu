@@ -745,7 +745,7 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
         }
     }
 
-    const size_t smem = 1024 + (size_t)p.num_stages * p.stage_bytes + p.staging_bytes + kBarrierBytes;
+    const size_t smem = smem_with_tmem(1024 + (size_t)p.num_stages * p.stage_bytes + p.staging_bytes + kBarrierBytes, 512);
     auto kern = p.ctas == 2 ? (ks == 2 ? tc_gemm_kernel<2, 2> : tc_gemm_kernel<2, 1>)
                             : (ks == 2 ? tc_gemm_kernel<1, 2> : tc_gemm_kernel<1, 1>);
     const cudaError_t attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);

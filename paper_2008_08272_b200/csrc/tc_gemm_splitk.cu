@@ -489,7 +489,7 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
         p.b_big = make_tmap(&tmBb, g.B, 4, dims, str, box, kTmapSwizzle128Atom32) ? 1 : 0;
     }
     p.recv_off = (uint32_t)p.num_stages * p.stage_bytes;
-    const size_t smem = 2048 + p.recv_off + std::max(recv_bytes, (size_t)kABytes);      // (at least what an MMA of the last stage reads)
+    const size_t smem = smem_with_tmem(2048 + p.recv_off + std::max(recv_bytes, (size_t)kABytes), kMaxBN);      // (at least what an MMA of the last stage reads)
     auto kern = ks == 2 ? tc_gemm_splitk_kernel<2> : tc_gemm_splitk_kernel<1>;
     const cudaError_t ae = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (ae != cudaSuccess) return (int)ae;

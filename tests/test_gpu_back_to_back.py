@@ -86,3 +86,52 @@ def test_back_to_back_chain_equals_the_synchronised_chain(shape):
         assert torch.equal(got3, want3)
     for o in ops:
         o[0].close()
+
+
+def test_clusters_of_several_streams(monkeypatch):
+    """Kernels that allocate all, half or a quarter of TMEM, in clusters of 1 to 8, on four streams at once, each stream in
+    an order of its own: all come to an end, with the bits of the same calls one after the other."""
+    from paper_2008_08272_b200 import binding
+    dev = torch.device("cuda:0")
+    g = torch.Generator(device=dev)
+    g.manual_seed(5)
+    rnd = lambda *s: torch.randn(s, generator=g, device=dev)
+
+    def gemm(M, N, K, pin):
+        A, B = rnd(M, K), rnd(N, K)
+
+        def call(Y):
+            monkeypatch.setenv("ONNXB_GEMM_SPLITK", pin)       # read at every launch
+            return binding.onnx_gemm(A, B, transB=True, Y=Y)
+        return call, (M, N)
+
+    def conv(xs, ws, split, **kw):
+        monkeypatch.setenv("ONNXB_CONV_SPLIT", split)          # read when the descriptor is created
+        d = binding.Conv2dDesc(xs, ws, **kw)
+        assert d.kernel_family == "mma_implicit"
+        X, W = rnd(*xs), rnd(*ws)
+        packed = d.prepack(W)
+        return (lambda Y: d.run_prepacked(X, W, packed, Y=Y)), d.y_shape
+
+    same = dict(pads=(1, 1, 1, 1))
+    calls = [gemm(1024, 512, 256, "0"), gemm(8, 256, 512, "32,8"), gemm(200, 512, 256, "64,4"), gemm(96, 160, 1024, "128,2"),
+             conv((2, 128, 12, 12), (48, 128, 3, 3), "16,16,8", **same), conv((2, 128, 12, 12), (176, 128, 3, 3), "256,16,4", **same),
+             conv((16, 128, 28, 28), (128, 128, 3, 3), "0", **same)]
+    want = []
+    for call, shape in calls:
+        want.append(call(torch.empty(shape, device=dev)))
+        torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    outs = [[torch.empty(shape, device=dev) for _, shape in calls] for _ in streams]
+    torch.cuda.synchronize()
+    for round_ in range(12):
+        for k in range(len(calls)):
+            for i, s in enumerate(streams):
+                j = (k * (1, 2, 3, 5)[i] + i + round_) % len(calls)
+                with torch.cuda.stream(s):
+                    calls[j][0](outs[i][j])
+    torch.cuda.synchronize()
+    assert binding.last_device_status() == 0
+    for out in outs:
+        for y, w in zip(out, want):
+            assert torch.equal(y, w)
