@@ -6,7 +6,8 @@ torch stream is passed through.  There is no CPU fallback: if the compiled
 library is missing, or a tensor is not on a CUDA device, the call raises.
 
 The operator calls go through ``ext/fast_binding.cpp``, which does the marshalling below natively; a call it
-declines (returning None, nothing launched) is repeated here, where every check raises its own error.
+declines (returning None, nothing launched) is repeated here, where every check raises its own error.  Where it cannot be
+built or loaded (no compiler, another torch), a warning says so and every call is made here.
 """
 from __future__ import annotations
 
@@ -55,6 +56,13 @@ _lib = None
 _fast_mod = None
 
 
+class _Declined:
+    """Stands in for the native call path where there is none: every call is declined."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def _fast():
     """The native call path, loaded with the first operator call (it needs torch's C++ libraries)."""
     global _fast_mod
@@ -62,12 +70,18 @@ def _fast():
         import importlib.util
         import torch  # noqa: F401  (its libraries must be loaded first)
         load()
-        if not os.path.exists(_build.EXT_PATH):
-            _build.build_ext()
-        spec = importlib.util.spec_from_file_location("_onnxb_fast", _build.EXT_PATH)
-        mod = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(mod)
-        mod.bind(_build.LIB_PATH)
+        try:
+            path = _build.ext_path()
+            if not os.path.exists(path):
+                _build.build_ext()
+            spec = importlib.util.spec_from_file_location("_onnxb_fast", path)
+            mod = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(mod)
+            mod.bind(_build.LIB_PATH)
+        except Exception as e:
+            import warnings
+            warnings.warn(f"no native call path ({e}): operator calls go through ctypes, some 10 us of host time each")
+            mod = _Declined()
         _fast_mod = mod
     return _fast_mod
 

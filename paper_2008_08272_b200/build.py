@@ -1,6 +1,7 @@
 """Builds libonnx_b200.so in-tree with nvcc for sm_100a, and the binding's native call path with g++.
 
-Usage: ``python -m paper_2008_08272_b200.build [--force] [--verbose]``.
+Usage: ``python -m paper_2008_08272_b200.build [--force] [--verbose]``.  The library needs nvcc alone; the native call
+path also needs torch's headers, and where it cannot be built the binding makes its calls through ctypes.
 """
 from __future__ import annotations
 
@@ -16,7 +17,6 @@ CSRC = os.path.join(HERE, "csrc")
 LIB_DIR = os.path.join(HERE, "_lib")
 LIB_PATH = os.path.join(LIB_DIR, "libonnx_b200.so")
 EXT_SRC = os.path.join(HERE, "ext", "fast_binding.cpp")
-EXT_PATH = os.path.join(LIB_DIR, "_onnxb_fast.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -40,17 +40,25 @@ def is_stale() -> bool:
     return any(os.path.getmtime(f) > t for f in _inputs())
 
 
+def ext_path() -> str:
+    """The native call path's file.  It calls into torch's C++ libraries and into CPython, neither of which keeps its ABI, so
+    their versions are part of the name: a file built for others is never loaded."""
+    import importlib.metadata
+    return os.path.join(LIB_DIR, "_onnxb_fast.%s.torch-%s.so" % (sys.implementation.cache_tag, importlib.metadata.version("torch")))
+
+
 def build_ext(force: bool = False, verbose: bool = False) -> str:
     """Compile the binding's native call path (a CPython extension on torch's C++ tensors)."""
     import sysconfig
+    path = ext_path()
     deps = [EXT_SRC, os.path.join(ROOT, "include", "onnx_b200.h")]
-    if not force and os.path.exists(EXT_PATH) and all(os.path.getmtime(EXT_PATH) >= os.path.getmtime(f) for f in deps):
-        return EXT_PATH
+    if not force and os.path.exists(path) and all(os.path.getmtime(path) >= os.path.getmtime(f) for f in deps):
+        return path
     import torch
     tdir = os.path.dirname(torch.__file__)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     os.makedirs(LIB_DIR, exist_ok=True)
-    tmp = EXT_PATH + ".%d.tmp" % os.getpid()
+    tmp = path + ".%d.tmp" % os.getpid()
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
            "-I" + os.path.join(ROOT, "include"), "-I" + os.path.join(tdir, "include"),
@@ -61,14 +69,13 @@ def build_ext(force: bool = False, verbose: bool = False) -> str:
     if verbose or proc.returncode != 0:
         sys.stderr.write(proc.stdout)
     if proc.returncode != 0:
-        raise RuntimeError("g++ failed building _onnxb_fast.so")
-    os.replace(tmp, EXT_PATH)
-    return EXT_PATH
+        raise RuntimeError("g++ failed building " + os.path.basename(path))
+    os.replace(tmp, path)
+    return path
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every CUDA source of the library into one shared object, and the binding's native call path."""
-    build_ext(force, verbose)
+    """Compile every CUDA source of the library into one shared object."""
     if not force and not is_stale():
         return LIB_PATH
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
@@ -89,4 +96,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 
 if __name__ == "__main__":
-    print(build(force="--force" in sys.argv, verbose="--verbose" in sys.argv))
+    flags = dict(force="--force" in sys.argv, verbose="--verbose" in sys.argv)
+    print(build(**flags))
+    try:
+        print(build_ext(**flags))
+    except Exception as e:
+        print("the binding's native call path was not built (%s): it will call through ctypes" % e, file=sys.stderr)
