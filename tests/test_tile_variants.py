@@ -63,16 +63,21 @@ def test_gemm_k_blocks_per_stage(binding, ks, pair, monkeypatch):
 @pytest.mark.parametrize("rows", [1, 7, 9, 65])
 def test_gemm_split_of_few_rows(binding, rows, monkeypatch):
     rng = np.random.default_rng(rows)
-    for shape in ("32,1", "32,8", "128,4"):
-        monkeypatch.setenv("ONNXB_GEMM_SPLITK", shape)
-        for N, K in ((1000, 768), (132, 356)):
-            A = rng.standard_normal((rows, K)).astype(np.float32)
-            B = rng.standard_normal((N, K)).astype(np.float32)
-            C = rng.standard_normal((N,)).astype(np.float32)
-            monkeypatch.setenv("ONNXB_FP32", "x")              # (not the dot-product kernel of tiny problems)
-            got = run_gemm_gpu(binding, torch, A, B, C, transB=True)
-            want, S = oracle.gemm(A, B, C, transB=True)
-            assert worst_ratio(got, want, S) <= 1.0, (shape, N, K)
+    binding.set_kernel_override("mma_gemm")                     # else the dot-product kernel takes the tiny ones
+    try:
+        for shape in ("32,1", "32,8", "128,4"):
+            monkeypatch.setenv("ONNXB_GEMM_SPLITK", shape)
+            for N, K in ((1000, 768), (132, 356)):
+                A = rng.standard_normal((rows, K)).astype(np.float32)
+                B = rng.standard_normal((N, K)).astype(np.float32)
+                C = rng.standard_normal((N,)).astype(np.float32)
+                before = binding.launch_count()
+                got = run_gemm_gpu(binding, torch, A, B, C, transB=True)
+                assert binding.launch_count() == before + 1     # the other tensor-core form has a rounding launch in front
+                want, S = oracle.gemm(A, B, C, transB=True)
+                assert worst_ratio(got, want, S) <= 1.0, (shape, N, K)
+    finally:
+        binding.set_kernel_override(None)
 
 
 @pytest.mark.parametrize("xs,pads", [((47, 126, 28, 28), (1, 1, 1, 1)), ((75, 128, 32, 32), (0, 1, 0, 1)), ((151, 128, 15, 16), (2, 1, 1, 1))])
