@@ -411,11 +411,11 @@ conv2d_depthwise_unit_kernel(const ConvGeom g, const float *__restrict__ X, cons
 // CTAs per SM, 20.9 with three and three, 22.4 with five and two).  Bound by HBM, at 5.1 TB/s there.
 constexpr int kRingStages = 2, kRingCtas = 4, kRingStageMax = 24576;
 
-template <int KH, int KW, int ROWS>
 __global__ void __launch_bounds__(256, kRingCtas)
 conv2d_depthwise_ring_kernel(const ConvGeom g, const float *__restrict__ X, const float *__restrict__ W, const float *__restrict__ B,
                              const float *__restrict__ R, float *__restrict__ Y, unsigned planes, unsigned per, unsigned Q4, unsigned P2,
                              const ConvDivisor dv_Q4, const ConvDivisor dv_P2, const ConvDivisor dv_C, unsigned int *err) {
+    constexpr int KH = 3, KW = 3, ROWS = 4;                    // the one filter and strip that the launch gives it
     extern __shared__ __align__(128) float ring[];
     __shared__ uint64_t full[kRingStages];
     const unsigned units = (planes + per - 1) / per, plane_floats = (unsigned)(g.H * g.W);
@@ -437,25 +437,19 @@ conv2d_depthwise_ring_kernel(const ConvGeom g, const float *__restrict__ X, cons
     int stage = 0;
     uint32_t phase = 0;
     for (unsigned u = blockIdx.x; u < units; u += gridDim.x) {
-        const unsigned items = min(per, planes - u * per) * P2 * Q4;
-        const float *base = ring + (size_t)stage * per * plane_floats;
-        bool landed = false;
-        for (unsigned i0 = 0; i0 < items; i0 += 256u) {
-            const unsigned i_own = i0 + threadIdx.x, i = min(i_own, items - 1);        // (the neighbours of a live lane must stay)
-            const unsigned t = (unsigned)conv_fdiv((int)i, (int)Q4, dv_Q4), pl = (unsigned)conv_fdiv((int)t, (int)P2, dv_P2);
-            const int q0 = (int)(i - t * Q4) * 4, p0 = (int)(t - pl * P2) * ROWS;
-            const unsigned plane = u * per + pl;
-            const unsigned c = plane - (unsigned)conv_fdiv((int)plane, g.C, dv_C) * (unsigned)g.C;
-            float w[KH * KW];
+        const unsigned items = min(per, planes - u * per) * P2 * Q4, i = min(threadIdx.x, items - 1);     // (at most 256; the neighbours of a live lane must stay)
+        const unsigned t = (unsigned)conv_fdiv((int)i, (int)Q4, dv_Q4), pl = (unsigned)conv_fdiv((int)t, (int)P2, dv_P2);
+        const int q0 = (int)(i - t * Q4) * 4, p0 = (int)(t - pl * P2) * ROWS;
+        const unsigned plane = u * per + pl;
+        const unsigned c = plane - (unsigned)conv_fdiv((int)plane, g.C, dv_C) * (unsigned)g.C;
+        float w[KH * KW];
 #pragma unroll
-            for (int k = 0; k < KH * KW; ++k) w[k] = __ldg(W + (size_t)c * (KH * KW) + k);
-            const float bias = B ? __ldg(B + c) : 0.f;
-            if (!landed) tc::mbar_wait(&full[stage], phase, err, 60);
-            landed = true;
-            float v[KH + ROWS - 1][KW + 3];
-            depthwise_window_vec<KH, KW, ROWS, true>(base + pl * plane_floats, g.H, g.W, p0 - g.pt, q0, v);
-            if (i_own < items) depthwise_strip<KH, KW, ROWS, true>(g, v, w, bias, R, Y, plane, p0, q0);
-        }
+        for (int k = 0; k < KH * KW; ++k) w[k] = __ldg(W + (size_t)c * (KH * KW) + k);
+        const float bias = B ? __ldg(B + c) : 0.f;
+        tc::mbar_wait(&full[stage], phase, err, 60);
+        float v[KH + ROWS - 1][KW + 3];
+        depthwise_window_vec<KH, KW, ROWS, true>(ring + ((size_t)stage * per + pl) * plane_floats, g.H, g.W, p0 - g.pt, q0, v);
+        if (threadIdx.x < items) depthwise_strip<KH, KW, ROWS, true>(g, v, w, bias, R, Y, plane, p0, q0);
         __syncthreads();                                       // every thread has read the stage
         if (threadIdx.x == 0 && u + kRingStages * gridDim.x < units) fetch(u + kRingStages * gridDim.x, stage);
         if (++stage == kRingStages) { stage = 0; phase ^= 1; }
@@ -478,11 +472,11 @@ int launch_depthwise_unit(const ConvGeom &g, const float *X, const float *W, con
     // units for every CTA, or the ring has nothing to run ahead of.  A 5x5 window does not leave room for four CTAs.
     const long long planes = (long long)g.N * g.C, plane_bytes = (long long)g.H * g.W * 4;
     const long long per = std::max(1LL, std::min(256LL / (P2 * Q4), kRingStageMax / plane_bytes)), strips = per * P2 * Q4;
-    if (KH == 3 && vec && rows4 && plane_bytes <= kRingStageMax && strips >= 224 && strips <= 256 &&
+    if (KH == 3 && KW == 3 && vec && rows4 && plane_bytes <= kRingStageMax && strips >= 224 && strips <= 256 &&
         planes >= per * 148 * kRingCtas * 2) {
         unsigned int *err = device_status_ptr();
         if (!err) return (int)cudaErrorUnknown;
-        auto ring = conv2d_depthwise_ring_kernel<3, 3, 4>;
+        auto ring = conv2d_depthwise_ring_kernel;
         const cudaError_t ae = cudaFuncSetAttribute(ring, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingStages * kRingStageMax);
         if (ae != cudaSuccess) return (int)ae;
         const unsigned units = (unsigned)((planes + per - 1) / per);
