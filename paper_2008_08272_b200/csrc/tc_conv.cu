@@ -686,8 +686,11 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                 }
                 char *yb = reinterpret_cast<char *>(Y);
                 const char *rb = reinterpret_cast<const char *>(R);
-                // fmaxf returns its other argument where one is NaN, and NaN where both are: without Relu nothing is changed
-                const float lowest = g.relu ? 0.f : __int_as_float(0x7FC00000);
+                // fmaxf returns its other argument where one is NaN, and NaN where both are: without Relu nothing is changed.
+                // (The constant is hidden from the compiler, which would otherwise choose between x and fmaxf(x, 0) for every
+                // output; that took the form with an addend from 145 to 185 us on a 3 -> 64, 7x7/2, 224x224 layer, batch 32.)
+                float lowest;
+                asm("mov.b32 %0, %1;" : "=f"(lowest) : "r"(g.relu ? 0 : 0x7FC00000));
                 for (int chunk = ch_lo; chunk < ch_hi; ++chunk) {
                     uint32_t v[32];
                     tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc_col + (uint32_t)(chunk * 32), v);
