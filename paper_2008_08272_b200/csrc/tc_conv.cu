@@ -117,8 +117,8 @@ __global__ void pack_weights_kernel(const TcConvPlan g, const float *__restrict_
 // same L2 lines at the same moment.
 __device__ __forceinline__ int cb_rotation(long long tile, int ncb) { return (int)((tile * 5 + 3) % ncb); }
 
-// TMEM columns of a split tile: its one accumulator (read in blocks of 32)
-__host__ __device__ constexpr uint32_t split_tmem_cols(int BN) { return BN <= 32 ? 32u : BN <= 64 ? 64u : BN <= 128 ? 128u : 256u; }
+// TMEM columns of a split tile: its one accumulator, in the sizes that smem_with_tmem knows
+__host__ __device__ constexpr uint32_t split_tmem_cols(int BN) { return BN <= 128 ? 128u : 256u; }
 // shared memory for its partial sums
 __host__ __device__ constexpr int split_recv_bytes(int split, int cols_per) { return split * cols_per * 512; }
 

@@ -43,7 +43,7 @@ constexpr uint32_t kStageBytes = 4 * kPart;                 // row hi, row lo, c
 constexpr int kTabBytes = kProducerWarps * 16 * 16;         // per producer warp: 16 reduction terms' offsets
 constexpr uint32_t kTmemCols = 256;                         // two accumulators
 constexpr size_t kSmem = 128 + (size_t)kStages * kStageBytes + kTabBytes + 256;
-static_assert(kSmem >= kTmemCols * kSmemPerTmemColumn, "see smem_with_tmem");
+static_assert(kSmem >= kSmemMoreTmem, "see smem_with_tmem");
 
 struct Bars {
     uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2];

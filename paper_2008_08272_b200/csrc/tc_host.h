@@ -41,15 +41,17 @@ double tc_gemm_estimate_ns(const TcGemmProblem &g);       // the persistent kern
 bool tc_gemm_splitk_fits(const TcGemmProblem &g);
 int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream);
 
-// Shared memory to launch a CTA with that uses `smem` bytes of it and allocates `columns` of TMEM.  tcgen05.alloc waits
-// for columns without limit, and the CTAs of a cluster wait for one another with theirs held: two clusters of different
-// streams could each hold on one SM what the other waits for on another.  So no CTA is to find too little: it reserves
-// shared memory in proportion to its columns (128 at least), and CTAs that need more than all 512 between them, 640 or
-// more then, do not fit one SM's 228 KB.  (At present their registers rule it out as well, and nearly every launch is
-// above its share anyway.)
-constexpr size_t kSmemPerTmemColumn = 368, kSmemPerSm = 228 * 1024;
-static_assert(640 * kSmemPerTmemColumn > kSmemPerSm && 512 * kSmemPerTmemColumn <= 227 * 1024, "share of a TMEM column");
-inline size_t smem_with_tmem(size_t smem, uint32_t columns) { return std::max(smem, std::max(columns, 128u) * kSmemPerTmemColumn); }
+// Shared memory to launch a CTA with that uses `smem` bytes of it and allocates `columns` of TMEM (128, 256 or 512).
+// tcgen05.alloc waits for columns without limit, and the CTAs of a cluster wait for one another with theirs held: two
+// clusters of different streams could each hold on one SM what the other waits for on another.  So no CTA is to find too
+// little, or what there is in pieces: one that allocates a quarter of TMEM reserves so much shared memory that five do not
+// fit an SM, one that allocates more so much that it does not fit beside another of either kind.  (At present their
+// registers rule both out as well, and nearly every launch uses more anyway.)
+constexpr size_t kSmemPerSm = 228 * 1024, kSmemPerCta = 1024;        // (the second: what the system adds for each CTA)
+constexpr size_t kSmemQuarterTmem = 46 * 1024, kSmemMoreTmem = 184 * 1024;
+static_assert(5 * (kSmemQuarterTmem + kSmemPerCta) > kSmemPerSm, "five quarters of TMEM on one SM");
+static_assert(kSmemMoreTmem + kSmemQuarterTmem + 2 * kSmemPerCta > kSmemPerSm, "more than TMEM on one SM");
+inline size_t smem_with_tmem(size_t smem, uint32_t columns) { return std::max(smem, columns <= 128 ? kSmemQuarterTmem : kSmemMoreTmem); }
 
 // Address of the device error word of the current device (NULL on failure).
 unsigned int *device_status_ptr();
