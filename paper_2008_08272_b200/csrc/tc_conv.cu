@@ -45,9 +45,10 @@ namespace {
 using namespace tc;
 
 // Warps: raw producer, weight producer, MMA issuer, relay, then 12 transform warps and 8 epilogue warps: 768 threads,
-// 80 registers each.  Both kernels below stay within them without a spill, on purpose: with 227 KB of shared memory
-// per CTA next to no L1 is left, and a value spilled in a transform loop is a trip to L2 (the same kernel with 40 to 90
-// bytes of spills took 51.6 us on the 64-channel 56x56 layer at batch 64, without them 44.3; the stem 101 -> 78).
+// 80 registers each.  The forms of the kernel below stay within them without a spill (one with an addend has two words),
+// on purpose: with 227 KB of shared memory per CTA next to no L1 is left, and a value spilled in a transform loop is a
+// trip to L2 (40 to 90 bytes of spills, while the loops were being written, cost 7 of 51 us on the 64-channel 56x56
+// layer at batch 64, 23 of 101 on the 7x7/2 first layer).
 constexpr int kXformWarps = 12, kXformThreads = kXformWarps * 32, kEpiWarps = 8;
 constexpr int kRelayWarp = 3;               // odd CTA of a pair: passes "operand stage written" on to the issuing CTA
 constexpr int kFirstXformWarp = 4, kFirstEpiWarp = kFirstXformWarp + kXformWarps;
@@ -1033,11 +1034,12 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
         } else if (MT == 2 && g.KB >= 16 &&
                    kSmemLimit - (1024 + 3LL * g.a_stage_bytes + kMaxRawStages * kSegBytes + kBiasBytes + kBarBytes) -
                            2LL * g.raw_stage_bytes >= 65536) {
-            // Two accumulators per CTA: a third operand stage instead of a third raw stage (64 -> 64
-            // channels at 56x56: 55.5 -> 52.3 us), and in a CTA pair the odd CTA's "stage written" message
-            // through its relay warp.  The message then arrives later, which three stages absorb, and the
-            // transform warps no longer wait for their cluster-scope fence (128 -> 128 channels at 28x28:
-            // 43.4 -> 41.0 us; with two stages the relay loses).
+            // Two accumulators per CTA: a third operand stage instead of a third raw stage, and in a CTA pair
+            // the odd CTA's "stage written" message through its relay warp.  The message then arrives later,
+            // which three stages absorb, and the transform warps no longer wait for their cluster-scope fence.
+            // Batch 64, the same tile; two operand and three raw stages without / with the relay, three and two
+            // without / with it: 64 -> 64 channels at 56x56 46.6 / 45.5, 47.2 / 38.2 us; 128 -> 128 at 28x28
+            // 34.1 / 37.0, 33.4 / 31.8; 256 -> 256 at 14x14 32.6 / 35.1, 31.7 / 31.8.
             g.na_stages = 3;
             g.relay = ctas == 2 ? 1 : 0;
         } else {
@@ -1211,8 +1213,9 @@ bool tc_conv_plan(const ConvGeom &c, TcConvPlan &plan, bool forced) {
         }
     }
     if (have) {
-        // Thin first layers in tap-pair mode are paced by the transform warps: take their fence off them too
-        // (ResNet-50 stem: 109.3 -> 106.6 us).  ONNXB_CONV_RELAY = 0 | 1 pins the choice for A/B measurements.
+        // Thin layers in tap-pair mode, where they run as pairs, are paced by the transform warps: take their fence off
+        // them too (4 -> 160 channels, 7x7/2, 112x112, batch 64, one accumulator: 46.0 -> 43.0 us; 3 -> 64 at 224x224,
+        // as a pair, 82.6 -> 75.7).  ONNXB_CONV_RELAY = 0 | 1 pins the choice for A/B measurements.
         if (plan.ctas == 2 && plan.KB == 4) plan.relay = 1;
         if (const char *e = getenv("ONNXB_CONV_RELAY"))
             if (e[0] == '0' || e[0] == '1') plan.relay = e[0] - '0';
