@@ -456,6 +456,112 @@ conv2d_depthwise_ring_kernel(const ConvGeom g, const float *__restrict__ X, cons
     }
 }
 
+// Depthwise convolution whose rows are no whole 16-byte pieces, or whose stride or dilation is not one: a thread owns
+// ROWS outputs of one column of a plane, lanes run along the output columns, so that a load touches one line (two at
+// column stride 2) where the strips above, four columns to a lane, touch four and more.  Bound by these loads' issue and by
+// HBM, so the rows of the window that the thread's outputs share are loaded once: at row stride 1 its outputs lie a dilation
+// apart, at row stride 2 (dilation 1) next to each other.  Column stride and dilation cost nothing and are any.  Against the
+// tiles of conv2d_depthwise_kernel: 160 channels 70x70 3x3/2 with an addend, batch 26: 165 -> 25 us (floor 19); 176 channels
+// 37x37 5x5/2, batch 38: 78 -> 26; 32 channels 179x114 dilation 2, batch 17: 105 -> 37.
+template <int KH, int KW, int SH, int ROWS>
+__global__ void __launch_bounds__(256)
+conv2d_depthwise_column_kernel(const ConvGeom g, const float *__restrict__ X, const float *__restrict__ W, const float *__restrict__ B,
+                               const float *__restrict__ R, float *__restrict__ Y, unsigned items, unsigned PG,
+                               const ConvDivisor dv_Q, const ConvDivisor dv_PG, const ConvDivisor dv_C, const ConvDivisor dv_dh) {
+    constexpr int NR = (ROWS - 1) * SH + KH;
+    tc::pdl_launch_dependents();
+    const unsigned i = blockIdx.x * 256u + threadIdx.x;
+    if (i >= items) return;
+    // i = (plane * PG + row group) * Q + column; a group's first row: a block of ROWS * dh rows, then one of its first dh
+    const unsigned t = (unsigned)conv_fdiv((int)i, g.Q, dv_Q), q = i - t * (unsigned)g.Q;
+    const unsigned plane = (unsigned)conv_fdiv((int)t, (int)PG, dv_PG), pg = t - plane * PG;
+    const unsigned dh = SH == 1 ? (unsigned)g.dh : 1u;
+    const unsigned blk = SH == 1 ? (unsigned)conv_fdiv((int)pg, g.dh, dv_dh) : pg;
+    const unsigned p0 = SH == 1 ? blk * (ROWS * dh) + (pg - blk * dh) : pg * ROWS;
+    const unsigned c = plane - (unsigned)conv_fdiv((int)plane, g.C, dv_C) * (unsigned)g.C;
+    const float *xp = X + (size_t)plane * g.H * g.W, *wp = W + (size_t)c * (KH * KW);
+    // (modulo 2^32: a row or column outside the image, however far, is no row or column of it)
+    const unsigned h0 = p0 * SH - (unsigned)g.pt, w0 = q * (unsigned)g.sw - (unsigned)g.pl;
+    tc::pdl_wait();
+    float v[NR][KW], w[KH * KW];
+#pragma unroll
+    for (int rr = 0; rr < NR; ++rr) {
+        const unsigned ih = h0 + rr * dh;
+        const float *row = xp + (size_t)ih * g.W;
+#pragma unroll
+        for (int s = 0; s < KW; ++s) {
+            const unsigned iw = w0 + s * (unsigned)g.dw;
+            v[rr][s] = ih < (unsigned)g.H && iw < (unsigned)g.W ? __ldg(row + iw) : 0.f;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < KH * KW; ++k) w[k] = __ldg(wp + k);
+    const float bias = B ? __ldg(B + c) : 0.f;
+    const size_t y0 = ((size_t)plane * g.P + p0) * g.Q + q, ystep = (size_t)dh * g.Q;
+    float r[ROWS];
+#pragma unroll
+    for (int k = 0; k < ROWS; ++k) r[k] = R && p0 + k * dh < (unsigned)g.P ? __ldg(R + y0 + k * ystep) : 0.f;
+#pragma unroll
+    for (int k = 0; k < ROWS; ++k) {
+        float a = bias;
+#pragma unroll
+        for (int rr = 0; rr < KH; ++rr)
+#pragma unroll
+            for (int s = 0; s < KW; ++s) a = fmaf(v[k * SH + rr][s], w[rr * KW + s], a);
+        if (R) a += r[k];
+        if (g.relu) a = a > 0.f ? a : 0.f;
+        if (p0 + k * dh < (unsigned)g.P) Y[y0 + k * ystep] = a;
+    }
+}
+
+// Rows per thread: the fewest loads per column of a plane (rows past the last one are loaded too) that leave every SM
+// 512 threads.
+struct ColumnPick {
+    int rows;
+    long long PG, items;
+};
+ColumnPick depthwise_column_pick(const ConvGeom &g) {
+    ColumnPick best{0, 0, 0};
+    long long best_loads = 0;
+    for (int rows : {8, 4, 2}) {
+        if (rows == 8 && (g.kH == 5 || g.sh == 2)) continue;      // windows of that many registers are slower
+        const long long dh = g.sh == 1 ? g.dh : 1, whole = g.P / (rows * dh), PG = whole * dh + std::min(dh, g.P - whole * rows * dh);
+        const long long items = (long long)g.N * g.C * PG * g.Q, loads = PG * ((rows - 1) * g.sh + g.kH);
+        if (best.rows && best.items >= 148LL * 512 && loads >= best_loads) continue;
+        best = {rows, PG, items};
+        best_loads = loads;
+    }
+    return best;
+}
+
+bool depthwise_column_fits(const ConvGeom &g) {
+    if (!(g.Cg == 1 && g.Mg == 1 && (g.sh == 1 || (g.sh == 2 && g.dh == 1)))) return false;
+    if (!((g.kH == 3 && g.kW == 3) || (g.kH == 5 && g.kW == 5))) return false;
+    return depthwise_column_pick(g).items < (1LL << 31) - 256;
+}
+
+template <int K>
+int launch_depthwise_column(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y, cudaStream_t st) {
+    const ColumnPick p = depthwise_column_pick(g);
+    auto kern = g.sh == 1 ? (p.rows == 8   ? conv2d_depthwise_column_kernel<K, K, 1, K == 3 ? 8 : 4>
+                             : p.rows == 4 ? conv2d_depthwise_column_kernel<K, K, 1, 4>
+                                           : conv2d_depthwise_column_kernel<K, K, 1, 2>)
+                          : (p.rows == 4 ? conv2d_depthwise_column_kernel<K, K, 2, 4> : conv2d_depthwise_column_kernel<K, K, 2, 2>);
+    const cudaError_t e = tc_host::launch_pdl(kern, dim3((unsigned)((p.items + 255) / 256)), dim3(256), 0, st, g, X, W, B, R, Y,
+                                              (unsigned)p.items, (unsigned)p.PG, conv_divisor(g.Q), conv_divisor((int)p.PG),
+                                              conv_divisor(g.C), conv_divisor(g.dh));
+    count_launch();
+    return (int)e;
+}
+
+// Every input and output row starts on a 16-byte boundary, as far as the sizes tell.
+bool depthwise_rows_vectorised(const ConvGeom &g) { return g.pl == (g.kW - 1) / 2 && g.W % 4 == 0 && g.Q == g.W; }
+
+// Where both kernels serve rows that are not: the strips' loads per output are fewer (2.25 against 3.75 at 3x3), the
+// columns' threads more and their lines per load a quarter.  3x3: 64 planes of 74x74 6.3 -> 2.8 us, 33 of 177x226 7.2 ->
+// 5.8, but 1170 of 59x59 12.5 -> 14.5; 5x5: 192 planes of 17x17 4.2 -> 2.8, but 800 of 51x39 10.4 -> 11.9.
+bool depthwise_columns_first(const ConvGeom &g) { return (long long)g.N * g.C * g.P * g.Q < (g.kH == 3 ? 2000000 : 500000); }
+
 template <int KH, int KW>
 int launch_depthwise_unit(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                           cudaStream_t st) {
@@ -466,7 +572,7 @@ int launch_depthwise_unit(const ConvGeom &g, const float *X, const float *W, con
     const long long items = (long long)g.N * g.C * P2 * Q4;
     const unsigned blocks = (unsigned)((items + 255) / 256);
     // aligned 16-byte accesses: every input and output row starts on a 16-byte boundary
-    const bool vec = g.pl == (KW - 1) / 2 && g.W % 4 == 0 && g.Q == g.W &&
+    const bool vec = depthwise_rows_vectorised(g) &&
                      (reinterpret_cast<uintptr_t>(X) & 15) == 0 && (reinterpret_cast<uintptr_t>(Y) & 15) == 0;
     // Planes per copy: a strip for every thread, and not many threads without one (56x56 has 196: 38.7 -> 39.4 us); several
     // units for every CTA, or the ring has nothing to run ahead of.  A 5x5 window does not leave room for four CTAs.
@@ -604,7 +710,11 @@ int launch_gather1x1(const ConvGeom &g, const float *X, float *Xg, long long pit
 
 int launch_simt_depthwise(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                           void *stream) {
-    if (depthwise_unit_fits(g)) {
+    const bool unit = depthwise_unit_fits(g);
+    if (depthwise_column_fits(g) && (!unit || (!depthwise_rows_vectorised(g) && depthwise_columns_first(g))))
+        return g.kH == 3 ? launch_depthwise_column<3>(g, X, W, B, R, Y, (cudaStream_t)stream)
+                         : launch_depthwise_column<5>(g, X, W, B, R, Y, (cudaStream_t)stream);
+    if (unit) {
         if (g.kH == 3) return launch_depthwise_unit<3, 3>(g, X, W, B, R, Y, (cudaStream_t)stream);
         return launch_depthwise_unit<5, 5>(g, X, W, B, R, Y, (cudaStream_t)stream);
     }
