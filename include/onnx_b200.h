@@ -67,7 +67,8 @@ typedef enum {
 
 /* Kernel family a descriptor resolved to (reported by onnx_conv2d_desc_query_kernel). */
 typedef enum {
-    ONNXB_KERNEL_SIMT_DIRECT = 0,  /* fp32 FMA direct convolution (thin contractions, any attributes) */
+    ONNXB_KERNEL_SIMT_DIRECT = 0,  /* fp32 direct convolution (thin contractions, images TMA cannot address, any attributes): FMA, or
+                                      where it is large split-TF32 products on the tensor cores, as exact */
     ONNXB_KERNEL_SIMT_DEPTHWISE = 1, /* fp32 FMA, one input channel per output channel, smem row tiles */
     ONNXB_KERNEL_MMA_GEMM = 2,     /* 1x1 stride-1: batched tcgen05 TF32 GEMM straight from NCHW via TMA */
     ONNXB_KERNEL_MMA_IMPLICIT = 3, /* general implicit GEMM: TMA staging + in-smem im2col + tcgen05 TF32 */
@@ -138,7 +139,8 @@ int onnx_conv2d_desc_query_kernel(onnxb_conv2d_desc_t desc);
  * X [N,C,H,W], W [M,C/g,kH,kW], B [M] (NULL exactly when has_bias == 0),
  * Y [N,M,P,Q]: device, fp32, dense.  workspace: device scratch of at least the
  * queried size (NULL allowed when that size is 0); its contents are undefined on
- * return and two runs that share a workspace must not overlap in time.
+ * return and two runs that share a workspace must not overlap in time.  With less
+ * than that a descriptor of ONNXB_KERNEL_SIMT_DIRECT runs all the same, on its FMA kernel.
  * Errors: ERR_NULL, ERR_WORKSPACE, ERR_UNSUPPORTED (misaligned pointer),
  * ERR_CUDA (launch failure).
  */
@@ -166,9 +168,11 @@ onnxb_status onnx_conv2d_add_run(onnxb_conv2d_desc_t desc, const float *X, const
  *
  * onnx_conv2d_prepack writes the derived copy of W that the descriptor's kernel reads (packed and
  * rounded to TF32 for ONNXB_KERNEL_MMA_IMPLICIT, rounded to TF32 for ONNXB_KERNEL_MMA_GEMM and
- * ONNXB_KERNEL_MMA_GATHER_GEMM) into `packed` (device, caller-owned, at least the workspace_bytes
- * of onnx_conv2d_desc_query, 16-byte aligned).  Descriptors of the SIMT kernels read W directly:
- * the call then does nothing and returns OK.
+ * ONNXB_KERNEL_MMA_GATHER_GEMM, split into two TF32 parts for ONNXB_KERNEL_SIMT_DIRECT with filters
+ * larger than 1x1 where its workspace_bytes is not 0) into `packed` (device, caller-owned, at least the
+ * workspace_bytes of onnx_conv2d_desc_query, 16-byte aligned).  Other descriptors of the SIMT kernels
+ * read W directly: the call then does nothing and returns OK, as it does for any of theirs when
+ * `packed` is NULL (the run call then uses none).
  * onnx_conv2d_run_prepacked computes what onnx_conv2d_run (R == NULL) or onnx_conv2d_add_run
  * (R != NULL) computes, from that copy, bit for bit.  W must still be passed (the kernels that use
  * no copy read it) and must be the tensor that was packed; `packed` is read only.  workspace /
@@ -218,7 +222,9 @@ size_t onnx_conv2d_static_scratch_bytes(void);
  * problem (0 when none).  Host only.  The tensor-core path keeps TF32-rounded
  * copies of A and B there (4 * (M*K + K*N) bytes; its split-K form for small M
  * rounds in shared memory and leaves the workspace untouched, but the size is
- * asked for all the same); the SIMT path needs none.
+ * asked for all the same); the fp32 path of large problems keeps both operands,
+ * split into two TF32 parts, there (8 bytes an element, padded to whole tiles)
+ * and runs on its FMA kernel, which needs none, where it is given less.
  */
 size_t onnx_gemm_workspace_bytes(int transA, int transB, int64_t M, int64_t N, int64_t K);
 

@@ -22,7 +22,7 @@ STATUS_NAMES = ["OK", "ERR_NULL", "ERR_ATTR", "ERR_SHAPE", "ERR_UNSUPPORTED", "E
                 "ERR_CUDA", "ERR_DEVICE_TIMEOUT"]
 AUTO_PAD = {"NOTSET": 0, "SAME_UPPER": 1, "SAME_LOWER": 2, "VALID": 3}
 KERNEL_FAMILIES = ["simt_direct", "simt_depthwise", "mma_gemm", "mma_implicit", "mma_gather_gemm"]
-WEIGHT_COPY_FAMILIES = ("mma_implicit", "mma_gemm", "mma_gather_gemm")   # prepack makes their derived copy of W once
+WEIGHT_COPY_FAMILIES = ("mma_implicit", "mma_gemm", "mma_gather_gemm")   # prepack always makes their derived copy of W once
 
 EXPORTS = [
     "onnx_conv2d_desc", "onnx_conv2d_desc_query", "onnx_conv2d_desc_query_kernel", "onnx_conv2d_run",
@@ -214,7 +214,7 @@ class Conv2dDesc:
         self.workspace_bytes = int(ws.value)
         self.kernel_family = KERNEL_FAMILIES[self._lib.onnx_conv2d_desc_query_kernel(self._h)]
         self._prepacked_needs_ws = bool(
-            (self.kernel_family not in WEIGHT_COPY_FAMILIES or self.kernel_family == "mma_gather_gemm")
+            (self.kernel_family == "mma_gather_gemm" or (self.kernel_family == "simt_direct" and tuple(w_shape[2:]) == (1, 1)))
             and self.workspace_bytes)
         self._plan = None
 
@@ -262,11 +262,10 @@ class Conv2dDesc:
         return Y
 
     def prepack(self, W, stream=None):
-        """``onnx_conv2d_prepack``: the packed copy of constant weights (a uint8 device tensor; empty when
+        """``onnx_conv2d_prepack``: the packed copy of constant weights (a uint8 device tensor; untouched when
         this descriptor's kernel reads W directly)."""
         import torch
-        packed = torch.empty(max(self.workspace_bytes, 16) if self.kernel_family in WEIGHT_COPY_FAMILIES else 16,
-                             dtype=torch.uint8, device=W.device)
+        packed = torch.empty(max(self.workspace_bytes, 16), dtype=torch.uint8, device=W.device)
         _check(self._lib.onnx_conv2d_prepack(self._h, _dev_ptr(W, "W"), ctypes.c_void_p(packed.data_ptr()),
                                              packed.numel(), _stream_ptr(stream)), "onnx_conv2d_prepack")
         return packed

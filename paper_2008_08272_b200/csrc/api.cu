@@ -151,7 +151,9 @@ static onnxb_status conv2d_run_impl(onnxb_conv2d_desc_t d, const float *X, const
     const size_t wr_bytes = (size_t)d->g.M * d->g.C * 4;           // the gather family's rounded weights
     size_t need = d->workspace_bytes;
     if (d->family == ONNXB_KERNEL_MMA_GATHER_GEMM) need = pack_only ? wr_bytes : w_copy ? need - wr_bytes : need;
-    if (need > 0 && (!workspace || workspace_bytes < need)) return ONNXB_ERR_WORKSPACE;
+    // (the fp32 kernels have a form that needs none)
+    const bool fp32_tc = d->fp32_tc && workspace && workspace_bytes >= need;
+    if (need > 0 && (!workspace || workspace_bytes < need) && d->family != ONNXB_KERNEL_SIMT_DIRECT) return ONNXB_ERR_WORKSPACE;
     if (misaligned(X) || misaligned(W) || misaligned(B) || misaligned(Y) || misaligned(workspace))
         return ONNXB_ERR_UNSUPPORTED;
 
@@ -161,7 +163,9 @@ static onnxb_status conv2d_run_impl(onnxb_conv2d_desc_t d, const float *X, const
             err = launch_simt_depthwise(d->g, X, W, B, R, Y, cuda_stream);
             break;
         case ONNXB_KERNEL_SIMT_DIRECT:
-            err = launch_simt_conv(d->g, X, W, B, R, Y, cuda_stream);
+            err = !fp32_tc          ? launch_simt_conv(d->g, X, W, B, R, Y, cuda_stream)
+                  : d->fp32_tc == 1 ? launch_tc_fp32_conv(d->g, d->fp32, X, W, B, R, Y, workspace, cuda_stream, phase)
+                                    : launch_tc_fp32_conv1x1(d->g, d->fp32_gemm, X, W, B, R, Y, workspace, cuda_stream);
             break;
         case ONNXB_KERNEL_MMA_GEMM: {
             // the workspace holds W rounded to TF32 (made here, or earlier by onnx_conv2d_prepack)
@@ -209,15 +213,16 @@ extern "C" onnxb_status onnx_conv2d_add_run(onnxb_conv2d_desc_t d, const float *
 
 // Weights known ahead of the run (an inference graph's constants, Sec. 3.4.4): the implicit-GEMM
 // kernel's packing step done once, and run calls that take the packed copy instead of redoing it.
-// Which kernel families keep a derived copy of W in their scratch (packed and/or rounded to TF32).
-static bool family_has_weight_copy(int family) {
-    return family == ONNXB_KERNEL_MMA_IMPLICIT || family == ONNXB_KERNEL_MMA_GEMM || family == ONNXB_KERNEL_MMA_GATHER_GEMM;
+// Whether the kernel keeps a derived copy of W in its scratch (packed, rounded to TF32 or split into TF32 parts).
+static bool has_weight_copy(onnxb_conv2d_desc_t d) {
+    return d->family == ONNXB_KERNEL_MMA_IMPLICIT || d->family == ONNXB_KERNEL_MMA_GEMM || d->family == ONNXB_KERNEL_MMA_GATHER_GEMM ||
+           d->fp32_tc == 1;
 }
 
 extern "C" onnxb_status onnx_conv2d_prepack(onnxb_conv2d_desc_t d, const float *W, void *packed, size_t packed_bytes,
                                             void *cuda_stream) {
     if (!d || !W) return ONNXB_ERR_NULL;
-    if (!family_has_weight_copy(d->family)) return ONNXB_OK;              // the other kernels read W as it is
+    if (!has_weight_copy(d) || (d->fp32_tc == 1 && !packed)) return ONNXB_OK;  // the other kernels read W as it is
     // (the gather family's copy is only the rounded W, the leading part of its workspace)
     const size_t need = d->family == ONNXB_KERNEL_MMA_GATHER_GEMM ? (size_t)d->g.M * d->g.C * 4 : d->workspace_bytes;
     if (!packed || packed_bytes < need) return ONNXB_ERR_WORKSPACE;
@@ -228,7 +233,7 @@ extern "C" onnxb_status onnx_conv2d_run_prepacked(onnxb_conv2d_desc_t d, const f
                                                   const void *packed, const float *B, const float *R, float *Y,
                                                   void *workspace, size_t workspace_bytes, void *cuda_stream) {
     if (!d) return ONNXB_ERR_NULL;
-    if (!family_has_weight_copy(d->family))
+    if (!has_weight_copy(d) || (d->fp32_tc == 1 && !packed))
         return conv2d_run_impl(d, X, W, B, R, Y, workspace, workspace_bytes, cuda_stream);
     if (!packed) return ONNXB_ERR_NULL;
     if (d->family == ONNXB_KERNEL_MMA_GATHER_GEMM)      // the copy of W from `packed`, the gathered input in the workspace
@@ -251,7 +256,10 @@ static bool gemm_tc_eligible(int transA, int transB, int64_t M, int64_t N, int64
 
 extern "C" size_t onnx_gemm_workspace_bytes(int transA, int transB, int64_t M, int64_t N, int64_t K) {
     if (M < 1 || N < 1 || K < 1) return 0;
-    return gemm_tc_eligible(transA, transB, M, N, K) ? (size_t)(M * K + K * N) * 4 : 0;
+    if (gemm_tc_eligible(transA, transB, M, N, K)) return (size_t)(M * K + K * N) * 4;
+    const int64_t lim = 2147483647LL;
+    if (M > lim || N > lim || K > lim || M * K > lim || K * N > lim || M * N > lim) return 0;
+    return simt_gemm_workspace_bytes((int)M, (int)N, (int)K);
 }
 
 extern "C" onnxb_status onnx_gemm_run(int transA, int transB, float alpha, float beta, int64_t M, int64_t N,
@@ -309,7 +317,7 @@ extern "C" onnxb_status onnx_gemm_run(int transA, int transB, float alpha, float
     } else if (forced_tc) {
         return ONNXB_ERR_UNSUPPORTED;
     } else {
-        err = launch_simt_gemm(p, A, B, C, Y, cuda_stream);
+        err = launch_simt_gemm(p, A, B, C, Y, workspace, workspace_bytes, cuda_stream);
     }
     return err == 0 ? ONNXB_OK : ONNXB_ERR_CUDA;
 }

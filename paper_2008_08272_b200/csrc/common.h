@@ -20,12 +20,21 @@ struct ConvGeom {
     int has_bias, relu;
 };
 
+struct Fp32GemmPlan {        // tile width, and CTAs that share a tile's reduction (tc_fp32.cu)
+    int BN, split;
+};
+
 }  // namespace onnxb
 
 struct onnxb_conv2d_desc_s {
     onnxb::ConvGeom g;
     int family;              // onnxb_kernel_family
     onnxb::TcConvPlan plan;  // valid when family == ONNXB_KERNEL_MMA_IMPLICIT
+    // ONNXB_KERNEL_SIMT_DIRECT on the tensor cores where it is given workspace: 1 by the convolution plan below, 2 as a Gemm of
+    // packed pixels
+    int fp32_tc;
+    onnxb::Fp32ConvPlan fp32;
+    onnxb::Fp32GemmPlan fp32_gemm;
     size_t workspace_bytes;
     int64_t y_dims[4];
     int64_t pads[4];
@@ -42,6 +51,9 @@ int kernel_override();   // -1 = automatic
 // R (everywhere below): optional addend with Y's shape, added before Relu (a residual connection); may be NULL.
 int launch_simt_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                      void *stream);
+// Whether the convolution belongs on the tensor cores (fp32 by split operands, tc_fp32.cu), and its plan there: the
+// descriptor's fp32_tc.
+int simt_conv_on_tensor_cores(const ConvGeom &g, Fp32ConvPlan &plan, Fp32GemmPlan &gemm);
 int launch_simt_depthwise(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                           void *stream);
 double small_conv_cost(const ConvGeom &g);           // estimated SM cycles; negative: not for this problem
@@ -68,13 +80,21 @@ struct GemmProblem {
     int relu;
 };
 bool simt_gemm_is_tiny(long long M, long long N, long long K);   // small enough for the dot-product kernel
-int launch_simt_gemm(const GemmProblem &p, const float *A, const float *B, const float *C, float *Y,
-                     void *stream);
-// fp32 through split TF32 operands on the tensor cores (tc_fp32.cu): the same problems, once they are large
-double tc_fp32_cost(long long rows, int cols, int K, int groups, bool pixels);     // estimated SM cycles
-int launch_tc_fp32_gemm(const GemmProblem &p, const float *A, const float *B, const float *C, float *Y, void *stream);
-bool tc_fp32_conv_fits(const ConvGeom &g);
-int launch_tc_fp32_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
-                        void *stream);
+// Scratch with which a Gemm of the fp32 family runs on the tensor cores (0: it does not); without it runs on the FMA units.
+size_t simt_gemm_workspace_bytes(int M, int N, int K);
+int launch_simt_gemm(const GemmProblem &p, const float *A, const float *B, const float *C, float *Y, void *workspace,
+                     size_t workspace_bytes, void *stream);
+// fp32 through split TF32 operands on the tensor cores (tc_fp32.cu): the same problems, once they are large.  The
+// plans return their estimated SM cycles, the packing launch included for Gemm (negative: no plan).
+double tc_fp32_gemm_plan(int M, int N, int K, Fp32GemmPlan &plan);
+size_t tc_fp32_gemm_workspace(int M, int N, int K, const Fp32GemmPlan &plan);
+int launch_tc_fp32_gemm(const GemmProblem &p, const Fp32GemmPlan &plan, const float *A, const float *B, const float *C, float *Y,
+                        void *workspace, void *stream);
+int launch_tc_fp32_conv1x1(const ConvGeom &g, const Fp32GemmPlan &plan, const float *X, const float *W, const float *B, const float *R,
+                           float *Y, void *workspace, void *stream);
+double tc_fp32_conv_plan(const ConvGeom &g, Fp32ConvPlan &plan);
+size_t tc_fp32_conv_workspace(const Fp32ConvPlan &plan);
+int launch_tc_fp32_conv(const ConvGeom &g, const Fp32ConvPlan &plan, const float *X, const float *W, const float *B, const float *R,
+                        float *Y, void *packed, void *stream, int phase);
 
 }  // namespace onnxb

@@ -148,9 +148,12 @@ extern "C" onnxb_status onnx_conv2d_desc(const onnxb_conv2d_attrs *a, onnxb_conv
         family = ONNXB_KERNEL_MMA_IMPLICIT;
     }
     d->family = family;
+    d->fp32_tc = family == ONNXB_KERNEL_SIMT_DIRECT ? simt_conv_on_tensor_cores(g, d->fp32, d->fp32_gemm) : 0;
     d->workspace_bytes = family == ONNXB_KERNEL_MMA_IMPLICIT     ? tc_conv_workspace_bytes(d->plan)
                          : family == ONNXB_KERNEL_MMA_GATHER_GEMM ? conv_gather_workspace_bytes(g) + (size_t)g.M * g.C * 4
                          : family == ONNXB_KERNEL_MMA_GEMM        ? (size_t)g.M * g.C * 4      // W rounded to TF32
+                         : d->fp32_tc == 1                        ? tc_fp32_conv_workspace(d->fp32)  // W split
+                         : d->fp32_tc == 2                        ? tc_fp32_gemm_workspace(g.M, g.N * g.P * g.Q, g.C, d->fp32_gemm)
                                                                   : 0;
     *out = d;
     return ONNXB_OK;

@@ -432,33 +432,38 @@ Pick search_shape(int M, int N, int K, int groups, bool pixels) {
     return best;
 }
 
-// What a launch is: a tile shape and split, or the tensor-core kernel.  The search costs about 2 us of host
-// time, as much as the launch itself, so each thread remembers the choices of the last few problems.
+// What a launch of Gemm is: a tile shape and split, or the tensor-core kernel.  The search costs some 2 us of host
+// time, as much as the launch itself, so each thread remembers the choices of the last few problems.  ONNXB_FP32 = "tc"
+// pins the tensor-core kernel, any other value the FMA one.
 struct Choice {
     int M, N, K, groups, pixels;
     Pick pick;
-    double tc_cost;
+    Fp32GemmPlan plan;
     bool tc;
 };
-bool fp32_on_tensor_cores(double fma_cost, double tc_cost);
+// The split operands' own error does not grow with the reduction, the FMA kernel's chain of additions does: relative to the
+// result (2-norm, against 64 bits) split operands err by 1.2 to 1.4e-7 up to some 1000 terms, the FMA kernel by 1.1e-7 where a
+// CTA adds 35 terms, 1.5e-7 at 69, 2.1e-7 at 144.  So the tensor cores are for what an FMA kernel's CTA would add some 60 terms
+// of; and for large problems (15 us by FMA) of 56 terms and more, where there is twice the time to gain.
+bool tc_is_as_exact(long long K, const Pick &fma) { return K >= 64LL * fma.split - 8 || (K >= 56 && fma.cost > 30000.0); }
+
+constexpr double kGemmScale = 0.85;        // the tensor-core estimate runs high by this (18 problems: 0.75 to 0.9)
 Choice choose(int M, int N, int K, int groups, bool pixels) {
     thread_local Choice memo[64] = {};
-    const bool pinned = getenv("ONNXB_FP32") != nullptr;
+    const char *pin = getenv("ONNXB_FP32");
     const unsigned h = ((unsigned)M * 2654435761u ^ (unsigned)N * 2246822519u ^ (unsigned)K * 3266489917u ^ (unsigned)groups * 668265263u ^
                         (unsigned)pixels) >> 7;
     Choice &c = memo[h % 64];
-    if (!pinned && c.M == M && c.N == N && c.K == K && c.groups == groups && c.pixels == (int)pixels) return c;
-    // (rows and columns change places there: its rows are the index contiguous in Y)
-    Choice r{M, N, K, groups, (int)pixels, search_shape(M, N, K, groups, pixels), tc_fp32_cost(N, M, K, groups, pixels), false};
-    r.tc = fp32_on_tensor_cores(r.pick.cost, r.tc_cost);
-    if (!pinned) c = r;
+    if (!pin && c.M == M && c.N == N && c.K == K && c.groups == groups && c.pixels == (int)pixels) return c;
+    Choice r{M, N, K, groups, (int)pixels, search_shape(M, N, K, groups, pixels), {0, 0}, false};
+    if (!pixels) {
+        const double tc = tc_fp32_gemm_plan(M, N, K, r.plan);
+        // (the packed copies are addressed in 32 bits of 16-byte pieces)
+        const bool fits = tc >= 0 && tc_fp32_gemm_workspace(M, N, K, r.plan) < (1ull << 33);
+        r.tc = fits && (pin ? pin[0] == 't' : kGemmScale * tc < r.pick.cost && tc_is_as_exact(K, r.pick));
+    }
+    if (!pin) c = r;
     return r;
-}
-
-// Large problems go to the split-TF32 tensor-core kernel, by the two estimates; ONNXB_FP32 = "tc" pins it.
-bool fp32_on_tensor_cores(double fma_cost, double tc_cost) {
-    if (const char *pin = getenv("ONNXB_FP32")) return pin[0] == 't';
-    return tc_cost < fma_cost;
 }
 
 template <int AM, int BMODE>
@@ -485,8 +490,8 @@ int launch_sgemm(SgemmArgs &a, int groups, const Pick &pick, cudaStream_t st) {
 // Up to this size the dot-product kernel beats any tiled launch (64 x 10 x 256: one launch of about 3 us).
 bool simt_gemm_is_tiny(long long M, long long N, long long K) { return M * N <= 4096 && M * N * K <= (1 << 20); }
 
-int launch_simt_gemm(const GemmProblem &p, const float *A, const float *B, const float *C, float *Y,
-                     void *stream) {
+int launch_simt_gemm(const GemmProblem &p, const float *A, const float *B, const float *C, float *Y, void *workspace,
+                     size_t workspace_bytes, void *stream) {
     SgemmArgs a{};
     a.A = A; a.B = B; a.Y = Y; a.M = p.M; a.N = p.N; a.K = p.K;
     a.a_ld = p.transA ? p.M : p.K;
@@ -502,10 +507,35 @@ int launch_simt_gemm(const GemmProblem &p, const float *A, const float *B, const
     }
     const Choice ch = choose(a.M, a.N, a.K, 1, false);
     const Pick pick = ch.pick;
-    if (ch.tc) return launch_tc_fp32_gemm(p, A, B, C, Y, stream);
+    if (ch.tc && workspace && workspace_bytes > 0 && workspace_bytes >= tc_fp32_gemm_workspace(p.M, p.N, p.K, ch.plan))
+        return launch_tc_fp32_gemm(p, ch.plan, A, B, C, Y, workspace, stream);
     if (p.transA)
         return p.transB ? launch_sgemm<kMnContig, kKContig>(a, 1, pick, st) : launch_sgemm<kMnContig, kMnContig>(a, 1, pick, st);
     return p.transB ? launch_sgemm<kKContig, kKContig>(a, 1, pick, st) : launch_sgemm<kKContig, kMnContig>(a, 1, pick, st);
+}
+
+size_t simt_gemm_workspace_bytes(int M, int N, int K) {
+    if ((long long)M * N * K < 2000000) return 0;              // (never on the tensor cores, and a call that short notices the search)
+    const Choice c = choose(M, N, K, 1, false);
+    return c.tc ? tc_fp32_gemm_workspace(M, N, K, c.plan) : 0;
+}
+
+// By the estimates: the small-image kernel's (the tiled ones run low where it applies), the FMA kernel's and the tensor-core
+// kernel's, where a 1x1 convolution, which has no taps to share a staged pixel, goes by packed pixels (2011 -> 1280 channels
+// 23x23, batch 3: 220 us staged, 58 packed, 134 by the im2col of 4-byte loads that both replace).  ONNXB_FP32 as above.
+int simt_conv_on_tensor_cores(const ConvGeom &g, Fp32ConvPlan &plan, Fp32GemmPlan &gemm) {
+    const char *pin = getenv("ONNXB_FP32");
+    if (pin && pin[0] != 't') return 0;
+    const long long pixels = (long long)g.N * g.P * g.Q, K = (long long)g.Cg * g.kH * g.kW;      // (each below 2^31)
+    const bool flat = g.kH == 1 && g.kW == 1 && g.group == 1 && !(g.pt | g.pl | g.pb | g.pr);
+    const double tc = flat ? kGemmScale * tc_fp32_gemm_plan(g.M, (int)pixels, g.C, gemm) : tc_fp32_conv_plan(g, plan);
+    if (tc < 0 || (flat && tc_fp32_gemm_workspace(g.M, (int)pixels, g.C, gemm) >= (1ull << 33))) return 0;
+    if (!pin) {
+        const double small = small_conv_cost(g);
+        const Pick fma = search_shape(g.Mg, (int)pixels, (int)K, g.group, true);
+        if (tc >= fma.cost || (small >= 0 && 0.85 * small < tc) || !tc_is_as_exact(K, fma)) return 0;
+    }
+    return flat ? 2 : 1;
 }
 
 int launch_simt_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
@@ -524,9 +554,8 @@ int launch_simt_conv(const ConvGeom &g, const float *X, const float *W, const fl
     const Pick pick = ch.pick;
     const double small = small_conv_cost(g);
     const char *pin = getenv("ONNXB_FP32");              // "small" pins the small-image kernel
-    if (small >= 0 && (pin ? pin[0] == 's' : 0.85 * small < std::min(ch.pick.cost, ch.tc_cost)))      // (the tiled estimates run low here)
+    if (small >= 0 && (pin ? pin[0] == 's' : 0.85 * small < ch.pick.cost))      // (the tiled estimate runs low here)
         return launch_small_conv(g, X, W, B, R, Y, stream);
-    if (ch.tc && tc_fp32_conv_fits(g)) return launch_tc_fp32_conv(g, X, W, B, R, Y, stream);
     return launch_sgemm<kKContig, kPixels>(a, g.group, pick, (cudaStream_t)stream);
 }
 

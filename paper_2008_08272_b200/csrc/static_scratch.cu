@@ -42,7 +42,8 @@ extern "C" size_t onnx_conv2d_static_scratch_bytes(void) { return kStaticScratch
 extern "C" onnxb_status onnx_conv2d_run_static(onnxb_conv2d_desc_t d, const float *X, const float *W,
                                                const float *B, float *Y, void *cuda_stream) {
     if (!d) return ONNXB_ERR_NULL;
-    if (d->workspace_bytes == 0)   // this descriptor's kernel needs no scratch at all
+    // this descriptor's kernel needs no scratch at all, or has a form that needs none
+    if (d->workspace_bytes == 0 || (d->fp32_tc && d->workspace_bytes > kStaticScratchBytes))
         return onnx_conv2d_run(d, X, W, B, Y, nullptr, 0, cuda_stream);
     if (d->workspace_bytes > kStaticScratchBytes) return ONNXB_ERR_WORKSPACE;
     void *scratch = static_scratch_ptr();

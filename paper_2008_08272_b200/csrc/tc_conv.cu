@@ -794,40 +794,6 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
 }
 
 // ------------------------------------------------------------------ planning (host)
-struct Axis {
-    int E, Amax, npar, par[kConvMaxPlanes];
-};
-
-// Slot extent along one axis: input size I, output size O, leading pad, stride s, dilation d, kernel k.
-bool plan_axis(int I, int O, int pad, int s, int d, int k, Axis &ax) {
-    int offmax[64];
-    bool used[64];
-    if (s > 64) return false;
-    for (int a = 0; a < s; ++a) { used[a] = false; offmax[a] = 0; }
-    ax.Amax = 0;
-    for (int t = 0; t < k; ++t) {
-        const int a = (t * d) % s, o = (t * d) / s;
-        used[a] = true;
-        offmax[a] = std::max(offmax[a], o);
-        ax.Amax = std::max(ax.Amax, o);
-    }
-    ax.npar = 0;
-    int a_min = -1;
-    long long e = O;
-    for (int a = 0; a < s; ++a) {
-        if (!used[a]) continue;
-        if (ax.npar == kConvMaxPlanes) return false;
-        ax.par[ax.npar++] = a;
-        if (a_min < 0) a_min = a;
-        const int z = pad > a ? (pad - a + s - 1) / s : 0;         // leading zero slots of this parity
-        e = std::max<long long>(e, (long long)O + offmax[a] - z);
-    }
-    e = std::max<long long>(e, ((long long)I + pad - a_min + s - 1) / s);
-    e = std::min<long long>(e, (long long)O + ax.Amax);
-    ax.E = (int)e;
-    return true;
-}
-
 int pick_conv_bn(int Mg) {
     if (Mg <= 256) return (Mg + 15) / 16 * 16;
     int best = 256, best_pad = 1 << 30;
@@ -849,9 +815,9 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     g.sh = c.sh; g.sw = c.sw; g.dh = c.dh; g.dw = c.dw; g.group = c.group; g.relu = c.relu;
     g.taps = c.kH * c.kW;
     if (g.taps > kConvMaxTaps) return false;
-    Axis ah, aw;
-    if (!plan_axis(c.H, c.P, c.pt, c.sh, c.dh, c.kH, ah)) return false;
-    if (!plan_axis(c.W, c.Q, c.pl, c.sw, c.dw, c.kW, aw)) return false;
+    ConvAxis ah, aw;
+    if (!conv_plan_axis(c.H, c.P, c.pt, c.sh, c.dh, c.kH, ah)) return false;
+    if (!conv_plan_axis(c.W, c.Q, c.pl, c.sw, c.dw, c.kW, aw)) return false;
     if (ah.npar * aw.npar > kConvMaxPlanes) return false;
     g.Hs = ah.E; g.Ws = aw.E;
     const long long L = (long long)g.Hs * g.Ws;

@@ -11,6 +11,7 @@
 // address.  Hs and Ws are chosen as small as possible: the trailing zero padding of one
 // row (image) is allowed to alias the leading zero padding of the next.
 #pragma once
+#include <algorithm>
 #include <cstdint>
 
 #if defined(__CUDACC__)
@@ -100,6 +101,88 @@ inline ConvDivisor conv_divisor(int d) {
     dv.s1 = l < 1 ? (uint32_t)l : 1u;
     dv.s2 = l > 1 ? (uint32_t)(l - 1) : 0u;
     return dv;
+}
+
+struct ConvAxis {
+    int E, Amax, npar, par[kConvMaxPlanes];
+};
+
+// Slot extent along one axis: input size I, output size O, leading pad, stride s, dilation d, kernel k.
+inline bool conv_plan_axis(int I, int O, int pad, int s, int d, int k, ConvAxis &ax) {
+    int offmax[64];
+    bool used[64];
+    if (s > 64) return false;
+    for (int a = 0; a < s; ++a) { used[a] = false; offmax[a] = 0; }
+    ax.Amax = 0;
+    for (int t = 0; t < k; ++t) {
+        const int a = (t * d) % s, o = (t * d) / s;
+        used[a] = true;
+        offmax[a] = std::max(offmax[a], o);
+        ax.Amax = std::max(ax.Amax, o);
+    }
+    ax.npar = 0;
+    int a_min = -1;
+    long long e = O;
+    for (int a = 0; a < s; ++a) {
+        if (!used[a]) continue;
+        if (ax.npar == kConvMaxPlanes) return false;
+        ax.par[ax.npar++] = a;
+        if (a_min < 0) a_min = a;
+        const int z = pad > a ? (pad - a + s - 1) / s : 0;         // leading zero slots of this parity
+        e = std::max<long long>(e, (long long)O + offmax[a] - z);
+    }
+    e = std::max<long long>(e, ((long long)I + pad - a_min + s - 1) / s);
+    e = std::min<long long>(e, (long long)O + ax.Amax);
+    ax.E = (int)e;
+    return true;
+}
+
+// Plan of the fp32 kernel (tc_fp32.cu): the same slot space, a tile is 128 consecutive slots and their halo.
+constexpr int kFp32MaxPlanes = 16, kFp32MaxSteps = 128, kFp32MaxSeg = 8;
+struct Fp32ConvPlan {
+    int N, C, H, W, M, Cg, Mg, kW, P, Q, pt, pl, sh, sw, dh, dw, group, taps;
+    int Hs, Ws, L, planes, SLOTS;        // slots per image; parity planes; slots of a plane in a stage
+    int a_min, a_max;                    // smallest / largest used row parity
+    int tiles_r, per_image;              // pixel tiles; of each image, or 0 where a tile may hold parts of several
+    int pitch;                           // floats from one channel's staged rows to the next's, congruent to H*W modulo 4
+    short pa[kFp32MaxPlanes], pb[kFp32MaxPlanes];
+    int nch, ncb;                        // four-channel chunks per block, blocks
+    int n_steps, n_groups, spg;          // K-steps of a block, and the partial sums they form
+    int BN, tiles_c, split;
+    uint32_t step_a[kFp32MaxSteps];      // slot of the step's first chunk in the stage | distance of its second << 16
+    short src_tap[kFp32MaxSteps][2], src_c0[kFp32MaxSteps][2];
+    ConvDivisor dv_L, dv_Ws, dv_slots, dv_SLOTS, dv_per_image;
+};
+// First slot of a pixel tile.
+ONNXB_HD inline int fp32_conv_first_slot(const Fp32ConvPlan &g, int rt) {
+    if (!g.per_image) return rt * 128;
+    const int n = conv_fdiv(rt, g.per_image, g.dv_per_image);
+    return n * g.L + (rt - n * g.per_image) * 128;
+}
+// The rows of the images that a tile's slots lie in: where each image's begin in X's plane and in a channel's staged rows.
+struct Fp32ConvSegs {
+    int n_first, nseg;
+    int f0[kFp32MaxSeg], len[kFp32MaxSeg], at[kFp32MaxSeg];
+};
+ONNXB_HD inline void fp32_conv_segments(const Fp32ConvPlan &g, int rt, int grp, Fp32ConvSegs &t) {
+    const long long G0 = fp32_conv_first_slot(g, rt), all = (long long)g.N * g.L, end = G0 + g.SLOTS < all ? G0 + g.SLOTS : all;
+    t.n_first = conv_fdiv((int)G0, g.L, g.dv_L);
+    t.nseg = conv_fdiv((int)(end - 1), g.L, g.dv_L) - t.n_first + 1;
+    int at = 4;                          // (a later channel's first copy may start up to three elements before its row)
+    for (int i = 0; i < t.nseg; ++i) {
+        const long long base = (long long)(t.n_first + i) * g.L;
+        const int lo = (int)(G0 > base ? G0 - base : 0), hi = (int)(end < base + g.L ? end - base : g.L);      // [lo, hi)
+        int h0 = conv_fdiv(lo, g.Ws, g.dv_Ws) * g.sh + g.a_min - g.pt, h1 = conv_fdiv(hi - 1, g.Ws, g.dv_Ws) * g.sh + g.a_max - g.pt;
+        if (h0 < 0) h0 = 0;
+        if (h1 > g.H - 1) h1 = g.H - 1;
+        t.f0[i] = h0 * g.W;
+        t.len[i] = h0 <= h1 ? (h1 - h0 + 1) * g.W : 0;
+        // as far from a 16-byte boundary as in X (the pitch keeps that for every channel), and clear of what the copy before,
+        // in whole 16-byte pieces, may write
+        const int e = ((t.n_first + i) * g.C + grp * g.Cg) * g.H * g.W + t.f0[i];
+        t.at[i] = (at + 3) / 4 * 4 + (e & 3);
+        at = t.at[i] + t.len[i] + 3;
+    }
 }
 
 struct TcConvSegs {
