@@ -645,11 +645,46 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             const int grp = ct_all / g.ctiles, ct = ct_all % g.ctiles;
             const long long G0 = ((t / cgt) * kCtas + rank) * tile_rows;
             const uint32_t ab = acc_dbl ? (it & 1u) : 0u, use = acc_dbl ? (it >> 1) : it;
+            const int nch = (g.BN + 31) / 32;
+            // eight warps: two per TMEM lane quarter, each taking half of the tile
+            const int hf = ew >> 2, mt = two ? hf : 0;
+            const int ch_lo = two ? 0 : hf ? (nch + 1) / 2 : 0, ch_hi = two || hf ? nch : (nch + 1) / 2;
+            const uint32_t PQ4 = (uint32_t)g.P * (uint32_t)g.Q * 4u;
+            bool valid = false;
+            uint32_t off = 0;                          // bytes from Y (and R): the launch keeps them below 2^32
+            if (it == 0) pdl_wait();
+            if (!kSplit) {
+                // What does not depend on the accumulators is fetched while they are being summed: the outputs' places, the first
+                // biases and, below, the first addends (each a trip to L2, next to no L1 being left).
+                const uint32_t G = (uint32_t)G0 + (uint32_t)(mt * 128 + quarter * 32 + lane);
+                valid = G < (uint32_t)g.total_slots;
+                if (valid) {
+                    const int n = conv_fdiv((int)G, g.L, g.dv_L), u = (int)G - n * g.L;
+                    const int p = conv_fdiv(u, g.Ws, g.dv_Ws), q = u - p * g.Ws;
+                    valid = p < g.P && q < g.Q;
+                    off = (uint32_t)(n * g.M + grp * g.Mg + ct * g.BN + ch_lo * 32) * PQ4 + (uint32_t)(p * g.Q + q) * 4u;
+                }
+            }
+            const char *rb = reinterpret_cast<const char *>(R);
+            const int tile_left = min(g.Mg - ct * g.BN, g.BN);         // channels of the tile
+            float b_next = 0.f, r[2][8];
+            auto fetch_bias = [&](int chunk) {
+                const int c = chunk * 32 + lane;
+                b_next = bias && chunk < ch_hi && c < tile_left ? __ldg(bias + grp * g.Mg + ct * g.BN + c) : 0.f;
+            };
+            // addends (at Y's own positions) of the eight channels `ahead` of those that `off` has come to, `left` of which exist
+            auto fetch_add = [&](float (&to)[8], int ahead, int left) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    to[j] = valid && ahead + j < left ? __ldg(reinterpret_cast<const float *>(rb + (off + (uint32_t)(ahead + j) * PQ4))) : 0.f;
+            };
+            if (!kSplit) {
+                fetch_bias(ch_lo);
+                if (kAdd) fetch_add(r[0], 0, min(tile_left, ch_hi * 32) - ch_lo * 32);
+            }
             mbar_wait(&bars->acc_full[ab], use & 1u, err, 18);
             tc_fence_after_sync();
-            if (it == 0) pdl_wait();        // long since satisfied: the producers passed theirs before the first load
             if (ew == 0 && lane == 0) LOG(8, 2);
-            const int nch = (g.BN + 31) / 32;
             if (kSplit) {
                 // every group of four channels goes to the CTA that finishes it, as [source CTA][group][pixel][4]:
                 // the lanes of a store write consecutive 16-byte pieces
@@ -671,22 +706,8 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                 }
             }
             if (!kSplit) {
-                // eight warps: two per TMEM lane quarter, each taking half of the tile
-                const int hf = ew >> 2, mt = two ? hf : 0;
-                const int ch_lo = two ? 0 : hf ? (nch + 1) / 2 : 0, ch_hi = two || hf ? nch : (nch + 1) / 2;
                 const uint32_t acc_col = ab * 256u + (uint32_t)mt * mt_cols;
-                const uint32_t G = (uint32_t)G0 + (uint32_t)(mt * 128 + quarter * 32 + lane);
-                const uint32_t PQ4 = (uint32_t)g.P * (uint32_t)g.Q * 4u;
-                bool valid = G < (uint32_t)g.total_slots;
-                uint32_t off = 0;                      // bytes from Y (and R): the launch keeps them below 2^32
-                if (valid) {
-                    const int n = conv_fdiv((int)G, g.L, g.dv_L), u = (int)G - n * g.L;
-                    const int p = conv_fdiv(u, g.Ws, g.dv_Ws), q = u - p * g.Ws;
-                    valid = p < g.P && q < g.Q;
-                    off = (uint32_t)(n * g.M + grp * g.Mg + ct * g.BN + ch_lo * 32) * PQ4 + (uint32_t)(p * g.Q + q) * 4u;
-                }
                 char *yb = reinterpret_cast<char *>(Y);
-                const char *rb = reinterpret_cast<const char *>(R);
                 // fmaxf returns its other argument where one is NaN, and NaN where both are: without Relu nothing is changed.
                 // (The constant is hidden from the compiler, which would otherwise choose between x and fmaxf(x, 0) for every
                 // output; that took the form with an addend from 145 to 185 us on a 3 -> 64, 7x7/2, 224x224 layer, batch 32.)
@@ -699,17 +720,13 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                     const int cnt = min(g.Mg, (ct + 1) * g.BN) - mg0;      // channels of the chunk that exist (above 32: all)
                     // the chunk's biases through shared memory: eight 16-byte broadcasts instead of 32 shuffles
                     __syncwarp();
-                    bias_w[lane] = bias && lane < cnt ? __ldg(bias + grp * g.Mg + mg0 + lane) : 0.f;
+                    bias_w[lane] = b_next;
                     __syncwarp();
+                    fetch_bias(chunk + 1);
                     tmem_ld_wait();
 #pragma unroll
                     for (int j0 = 0; j0 < 32; j0 += 8) {
-                        float r[8];
-                        if (kAdd) {                                        // residual addend at Y's own position
-#pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                r[j] = valid && j0 + j < cnt ? __ldg(reinterpret_cast<const float *>(rb + (off + (uint32_t)j * PQ4))) : 0.f;
-                        }
+                        if (kAdd) fetch_add(r[(j0 >> 3) + 1 & 1], 8, min(tile_left, ch_hi * 32) - chunk * 32 - j0);
 #pragma unroll
                         for (int j = 0; j < 8; j += 4) {
                             const float4 b4 = *reinterpret_cast<const float4 *>(bias_w + j0 + j);
@@ -717,7 +734,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 float x = __uint_as_float(v[j0 + j + e]) + b[e];
-                                if (kAdd) x += r[j + e];
+                                if (kAdd) x += r[(j0 >> 3) & 1][j + e];
                                 x = fmaxf(x, lowest);
                                 if (valid && j0 + j + e < cnt) *reinterpret_cast<float *>(yb + off) = x;
                                 off += PQ4;
