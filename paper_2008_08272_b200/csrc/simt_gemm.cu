@@ -441,11 +441,20 @@ struct Choice {
     Fp32GemmPlan plan;
     bool tc;
 };
-// The split operands' own error does not grow with the reduction, the FMA kernel's chain of additions does: relative to the
-// result (2-norm, against 64 bits) split operands err by 1.2 to 1.4e-7 up to some 1000 terms, the FMA kernel by 1.1e-7 where a
-// CTA adds 35 terms, 1.5e-7 at 69, 2.1e-7 at 144.  So the tensor cores are for what an FMA kernel's CTA would add some 60 terms
-// of; and for large problems (15 us by FMA) of 56 terms and more, where there is twice the time to gain.
-bool tc_is_as_exact(long long K, const Pick &fma) { return K >= 64LL * fma.split - 8 || (K >= 56 && fma.cost > 30000.0); }
+// Whether a problem may go to the tensor cores, faster there or not.  The split operands' own error does not grow with the
+// reduction, the FMA kernel's chain of additions does: relative to the result (2-norm, against 64 bits) split operands err by
+// 1.2 to 1.4e-7 up to some 1000 terms, the FMA kernel by 1.1e-7 where a CTA adds 35 terms, 1.5e-7 at 69, 2.1e-7 at 144.  So
+// the tensor cores are for what an FMA kernel's CTA would add some 60 terms of; and, with fewer, for problems of much work per
+// output tile (12,000 cycles' worth: 563 x 3424 x 27 16.5 us by FMA, 10 there; 5230 x 5956 x 33 stays).
+bool tc_is_as_exact(int M, int N, long long K, int groups, bool pixels, const Pick &fma) {
+    if (K >= 64LL * fma.split - 8) return true;
+    for (int bn = 16; bn <= 128 && bn <= (M + 15) / 16 * 16; bn += 16) {
+        const long long tiles = (N + 127LL) / 128 * ((M + bn - 1) / bn) * groups;
+        const double blk = pixels ? 2120.0 + 8.0 * bn : 1750.0 + 5.0 * bn;
+        if ((double)((tiles + 147) / 148) * ((double)((K + 31) / 32) * blk + 12000.0) + 4500.0 < fma.cost) return true;
+    }
+    return false;
+}
 
 constexpr double kGemmScale = 0.85;        // the tensor-core estimate runs high by this (18 problems: 0.75 to 0.9)
 Choice choose(int M, int N, int K, int groups, bool pixels) {
@@ -460,7 +469,7 @@ Choice choose(int M, int N, int K, int groups, bool pixels) {
         const double tc = tc_fp32_gemm_plan(M, N, K, r.plan);
         // (the packed copies are addressed in 32 bits of 16-byte pieces)
         const bool fits = tc >= 0 && tc_fp32_gemm_workspace(M, N, K, r.plan) < (1ull << 33);
-        r.tc = fits && (pin ? pin[0] == 't' : kGemmScale * tc < r.pick.cost && tc_is_as_exact(K, r.pick));
+        r.tc = fits && (pin ? pin[0] == 't' : kGemmScale * tc < r.pick.cost && tc_is_as_exact(M, N, K, 1, false, r.pick));
     }
     if (!pin) c = r;
     return r;
@@ -533,7 +542,7 @@ int simt_conv_on_tensor_cores(const ConvGeom &g, Fp32ConvPlan &plan, Fp32GemmPla
     if (!pin) {
         const double small = small_conv_cost(g);
         const Pick fma = search_shape(g.Mg, (int)pixels, (int)K, g.group, true);
-        if (tc >= fma.cost || (small >= 0 && 0.85 * small < tc) || !tc_is_as_exact(K, fma)) return 0;
+        if (tc >= fma.cost || (small >= 0 && 0.85 * small < tc) || !tc_is_as_exact(g.Mg, (int)pixels, K, g.group, true, fma)) return 0;
     }
     return flat ? 2 : 1;
 }
