@@ -295,7 +295,7 @@ extern "C" onnxb_status onnx_gemm_run(int transA, int transB, float alpha, float
     t.A = A; t.B = B;
     t.a_mn_major = p.transA; t.a_ld = p.transA ? p.M : p.K;
     t.b_mn_major = !p.transB; t.b_ld = p.transB ? p.K : p.N;
-    t.alpha = alpha; t.beta = beta; t.C = C; t.c_si = p.c_stride_i; t.c_sj = p.c_stride_j; t.c_sb = 0;
+    t.alpha = alpha; t.beta = beta; t.C = C; t.c_si = p.c_stride_i; t.c_sj = p.c_stride_j;
     t.row_bias = nullptr; t.relu = p.relu; t.round_operands = 1;
     t.Y = Y; t.y_ld = p.N; t.y_bs = 0;
     const int forced = kernel_override();

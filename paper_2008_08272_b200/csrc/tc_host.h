@@ -20,7 +20,7 @@ struct TcGemmProblem {
     int a_batched, b_batched;
     float alpha, beta;
     const float *C;
-    long long c_si, c_sj, c_sb;
+    long long c_si, c_sj;
     const float *row_bias;
     const float *residual;   // optional addend with Y's own layout, added before Relu (ignored when C is given)
     int relu;

@@ -86,3 +86,17 @@ def test_depthwise_streamed_planes(binding, xs, pads):
     images = [0, xs[0] // 2, xs[0] - 1]
     ratio, family = check_conv(binding, torch, X, W, B, relu=True, pads=pads, group=xs[1], images=images)
     assert family == "simt_depthwise" and ratio <= 1.0
+
+
+@pytest.mark.parametrize("cs", [(), (1,), ("N",), (1, "N"), ("M", 1), ("M", "N")], ids=str)
+def test_gemm_addend_forms(binding, cs, monkeypatch):
+    """C of every broadcast form in the persistent kernel's epilogue, where Y goes out by TMA and where it does not (rows that
+    are no multiples of 16 bytes), on tiles that end inside a block of rows and of columns."""
+    monkeypatch.setenv("ONNXB_GEMM_SPLITK", "0")
+    rng = np.random.default_rng(2)
+    for M, N, K in ((300, 332, 96), (300, 330, 96), (20, 37, 64)):
+        A, B = rng.standard_normal((M, K)).astype(np.float32), rng.standard_normal((N, K)).astype(np.float32)
+        C = rng.standard_normal([{"M": M, "N": N}.get(d, d) for d in cs]).astype(np.float32)
+        got = run_gemm_gpu(binding, torch, A, B, C, transB=True, alpha=0.5, beta=-1.5, fuse_relu=True)
+        want, S = oracle.gemm(A, B, C, transB=True, alpha=0.5, beta=-1.5, relu=True)
+        assert worst_ratio(got, want, S) <= 1.0, (M, N)
