@@ -188,6 +188,13 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *m, const void *s
                  ::"l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(src)), "r"(c0), "r"(c1), "r"(c2)
                  : "memory");
 }
+// *p where i < n, else 0 (volatile: issued where it stands among other such instructions)
+__device__ __forceinline__ float ldg_where(const void *p, int i, int n) {
+    float v;
+    asm volatile("{\n.reg .pred w;\nsetp.lt.s32 w, %2, %3;\nmov.f32 %0, 0f00000000;\n@w ld.global.nc.f32 %0, [%1];\n}" : "=f"(v) : "l"(p), "r"(i), "r"(n));
+    return v;
+}
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 // plain (untiled) bulk copy global -> shared; both addresses 16-byte aligned, size a multiple of 16
 __device__ __forceinline__ void bulk_load_1d(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
     asm volatile(

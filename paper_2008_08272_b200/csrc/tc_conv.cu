@@ -45,7 +45,7 @@ namespace {
 using namespace tc;
 
 // Warps: raw producer, weight producer, MMA issuer, relay, then 12 transform warps and 8 epilogue warps: 768 threads,
-// 80 registers each.  The forms of the kernel below stay within them without a spill (one with an addend has two words),
+// 80 registers each.  The forms of the kernel below stay within them without a spill (those with an addend have one to three words),
 // on purpose: with 227 KB of shared memory per CTA next to no L1 is left, and a value spilled in a transform loop is a
 // trip to L2 (40 to 90 bytes of spills, while the loops were being written, cost 7 of 51 us on the 64-channel 56x56
 // layer at batch 64, 23 of 101 on the 7x7/2 first layer).
@@ -65,6 +65,8 @@ constexpr int kBarBytes = 512;
 constexpr int kSegBytes = 256;             // >= sizeof(TcConvSegs)
 constexpr int kBiasBytes = 8 * 128;        // 32 biases per epilogue warp
 static_assert(sizeof(TcConvSegs) <= kSegBytes, "segment table does not fit its slot");
+
+enum { kNoAddend, kAddendNear, kAddendFar };
 
 struct Bars {
     uint64_t raw_full[kMaxRawStages], raw_empty[kMaxRawStages], a_full[kMaxAStages], a_empty[kMaxAStages];
@@ -124,8 +126,9 @@ __host__ __device__ constexpr uint32_t split_tmem_cols(int BN) { return BN <= 12
 __host__ __device__ constexpr int split_recv_bytes(int split, int cols_per) { return split * cols_per * 512; }
 
 // ------------------------------------------------------------------ main kernel
-// kAdd: the epilogue also adds a tensor laid out like Y (a residual connection) before the Relu.  A
-// separate instantiation, so that the plain kernel's register allocation is not disturbed.
+// kAddend: the epilogue also adds a tensor laid out like Y (a residual connection) before the Relu; kAddendFar asks for it ahead
+// of time.  Separate instantiations, so that one form's register allocation and instruction schedule do not disturb another's
+// (the code that asks ahead, present but not executed, cost others of the layers with an addend up to 13 %).
 // kSplit: the problem has few tiles, so a cluster of g.split CTAs shares one: CTA r reduces the channel blocks
 // [r * cb_per, (r + 1) * cb_per) and finishes one slice of the tile's channels.  The epilogue warps write each partial
 // sum from TMEM straight into the shared memory of the CTA that finishes it (st.async, counted on an mbarrier there);
@@ -134,12 +137,16 @@ __host__ __device__ constexpr int split_recv_bytes(int split, int cols_per) { re
 // the peers' partial tiles between two cluster barriers took 2,200 more).  One 14x14 image, 256 -> 256 channels: 24 us
 // unsplit, 8.6 split over 8; 28x28, 128 channels 15.7 -> 8.3.
 // kThin: blocks of one 4-channel chunk (tap pairs).
-template <int kCtas, bool kAdd, bool kThin, bool kSplit>
+template <int kCtas, int kAddend, bool kThin, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, const float *__restrict__ X,
                const float *__restrict__ Wpk, const float *__restrict__ bias, const float *__restrict__ R,
                float *__restrict__ Y, unsigned int *err) {
     constexpr int kOwned = kThin ? kOwnedThin : kOwnedThick;
+    constexpr bool kAdd = kAddend != kNoAddend, kLinear = kThin && kAddend != kAddendNear;
+    // may stage rows (raw_mode 2): the thin ones; but the schedule that the compiler finds for those with an addend, whose epilogue has
+    // no register to spare, is the better one with that code in place (64 -> 64 3x3 56x56 batch 32 23.8 against 25.3 us)
+    constexpr bool kRows = kThin || kAdd;
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment by pointer arithmetic on the shared array itself, so that the compiler
     // keeps treating everything derived from it as shared memory (LDS/STS, not generic accesses)
@@ -279,6 +286,17 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                             float *d = dst + segs->base[i];
                             for (int j = 0; j < nbox; ++j)
                                 tma_load_2d(d + j * box_floats, &tmX, &bars->raw_full[rs], f0 + j * g.BOXP, plane0);
+                        }
+                    } else if (kRows && g.raw_mode == 2) {
+                        // the rows of every channel that exists, one copy each
+                        const int chans = min(KB, g.Cg - cbx * KB);
+                        mbar_arrive_expect_tx(&bars->raw_full[rs], (uint32_t)chans * tile_bytes);
+                        for (int i = 0; i < nseg; ++i) {
+                            const uint32_t bytes = (uint32_t)segs->nbox[i] * 4u;
+                            const float *x = X + ((long long)(segs->n_first + i) * g.C + c0) * HW + segs->f0[i];
+                            float *d = dst + segs->base[i];
+                            if (bytes)
+                                for (int c = 0; c < chans; ++c) bulk_load_1d(d + c * g.BOXP, x + c * HW, bytes, &bars->raw_full[rs]);
                         }
                     } else {
                         // whole-image slabs [channel][H*W]; clip at the end of X
@@ -470,29 +488,32 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
         const uint32_t a_full_addr = kCtas == 2 ? map_to_cta(smem_u32(&bars->a_full[0]), 0) : 0u;
         // What does not depend on the tile is worked out once: where a unit's operand row goes, and
         // which slot of which parity plane it reads.
-        uint32_t udst[kOwned];                     // byte offset of the unit's operand row inside an A stage | chunk group
-        uint32_t ujp[kOwned];                      // slot rows << 12 | slot columns from the tile's first slot
+        uint32_t udst[kOwned];                     // byte offset of the unit's operand row inside an A stage | chunk group (thin: just xt * 16, and on from there)
+        uint32_t ujp[kOwned];                      // slot columns << 16 | slot rows from the tile's first slot (rows << 12 | columns where no rule below compares them)
         uint32_t upix[kOwned];                     // the same distance in pixels, the plane's and the padding's share added: rows << 16 | columns (signed)
+        int ulin[kLinear ? kOwned : 1];              // and as one number, rows * W + columns
 #pragma unroll
         for (int i = 0; i < kOwned; ++i) {
-            udst[i] = 0;
+            udst[i] = kThin ? (uint32_t)xt * 16u + (uint32_t)i * (kXformThreads * 16u) : 0u;
             ujp[i] = 0;
             upix[i] = 0;
+            if (kLinear) ulin[i] = 0;
             if (i < nu) {
                 const int u = xt + i * kXformThreads;
                 const int cg = kThin ? 0 : conv_fdiv(u, g.planes * g.SLOTS, g.dv_pss), idx = u - cg * per_stage_slots;
                 // operand rows are 16 bytes apart: the low four bits carry the unit's chunk group
-                udst[i] = ((uint32_t)(cg * cpu) * (uint32_t)g.chunk_pitch + (uint32_t)idx * 16u) | (uint32_t)cg;
+                if (!kThin) udst[i] = ((uint32_t)(cg * cpu) * (uint32_t)g.chunk_pitch + (uint32_t)idx * 16u) | (uint32_t)cg;
                 const int pl = conv_fdiv(idx, g.SLOTS, g.dv_SLOTS), j = idx - pl * g.SLOTS;
                 // the slot's distance from the tile's first slot, as whole slot rows and columns
                 // (both below 2^12: a stage holds at most 2560 slots)
                 const int dh = conv_fdiv(j, g.Ws, g.dv_Ws), dw = j - dh * g.Ws;
-                ujp[i] = (uint32_t)dw | ((uint32_t)dh << 12);
+                ujp[i] = kRows ? (uint32_t)dh | ((uint32_t)dw << 16) : (uint32_t)dw | ((uint32_t)dh << 12);
                 // fixed-index reads of the parity tables (a dynamic index into kernel parameters costs an indexed
                 // constant load per use)
                 const int pa = pl == 0 ? g.pa[0] : pl == 1 ? g.pa[1] : pl == 2 ? g.pa[2] : g.pa[3];
                 const int pb = pl == 0 ? g.pb[0] : pl == 1 ? g.pb[1] : pl == 2 ? g.pb[2] : g.pb[3];
                 upix[i] = ((uint32_t)(dh * g.sh + pa - g.pt) << 16) | ((uint32_t)(dw * g.sw + pb - g.pl) & 0xFFFFu);
+                if (kLinear) ulin[i] = (dh * g.sh + pa - g.pt) * g.W + dw * g.sw + pb - g.pl;
             }
         }
         for (long long t = first_tile; t < g.total_tiles; t += tile_step) {
@@ -511,7 +532,21 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                 // was the larger part of the thin first layer's time).  Slot -> (image, slot row, slot column) without
                 // dividing the slot number: the tile's first slot was decomposed once (by the producer, in the
                 // segment table), and this unit lies a fixed number of slot rows and columns further on.
-                {
+                if (kLinear && g.raw_mode == 2 && segs->one_image) {
+                    // Nearly every tile of a large image: rows lie as in X, so a pixel's place in X's plane less the
+                    // segment's is its offset, and its row exists where that place does (its column exists too).  A third
+                    // of the instructions of the general form below, which were nearly half of a thin layer's re-lay: 7x7/2 first
+                    // layer at batch 64 67.0 -> 63.8 us, 10 -> 16 channels 3x3 144x144 at batch 56 113.5 -> 99.2.
+                    const uint32_t wrap = (uint32_t)(g.Ws - wq0) << 16;
+                    const int w0 = wq0 * g.sw, w1 = w0 - g.Ws * g.sw, HW = g.H * g.W;
+                    const int p0 = hq0 * g.sh * g.W + w0, p1 = p0 + g.sh * g.W - g.Ws * g.sw, rel = segs->base[0] - segs->f0[0];
+#pragma unroll
+                    for (int i = 0; i < kOwned; ++i) {
+                        const bool carry = ujp[i] >= wrap;
+                        const int at = ulin[kLinear ? i : 0] + (carry ? p1 : p0), w = (int)(short)upix[i] + (carry ? w1 : w0);
+                        uoff[i] = (unsigned)w < (unsigned)g.W && (unsigned)at < (unsigned)HW ? at + rel : -1;
+                    }
+                } else {
                     const int nseg = segs->nseg, hbase = hq0 * g.sh, wbase = wq0 * g.sw, Wssw = g.Ws * g.sw, Hssh = g.Hs * g.sh;
                     // the table's first two entries in registers: a tile of a large image touches no more than two
                     const int f0a = segs->f0[0], f0b = segs->f0[1], ba = segs->base[0], bb = segs->base[1];
@@ -519,8 +554,8 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
 #pragma unroll
                     for (int i = 0; i < kOwned; ++i) {
                         const int ch = kThin ? 0 : (int)(udst[i] & 15u) * cpu;
-                        const int carry = wq0 + (int)(ujp[i] & 0xFFFu) >= g.Ws ? 1 : 0;
-                        const int hq = hq0 + (int)(ujp[i] >> 12) + carry;
+                        const int carry = wq0 + (int)(kRows ? ujp[i] >> 16 : ujp[i] & 0xFFFu) >= g.Ws ? 1 : 0;
+                        const int hq = hq0 + (int)(kRows ? ujp[i] & 0xFFFFu : ujp[i] >> 12) + carry;
                         int k = hq >= g.Hs ? 1 : 0, f0 = k ? f0b : f0a, base = k ? bb : ba;        // images crossed
                         if (nseg > 2) {                                                            // (small images: several)
                             k = conv_fdiv(hq, g.Hs, g.dv_Hs);
@@ -532,8 +567,8 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                         const int w = wbase + (int)(short)upix[i] - carry * Wssw;
                         const bool ok = i < nu && k < images && (unsigned)h < (unsigned)g.H && (unsigned)w < (unsigned)g.W;
                         const int f = h * g.W + w - f0;
-                        int o = base + f;                                                          // whole-image slabs
-                        if (g.raw_mode != 1) {
+                        int o = base + f;                                                          // slabs, rows
+                        if (kRows ? g.raw_mode == 0 : g.raw_mode != 1) {
                             if (g.boxp_shift >= 0) {
                                 o = base + (f >> g.boxp_shift) * box_floats + (f & (g.BOXP - 1));
                             } else {
@@ -666,6 +701,24 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                 }
             }
             const char *rb = reinterpret_cast<const char *>(R);
+            if (kAddend == kAddendFar) {
+                // The next tile's addends (the first time this one's too) are asked into L2: eight in flight per lane below, all
+                // that its registers hold, are too few for a trip to memory each.  3 -> 64
+                // channels 7x7/2 224x224 at batch 32 78.7 -> 65.8 us, 10 -> 80 3x3 130x198 at batch 23 142 -> 122.
+                for (long long u = it == 0 ? t : t + tile_step; u <= t + tile_step && u < g.total_tiles; u += tile_step) {
+                    const int cta = (int)(u % cgt), gr = cta / g.ctiles, m0 = cta % g.ctiles * g.BN;
+                    const uint32_t Gw = (uint32_t)(((u / cgt) * kCtas + rank) * tile_rows) + (uint32_t)(mt * 128 + quarter * 32);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {               // the two lines that the warp's 32 pixels lie in
+                        const uint32_t G = Gw + 31u * e;
+                        const int n = conv_fdiv((int)G, g.L, g.dv_L), w = (int)G - n * g.L, p = conv_fdiv(w, g.Ws, g.dv_Ws);
+                        if (n >= g.N || p >= g.P) continue;
+                        const char *at = rb + (uint32_t)(p * g.Q + min(w - p * g.Ws, g.Q - 1)) * 4u;
+                        for (int c = m0 + ch_lo * 32 + lane; c < min(g.Mg, m0 + min(g.BN, ch_hi * 32)); c += 32)
+                            prefetch_l2(at + (uint32_t)(n * g.M + gr * g.Mg + c) * PQ4);
+                    }
+                }
+            }
             const int tile_left = min(g.Mg - ct * g.BN, g.BN);         // channels of the tile
             float b_next = 0.f, r[2][8];
             auto fetch_bias = [&](int chunk) {
@@ -674,9 +727,14 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             };
             // addends (at Y's own positions) of the eight channels `ahead` of those that `off` has come to, `left` of which exist
             auto fetch_add = [&](float (&to)[8], int ahead, int left) {
+                const int lane_left = valid ? left : 0;
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    to[j] = valid && ahead + j < left ? __ldg(reinterpret_cast<const float *>(rb + (off + (uint32_t)(ahead + j) * PQ4))) : 0.f;
+                for (int j = 0; j < 8; ++j) {
+                    // (the form that does not ask ahead gains from having them issued where they stand, 7 to 20 % on layers with a
+                    // large addend; the other, 3 %, from having them where the compiler puts them)
+                    if (kAddend == kAddendNear) to[j] = ldg_where(rb + (off + (uint32_t)(ahead + j) * PQ4), ahead + j, lane_left);
+                    else to[j] = ahead + j < lane_left ? __ldg(reinterpret_cast<const float *>(rb + (off + (uint32_t)(ahead + j) * PQ4))) : 0.f;
+                }
             };
             if (!kSplit) {
                 fetch_bias(ch_lo);
@@ -941,7 +999,9 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     // raw staging mode
     const long long HW = (long long)c.H * c.W;
     if (HW % 4 == 0) {
-        g.raw_mode = 0;
+        // Blocks of 4 channels of images that a tile touches two of at most: a copy per channel (a box per 256 pixels is more
+        // copies there, and its places cost the transform a shift and a mask per unit).
+        g.raw_mode = g.KB == 4 && (g.SLOTS + L - 2) / L + 1 <= 2 ? 2 : 0;
     } else if (c.Cg % 4 == 0 && c.C % 4 == 0 && HW * g.KB * 4 <= 32768) {
         g.raw_mode = 1;
     } else {
@@ -977,6 +1037,9 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     int worst, boxes;
     if (g.raw_mode == 1) {
         worst = stage_floats(256, boxes);
+    } else if (g.raw_mode == 2) {
+        g.BOXP = std::max(4, stage_floats(4, boxes));
+        worst = g.BOXP * g.KBR;
     } else if (g.KB == 4) {
         // Blocks of 4 channels (the thin first layer of a network) stage little per pixel: 256-pixel boxes, and
         // a power of two spares the transform a division per unit.
@@ -1223,7 +1286,7 @@ static int max_pairs() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_conv_kernel<2, false, false, false>, &cfg) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, tc_conv_kernel<2, kNoAddend, false, false>, &cfg) != cudaSuccess || n < 1) {
         cudaGetLastError();
         n = tc_host::num_sms() / 2;
     }
@@ -1290,11 +1353,18 @@ static int launch_images(const TcConvPlan &plan, const float *X, const float *B,
     const bool add = R != nullptr;
     const bool split = plan.split > 1;
     const bool thin = plan.KB == 4;
-    auto kern = split  ? (add ? tc_conv_kernel<1, true, false, true> : tc_conv_kernel<1, false, false, true>)
-                : thin ? (pair ? (add ? tc_conv_kernel<2, true, true, false> : tc_conv_kernel<2, false, true, false>)
-                               : (add ? tc_conv_kernel<1, true, true, false> : tc_conv_kernel<1, false, true, false>))
-                       : (pair ? (add ? tc_conv_kernel<2, true, false, false> : tc_conv_kernel<2, false, false, false>)
-                               : (add ? tc_conv_kernel<1, true, false, false> : tc_conv_kernel<1, false, false, false>));
+    // Asking ahead for an addend is worth it where L2 is unlikely to hold it still (64 -> 64 channels 3x3 56x56 batch 32, 26 MB:
+    // 23.9 -> 25.1 us with it) and the main loop is too short to hide the epilogue (64 -> 64 3x3 112x112 batch 32, 72 steps:
+    // 97 -> 102; 32 -> 128, 36 steps of 128 columns: 132 -> 138; 32 -> 64, 36 of 64: 77 -> 69; thin layers:
+    // 3 -> 256 7x7 64x64 batch 64 197 -> 173, 12 -> 64 5x5 112x112 batch 32 82 -> 72).
+    const bool far = add && 4LL * plan.N * plan.M * plan.P * plan.Q >= (64LL << 20) && (thin || plan.ncb * plan.n_steps * plan.BN <= 2560);
+    auto kern = split  ? (add ? tc_conv_kernel<1, kAddendNear, false, true> : tc_conv_kernel<1, kNoAddend, false, true>)
+                : thin ? (far   ? (pair ? tc_conv_kernel<2, kAddendFar, true, false> : tc_conv_kernel<1, kAddendFar, true, false>)
+                          : add ? (pair ? tc_conv_kernel<2, kAddendNear, true, false> : tc_conv_kernel<1, kAddendNear, true, false>)
+                                : (pair ? tc_conv_kernel<2, kNoAddend, true, false> : tc_conv_kernel<1, kNoAddend, true, false>))
+                       : (far   ? (pair ? tc_conv_kernel<2, kAddendFar, false, false> : tc_conv_kernel<1, kAddendFar, false, false>)
+                          : add ? (pair ? tc_conv_kernel<2, kAddendNear, false, false> : tc_conv_kernel<1, kAddendNear, false, false>)
+                                : (pair ? tc_conv_kernel<2, kNoAddend, false, false> : tc_conv_kernel<1, kNoAddend, false, false>));
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return (int)e;
     const int sms = num_sms();

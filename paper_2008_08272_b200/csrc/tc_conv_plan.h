@@ -59,7 +59,8 @@ struct TcConvPlan {
     int pix_tiles;                   // ceil(total_slots / (ctas*MT*128))
     long long total_tiles;
     // raw staging
-    int raw_mode;                    // 0: tensor-map boxes [KB][BOXP] over X seen as (H*W, N*C); 1: whole-image slabs
+    int raw_mode;                    // 0: tensor-map boxes [KB][BOXP] over X seen as (H*W, N*C); 1: whole-image slabs;
+                                     // 2: one copy of rows per channel, [channel][BOXP]
     int BOXP;
     int KBR;                         // channels staged per block: KB, or all of a group's if it has fewer
     // shared memory carve-up (bytes)
@@ -190,8 +191,9 @@ struct TcConvSegs {
     int hq0, wq0;                    // slot row / column of the tile's first slot within image n_first
     int f0[kConvMaxSeg];             // first flat pixel (h*W + w) staged for the image
     int base[kConvMaxSeg];           // float offset of the image's data inside the raw stage
-    int nbox[kConvMaxSeg];           // boxes (mode 0) / 1 (mode 1) / 0 when nothing of the image is needed
-    int total_floats;
+    int nbox[kConvMaxSeg];           // boxes (mode 0) / 1 (mode 1) / pixels (mode 2) / 0 when nothing of the image is needed
+    int total_floats;                // of the stage (mode 2: of a channel)
+    int one_image;                   // every slot of the tile lies in image n_first
 };
 
 // Which part of which images the A stage of the tile starting at global slot G0 needs.
@@ -203,6 +205,7 @@ ONNXB_HD inline void tc_conv_segments(const TcConvPlan &g, long long G0, TcConvS
         t.nseg = 0;
         t.hq0 = t.wq0 = 0;
         t.total_floats = 0;
+        t.one_image = 0;
         return;
     }
     t.n_first = conv_fdiv((int)G0, g.L, g.dv_L);
@@ -214,6 +217,7 @@ ONNXB_HD inline void tc_conv_segments(const TcConvPlan &g, long long G0, TcConvS
     const int n_last = conv_fdiv((int)(Gend - 1), g.L, g.dv_L);
     t.nseg = n_last - t.n_first + 1;
     if (t.nseg > kConvMaxSeg) t.nseg = kConvMaxSeg;   // excluded by the planner
+    t.one_image = t.nseg == 1 && Gend == G0 + g.SLOTS;
     int base = 0;
     for (int i = 0; i < t.nseg; ++i) {
         const long long n = t.n_first + i;
@@ -237,6 +241,11 @@ ONNXB_HD inline void tc_conv_segments(const TcConvPlan &g, long long G0, TcConvS
             const int f0 = (h_min * g.W) & ~3;
             const int len = (h_max + 1) * g.W - f0;
             t.f0[i] = f0;
+            if (g.raw_mode == 2) {
+                t.nbox[i] = (len + 3) & ~3;          // (within the plane: H * W is a multiple of 4)
+                base += t.nbox[i];
+                continue;
+            }
             t.nbox[i] = conv_fdiv(len + g.BOXP - 1, g.BOXP, g.dv_BOXP);
             base += t.nbox[i] * g.BOXP * g.KBR;
         }
