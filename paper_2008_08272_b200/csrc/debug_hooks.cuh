@@ -1,7 +1,6 @@
 // Optional in-kernel instrumentation of the two tensor-core kernels.  Nothing here is compiled unless the
-// library is built with -DONNXB_PROFILE (cycle accounting per warp role and an event log of CTA 0) or
-// -DONNXB_CHECK (index checks in the weight-packing kernel); in a normal build every macro below is
-// empty and no symbol is added.  The including file selects its part with ONNXB_DEBUG_HOOKS_CONV or
+// library is built with -DONNXB_PROFILE (cycle accounting per warp role and an event log of CTA 0); in a normal
+// build every macro below is empty and no symbol is added.  The including file selects its part with ONNXB_DEBUG_HOOKS_CONV or
 // ONNXB_DEBUG_HOOKS_GEMM.
 #pragma once
 #include <cuda_runtime.h>
@@ -31,18 +30,6 @@ extern "C" int onnxb_dbg_log(long long *out) {
 #define PROF_DECL do {} while (0)
 #define PROF_MARK(k) do {} while (0)
 #define PROF_FLUSH(base) do {} while (0)
-#endif
-
-#if defined(ONNXB_CHECK) && defined(ONNXB_DEBUG_HOOKS_CONV)
-__device__ long long g_chk[8];
-#define CHK(cond, code, val) if (!(cond)) { if (atomicCAS((unsigned long long *)&g_chk[0], 0ull, (unsigned long long)(code)) == 0ull) { g_chk[1] = (long long)(val); g_chk[2] = blockIdx.x; g_chk[3] = threadIdx.x; } continue; }
-extern "C" int onnxb_dbg_check(long long *out) {
-    cudaDeviceSynchronize();
-    cudaMemcpyFromSymbol(out, g_chk, sizeof(long long) * 8);
-    return 0;
-}
-#else
-#define CHK(cond, code, val)
 #endif
 
 #if defined(ONNXB_PROFILE) && defined(ONNXB_DEBUG_HOOKS_GEMM)

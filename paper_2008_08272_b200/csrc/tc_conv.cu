@@ -34,6 +34,7 @@
 #include "common.h"
 #define ONNXB_DEBUG_HOOKS_CONV
 #include "debug_hooks.cuh"
+#include "pack_weights.cuh"
 #include "tc_common.cuh"
 #include "tc_conv_plan.h"
 #include "tc_host.h"
@@ -86,33 +87,11 @@ static_assert(sizeof(Bars) <= kBarBytes, "barrier block too large");
 // rows past the group's channels, channels past Cg and unpaired taps are zero.
 // Launched with programmatic stream serialization: it may become resident while the previous kernel
 // of the stream drains, and waits (pdl_wait) before it touches W or the workspace.
-__global__ void pack_weights_kernel(const TcConvPlan g, const float *__restrict__ W, float4 *__restrict__ out) {
+__global__ void __launch_bounds__(kPackThreads) pack_weights_kernel(const __grid_constant__ TcConvPlan g, const float *__restrict__ W, float4 *__restrict__ out) {
     pdl_launch_dependents();
-    const unsigned total = (unsigned)(g.packed_floats / 4);          // the planner keeps this below 2^31
-    pdl_wait();
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        unsigned t = i;
-        const int row = (int)(t % (unsigned)g.BNH); t /= (unsigned)g.BNH;
-        const int k = (int)(t & 1u); t >>= 1;
-        const int step = (int)(t % (unsigned)g.n_steps); t /= (unsigned)g.n_steps;
-        const int cb = (int)(t % (unsigned)g.ncb); t /= (unsigned)g.ncb;
-        const unsigned cts = (unsigned)(g.ctiles * g.ctas);
-        const int ct = (int)(t % cts); t /= cts;                     // BNH-wide tile: (tile, CTA of the pair)
-        const int grp = (int)t;
-        const int mg = ct * g.BNH + row;
-        const int tap = g.src_tap[step][k];
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-        if (mg < g.Mg && tap >= 0) {
-            const int m = grp * g.Mg + mg;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int c = cb * g.KB + g.src_c0[step][k] + e;
-                CHK(((size_t)m * g.Cg + (c < g.Cg ? c : 0)) * g.taps + tap < (size_t)g.M * g.Cg * g.taps, 1, ((size_t)m * g.Cg + c) * g.taps + tap)
-                if (c < g.Cg) v[e] = round_tf32(__ldg(W + ((size_t)m * g.Cg + c) * g.taps + tap));
-            }
-        }
-        out[i] = make_float4(v[0], v[1], v[2], v[3]);
-    }
+    pack_weights(g, W, g.ctiles * g.ctas, g.BNH, g.KB, [&](size_t tile, int cb, int step, int half, int row, const float (&v)[4]) {
+        out[(((tile * g.ncb + cb) * g.n_steps + step) * 2 + half) * g.BNH + row] = make_float4(round_tf32(v[0]), round_tf32(v[1]), round_tf32(v[2]), round_tf32(v[3]));
+    });
 }
 
 // Channel blocks are summed in a rotated order that differs from tile to tile: CTAs working at the
@@ -1308,10 +1287,8 @@ int launch_tc_conv(const TcConvPlan &plan, const float *X, const float *W, const
 
     // 1. pack + round the weights into the workspace (skipped when the caller packed them earlier)
     if (phase != kTcConvRunOnly) {
-        const long long vec = plan.packed_floats / 4;
-        const int blocks = (int)std::min<long long>((vec + 255) / 256, 148 * 16);
-        const cudaError_t e = launch_pdl(pack_weights_kernel, dim3(blocks), dim3(256), 0, st, plan, W,
-                                         reinterpret_cast<float4 *>(workspace));
+        const dim3 grid = pack_weights_grid(plan, plan.ctiles * plan.ctas, plan.BNH);
+        const cudaError_t e = launch_pdl(pack_weights_kernel, grid, dim3(kPackThreads), 0, st, plan, W, reinterpret_cast<float4 *>(workspace));
         count_launch();
         if (e != cudaSuccess) return (int)e;
     }

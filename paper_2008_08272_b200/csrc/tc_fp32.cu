@@ -29,6 +29,7 @@
 #include <cstdlib>
 
 #include "common.h"
+#include "pack_weights.cuh"
 #include "tc_common.cuh"
 #include "tc_host.h"
 
@@ -168,28 +169,15 @@ __global__ void __launch_bounds__(256) pack_split_kernel(const __grid_constant__
 }
 
 // The filters of a convolution, split: [group][channel tile][block][K-step][chunk][hi, lo][channel of the tile][4].
-__global__ void __launch_bounds__(256) pack_filters_split_kernel(const __grid_constant__ Fp32ConvPlan p, const float *__restrict__ W, float4 *__restrict__ out) {
+__global__ void __launch_bounds__(kPackThreads) pack_filters_split_kernel(const __grid_constant__ Fp32ConvPlan p, const float *__restrict__ W, float4 *__restrict__ out) {
     pdl_launch_dependents();
-    const unsigned BN = (unsigned)p.BN, total = (unsigned)(p.group * p.tiles_c * p.ncb * p.n_steps) * 2u * BN;
-    pdl_wait();
-    for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < total; i += gridDim.x * 256u) {
-        unsigned t = i;
-        const int row = (int)(t % BN); t /= BN;
-        const int k = (int)(t & 1u); t >>= 1;
-        const int step = (int)(t % (unsigned)p.n_steps); t /= (unsigned)p.n_steps;
-        const int cb = (int)(t % (unsigned)p.ncb); t /= (unsigned)p.ncb;
-        const int ct = (int)(t % (unsigned)p.tiles_c), grp = (int)(t / (unsigned)p.tiles_c);
-        const int mg = ct * p.BN + row, tap = p.src_tap[step][k], c0 = cb * p.nch * 4 + p.src_c0[step][k];
-        float v[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            v[e] = mg < p.Mg && tap >= 0 && c0 + e < p.Cg ? __ldg(W + ((size_t)(grp * p.Mg + mg) * p.Cg + c0 + e) * p.taps + tap) : 0.f;
+    pack_weights(p, W, p.tiles_c, p.BN, p.nch * 4, [&](size_t tile, int cb, int step, int half, int row, const float (&v)[4]) {
         float4 hi, lo;
         split4(v, hi, lo);
-        float4 *d = out + ((size_t)(i / (2u * BN)) * 2u + k) * 2u * BN + row;
+        float4 *d = out + (((tile * p.ncb + cb) * p.n_steps + step) * 2 + half) * 2 * p.BN + row;
         d[0] = hi;
-        d[BN] = lo;
-    }
+        d[p.BN] = lo;
+    });
 }
 
 // ------------------------------------------------------------------ tiles and pixels
@@ -925,8 +913,7 @@ int launch_tc_fp32_conv(const ConvGeom &g, const Fp32ConvPlan &p, const float *X
                         void *packed, void *stream, int phase) {
     cudaStream_t st = (cudaStream_t)stream;
     if (phase != kTcConvRunOnly) {
-        const unsigned items = (unsigned)(tc_fp32_conv_workspace(p) / 32);
-        const cudaError_t e = tc_host::launch_pdl(pack_filters_split_kernel, dim3(std::min((items + 255) / 256, 148u * 16)), dim3(256), 0, st, p, W,
+        const cudaError_t e = tc_host::launch_pdl(pack_filters_split_kernel, pack_weights_grid(p, p.tiles_c, p.BN), dim3(kPackThreads), 0, st, p, W,
                                                   static_cast<float4 *>(packed));
         count_launch();
         if (e != cudaSuccess) return (int)e;
