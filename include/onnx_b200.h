@@ -200,7 +200,8 @@ void onnx_conv2d_desc_destroy(onnxb_conv2d_desc_t desc);
  * (10 MiB) that is part of the library image: every GPU the library is loaded on holds it
  * until the process exits.  The call allocates and frees nothing.  A descriptor whose
  * queried workspace_bytes exceeds that size is rejected with ONNXB_ERR_WORKSPACE and
- * nothing is launched; use onnx_conv2d_run with your own workspace for such layers.
+ * nothing is launched (use onnx_conv2d_run with your own workspace for such layers);
+ * one of ONNXB_KERNEL_SIMT_DIRECT runs on its FMA kernel instead.
  *
  * X, W, B, Y, cuda_stream: exactly as for onnx_conv2d_run (device pointers, caller-owned).
  * The first call on each device looks up the array's device address (a host-side query,

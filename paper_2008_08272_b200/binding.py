@@ -216,6 +216,9 @@ class Conv2dDesc:
         self._prepacked_needs_ws = bool(
             (self.kernel_family == "mma_gather_gemm" or (self.kernel_family == "simt_direct" and tuple(w_shape[2:]) == (1, 1)))
             and self.workspace_bytes)
+        # a copy of fewer bytes than this descriptor's is none of its own (one of the fp32 family kept from a time when that family
+        # made no copy, say): its fp32 kernels then read W
+        self._copy_bytes = self.workspace_bytes if self.kernel_family == "simt_direct" else 0
         self._plan = None
 
     def _native(self, X, W, packed, B, R, Y, workspace, stream):
@@ -272,6 +275,8 @@ class Conv2dDesc:
 
     def run_prepacked(self, X, W, packed, B=None, R=None, Y=None, workspace=None, stream=None):
         """``onnx_conv2d_run_prepacked``: run (R None) or run_add (R given) from a packed copy of W."""
+        if self._copy_bytes and packed is not None and packed.numel() * packed.element_size() < self._copy_bytes:
+            return self.run(X, W, B, Y, workspace, stream) if R is None else self.run_add(X, W, B, R, Y, workspace, stream)
         if packed is not None:
             y = self._native(X, W, packed, B, R, Y, workspace, stream)
             if y is not None:

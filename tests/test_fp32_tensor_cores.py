@@ -51,6 +51,8 @@ def test_conv(binding, c, tile, monkeypatch):
     assert ok(got, want, S) and ok(added, want + R, S + np.abs(R))
     packed = d.prepack(w)
     assert torch.equal(d.run_prepacked(x, w, packed, b), got) and torch.equal(d.run_prepacked(x, w, packed, b, r), added)
+    short = packed[:16]                                   # not this descriptor's copy: W is read instead
+    assert torch.equal(d.run_prepacked(x, w, short, b), got) and torch.equal(d.run_prepacked(x, w, short, b, r), added)
     # without a workspace: the kernel on the FMA units
     y, stream = torch.empty_like(got), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     ptr = lambda t: ctypes.c_void_p(t.data_ptr())
