@@ -645,6 +645,7 @@ static bool gemm_pairs(const TcGemmProblem &g) {
 }
 
 // Fitted together with the split-K form's estimate (see there); includes ONNX Gemm's rounding pre-pass.
+double tc_gemm_prepass_ns(const TcGemmProblem &g) { return 2030.0 + 283e-6 * 4.0 * ((double)g.M * g.K + (double)g.K * g.N); }
 double tc_gemm_estimate_ns(const TcGemmProblem &g) {
     const int ctas = gemm_pairs(g) ? 2 : 1, units = ctas == 2 ? gemm_max_pairs() : tc_host::num_sms();
     const long long tiles_m = (g.M + kBM * ctas - 1) / (kBM * ctas);
@@ -652,7 +653,7 @@ double tc_gemm_estimate_ns(const TcGemmProblem &g) {
     const long long tiles = tiles_m * ((g.N + bn - 1) / bn) * g.batch;
     const double waves = (double)((tiles + units - 1) / units);
     const double t = waves * ((g.K + kBK - 1) / kBK * (52.0 + 3.06 * bn / ctas + (ctas == 2 ? 8.0 : 0.0)) + 14.9 * bn) + 2470.0;
-    return t + (g.round_operands ? 2030.0 + 283e-6 * 4.0 * ((double)g.M * g.K + (double)g.K * g.N) : 0.0);
+    return t + (g.round_operands ? tc_gemm_prepass_ns(g) : 0.0);
 }
 
 int launch_tc_gemm(const TcGemmProblem &g, void *stream) {

@@ -364,11 +364,18 @@ int resident_ctas(int S) {
 // convolutions of ResNet-50 at batch 1 to 32 and Gemms from 1 x 1000 x 2048 to 1024 x 1024 x 4096; the choice is
 // within 1 % of the best on average).  A wave of CTAs costs 1.4 us and more for its first fill and exchange, and a
 // K block 160-420 ns (rounded in shared memory first: 130-620, with the rows of A there are).
+// ONNX Gemm's operands may also be rounded by the pre-pass and then come here: half of a K block's time is the rounding, and where
+// no operand is large the pre-pass is the shorter (1072 x 384 x 1696 17.4 -> 14.6 us, 416 x 736 x 4416 30.9 -> 24.1, 1024 x 80 x
+// 5232 20.9 -> 15.8; but 128 x 4304 x 3136 27 -> 36, 32 x 4704 x 2432 14.8 -> 27).  The choice then is "not in this kernel", and
+// falls again once they are rounded.
+constexpr double kAhead = 0.85;      // of 0.75 to 1 the best against the estimate above on 104 problems (the pick is within 1.3 % of the better)
 SkChoice search(const TcGemmProblem &g) {
     SkChoice c{0, 0};
     if ((g.a_batched && g.batch > 1) || (g.batch > 1 && g.b_batched && g.b_bs % 4)) return c;
     const int num_kb = (g.K + kBK - 1) / kBK;
     double best = 0.97 * tc_gemm_estimate_ns(g);
+    const double pre = tc_gemm_prepass_ns(g);
+    double ahead = 1e30;                                    // rounded by the pre-pass, then here
     for (int BN = 32; BN <= kMaxBN; BN *= 2)
         for (int S = 1; S <= 8 && S <= num_kb; S *= 2) {
             const long long tiles = (long long)((g.M + kBM - 1) / kBM) * ((g.N + BN - 1) / BN) * g.batch;
@@ -376,13 +383,24 @@ SkChoice search(const TcGemmProblem &g) {
             if (ctas > 4 * 148) break;
             const int units = resident_ctas(S);
             const double waves = (double)((ctas + units - 1) / units);
-            const double blk = g.round_operands ? 64.0 + 1.94 * BN + 2.38 * std::min(g.M, kBM) : 72.0 + 2.71 * BN;
-            const double t = waves * ((num_kb + S - 1) / S * blk + 1390.0 + 23.0 * BN) + 1790.0;
+            const double rest = 1390.0 + 23.0 * BN, kb = (double)((num_kb + S - 1) / S);
+            const double plain = waves * (kb * (72.0 + 2.71 * BN) + rest) + 1790.0;
+            if (!g.round_operands) {
+                if (plain < best) {
+                    best = plain;
+                    c = {BN, S};
+                }
+                continue;
+            }
+            const double t = waves * (kb * (64.0 + 1.94 * BN + 2.38 * std::min(g.M, kBM)) + rest) + 1790.0;
             if (t < best) {
                 best = t;
                 c = {BN, S};
             }
+            ahead = std::min(ahead, kAhead * (pre + plain));
         }
+    // (two launches keep the host busy for some 8 us where one takes 5: not for calls about as short as that)
+    if (ahead < best && best > 10000.0) c = {0, 0};
     return c;
 }
 

@@ -38,6 +38,7 @@ bool tc_gemm_supports(const TcGemmProblem &g);
 int launch_tc_gemm(const TcGemmProblem &g, void *stream);
 // Split-K form for few output tiles (tc_gemm_splitk.cu); launch_tc_gemm uses it where it fits.
 double tc_gemm_estimate_ns(const TcGemmProblem &g);       // the persistent kernel's estimated time
+double tc_gemm_prepass_ns(const TcGemmProblem &g);        // and that of the launch that rounds ONNX Gemm's operands in front of it
 bool tc_gemm_splitk_fits(const TcGemmProblem &g);
 int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream);
 

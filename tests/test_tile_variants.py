@@ -100,3 +100,18 @@ def test_gemm_addend_forms(binding, cs, monkeypatch):
         got = run_gemm_gpu(binding, torch, A, B, C, transB=True, alpha=0.5, beta=-1.5, fuse_relu=True)
         want, S = oracle.gemm(A, B, C, transB=True, alpha=0.5, beta=-1.5, relu=True)
         assert worst_ratio(got, want, S) <= 1.0, (M, N)
+
+
+@pytest.mark.parametrize("tA,tB", [(False, True), (True, False)])
+@pytest.mark.parametrize("M,N,K", [(640, 640, 1280), (704, 304, 2640), (144, 176, 4784)])
+def test_gemm_rounded_ahead_of_the_split(binding, M, N, K, tA, tB):
+    """Problems whose operands are rounded by a launch of their own and whose tiles are then shared by clusters."""
+    rng = np.random.default_rng(M)
+    A = rng.standard_normal((K, M) if tA else (M, K)).astype(np.float32)
+    B = rng.standard_normal((N, K) if tB else (K, N)).astype(np.float32)
+    C = rng.standard_normal((N,)).astype(np.float32)
+    before = binding.launch_count()
+    got = run_gemm_gpu(binding, torch, A, B, C, transA=tA, transB=tB, alpha=0.5, beta=-1.5)
+    assert binding.launch_count() == before + 2
+    want, S = oracle.gemm(A, B, C, transA=tA, transB=tB, alpha=0.5, beta=-1.5)
+    assert worst_ratio(got, want, S) <= 1.0
