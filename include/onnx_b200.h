@@ -221,8 +221,8 @@ size_t onnx_conv2d_static_scratch_bytes(void);
 /*
  * onnx_gemm_workspace_bytes - device scratch onnx_gemm_run needs for this
  * problem (0 when none).  Host only.  The tensor-core path keeps TF32-rounded
- * copies of A and B there (4 * (M*K + K*N) bytes; its split-K form for small M
- * rounds in shared memory and leaves the workspace untouched, but the size is
+ * copies of A and B there (4 * (M*K + K*N) bytes; its split-K form, where
+ * it rounds in shared memory, leaves the workspace untouched, but the size is
  * asked for all the same); the fp32 path of large problems keeps both operands,
  * split into two TF32 parts, there (8 bytes an element, padded to whole tiles)
  * and runs on its FMA kernel, which needs none, where it is given less.
