@@ -516,7 +516,8 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                     // segment's is its offset, and its row exists where that place does (its column exists too).  A third
                     // of the instructions of the general form below, which were nearly half of a thin layer's re-lay: 7x7/2 first
                     // layer at batch 64 67.0 -> 63.8 us, 10 -> 16 channels 3x3 144x144 at batch 56 113.5 -> 99.2.
-                    const uint32_t wrap = (uint32_t)(g.Ws - wq0) << 16;
+                    // (saturated: a unit's columns are below 2^12, a slot row of far padding at its end has 2^16 and more)
+                    const uint32_t wrap = (uint32_t)min(g.Ws - wq0, 0xFFFF) << 16;
                     const int w0 = wq0 * g.sw, w1 = w0 - g.Ws * g.sw, HW = g.H * g.W;
                     const int p0 = hq0 * g.sh * g.W + w0, p1 = p0 + g.sh * g.W - g.Ws * g.sw, rel = segs->base[0] - segs->f0[0];
 #pragma unroll

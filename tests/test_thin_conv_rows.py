@@ -39,6 +39,22 @@ def test_thin_rows(xs, ws, kw, tile, monkeypatch):
     assert family == "mma_implicit" and ratio <= 1.0
 
 
+@pytest.mark.parametrize("tile", [None, "1,1,32", "2,2,32"])
+@pytest.mark.parametrize("xs,ws,pads", [((1, 1, 1, 20000), (64, 1, 1, 33), (0, 16, 0, 50000)), ((2, 8, 2, 2000), (16, 8, 1, 25), (0, 0, 0, 64000)),
+                                        ((1, 4, 1, 2000), (16, 4, 1, 9), (0, 4, 0, 63536))], ids=str)
+def test_slot_rows_of_65536_and_more(xs, ws, pads, tile, monkeypatch):
+    """Padding at the end of the rows that makes a slot row longer than 16 bits count."""
+    from paper_2008_08272_b200 import binding
+    if tile:
+        monkeypatch.setenv("ONNXB_CONV_TILE", tile)
+    binding.set_kernel_override("mma_implicit")
+    try:
+        ratio, family = check_conv(binding, torch, *_operands(xs, ws), pads=pads)
+    finally:
+        binding.set_kernel_override(None)
+    assert family == "mma_implicit" and ratio <= 1.0
+
+
 @pytest.mark.parametrize("xs,ws", [((3, 8, 472, 500), (24, 8, 3, 3)), ((6, 16, 240, 180), (65, 16, 3, 3))])
 def test_far_addend(xs, ws):
     from paper_2008_08272_b200 import binding
