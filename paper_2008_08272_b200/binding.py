@@ -177,6 +177,26 @@ def _stream_ptr(stream=None):
     return ctypes.c_void_p(s.cuda_stream)
 
 
+def _new(size, device, stream, dtype="float32", kept=True):
+    """Memory for a call on ``stream`` (None: the current one).  The allocator hands a block out and takes it back in the order of
+    the stream it was made on: made on another than the call's, the block's last user may not have finished when the call's kernels
+    begin, nor they when its next one does.  What the caller keeps goes on to be used from the current stream, too."""
+    import torch
+    dtype = getattr(torch, dtype)
+    if stream is None or not str(device).startswith("cuda"):
+        return torch.empty(size, dtype=dtype, device=device)
+    current = torch.cuda.current_stream(device)
+    if stream.cuda_stream == current.cuda_stream:
+        return torch.empty(size, dtype=dtype, device=device)
+    if not isinstance(stream, torch.cuda.Stream):        # anything with a handle
+        stream = torch.cuda.ExternalStream(stream.cuda_stream, device) if stream.cuda_stream else torch.cuda.default_stream(device)
+    with torch.cuda.stream(stream):
+        t = torch.empty(size, dtype=dtype, device=device)
+    if kept:
+        t.record_stream(current)
+    return t
+
+
 def make_attrs(x_shape, w_shape, *, kernel_shape=None, pads=None, strides=None, dilations=None, group=0,
                auto_pad="NOTSET", has_bias=False, fuse_relu=False) -> ConvAttrs:
     a = ConvAttrs()
@@ -234,11 +254,10 @@ class Conv2dDesc:
         y = self._native(X, W, None, B, None, Y, workspace, stream)
         if y is not None:
             return y
-        import torch
         if Y is None:
-            Y = torch.empty(self.y_shape, dtype=torch.float32, device=X.device)
+            Y = _new(self.y_shape, X.device, stream)
         if workspace is None and self.workspace_bytes:
-            workspace = torch.empty(self.workspace_bytes, dtype=torch.uint8, device=X.device)
+            workspace = _new(self.workspace_bytes, X.device, stream, "uint8", kept=False)
         ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
         ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
         _check(self._lib.onnx_conv2d_run(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
@@ -252,11 +271,10 @@ class Conv2dDesc:
             y = self._native(X, W, None, B, R, Y, workspace, stream)
             if y is not None:
                 return y
-        import torch
         if Y is None:
-            Y = torch.empty(self.y_shape, dtype=torch.float32, device=X.device)
+            Y = _new(self.y_shape, X.device, stream)
         if workspace is None and self.workspace_bytes:
-            workspace = torch.empty(self.workspace_bytes, dtype=torch.uint8, device=X.device)
+            workspace = _new(self.workspace_bytes, X.device, stream, "uint8", kept=False)
         ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
         ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
         _check(self._lib.onnx_conv2d_add_run(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
@@ -267,8 +285,7 @@ class Conv2dDesc:
     def prepack(self, W, stream=None):
         """``onnx_conv2d_prepack``: the packed copy of constant weights (a uint8 device tensor; untouched when
         this descriptor's kernel reads W directly)."""
-        import torch
-        packed = torch.empty(max(self.workspace_bytes, 16), dtype=torch.uint8, device=W.device)
+        packed = _new(max(self.workspace_bytes, 16), W.device, stream, "uint8")
         _check(self._lib.onnx_conv2d_prepack(self._h, _dev_ptr(W, "W"), ctypes.c_void_p(packed.data_ptr()),
                                              packed.numel(), _stream_ptr(stream)), "onnx_conv2d_prepack")
         return packed
@@ -281,11 +298,10 @@ class Conv2dDesc:
             y = self._native(X, W, packed, B, R, Y, workspace, stream)
             if y is not None:
                 return y
-        import torch
         if Y is None:
-            Y = torch.empty(self.y_shape, dtype=torch.float32, device=X.device)
+            Y = _new(self.y_shape, X.device, stream)
         if workspace is None and self._prepacked_needs_ws:
-            workspace = torch.empty(self.workspace_bytes, dtype=torch.uint8, device=X.device)
+            workspace = _new(self.workspace_bytes, X.device, stream, "uint8", kept=False)
         ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
         ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
         _check(self._lib.onnx_conv2d_run_prepacked(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
@@ -299,9 +315,8 @@ class Conv2dDesc:
         """``onnx_conv2d_run_static``: like run(), but the library's built-in scratch array
         stands in for the workspace, so no device memory is allocated for scratch.  (Y is
         still allocated here with torch when the caller does not pass one.)"""
-        import torch
         if Y is None:
-            Y = torch.empty(self.y_shape, dtype=torch.float32, device=X.device)
+            Y = _new(self.y_shape, X.device, stream)
         _check(self._lib.onnx_conv2d_run_static(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
                                                 _dev_ptr(B, "B", allow_none=True), _dev_ptr(Y, "Y"),
                                                 _stream_ptr(stream)), "onnx_conv2d_run_static")
@@ -342,7 +357,6 @@ def onnx_gemm(A, B, C=None, *, alpha=1.0, beta=1.0, transA=False, transB=False, 
     y = (_fast_mod or _fast()).gemm(A, B, C, alpha, beta, transA, transB, fuse_relu, Y, workspace, stream)
     if y is not None:
         return y
-    import torch
     lib = load()
     M, K = (A.shape[1], A.shape[0]) if transA else (A.shape[0], A.shape[1])
     N = B.shape[0] if transB else B.shape[1]
@@ -350,14 +364,14 @@ def onnx_gemm(A, B, C=None, *, alpha=1.0, beta=1.0, transA=False, transB=False, 
     if kb != K:
         raise OnnxB200Error(3, "onnx_gemm: inner dimensions differ")
     if Y is None:
-        Y = torch.empty((M, N), dtype=torch.float32, device=A.device)
+        Y = _new((M, N), A.device, stream)
     c_rank, c_dims = 0, None
     if C is not None:
         c_rank = C.dim()
         c_dims = (ctypes.c_int64 * max(c_rank, 1))(*[int(v) for v in C.shape])
     need = gemm_workspace_bytes(transA, transB, M, N, K)
     if workspace is None and need:
-        workspace = torch.empty(need, dtype=torch.uint8, device=A.device)
+        workspace = _new(need, A.device, stream, "uint8", kept=False)
     ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
     ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
     _check(lib.onnx_gemm_run(int(bool(transA)), int(bool(transB)), float(alpha), float(beta), M, N, K,
@@ -406,21 +420,20 @@ def onnx_matmul_add(A, B, C=None, *, fuse_relu=False, Y=None, workspace=None, st
     y = (_fast_mod or _fast()).gemm(A, B, C, 1.0, 1.0, False, False, fuse_relu, Y, workspace, stream)
     if y is not None:
         return y
-    import torch
     lib = load()
     M, K = A.shape
     if B.shape[0] != K:
         raise OnnxB200Error(3, "onnx_matmul_add: inner dimensions differ")
     N = B.shape[1]
     if Y is None:
-        Y = torch.empty((M, N), dtype=torch.float32, device=A.device)
+        Y = _new((M, N), A.device, stream)
     c_rank, c_dims = 0, None
     if C is not None:
         c_rank = C.dim()
         c_dims = (ctypes.c_int64 * max(c_rank, 1))(*[int(v) for v in C.shape])
     need = gemm_workspace_bytes(False, False, M, N, K)
     if workspace is None and need:
-        workspace = torch.empty(need, dtype=torch.uint8, device=A.device)
+        workspace = _new(need, A.device, stream, "uint8", kept=False)
     ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
     ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
     _check(lib.onnx_matmul_add_run(M, N, K, _dev_ptr(A, "A"), _dev_ptr(B, "B"), _dev_ptr(C, "C", allow_none=True),
@@ -448,10 +461,9 @@ def onnx_maxpool2d(X, kernel_shape, *, pads=None, strides=None, Y=None, stream=N
     y = (_fast_mod or _fast()).maxpool(X, kernel_shape, pads, strides, Y, stream)
     if y is not None:
         return y
-    import torch
     y_shape = maxpool2d_shape(tuple(X.shape), kernel_shape, pads, strides)
     if Y is None:
-        Y = torch.empty(y_shape, dtype=torch.float32, device=X.device)
+        Y = _new(y_shape, X.device, stream)
     _check(load().onnx_maxpool2d_run(_i64(tuple(X.shape), 4), _i64(kernel_shape, 2), _i64(pads, 4), _i64(strides, 2),
                                      _dev_ptr(X, "X"), _dev_ptr(Y, "Y"), _stream_ptr(stream)), "onnx_maxpool2d_run")
     return Y
@@ -462,9 +474,8 @@ def onnx_global_average_pool(X, *, Y=None, stream=None):
     y = (_fast_mod or _fast()).gap(X, Y, stream)
     if y is not None:
         return y
-    import torch
     if Y is None:
-        Y = torch.empty((X.shape[0], X.shape[1], 1, 1), dtype=torch.float32, device=X.device)
+        Y = _new((X.shape[0], X.shape[1], 1, 1), X.device, stream)
     _check(load().onnx_global_average_pool_run(_i64(tuple(X.shape), 4), _dev_ptr(X, "X"), _dev_ptr(Y, "Y"),
                                                _stream_ptr(stream)), "onnx_global_average_pool_run")
     return Y

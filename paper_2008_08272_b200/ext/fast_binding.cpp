@@ -11,6 +11,8 @@
 
 #include <ATen/core/Tensor.h>
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDACachingAllocator.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -69,7 +71,19 @@ inline void *stream_ptr(PyObject *o, bool &fine) {
     return p;
 }
 
-inline at::Tensor new_tensor(at::IntArrayRef size, at::ScalarType type, const at::Device &dev) {
+// Memory for a call on `st`; `given` is the stream argument it came from.  The allocator hands a block out and takes it back in
+// the order of the stream it was made on: made on another than the call's, the block's last user may not have finished when the
+// call's kernels begin, nor they when its next one does.  A result goes on to be used from the current stream, too.
+inline at::Tensor new_tensor(at::IntArrayRef size, at::ScalarType type, const at::Device &dev, PyObject *given, void *st, bool is_result) {
+    if (given != Py_None) {
+        const c10::cuda::CUDAStream current = c10::cuda::getCurrentCUDAStream(dev.index());
+        if (current.stream() != st) {
+            const c10::cuda::CUDAStreamGuard on(c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(st), dev.index()));
+            at::Tensor t(at::detail::empty_cuda(size, type, dev, c10::nullopt));
+            if (is_result) c10::cuda::CUDACachingAllocator::recordStream(t.storage().data_ptr(), current);
+            return t;
+        }
+    }
     return at::Tensor(at::detail::empty_cuda(size, type, dev, c10::nullopt));
 }
 
@@ -137,11 +151,11 @@ PyObject *py_conv(PyObject *, PyObject *const *a, Py_ssize_t n) {
     const bool pre = a[3] != Py_None;
     at::Tensor ym, wm;
     if (!y) {
-        ym = new_tensor(p->y, at::kFloat, xt->device());
+        ym = new_tensor(p->y, at::kFloat, xt->device(), a[8], st, true);
         y = static_cast<float *>(ym.data_ptr());
     }
     if (!ws && p->workspace && (!pre || p->prepacked_needs_ws)) {
-        wm = new_tensor({(int64_t)p->workspace}, at::kByte, xt->device());
+        wm = new_tensor({(int64_t)p->workspace}, at::kByte, xt->device(), a[8], st, false);
         ws = wm.data_ptr();
         ws_bytes = p->workspace;
     }
@@ -171,13 +185,13 @@ PyObject *py_gemm(PyObject *, PyObject *const *a, Py_ssize_t n) {
     for (int i = 0; i < c_rank; ++i) c_dims[i] = ct->size(i);
     at::Tensor ym, wm;
     if (!y) {
-        ym = new_tensor({M, N}, at::kFloat, at_->device());
+        ym = new_tensor({M, N}, at::kFloat, at_->device(), a[10], st, true);
         y = static_cast<float *>(ym.data_ptr());
     }
     if (!ws) {
         const size_t need = abi.gemm_workspace_bytes(ta, tb, M, N, K);
         if (need) {
-            wm = new_tensor({(int64_t)need}, at::kByte, at_->device());
+            wm = new_tensor({(int64_t)need}, at::kByte, at_->device(), a[10], st, false);
             ws = wm.data_ptr();
             ws_bytes = need;
         }
@@ -217,7 +231,7 @@ PyObject *py_maxpool(PyObject *, PyObject *const *a, Py_ssize_t n) {
     if (abi.maxpool2d_shape(xd, ks, pads, st, yd) != ONNXB_OK) return slow_path();
     at::Tensor ym;
     if (!y) {
-        ym = new_tensor(yd, at::kFloat, xt->device());
+        ym = new_tensor(yd, at::kFloat, xt->device(), a[5], stream, true);
         y = static_cast<float *>(ym.data_ptr());
     }
     return abi.maxpool2d_run(xd, ks, pads, st, x, y, stream) == ONNXB_OK ? result(a[4], ym) : slow_path();
@@ -234,7 +248,7 @@ PyObject *py_gap(PyObject *, PyObject *const *a, Py_ssize_t n) {
     if (!fine || !x || xt->dim() != 4) return slow_path();
     at::Tensor ym;
     if (!y) {
-        ym = new_tensor({xt->size(0), xt->size(1), 1, 1}, at::kFloat, xt->device());
+        ym = new_tensor({xt->size(0), xt->size(1), 1, 1}, at::kFloat, xt->device(), a[2], stream, true);
         y = static_cast<float *>(ym.data_ptr());
     }
     return abi.global_average_pool_run(xt->sizes().data(), x, y, stream) == ONNXB_OK ? result(a[1], ym) : slow_path();
