@@ -434,7 +434,7 @@ Pick search_shape(int M, int N, int K, int groups, bool pixels) {
 
 // What a launch of Gemm is: a tile shape and split, or the tensor-core kernel.  The search costs some 2 us of host
 // time, as much as the launch itself, so each thread remembers the choices of the last few problems.  ONNXB_FP32 = "tc"
-// pins the tensor-core kernel, any other value the FMA one.
+// pins the tensor-core kernel (but for the dot-product kernel's problems), any other value the FMA one.
 struct Choice {
     int M, N, K, groups, pixels;
     Pick pick;
@@ -524,7 +524,8 @@ int launch_simt_gemm(const GemmProblem &p, const float *A, const float *B, const
 }
 
 size_t simt_gemm_workspace_bytes(int M, int N, int K) {
-    if ((long long)M * N * K < 2000000) return 0;              // (never on the tensor cores, and a call that short notices the search)
+    // (never on the tensor cores unless pinned, and a call that short notices the search)
+    if (simt_gemm_is_tiny(M, N, K) || ((long long)M * N * K < 2000000 && !getenv("ONNXB_FP32"))) return 0;
     const Choice c = choose(M, N, K, 1, false);
     return c.tc ? tc_fp32_gemm_workspace(M, N, K, c.plan) : 0;
 }

@@ -104,6 +104,16 @@ def test_descriptor_defaults_and_error_codes():
     lib.onnx_conv2d_desc_destroy(None)                           # must be a no-op
 
 
+def test_pinned_fp32_gemm_is_on_the_tensor_cores_whatever_its_size(monkeypatch):
+    """Its workspace is what takes it there: asked for below the size at which the automatic choice looks, too."""
+    assert binding.gemm_workspace_bytes(False, False, 70, 131, 75) == 0
+    monkeypatch.setenv("ONNXB_FP32", "tc")
+    assert binding.gemm_workspace_bytes(False, False, 70, 131, 75) > 0
+    assert binding.gemm_workspace_bytes(False, False, 1, 130, 65) == 0      # the dot-product kernel's
+    monkeypatch.setenv("ONNXB_FP32", "0,1")
+    assert binding.gemm_workspace_bytes(False, False, 1001, 1530, 777) == 0
+
+
 def test_run_calls_reject_bad_arguments_before_any_launch():
     """Argument errors are reported before CUDA is touched, so this runs without a GPU."""
     lib = binding.load()

@@ -38,6 +38,8 @@ def test_fp32_gemm_and_conv_tiles(binding, pin, monkeypatch):
             B = rng.standard_normal((N, K) if tB else (K, N)).astype(np.float32)
             C = rng.standard_normal((M, 1)).astype(np.float32)
             kw = dict(alpha=0.5, beta=-1.5, transA=tA, transB=tB)
+            # (the first is the dot-product kernel's under every pin)
+            assert (binding.gemm_workspace_bytes(tA, tB, M, N, K) > 0) == (pin == "tc" and M > 1)
             got = run_gemm_gpu(binding, torch, A, B, C, fuse_relu=True, **kw)
             want, S = oracle.gemm(A, B, C, relu=True, **kw)
             assert (np.abs(got - want) <= REL * S + 1e-5).all(), (M, N, K)
@@ -47,6 +49,7 @@ def test_fp32_gemm_and_conv_tiles(binding, pin, monkeypatch):
             B = rng.standard_normal((c["w"][0],)).astype(np.float32)
             kw = dict(pads=c.get("pads", (0, 0, 0, 0)), strides=c.get("strides", (1, 1)),
                       dilations=c.get("dilations", (1, 1)), group=c.get("group", 1))
+            assert (binding.Conv2dDesc(X.shape, W.shape, **kw).workspace_bytes > 0) == (pin == "tc")
             got, fam = run_conv_gpu(binding, torch, X, W, B, relu=True, **kw)
             assert fam == "simt_direct"
             want, S = oracle.conv2d(X, W, B, relu=True, **kw)
@@ -98,10 +101,20 @@ def test_tiny_gemm(binding, shape, tA):
         assert (np.abs(got - want) <= REL * S + 1e-6).all()
 
 
-def test_split_operands_that_overflow(binding, monkeypatch):
+def _as_an_fp32_sum(got, want):
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
+    ok = np.isfinite(want)
+    assert np.isnan(want).any() and np.isinf(want).any() and np.allclose(got[ok], want[ok], rtol=1e-5, atol=1e-4)
+
+
+@pytest.mark.parametrize("tile", [None, "16,1", "32,2"])        # (a reduction shared by two CTAs)
+def test_split_operands_that_overflow(binding, tile, monkeypatch):
     """Infinite, NaN and near-overflow operands have no hi/lo split: the outputs they reach are summed in
     plain fp32 and come out as an fp32 sum gives them."""
     monkeypatch.setenv("ONNXB_FP32", "tc")
+    if tile:
+        monkeypatch.setenv("ONNXB_FP32_GEMM", tile)
+    assert binding.gemm_workspace_bytes(False, False, 70, 131, 75) > 0
     rng = np.random.default_rng(8)
     A = rng.standard_normal((70, 75)).astype(np.float32)
     B = rng.standard_normal((75, 131)).astype(np.float32)
@@ -110,9 +123,25 @@ def test_split_operands_that_overflow(binding, monkeypatch):
     got = run_gemm_gpu(binding, torch, A, B, None)
     with np.errstate(all="ignore"):
         want = A.astype(np.float64) @ B.astype(np.float64)
-    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
-    ok = np.isfinite(want)
-    assert np.allclose(got[ok], want[ok], rtol=1e-5, atol=1e-4)
+    _as_an_fp32_sum(got, want)
+
+
+@pytest.mark.parametrize("split", [1, 8])                       # CTAs that share a reduction
+@pytest.mark.parametrize("xs,ws,pads", [((2, 58, 11, 13), (21, 58, 3, 3), (1, 1, 1, 1)), ((2, 1130, 7, 9), (33, 1130, 1, 1), (0, 0, 0, 0))],
+                         ids=["staged", "packed pixels"])
+def test_split_conv_operands_that_overflow(binding, xs, ws, pads, split, monkeypatch):
+    monkeypatch.setenv("ONNXB_FP32", "tc")
+    monkeypatch.setenv("ONNXB_FP32_TILE", f"1,16,{split}")
+    monkeypatch.setenv("ONNXB_FP32_GEMM", f"16,{split}")
+    rng = np.random.default_rng(9)
+    X = rng.standard_normal(xs).astype(np.float32)
+    W = (rng.standard_normal(ws) * 0.05).astype(np.float32)
+    X[0, 5, 1, 2], X[1, 7, 6, 3], X[1, 31, 2, 6] = np.inf, np.nan, 3.40282e38
+    W[:, 31] = 1e-3
+    assert binding.Conv2dDesc(xs, ws, pads=pads).workspace_bytes > 0
+    got, fam = run_conv_gpu(binding, torch, X, W, None, pads=pads)
+    assert fam == "simt_direct"
+    _as_an_fp32_sum(got, oracle.conv2d(X, W, None, pads=pads)[0])
 
 
 @pytest.mark.parametrize("pin", ["tc", "0,1", "2,3", "3,1", "4,8"])

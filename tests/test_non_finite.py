@@ -104,12 +104,20 @@ def test_gemm_keeps_nan(binding, split, pattern, monkeypatch):
 
 
 @pytest.mark.parametrize("pattern", PATTERNS, ids=hex)
-def test_split_fp32_keeps_nan(binding, pattern, monkeypatch):
-    """fp32 on the tensor cores, by two TF32 parts of every operand: Gemm and Conv."""
+@pytest.mark.parametrize("split", [1, 2])                  # CTAs that share a reduction
+def test_split_fp32_keeps_nan(binding, split, pattern, monkeypatch):
+    """fp32 on the tensor cores, by two TF32 parts of every operand: Gemm, and Conv with staged pixels and with packed ones."""
     monkeypatch.setenv("ONNXB_FP32", "tc")
+    monkeypatch.setenv("ONNXB_FP32_GEMM", f"16,{split}")
+    if split > 1:
+        monkeypatch.setenv("ONNXB_FP32_TILE", f"1,16,{split}")
     binding.set_kernel_override("simt_direct")
     try:
+        assert binding.gemm_workspace_bytes(False, False, 70, 131, 75) > 0
         _gemm(binding, 70, 131, 75, pattern)
-        _conv(binding, (2, 6, 19, 23), (130, 3, 3, 3), pattern, "simt_direct", pads=(1, 1, 1, 1), group=2)
+        for xs, ws, kw in (((2, 6, 19, 23), (130, 3, 3, 3), dict(pads=(1, 1, 1, 1), group=2)) if split == 1 else
+                           ((2, 58, 11, 13), (21, 58, 3, 3), dict(pads=(1, 1, 1, 1))), ((2, 70, 11, 13), (31, 70, 1, 1), {})):
+            assert binding.Conv2dDesc(xs, ws, **kw).workspace_bytes > 0
+            _conv(binding, xs, ws, pattern, "simt_direct", **kw)
     finally:
         binding.set_kernel_override(None)
