@@ -253,13 +253,17 @@ static bool gemm_tc_eligible(int transA, int transB, int64_t M, int64_t N, int64
     const int64_t a_ld = transA ? M : K, b_ld = transB ? K : N;
     return a_ld % 4 == 0 && b_ld % 4 == 0;          // tensor-map strides are multiples of 16 bytes
 }
+// ... and a family pinned by the override that is none of Gemm's leaves them to the fp32 kernels.
+static bool gemm_forced_tc() { return kernel_override() == ONNXB_KERNEL_MMA_GEMM || kernel_override() == ONNXB_KERNEL_MMA_IMPLICIT; }
+static bool gemm_forced_fp32() { return kernel_override() >= 0 && !gemm_forced_tc(); }
 
 extern "C" size_t onnx_gemm_workspace_bytes(int transA, int transB, int64_t M, int64_t N, int64_t K) {
     if (M < 1 || N < 1 || K < 1) return 0;
-    if (gemm_tc_eligible(transA, transB, M, N, K)) return (size_t)(M * K + K * N) * 4;
+    const size_t tf32 = gemm_tc_eligible(transA, transB, M, N, K) ? (size_t)(M * K + K * N) * 4 : 0;
+    if (tf32 && !gemm_forced_fp32()) return tf32;
     const int64_t lim = 2147483647LL;
-    if (M > lim || N > lim || K > lim || M * K > lim || K * N > lim || M * N > lim) return 0;
-    return simt_gemm_workspace_bytes((int)M, (int)N, (int)K);
+    if (M > lim || N > lim || K > lim || M * K > lim || K * N > lim || M * N > lim) return tf32;
+    return std::max(tf32, simt_gemm_workspace_bytes((int)M, (int)N, (int)K));      // (enough if the override has gone by the run)
 }
 
 extern "C" onnxb_status onnx_gemm_run(int transA, int transB, float alpha, float beta, int64_t M, int64_t N,
@@ -298,11 +302,10 @@ extern "C" onnxb_status onnx_gemm_run(int transA, int transB, float alpha, float
     t.alpha = alpha; t.beta = beta; t.C = C; t.c_si = p.c_stride_i; t.c_sj = p.c_stride_j;
     t.row_bias = nullptr; t.relu = p.relu; t.round_operands = 1;
     t.Y = Y; t.y_ld = p.N; t.y_bs = 0;
-    const int forced = kernel_override();
-    const bool forced_tc = forced == ONNXB_KERNEL_MMA_GEMM || forced == ONNXB_KERNEL_MMA_IMPLICIT;
+    const bool forced_tc = gemm_forced_tc();
     const bool eligible = gemm_tc_eligible(transA, transB, M, N, K) && tc_gemm_supports(t);
     int err;
-    if (eligible && (forced_tc || forced < 0)) {
+    if (eligible && !gemm_forced_fp32()) {
         const size_t need = onnx_gemm_workspace_bytes(transA, transB, M, N, K);
         if (!workspace || workspace_bytes < need) return ONNXB_ERR_WORKSPACE;
         if (tc_gemm_splitk_fits(t)) {

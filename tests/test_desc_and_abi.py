@@ -114,6 +114,16 @@ def test_pinned_fp32_gemm_is_on_the_tensor_cores_whatever_its_size(monkeypatch):
     assert binding.gemm_workspace_bytes(False, False, 1001, 1530, 777) == 0
 
 
+def test_gemm_workspace_is_that_of_the_family_the_override_leaves():
+    split, rounded = 8 * 2 * 2048 * 2048, 4 * 2 * 2048 * 2048                # bytes: both operands, in two parts or rounded
+    for family, want in ((None, rounded), ("mma_gemm", rounded), ("simt_direct", split)):
+        binding.set_kernel_override(family)
+        try:
+            assert binding.gemm_workspace_bytes(False, False, 2048, 2048, 2048) == want
+        finally:
+            binding.set_kernel_override(None)
+
+
 def test_run_calls_reject_bad_arguments_before_any_launch():
     """Argument errors are reported before CUDA is touched, so this runs without a GPU."""
     lib = binding.load()

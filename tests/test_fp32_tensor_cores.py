@@ -87,6 +87,15 @@ def test_conv(binding, c, tile, monkeypatch):
     assert binding.last_device_status() == 0
 
 
+def test_gemm_of_the_fp32_family_whose_rows_tma_could_address(binding, monkeypatch):
+    """The kernel override of this module's descriptors holds for Gemm, too."""
+    A, B = (torch.randn(1024, 1024, generator=torch.Generator().manual_seed(s)) for s in (1, 2))
+    a, b = A.cuda(), B.cuda()
+    got, launches = _launches(binding, lambda: binding.onnx_gemm(a, b, transB=True))
+    want, S = oracle.gemm(A.numpy(), B.numpy(), None, transB=True)
+    assert launches == 2 and (np.abs(got.cpu().numpy() - want) <= REL * S + 1e-5).all()
+
+
 @pytest.mark.parametrize("tile", ["16,1", "48,1", "128,1", "64,2", "32,4", "16,8"])
 def test_gemm(binding, tile, monkeypatch):
     monkeypatch.setenv("ONNXB_FP32", "tc")
