@@ -9,7 +9,7 @@ in HBM; `e2e` repeats the measurement with host (pinned) inputs copied in and th
 outputs copied back inside the timed region.  `--impl reference` times the fp64
 CPU oracle on a bounded sample of the same workload.  The weights are constants of
 the graph, so their packed / TF32-rounded copies are made once at set-up
-(onnx_conv2d_prepack) and the timed region runs onnx_conv2d_run_prepacked;
+(onnx_conv2d_prepack) and the timed region runs onnx_conv2d_run_packed;
 `--repack` times onnx_conv2d_run instead, which redoes that copy at every call.
 With `--gpus N` and no launcher (WORLD_SIZE unset) the script starts its N ranks itself.
 

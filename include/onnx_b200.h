@@ -162,27 +162,33 @@ onnxb_status onnx_conv2d_add_run(onnxb_conv2d_desc_t desc, const float *X, const
                                  void *cuda_stream);
 
 /*
- * onnx_conv2d_prepack / onnx_conv2d_run_prepacked - for weights that are constants of the graph
+ * onnx_conv2d_prepack / onnx_conv2d_run_packed / onnx_conv2d_run_prepacked - for weights that are constants of the graph
  * (the usual case in inference; the compiler propagates constants ahead of time, Sec. 3.4.4):
  * the weight re-layout that onnx_conv2d_run performs at every call is done once.
  *
  * onnx_conv2d_prepack writes the derived copy of W that the descriptor's kernel reads (packed and
  * rounded to TF32 for ONNXB_KERNEL_MMA_IMPLICIT, rounded to TF32 for ONNXB_KERNEL_MMA_GEMM and
  * ONNXB_KERNEL_MMA_GATHER_GEMM, split into two TF32 parts for ONNXB_KERNEL_SIMT_DIRECT with filters
- * larger than 1x1 where its workspace_bytes is not 0) into `packed` (device, caller-owned, at least the
- * workspace_bytes of onnx_conv2d_desc_query, 16-byte aligned).  Other descriptors of the SIMT kernels
- * read W directly: the call then does nothing and returns OK, as it does for any of theirs when
- * `packed` is NULL (the run call then uses none).
- * onnx_conv2d_run_prepacked computes what onnx_conv2d_run (R == NULL) or onnx_conv2d_add_run
+ * larger than 1x1 where its workspace_bytes is not 0) into `packed` (device, caller-owned, at least
+ * onnx_conv2d_packed_bytes, which never exceeds the workspace_bytes of onnx_conv2d_desc_query; 16-byte
+ * aligned).  Where that is 0 the kernel reads W directly: the call then does nothing and returns OK, as it
+ * does for a descriptor of ONNXB_KERNEL_SIMT_DIRECT when `packed` is smaller or NULL.
+ * onnx_conv2d_run_packed computes what onnx_conv2d_run (R == NULL) or onnx_conv2d_add_run
  * (R != NULL) computes, from that copy, bit for bit.  W must still be passed (the kernels that use
- * no copy read it) and must be the tensor that was packed; `packed` is read only.  workspace /
- * workspace_bytes: as for onnx_conv2d_run for the SIMT kernels and for
- * ONNXB_KERNEL_MMA_GATHER_GEMM (whose gathered input still needs scratch: the queried
- * workspace_bytes always suffice), ignored (may be NULL / 0) otherwise.  Errors: as the calls they
+ * no copy read it, and those of ONNXB_KERNEL_SIMT_DIRECT where packed_bytes is less than their copy has)
+ * and must be the tensor that was packed; `packed` is read only.  workspace / workspace_bytes: as for
+ * onnx_conv2d_run where W is read and for ONNXB_KERNEL_MMA_GATHER_GEMM (whose gathered input still
+ * needs scratch: the queried workspace_bytes always suffice), ignored (may be NULL / 0) otherwise.
+ * onnx_conv2d_run_prepacked is the same without the size: every descriptor of a SIMT kernel reads W, whatever
+ * `packed` is, and the others take it to be as large as their copy.  Errors: as the calls they
  * stand for; ERR_WORKSPACE when `packed` is too small, ERR_NULL when it is missing where needed.
  */
+size_t onnx_conv2d_packed_bytes(onnxb_conv2d_desc_t desc);      /* host only; 0 for NULL */
 onnxb_status onnx_conv2d_prepack(onnxb_conv2d_desc_t desc, const float *W, void *packed, size_t packed_bytes,
                                  void *cuda_stream);
+onnxb_status onnx_conv2d_run_packed(onnxb_conv2d_desc_t desc, const float *X, const float *W, const void *packed,
+                                    size_t packed_bytes, const float *B, const float *R, float *Y, void *workspace,
+                                    size_t workspace_bytes, void *cuda_stream);
 onnxb_status onnx_conv2d_run_prepacked(onnxb_conv2d_desc_t desc, const float *X, const float *W, const void *packed,
                                        const float *B, const float *R, float *Y, void *workspace,
                                        size_t workspace_bytes, void *cuda_stream);

@@ -31,7 +31,8 @@ EXPORTS = [
     "onnxb_last_device_status", "onnxb_set_kernel_override", "onnxb_launch_count",
     "onnxb_probe_tf32_mma_rate", "onnx_matmul_add_run",
     "onnx_maxpool2d_shape", "onnx_maxpool2d_run", "onnx_global_average_pool_run", "onnx_conv2d_add_run",
-    "onnx_conv2d_prepack", "onnx_conv2d_run_prepacked", "onnxb_probe_wait_timeout",
+    "onnx_conv2d_prepack", "onnx_conv2d_run_prepacked", "onnx_conv2d_packed_bytes", "onnx_conv2d_run_packed",
+    "onnxb_probe_wait_timeout",
 ]
 
 
@@ -114,6 +115,10 @@ def load(build_if_missing: bool = True):
     lib.onnx_conv2d_add_run.argtypes = [vp, vp, vp, vp, vp, vp, vp, sz, vp]
     lib.onnx_conv2d_prepack.restype = ctypes.c_int
     lib.onnx_conv2d_prepack.argtypes = [vp, vp, vp, sz, vp]
+    lib.onnx_conv2d_packed_bytes.restype = sz
+    lib.onnx_conv2d_packed_bytes.argtypes = [vp]
+    lib.onnx_conv2d_run_packed.restype = ctypes.c_int
+    lib.onnx_conv2d_run_packed.argtypes = [vp, vp, vp, vp, sz, vp, vp, vp, vp, sz, vp]
     lib.onnx_conv2d_run_prepacked.restype = ctypes.c_int
     lib.onnx_conv2d_run_prepacked.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]
     lib.onnx_conv2d_run_static.restype = ctypes.c_int
@@ -233,12 +238,8 @@ class Conv2dDesc:
         self.pads = tuple(int(v) for v in p)
         self.workspace_bytes = int(ws.value)
         self.kernel_family = KERNEL_FAMILIES[self._lib.onnx_conv2d_desc_query_kernel(self._h)]
-        self._prepacked_needs_ws = bool(
-            (self.kernel_family == "mma_gather_gemm" or (self.kernel_family == "simt_direct" and tuple(w_shape[2:]) == (1, 1)))
-            and self.workspace_bytes)
-        # a copy of fewer bytes than this descriptor's is none of its own (one of the fp32 family kept from a time when that family
-        # made no copy, say): its fp32 kernels then read W
-        self._copy_bytes = self.workspace_bytes if self.kernel_family == "simt_direct" else 0
+        self.packed_bytes = int(self._lib.onnx_conv2d_packed_bytes(self._h))
+        self._packed_needs_ws = self.workspace_bytes > self.packed_bytes
         self._plan = None
 
     def _native(self, X, W, packed, B, R, Y, workspace, stream):
@@ -246,7 +247,7 @@ class Conv2dDesc:
         if self._plan is None:
             if not self._h:
                 return None
-            self._plan = _fast().plan(self._h.value, self.y_shape, self.workspace_bytes, self._prepacked_needs_ws)
+            self._plan = _fast().plan(self._h.value, self.y_shape, self.workspace_bytes, self.packed_bytes, self._packed_needs_ws)
         return _fast_mod.conv(self._plan, X, W, packed, B, R, Y, workspace, stream)
 
     def run(self, X, W, B=None, Y=None, workspace=None, stream=None):
@@ -285,30 +286,29 @@ class Conv2dDesc:
     def prepack(self, W, stream=None):
         """``onnx_conv2d_prepack``: the packed copy of constant weights (a uint8 device tensor; untouched when
         this descriptor's kernel reads W directly)."""
-        packed = _new(max(self.workspace_bytes, 16), W.device, stream, "uint8")
+        packed = _new(max(self.packed_bytes, 16), W.device, stream, "uint8")
         _check(self._lib.onnx_conv2d_prepack(self._h, _dev_ptr(W, "W"), ctypes.c_void_p(packed.data_ptr()),
                                              packed.numel(), _stream_ptr(stream)), "onnx_conv2d_prepack")
         return packed
 
     def run_prepacked(self, X, W, packed, B=None, R=None, Y=None, workspace=None, stream=None):
-        """``onnx_conv2d_run_prepacked``: run (R None) or run_add (R given) from a packed copy of W."""
-        if self._copy_bytes and packed is not None and packed.numel() * packed.element_size() < self._copy_bytes:
-            return self.run(X, W, B, Y, workspace, stream) if R is None else self.run_add(X, W, B, R, Y, workspace, stream)
+        """``onnx_conv2d_run_packed``: run (R None) or run_add (R given) from a packed copy of W."""
         if packed is not None:
             y = self._native(X, W, packed, B, R, Y, workspace, stream)
             if y is not None:
                 return y
         if Y is None:
             Y = _new(self.y_shape, X.device, stream)
-        if workspace is None and self._prepacked_needs_ws:
+        packed_len = packed.numel() * packed.element_size()
+        if workspace is None and self.workspace_bytes and (self._packed_needs_ws or packed_len < self.packed_bytes):
             workspace = _new(self.workspace_bytes, X.device, stream, "uint8", kept=False)
         ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
         ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
-        _check(self._lib.onnx_conv2d_run_prepacked(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
-                                                   ctypes.c_void_p(packed.data_ptr()),
-                                                   _dev_ptr(B, "B", allow_none=True), _dev_ptr(R, "R", allow_none=True),
-                                                   _dev_ptr(Y, "Y"), ws_ptr, ws_len, _stream_ptr(stream)),
-               "onnx_conv2d_run_prepacked")
+        _check(self._lib.onnx_conv2d_run_packed(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
+                                                ctypes.c_void_p(packed.data_ptr()), packed_len,
+                                                _dev_ptr(B, "B", allow_none=True), _dev_ptr(R, "R", allow_none=True),
+                                                _dev_ptr(Y, "Y"), ws_ptr, ws_len, _stream_ptr(stream)),
+               "onnx_conv2d_run_packed")
         return Y
 
     def run_static(self, X, W, B=None, Y=None, stream=None):

@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cstdint>
 
 #include "common.h"
 #include "tc_common.cuh"
@@ -213,34 +214,45 @@ extern "C" onnxb_status onnx_conv2d_add_run(onnxb_conv2d_desc_t d, const float *
 
 // Weights known ahead of the run (an inference graph's constants, Sec. 3.4.4): the implicit-GEMM
 // kernel's packing step done once, and run calls that take the packed copy instead of redoing it.
-// Whether the kernel keeps a derived copy of W in its scratch (packed, rounded to TF32 or split into TF32 parts).
-static bool has_weight_copy(onnxb_conv2d_desc_t d) {
-    return d->family == ONNXB_KERNEL_MMA_IMPLICIT || d->family == ONNXB_KERNEL_MMA_GEMM || d->family == ONNXB_KERNEL_MMA_GATHER_GEMM ||
-           d->fp32_tc == 1;
+// The copy of W (packed, rounded to TF32 or split into TF32 parts) is what the scratch holds, or the leading part of it (the
+// gather family's, next to the gathered input).
+extern "C" size_t onnx_conv2d_packed_bytes(onnxb_conv2d_desc_t d) {
+    if (!d) return 0;
+    if (d->family == ONNXB_KERNEL_MMA_GATHER_GEMM) return (size_t)d->g.M * d->g.C * 4;
+    return d->family == ONNXB_KERNEL_MMA_IMPLICIT || d->family == ONNXB_KERNEL_MMA_GEMM || d->fp32_tc == 1 ? d->workspace_bytes : 0;
 }
 
 extern "C" onnxb_status onnx_conv2d_prepack(onnxb_conv2d_desc_t d, const float *W, void *packed, size_t packed_bytes,
                                             void *cuda_stream) {
     if (!d || !W) return ONNXB_ERR_NULL;
-    if (!has_weight_copy(d) || (d->fp32_tc == 1 && !packed)) return ONNXB_OK;  // the other kernels read W as it is
-    // (the gather family's copy is only the rounded W, the leading part of its workspace)
-    const size_t need = d->family == ONNXB_KERNEL_MMA_GATHER_GEMM ? (size_t)d->g.M * d->g.C * 4 : d->workspace_bytes;
-    if (!packed || packed_bytes < need) return ONNXB_ERR_WORKSPACE;
+    const size_t need = onnx_conv2d_packed_bytes(d);
+    if (need == 0) return ONNXB_OK;                                       // the other kernels read W as it is
+    if (!packed || packed_bytes < need) return d->fp32_tc ? ONNXB_OK : ONNXB_ERR_WORKSPACE;      // (the fp32 kernels can)
     return conv2d_run_impl(d, nullptr, W, nullptr, nullptr, nullptr, packed, packed_bytes, cuda_stream, kTcConvPackOnly);
 }
 
-extern "C" onnxb_status onnx_conv2d_run_prepacked(onnxb_conv2d_desc_t d, const float *X, const float *W,
-                                                  const void *packed, const float *B, const float *R, float *Y,
-                                                  void *workspace, size_t workspace_bytes, void *cuda_stream) {
+extern "C" onnxb_status onnx_conv2d_run_packed(onnxb_conv2d_desc_t d, const float *X, const float *W, const void *packed,
+                                               size_t packed_bytes, const float *B, const float *R, float *Y, void *workspace,
+                                               size_t workspace_bytes, void *cuda_stream) {
     if (!d) return ONNXB_ERR_NULL;
-    if (!has_weight_copy(d) || (d->fp32_tc == 1 && !packed))
+    const size_t need = onnx_conv2d_packed_bytes(d);
+    if (need == 0 || (d->fp32_tc && (!packed || packed_bytes < need)))
         return conv2d_run_impl(d, X, W, B, R, Y, workspace, workspace_bytes, cuda_stream);
     if (!packed) return ONNXB_ERR_NULL;
+    if (packed_bytes < need) return ONNXB_ERR_WORKSPACE;
     if (d->family == ONNXB_KERNEL_MMA_GATHER_GEMM)      // the copy of W from `packed`, the gathered input in the workspace
         return conv2d_run_impl(d, X, W, B, R, Y, workspace, workspace_bytes, cuda_stream, kTcConvRunOnly,
                                static_cast<const float *>(packed));
-    // the packed copy stands in for the workspace; its size was checked when it was made
-    return conv2d_run_impl(d, X, W, B, R, Y, const_cast<void *>(packed), d->workspace_bytes, cuda_stream, kTcConvRunOnly);
+    // the packed copy stands in for the workspace
+    return conv2d_run_impl(d, X, W, B, R, Y, const_cast<void *>(packed), need, cuda_stream, kTcConvRunOnly);
+}
+
+// Not told the size of `packed`, which for a descriptor of the fp32 kernels may be no copy at all: these have only come to make
+// one, and a caller's `packed` is anything that was left untouched until then.
+extern "C" onnxb_status onnx_conv2d_run_prepacked(onnxb_conv2d_desc_t d, const float *X, const float *W,
+                                                  const void *packed, const float *B, const float *R, float *Y,
+                                                  void *workspace, size_t workspace_bytes, void *cuda_stream) {
+    return onnx_conv2d_run_packed(d, X, W, packed, d && d->fp32_tc ? 0 : SIZE_MAX, B, R, Y, workspace, workspace_bytes, cuda_stream);
 }
 
 // ONNX Gemm on the tensor cores reads rounded copies of both operands: the tensor core would otherwise

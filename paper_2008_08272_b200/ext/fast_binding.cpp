@@ -23,7 +23,7 @@ namespace {
 struct Abi {
     decltype(&onnx_conv2d_run) conv_run;
     decltype(&onnx_conv2d_add_run) conv_add_run;
-    decltype(&onnx_conv2d_run_prepacked) conv_run_prepacked;
+    decltype(&onnx_conv2d_run_packed) conv_run_packed;
     decltype(&onnx_gemm_workspace_bytes) gemm_workspace_bytes;
     decltype(&onnx_gemm_run) gemm_run;
     decltype(&onnx_maxpool2d_shape) maxpool2d_shape;
@@ -35,7 +35,8 @@ struct Plan {                    // what a convolution descriptor resolved to
     onnxb_conv2d_desc_t desc;
     int64_t y[4];
     size_t workspace;            // bytes onnx_conv2d_run needs
-    bool prepacked_needs_ws;     // onnx_conv2d_run_prepacked needs them too
+    size_t packed;               // bytes of the copy of W (0: none)
+    bool packed_needs_ws;        // onnx_conv2d_run_packed needs the workspace too
 };
 
 // An argument as the library takes it: nullptr for None; `fine` cleared when it is anything but a contiguous
@@ -113,7 +114,7 @@ PyObject *py_bind(PyObject *, PyObject *arg) {
     };
     get(abi.conv_run, "onnx_conv2d_run");
     get(abi.conv_add_run, "onnx_conv2d_add_run");
-    get(abi.conv_run_prepacked, "onnx_conv2d_run_prepacked");
+    get(abi.conv_run_packed, "onnx_conv2d_run_packed");
     get(abi.gemm_workspace_bytes, "onnx_gemm_workspace_bytes");
     get(abi.gemm_run, "onnx_gemm_run");
     get(abi.maxpool2d_shape, "onnx_maxpool2d_shape");
@@ -123,18 +124,18 @@ PyObject *py_bind(PyObject *, PyObject *arg) {
     Py_RETURN_NONE;
 }
 
-// plan(desc address, (n, m, p, q), workspace bytes, prepacked needs workspace) -> capsule
+// plan(desc address, (n, m, p, q), workspace bytes, packed bytes, whether a run from the copy needs workspace) -> capsule
 PyObject *py_plan(PyObject *, PyObject *args) {
-    unsigned long long desc, ws;
+    unsigned long long desc, ws, packed;
     long long y[4];
     int needs;
-    if (!PyArg_ParseTuple(args, "K(LLLL)Kp", &desc, &y[0], &y[1], &y[2], &y[3], &ws, &needs)) return nullptr;
-    Plan *p = new Plan{reinterpret_cast<onnxb_conv2d_desc_t>(desc), {y[0], y[1], y[2], y[3]}, (size_t)ws, needs != 0};
+    if (!PyArg_ParseTuple(args, "K(LLLL)KKp", &desc, &y[0], &y[1], &y[2], &y[3], &ws, &packed, &needs)) return nullptr;
+    Plan *p = new Plan{reinterpret_cast<onnxb_conv2d_desc_t>(desc), {y[0], y[1], y[2], y[3]}, (size_t)ws, (size_t)packed, needs != 0};
     return PyCapsule_New(p, "onnxb.plan", plan_free);
 }
 
 // conv(plan, X, W, packed, B, R, Y, workspace, stream): run (packed and R None), run_add (R given) or
-// run_prepacked (packed given)
+// run_packed (packed given)
 PyObject *py_conv(PyObject *, PyObject *const *a, Py_ssize_t n) {
     if (n != 9) return slow_path();
     Plan *p = plan_of(a[0]);
@@ -154,12 +155,12 @@ PyObject *py_conv(PyObject *, PyObject *const *a, Py_ssize_t n) {
         ym = new_tensor(p->y, at::kFloat, xt->device(), a[8], st, true);
         y = static_cast<float *>(ym.data_ptr());
     }
-    if (!ws && p->workspace && (!pre || p->prepacked_needs_ws)) {
+    if (!ws && p->workspace && (!pre || p->packed_needs_ws || packed_bytes < p->packed)) {
         wm = new_tensor({(int64_t)p->workspace}, at::kByte, xt->device(), a[8], st, false);
         ws = wm.data_ptr();
         ws_bytes = p->workspace;
     }
-    const onnxb_status s = pre ? abi.conv_run_prepacked(p->desc, x, w, packed, b, r, y, ws, ws_bytes, st)
+    const onnxb_status s = pre ? abi.conv_run_packed(p->desc, x, w, packed, packed_bytes, b, r, y, ws, ws_bytes, st)
                            : r ? abi.conv_add_run(p->desc, x, w, b, r, y, ws, ws_bytes, st)
                                : abi.conv_run(p->desc, x, w, b, y, ws, ws_bytes, st);
     return s == ONNXB_OK ? result(a[6], ym) : slow_path();

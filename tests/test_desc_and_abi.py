@@ -114,6 +114,26 @@ def test_pinned_fp32_gemm_is_on_the_tensor_cores_whatever_its_size(monkeypatch):
     assert binding.gemm_workspace_bytes(False, False, 1001, 1530, 777) == 0
 
 
+def test_copies_of_the_weights():
+    """A descriptor of the fp32 kernels takes any `packed`, or none, as before these made a copy; those that cannot do without
+    one refuse one too small.  (Host only: nothing here reaches a launch.)"""
+    lib, fake, before = binding.load(), ctypes.c_void_p(0x1000), binding.launch_count()
+    staged = binding.Conv2dDesc((4, 96, 75, 61), (192, 48, 3, 3), pads=(1, 1, 1, 1), group=2)
+    pixels = binding.Conv2dDesc((3, 2011, 23, 23), (1280, 2011, 1, 1))
+    for d in (staged, pixels):
+        assert d.kernel_family == "simt_direct" and d.workspace_bytes > 0
+        for packed, size in ((None, 0), (fake, 0), (fake, 16)):
+            assert lib.onnx_conv2d_prepack(d._h, fake, packed, size, None) == 0
+    assert staged.packed_bytes == staged.workspace_bytes and pixels.packed_bytes == 0
+    for x, w, kw in (((2, 64, 28, 28), (96, 64, 3, 3), {}), ((2, 64, 28, 28), (96, 64, 1, 1), {}), ((2, 64, 28, 28), (96, 64, 1, 1), dict(strides=(2, 2)))):
+        d = binding.Conv2dDesc(x, w, **kw)
+        assert 0 < d.packed_bytes <= d.workspace_bytes and d.kernel_family in binding.WEIGHT_COPY_FAMILIES
+        assert lib.onnx_conv2d_prepack(d._h, fake, fake, d.packed_bytes - 1, None) == 5
+        assert lib.onnx_conv2d_run_packed(d._h, fake, fake, fake, d.packed_bytes - 1, None, None, fake, fake, 1 << 30, None) == 5
+        assert lib.onnx_conv2d_run_packed(d._h, fake, fake, None, 0, None, None, fake, fake, 1 << 30, None) == 1
+    assert lib.onnx_conv2d_packed_bytes(None) == 0 and binding.launch_count() == before
+
+
 def test_gemm_workspace_is_that_of_the_family_the_override_leaves():
     split, rounded = 8 * 2 * 2048 * 2048, 4 * 2 * 2048 * 2048                # bytes: both operands, in two parts or rounded
     for family, want in ((None, rounded), ("mma_gemm", rounded), ("simt_direct", split)):

@@ -79,10 +79,15 @@ def test_conv(binding, c, tile, monkeypatch):
     assert torch.equal(d.run_prepacked(x, w, packed, b), got) and torch.equal(d.run_prepacked(x, w, packed, b, r), added)
     short = packed[:16]                                   # not this descriptor's copy: W is read instead
     assert torch.equal(d.run_prepacked(x, w, short, b), got) and torch.equal(d.run_prepacked(x, w, short, b, r), added)
-    # without a workspace: the kernel on the FMA units
+    assert packed.numel() == max(16, d.packed_bytes)
     y, stream = torch.empty_like(got), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     ptr = lambda t: ctypes.c_void_p(t.data_ptr())
-    assert binding.load().onnx_conv2d_run(d._h, ptr(x), ptr(w), ptr(b), ptr(y), None, 0, stream) == 0 and ok(y, want, S)
+    # the entry that is not told the copy's size: no byte of a pointer that may be no copy is read
+    wsp = torch.empty(d.workspace_bytes, dtype=torch.uint8, device="cuda")
+    assert binding.load().onnx_conv2d_run_prepacked(d._h, ptr(x), ptr(w), ptr(torch.zeros(16, dtype=torch.uint8, device="cuda")), ptr(b), None, ptr(y),
+                                                    ptr(wsp), wsp.numel(), stream) == 0 and torch.equal(y, got)
+    # without a workspace: the kernel on the FMA units
+    assert binding.load().onnx_conv2d_run(d._h, ptr(x), ptr(w), ptr(b), ptr(y.zero_()), None, 0, stream) == 0 and ok(y, want, S)
     assert binding.load().onnx_conv2d_prepack(d._h, ptr(w), None, 0, stream) == 0
     assert binding.last_device_status() == 0
 
