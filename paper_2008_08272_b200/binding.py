@@ -158,7 +158,10 @@ def load(build_if_missing: bool = True):
     return lib
 
 
-def _check(status: int, where: str):
+def _check(status: int, where: str, no_memory=None):
+    """``no_memory``: what stood in the way of a workspace (``_scratch``)."""
+    if no_memory is not None and STATUS_NAMES[status] == "ERR_WORKSPACE":
+        raise no_memory
     if status != OK:
         raise OnnxB200Error(status, where)
 
@@ -200,6 +203,23 @@ def _new(size, device, stream, dtype="float32", kept=True):
     if kept:
         t.record_stream(current)
     return t
+
+
+def _scratch(size, device, stream):
+    """A workspace of ``size`` bytes as (tensor, pointer, bytes, None), or where there is no memory for it (None, None, 0, the error):
+    the fp32 kernels do without, and for the others ``_check`` raises the error."""
+    import torch
+    try:
+        t = _new(size, device, stream, "uint8", kept=False)
+    except torch.OutOfMemoryError as e:
+        return None, None, 0, e.with_traceback(None)     # (whose frames would hold the caller's tensors)
+    return t, ctypes.c_void_p(t.data_ptr()), size, None
+
+
+def _given(workspace):
+    if workspace is None:
+        return None, None, 0, None
+    return workspace, ctypes.c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size(), None
 
 
 def make_attrs(x_shape, w_shape, *, kernel_shape=None, pads=None, strides=None, dilations=None, group=0,
@@ -257,13 +277,11 @@ class Conv2dDesc:
             return y
         if Y is None:
             Y = _new(self.y_shape, X.device, stream)
-        if workspace is None and self.workspace_bytes:
-            workspace = _new(self.workspace_bytes, X.device, stream, "uint8", kept=False)
-        ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
-        ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
+        needs = workspace is None and self.workspace_bytes
+        workspace, ws_ptr, ws_len, no_memory = _scratch(self.workspace_bytes, X.device, stream) if needs else _given(workspace)
         _check(self._lib.onnx_conv2d_run(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
                                          _dev_ptr(B, "B", allow_none=True), _dev_ptr(Y, "Y"),
-                                         ws_ptr, ws_len, _stream_ptr(stream)), "onnx_conv2d_run")
+                                         ws_ptr, ws_len, _stream_ptr(stream)), "onnx_conv2d_run", no_memory)
         return Y
 
     def run_add(self, X, W, B, R, Y=None, workspace=None, stream=None):
@@ -274,19 +292,23 @@ class Conv2dDesc:
                 return y
         if Y is None:
             Y = _new(self.y_shape, X.device, stream)
-        if workspace is None and self.workspace_bytes:
-            workspace = _new(self.workspace_bytes, X.device, stream, "uint8", kept=False)
-        ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
-        ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
+        needs = workspace is None and self.workspace_bytes
+        workspace, ws_ptr, ws_len, no_memory = _scratch(self.workspace_bytes, X.device, stream) if needs else _given(workspace)
         _check(self._lib.onnx_conv2d_add_run(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
                                              _dev_ptr(B, "B", allow_none=True), _dev_ptr(R, "R"), _dev_ptr(Y, "Y"),
-                                             ws_ptr, ws_len, _stream_ptr(stream)), "onnx_conv2d_add_run")
+                                             ws_ptr, ws_len, _stream_ptr(stream)), "onnx_conv2d_add_run", no_memory)
         return Y
 
     def prepack(self, W, stream=None):
         """``onnx_conv2d_prepack``: the packed copy of constant weights (a uint8 device tensor; untouched when
         this descriptor's kernel reads W directly)."""
-        packed = _new(max(self.packed_bytes, 16), W.device, stream, "uint8")
+        import torch
+        try:
+            packed = _new(max(self.packed_bytes, 16), W.device, stream, "uint8")
+        except torch.OutOfMemoryError:
+            if self.kernel_family != "simt_direct":      # (the fp32 kernels take W itself)
+                raise
+            packed = _new(16, W.device, stream, "uint8")
         _check(self._lib.onnx_conv2d_prepack(self._h, _dev_ptr(W, "W"), ctypes.c_void_p(packed.data_ptr()),
                                              packed.numel(), _stream_ptr(stream)), "onnx_conv2d_prepack")
         return packed
@@ -300,15 +322,13 @@ class Conv2dDesc:
         if Y is None:
             Y = _new(self.y_shape, X.device, stream)
         packed_len = packed.numel() * packed.element_size()
-        if workspace is None and self.workspace_bytes and (self._packed_needs_ws or packed_len < self.packed_bytes):
-            workspace = _new(self.workspace_bytes, X.device, stream, "uint8", kept=False)
-        ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
-        ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
+        needs = workspace is None and self.workspace_bytes and (self._packed_needs_ws or packed_len < self.packed_bytes)
+        workspace, ws_ptr, ws_len, no_memory = _scratch(self.workspace_bytes, X.device, stream) if needs else _given(workspace)
         _check(self._lib.onnx_conv2d_run_packed(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
                                                 ctypes.c_void_p(packed.data_ptr()), packed_len,
                                                 _dev_ptr(B, "B", allow_none=True), _dev_ptr(R, "R", allow_none=True),
                                                 _dev_ptr(Y, "Y"), ws_ptr, ws_len, _stream_ptr(stream)),
-               "onnx_conv2d_run_packed")
+               "onnx_conv2d_run_packed", no_memory)
         return Y
 
     def run_static(self, X, W, B=None, Y=None, stream=None):
@@ -370,14 +390,11 @@ def onnx_gemm(A, B, C=None, *, alpha=1.0, beta=1.0, transA=False, transB=False, 
         c_rank = C.dim()
         c_dims = (ctypes.c_int64 * max(c_rank, 1))(*[int(v) for v in C.shape])
     need = gemm_workspace_bytes(transA, transB, M, N, K)
-    if workspace is None and need:
-        workspace = _new(need, A.device, stream, "uint8", kept=False)
-    ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
-    ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
+    workspace, ws_ptr, ws_len, no_memory = _scratch(need, A.device, stream) if workspace is None and need else _given(workspace)
     _check(lib.onnx_gemm_run(int(bool(transA)), int(bool(transB)), float(alpha), float(beta), M, N, K,
                              _dev_ptr(A, "A"), _dev_ptr(B, "B"), _dev_ptr(C, "C", allow_none=True),
                              c_rank, c_dims, int(bool(fuse_relu)), _dev_ptr(Y, "Y"), ws_ptr, ws_len,
-                             _stream_ptr(stream)), "onnx_gemm_run")
+                             _stream_ptr(stream)), "onnx_gemm_run", no_memory)
     return Y
 
 
@@ -432,13 +449,10 @@ def onnx_matmul_add(A, B, C=None, *, fuse_relu=False, Y=None, workspace=None, st
         c_rank = C.dim()
         c_dims = (ctypes.c_int64 * max(c_rank, 1))(*[int(v) for v in C.shape])
     need = gemm_workspace_bytes(False, False, M, N, K)
-    if workspace is None and need:
-        workspace = _new(need, A.device, stream, "uint8", kept=False)
-    ws_ptr = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
-    ws_len = workspace.numel() * workspace.element_size() if workspace is not None else 0
+    workspace, ws_ptr, ws_len, no_memory = _scratch(need, A.device, stream) if workspace is None and need else _given(workspace)
     _check(lib.onnx_matmul_add_run(M, N, K, _dev_ptr(A, "A"), _dev_ptr(B, "B"), _dev_ptr(C, "C", allow_none=True),
                                    c_rank, c_dims, int(bool(fuse_relu)), _dev_ptr(Y, "Y"), ws_ptr, ws_len,
-                                   _stream_ptr(stream)), "onnx_matmul_add_run")
+                                   _stream_ptr(stream)), "onnx_matmul_add_run", no_memory)
     return Y
 
 
