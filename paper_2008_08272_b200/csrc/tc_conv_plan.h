@@ -185,6 +185,9 @@ ONNXB_HD inline void fp32_conv_segments(const Fp32ConvPlan &g, int rt, int grp, 
         at = t.at[i] + t.len[i] + 3;
     }
 }
+// Where a copy of X that has to reach element `last` (exclusive) ends: a whole number of 16-byte pieces, none past the x_whole
+// elements of X that are such pieces.  (The smaller of the two is rounded up: last + 3 may not fit an int.)
+ONNXB_HD inline int fp32_conv_copy_end(int last, int x_whole) { return ((last < x_whole ? last : x_whole) + 3) & ~3; }
 
 struct TcConvSegs {
     int n_first, nseg;

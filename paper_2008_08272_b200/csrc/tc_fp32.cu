@@ -399,7 +399,7 @@ tc_fp32_kernel(const __grid_constant__ Args g, unsigned int *err) {
                         const int last = e + segs->len[i];
                         from[k] = e & ~3;
                         to[k] = d - (e & 3);
-                        bytes[k] = (min((last + 3) & ~3, x_whole) - from[k]) * 4;
+                        bytes[k] = (fp32_conv_copy_end(last, x_whole) - from[k]) * 4;
                         if (last > x_whole)
                             for (int x = max(e, x_whole); x < x_end; ++x) stage[d + x - e] = __ldg(g.R + x);
                     }
