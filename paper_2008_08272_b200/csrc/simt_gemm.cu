@@ -445,7 +445,9 @@ struct Choice {
 // reduction, the FMA kernel's chain of additions does: relative to the result (2-norm, against 64 bits) split operands err by
 // 1.2 to 1.4e-7 up to some 1000 terms, the FMA kernel by 1.1e-7 where a CTA adds 35 terms, 1.5e-7 at 69, 2.1e-7 at 144.  So
 // the tensor cores are for what an FMA kernel's CTA would add some 60 terms of; and, with fewer, for problems of much work per
-// output tile (12,000 cycles' worth: 563 x 3424 x 27 16.5 us by FMA, 10 there; 5230 x 5956 x 33 stays).
+// output tile (12,000 cycles' worth: 4119 x 1513 x 56 33 us by FMA, 20 there; 5230 x 5956 x 33 stays).  One round of 128 x 128 tiles
+// of 17 to 32 terms also stays, by the estimates (563 x 3424 x 27: 10.6 us against 10.7; 15.2 and 9.7 measured), and is the more
+// exact for it (0.9e-7 against 1.3e-7).
 bool tc_is_as_exact(int M, int N, long long K, int groups, bool pixels, const Pick &fma) {
     if (K >= 64LL * fma.split - 8) return true;
     for (int bn = 16; bn <= 128 && bn <= (M + 15) / 16 * 16; bn += 16) {

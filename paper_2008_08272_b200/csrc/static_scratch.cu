@@ -4,8 +4,9 @@
 // a plugin hosted by a framework that owns the allocator, or a process whose device heap is
 // already fully reserved.  Whatever scratch the descriptor's kernel needs lives in a fixed
 // array inside the library image instead: the packed, TF32-rounded weights of the implicit-GEMM
-// kernel, the TF32-rounded weights of the 1x1 GEMM kernel, or the gathered input copy of the
-// gather-then-GEMM kernel.
+// kernel, the TF32-rounded weights of the 1x1 GEMM kernel, the gathered input copy of the
+// gather-then-GEMM kernel, or the split filters (of 1x1 layers: pixels and filters) of the fp32 tensor-core
+// kernel, whose layers of more than the array run on the FMA kernel.
 #include <cuda_runtime.h>
 
 #include <atomic>

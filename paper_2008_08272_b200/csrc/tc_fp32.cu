@@ -13,9 +13,9 @@
 // workspace (filters that are constants once, when they are packed), laid out as the tensor core reads them, so that
 // one bulk copy brings a block of 32 terms: split by the warps of every tile that reads them, through registers by
 // 4-byte loads, the same blocks took 1800 to 3100 cycles against the 768 of their MMAs.  The pixels of a convolution are
-// split by six warps on their way into shared memory, ONCE for all taps of a filter: a tile is a grid of pixels with its
-// halo (16 rows of 8, or 128 consecutive pixels of narrow images), one 16-byte row per pixel and four channels, and a
-// tap reads the same grid from another start (plan of the slot grid: conv_fp32_plan).  The MMA's rows are the pixels, or
+// split by five warps on their way into shared memory, ONCE for all taps of a filter: a tile is 128 consecutive slots of the
+// padded images with the halo behind them, one 16-byte row per slot and four channels, and a tap reads the same rows from
+// another start (plan of the slots: conv_plan_axis, fill, fill_steps).  The MMA's rows are the pixels, or
 // the columns of Gemm (what is contiguous in Y: TMEM lanes then store consecutive addresses), its columns the
 // channels, or the rows of Gemm.
 //
