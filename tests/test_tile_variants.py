@@ -97,15 +97,22 @@ def test_gemm_addend_forms(binding, cs, monkeypatch):
     for M, N, K in ((300, 332, 96), (300, 330, 96), (20, 37, 64)):
         A, B = rng.standard_normal((M, K)).astype(np.float32), rng.standard_normal((N, K)).astype(np.float32)
         C = rng.standard_normal([{"M": M, "N": N}.get(d, d) for d in cs]).astype(np.float32)
-        got = run_gemm_gpu(binding, torch, A, B, C, transB=True, alpha=0.5, beta=-1.5, fuse_relu=True)
+        before = binding.launch_count()
+        binding.set_kernel_override("mma_gemm")                 # else the dot-product kernel takes the last one
+        try:
+            got = run_gemm_gpu(binding, torch, A, B, C, transB=True, alpha=0.5, beta=-1.5, fuse_relu=True)
+        finally:
+            binding.set_kernel_override(None)
+        assert binding.launch_count() == before + 2             # operands rounded by a launch in front: not the split form
         want, S = oracle.gemm(A, B, C, transB=True, alpha=0.5, beta=-1.5, relu=True)
         assert worst_ratio(got, want, S) <= 1.0, (M, N)
 
 
 @pytest.mark.parametrize("tA,tB", [(False, True), (True, False)])
 @pytest.mark.parametrize("M,N,K", [(640, 640, 1280), (704, 304, 2640), (144, 176, 4784)])
-def test_gemm_rounded_ahead_of_the_split(binding, M, N, K, tA, tB):
-    """Problems whose operands are rounded by a launch of their own and whose tiles are then shared by clusters."""
+def test_gemm_rounded_ahead_of_the_split(binding, M, N, K, tA, tB, monkeypatch):
+    """Problems whose operands are rounded by a launch of their own and then go to the split kernel: the first one's tiles to a CTA
+    each, the others' to clusters."""
     rng = np.random.default_rng(M)
     A = rng.standard_normal((K, M) if tA else (M, K)).astype(np.float32)
     B = rng.standard_normal((N, K) if tB else (K, N)).astype(np.float32)
@@ -115,3 +122,6 @@ def test_gemm_rounded_ahead_of_the_split(binding, M, N, K, tA, tB):
     assert binding.launch_count() == before + 2
     want, S = oracle.gemm(A, B, C, transA=tA, transB=tB, alpha=0.5, beta=-1.5)
     assert worst_ratio(got, want, S) <= 1.0
+    monkeypatch.setenv("ONNXB_GEMM_SPLITK", "0")                # the persistent kernel, also with a launch in front: a sum in one piece
+    whole = run_gemm_gpu(binding, torch, A, B, C, transA=tA, transB=tB, alpha=0.5, beta=-1.5)
+    assert np.array_equal(whole, got) == (K == 1280)
