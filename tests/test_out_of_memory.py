@@ -9,17 +9,26 @@ torch = pytest.importorskip("torch")
 from paper_2008_08272_b200 import binding  # noqa: E402
 
 
+ENOUGH = 20 << 20           # bytes that a call here needs and does not get
+
+
 @pytest.fixture
 def launches_without_memory():
-    """launches(call): those of a call for which the allocator has little more than it holds already."""
+    """launches(call): those of a call for which the allocator has no block of ENOUGH bytes: neither new ones nor, in what it holds,
+    parts that earlier tensors have left."""
     def launches(call):
         torch.cuda.synchronize()
         torch.cuda.empty_cache()
         total, before = torch.cuda.get_device_properties(0).total_memory, binding.launch_count()
         torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (8 << 20)) / total)
+        taken = []
         try:
+            with pytest.raises(torch.OutOfMemoryError):
+                while True:
+                    taken.append(torch.empty(ENOUGH, dtype=torch.uint8, device="cuda"))
             call()
         finally:
+            del taken
             torch.cuda.set_per_process_memory_fraction(1.0)
         return binding.launch_count() - before
     return launches
@@ -31,7 +40,7 @@ def _same(got, want):
 
 def test_fp32_gemm(launches_without_memory):
     A, B, Y, want = (torch.randn(s, device="cuda") for s in ((3001, 1001), (1001, 2999), (3001, 2999), (3001, 2999)))
-    assert binding.gemm_workspace_bytes(False, False, 3001, 2999, 1001) > 20 << 20      # more than a block that happens to be free
+    assert binding.gemm_workspace_bytes(False, False, 3001, 2999, 1001) > ENOUGH
     binding.onnx_gemm(A, B, Y=want)
     for call in (binding.onnx_gemm, binding.onnx_matmul_add):
         assert launches_without_memory(lambda: call(A, B, Y=Y.zero_())) == 1 and _same(Y, want)
@@ -41,7 +50,7 @@ def test_fp32_gemm(launches_without_memory):
                          ids=["packed pixels", "staged"])
 def test_fp32_conv(launches_without_memory, xs, ws, kw):
     d = binding.Conv2dDesc(xs, ws, **kw)
-    assert d.kernel_family == "simt_direct" and d.workspace_bytes > 20 << 20
+    assert d.kernel_family == "simt_direct" and d.workspace_bytes > ENOUGH
     X, W, R, Y, want, added = (torch.randn(s, device="cuda") for s in (xs, ws) + (d.y_shape,) * 4)
     d.run(X, W, Y=want)
     d.run_add(X, W, None, R, Y=added)
