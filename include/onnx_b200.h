@@ -215,7 +215,8 @@ void onnx_conv2d_desc_destroy(onnxb_conv2d_desc_t desc);
  * All calls on a device share the one array, and it keeps whatever the previous call left
  * there.  Each call overwrites all of the scratch it later reads, so stale contents are
  * harmless, but two calls whose kernels may overlap on the GPU (different streams, or
- * several host threads) race on it: serialise them, e.g. by using one stream.
+ * several host threads) race on it: serialise them, e.g. by using one stream.  Only
+ * descriptors whose queried workspace_bytes is 0, whatever their family, use none of it.
  * Errors: as onnx_conv2d_run, plus ONNXB_ERR_WORKSPACE as described above.
  */
 onnxb_status onnx_conv2d_run_static(onnxb_conv2d_desc_t desc, const float *X, const float *W,
