@@ -193,6 +193,22 @@ onnxb_status onnx_conv2d_run_prepacked(onnxb_conv2d_desc_t desc, const float *X,
                                        const float *B, const float *R, float *Y, void *workspace,
                                        size_t workspace_bytes, void *cuda_stream);
 
+/*
+ * onnx_conv2d_run_packed_sampled - onnx_conv2d_run_packed with an addend that is read at every
+ * r_strides[0]-th row and r_strides[1]-th column of images of r_dims[0] x r_dims[1]: R is [N, M, r_dims[0], r_dims[1]],
+ * and Y = relu?( Conv(X, W) + B + R[:, :, ::r_strides[0], ::r_strides[1]] ).  For a residual connection across a block that
+ * is computed only at the places a following strided 1x1 convolution reads.  Y_rounded (may be NULL), laid out like Y: a second
+ * output, Y rounded to TF32 (nearest), for tensor-core layers of unit stride to read (which would truncate Y where a strided one
+ * rounds it).
+ * Errors: as onnx_conv2d_run_packed; ERR_NULL when R, r_dims or r_strides is; ERR_SHAPE when the places read are not
+ * P x Q; ERR_UNSUPPORTED for descriptors other than of ONNXB_KERNEL_MMA_GEMM and ONNXB_KERNEL_MMA_GATHER_GEMM (those of
+ * group-1, unpadded 1x1 convolutions of 32 channels and more), and for an R of 2^31 elements and more.
+ */
+onnxb_status onnx_conv2d_run_packed_sampled(onnxb_conv2d_desc_t desc, const float *X, const float *W, const void *packed,
+                                            size_t packed_bytes, const float *B, const float *R, const int64_t r_dims[2],
+                                            const int64_t r_strides[2], float *Y, float *Y_rounded, void *workspace,
+                                            size_t workspace_bytes, void *cuda_stream);
+
 void onnx_conv2d_desc_destroy(onnxb_conv2d_desc_t desc);
 
 /*

@@ -32,6 +32,7 @@ EXPORTS = [
     "onnxb_probe_tf32_mma_rate", "onnx_matmul_add_run",
     "onnx_maxpool2d_shape", "onnx_maxpool2d_run", "onnx_global_average_pool_run", "onnx_conv2d_add_run",
     "onnx_conv2d_prepack", "onnx_conv2d_run_prepacked", "onnx_conv2d_packed_bytes", "onnx_conv2d_run_packed",
+    "onnx_conv2d_run_packed_sampled",
     "onnxb_probe_wait_timeout",
 ]
 
@@ -119,6 +120,9 @@ def load(build_if_missing: bool = True):
     lib.onnx_conv2d_packed_bytes.argtypes = [vp]
     lib.onnx_conv2d_run_packed.restype = ctypes.c_int
     lib.onnx_conv2d_run_packed.argtypes = [vp, vp, vp, vp, sz, vp, vp, vp, vp, sz, vp]
+    lib.onnx_conv2d_run_packed_sampled.restype = ctypes.c_int
+    lib.onnx_conv2d_run_packed_sampled.argtypes = [vp, vp, vp, vp, sz, vp, vp, ctypes.POINTER(i64), ctypes.POINTER(i64),
+                                                   vp, vp, vp, sz, vp]
     lib.onnx_conv2d_run_prepacked.restype = ctypes.c_int
     lib.onnx_conv2d_run_prepacked.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]
     lib.onnx_conv2d_run_static.restype = ctypes.c_int
@@ -262,13 +266,13 @@ class Conv2dDesc:
         self._packed_needs_ws = self.workspace_bytes > self.packed_bytes
         self._plan = None
 
-    def _native(self, X, W, packed, B, R, Y, workspace, stream):
+    def _native(self, X, W, packed, B, R, Y, workspace, stream, *sampled):
         """The call through the native path; None when it declined."""
         if self._plan is None:
             if not self._h:
                 return None
             self._plan = _fast().plan(self._h.value, self.y_shape, self.workspace_bytes, self.packed_bytes, self._packed_needs_ws)
-        return _fast_mod.conv(self._plan, X, W, packed, B, R, Y, workspace, stream)
+        return _fast_mod.conv(self._plan, X, W, packed, B, R, Y, workspace, stream, *sampled)
 
     def run(self, X, W, B=None, Y=None, workspace=None, stream=None):
         """``onnx_conv2d_run``; allocates Y (and a workspace) with torch when not supplied."""
@@ -329,6 +333,26 @@ class Conv2dDesc:
                                                 _dev_ptr(B, "B", allow_none=True), _dev_ptr(R, "R", allow_none=True),
                                                 _dev_ptr(Y, "Y"), ws_ptr, ws_len, _stream_ptr(stream)),
                "onnx_conv2d_run_packed", no_memory)
+        return Y
+
+    def run_prepacked_sampled(self, X, W, packed, B, R, strides, Y=None, Y_rounded=None, workspace=None, stream=None):
+        """``onnx_conv2d_run_packed_sampled``: run_prepacked with the addend R[:, :, ::strides[0], ::strides[1]]; Y rounded to TF32
+        goes to ``Y_rounded`` where it is given."""
+        if R.dim() != 4 or tuple(R.shape[:2]) != self.y_shape[:2]:
+            raise OnnxB200Error(3, "run_prepacked_sampled: the addend's images and channels are not the output's")
+        y = self._native(X, W, packed, B, R, Y, workspace, stream, strides, Y_rounded)
+        if y is not None:
+            return y
+        if Y is None:
+            Y = _new(self.y_shape, X.device, stream)
+        needs = workspace is None and self.workspace_bytes and self._packed_needs_ws
+        workspace, ws_ptr, ws_len, no_memory = _scratch(self.workspace_bytes, X.device, stream) if needs else _given(workspace)
+        _check(self._lib.onnx_conv2d_run_packed_sampled(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
+                                                        ctypes.c_void_p(packed.data_ptr()), packed.numel() * packed.element_size(),
+                                                        _dev_ptr(B, "B", allow_none=True), _dev_ptr(R, "R"),
+                                                        _i64(R.shape[2:], 2), _i64(strides, 2), _dev_ptr(Y, "Y"),
+                                                        _dev_ptr(Y_rounded, "Y_rounded", allow_none=True), ws_ptr, ws_len, _stream_ptr(stream)),
+               "onnx_conv2d_run_packed_sampled", no_memory)
         return Y
 
     def run_static(self, X, W, B=None, Y=None, stream=None):

@@ -140,11 +140,27 @@ size_t conv_gather_workspace_bytes(const ConvGeom &g) {
 
 static inline bool misaligned(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
 
+// An addend that is read at every sh-th row and sw-th column of images of H x W.
+struct SampledAddend {
+    int H, W, sh, sw;
+    float *Y_rounded;
+};
+static TcGemmProblem sample(TcGemmProblem t, const ConvGeom &g, const SampledAddend *a) {
+    if (a) {
+        t.r_q = g.Q;
+        t.r_ld = (long long)a->H * a->W; t.r_bs = t.r_ld * g.M;
+        t.r_row = a->sh * a->W; t.r_col = a->sw;
+        t.Y_rounded = a->Y_rounded;
+    }
+    return t;
+}
+
 // w_copy (gather family only): a TF32-rounded copy of W made earlier by onnx_conv2d_prepack; the workspace
 // then only has to hold the gathered input.
 static onnxb_status conv2d_run_impl(onnxb_conv2d_desc_t d, const float *X, const float *W, const float *B,
                                     const float *R, float *Y, void *workspace, size_t workspace_bytes,
-                                    void *cuda_stream, int phase = kTcConvPackAndRun, const float *w_copy = nullptr) {
+                                    void *cuda_stream, int phase = kTcConvPackAndRun, const float *w_copy = nullptr,
+                                    const SampledAddend *sampled = nullptr) {
     const bool pack_only = phase == kTcConvPackOnly;
     if (!d || !W || (!pack_only && (!X || !Y))) return ONNXB_ERR_NULL;
     if (misaligned(R)) return ONNXB_ERR_UNSUPPORTED;
@@ -173,7 +189,7 @@ static onnxb_status conv2d_run_impl(onnxb_conv2d_desc_t d, const float *X, const
             float *Wr = static_cast<float *>(workspace);
             err = 0;
             if (phase != kTcConvRunOnly) err = launch_round_tf32_copy(W, Wr, (long long)d->g.M * d->g.C, nullptr, nullptr, 0, cuda_stream);
-            if (err == 0 && phase != kTcConvPackOnly) err = launch_tc_gemm(conv1x1_as_gemm(d->g, X, Wr, B, Y, R), cuda_stream);
+            if (err == 0 && phase != kTcConvPackOnly) err = launch_tc_gemm(sample(conv1x1_as_gemm(d->g, X, Wr, B, Y, R), d->g, sampled), cuda_stream);
             break;
         }
         case ONNXB_KERNEL_MMA_GATHER_GEMM: {
@@ -185,7 +201,7 @@ static onnxb_status conv2d_run_impl(onnxb_conv2d_desc_t d, const float *X, const
             if (!w_copy) err = launch_round_tf32_copy(W, ws, (long long)d->g.M * d->g.C, nullptr, nullptr, 0, cuda_stream);
             if (pack_only) break;
             if (err == 0) err = launch_gather1x1(d->g, X, Xg, gather_pitch(d->g), gather_merged(d->g), cuda_stream);
-            if (err == 0) err = launch_tc_gemm(conv1x1_gathered_as_gemm(d->g, Xg, Wr, B, Y, R), cuda_stream);
+            if (err == 0) err = launch_tc_gemm(sample(conv1x1_gathered_as_gemm(d->g, Xg, Wr, B, Y, R), d->g, sampled), cuda_stream);
             break;
         }
         case ONNXB_KERNEL_MMA_IMPLICIT:
@@ -231,9 +247,9 @@ extern "C" onnxb_status onnx_conv2d_prepack(onnxb_conv2d_desc_t d, const float *
     return conv2d_run_impl(d, nullptr, W, nullptr, nullptr, nullptr, packed, packed_bytes, cuda_stream, kTcConvPackOnly);
 }
 
-extern "C" onnxb_status onnx_conv2d_run_packed(onnxb_conv2d_desc_t d, const float *X, const float *W, const void *packed,
-                                               size_t packed_bytes, const float *B, const float *R, float *Y, void *workspace,
-                                               size_t workspace_bytes, void *cuda_stream) {
+static onnxb_status run_packed(onnxb_conv2d_desc_t d, const float *X, const float *W, const void *packed, size_t packed_bytes,
+                               const float *B, const float *R, float *Y, void *workspace, size_t workspace_bytes,
+                               void *cuda_stream, const SampledAddend *sampled = nullptr) {
     if (!d) return ONNXB_ERR_NULL;
     const size_t need = onnx_conv2d_packed_bytes(d);
     if (need == 0 || (d->fp32_tc && (!packed || packed_bytes < need)))
@@ -242,9 +258,32 @@ extern "C" onnxb_status onnx_conv2d_run_packed(onnxb_conv2d_desc_t d, const floa
     if (packed_bytes < need) return ONNXB_ERR_WORKSPACE;
     if (d->family == ONNXB_KERNEL_MMA_GATHER_GEMM)      // the copy of W from `packed`, the gathered input in the workspace
         return conv2d_run_impl(d, X, W, B, R, Y, workspace, workspace_bytes, cuda_stream, kTcConvRunOnly,
-                               static_cast<const float *>(packed));
+                               static_cast<const float *>(packed), sampled);
     // the packed copy stands in for the workspace
-    return conv2d_run_impl(d, X, W, B, R, Y, const_cast<void *>(packed), need, cuda_stream, kTcConvRunOnly);
+    return conv2d_run_impl(d, X, W, B, R, Y, const_cast<void *>(packed), need, cuda_stream, kTcConvRunOnly, nullptr, sampled);
+}
+
+extern "C" onnxb_status onnx_conv2d_run_packed(onnxb_conv2d_desc_t d, const float *X, const float *W, const void *packed,
+                                               size_t packed_bytes, const float *B, const float *R, float *Y, void *workspace,
+                                               size_t workspace_bytes, void *cuda_stream) {
+    return run_packed(d, X, W, packed, packed_bytes, B, R, Y, workspace, workspace_bytes, cuda_stream);
+}
+
+// The addend read at every other place, say: a residual connection across a block whose output is only computed there.
+extern "C" onnxb_status onnx_conv2d_run_packed_sampled(onnxb_conv2d_desc_t d, const float *X, const float *W, const void *packed,
+                                                       size_t packed_bytes, const float *B, const float *R,
+                                                       const int64_t *r_dims, const int64_t *r_strides, float *Y, float *Y_rounded,
+                                                       void *workspace, size_t workspace_bytes, void *cuda_stream) {
+    if (!d || !R || !r_dims || !r_strides) return ONNXB_ERR_NULL;
+    if (d->family != ONNXB_KERNEL_MMA_GEMM && d->family != ONNXB_KERNEL_MMA_GATHER_GEMM) return ONNXB_ERR_UNSUPPORTED;
+    const int64_t out[2] = {d->g.P, d->g.Q};
+    for (int i = 0; i < 2; ++i)
+        if (r_dims[i] < 1 || r_strides[i] < 1 || r_dims[i] > 2147483647LL || (r_dims[i] - 1) / r_strides[i] + 1 != out[i]) return ONNXB_ERR_SHAPE;
+    if (misaligned(Y_rounded) || r_strides[0] > 2147483647LL || r_strides[1] > 2147483647LL || r_dims[0] * r_dims[1] > 2147483647LL / d->g.M / d->g.N)
+        return ONNXB_ERR_UNSUPPORTED;
+    // (a stride that reads no second row or column is as good as that dimension's length)
+    const SampledAddend a{(int)r_dims[0], (int)r_dims[1], (int)std::min(r_strides[0], r_dims[0]), (int)std::min(r_strides[1], r_dims[1]), Y_rounded};
+    return run_packed(d, X, W, packed, packed_bytes, B, R, Y, workspace, workspace_bytes, cuda_stream, &a);
 }
 
 // Not told the size of `packed`, which for a descriptor of the fp32 kernels may be no copy at all: these have only come to make

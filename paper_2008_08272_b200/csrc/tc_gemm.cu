@@ -67,6 +67,11 @@ struct Params {
     const float *row_bias;     // optional per-row addend (convolution bias)
     const float *R;            // optional addend laid out exactly like Y (a residual connection, or Gemm's whole C), scaled and
     float r_scale;             // added before Relu
+    int r_q;                   // R sampled: see TcGemmProblem
+    int r_row, r_col;
+    float *Yr;                 // Y rounded to TF32, a second output (by tmR where Y is stored by TMA), or NULL
+    long long r_ld, r_bs;      // R's planes and images are that far apart
+    ConvDivisor dv_rq, dv_split;
     int r_tma;                 // R is fetched by TMA (when Y is stored by TMA: same geometry), r_bufs blocks ahead
     int r_bufs;                // 1 or 2 blocks of R in flight per epilogue warp
     uint32_t staging_bytes;    // Y staging blocks, plus the R blocks when r_tma
@@ -392,7 +397,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         }
                     } else if (!kC) {
                         // Residual addend R, laid out like Y.  A lane owns a ROW of the block, but rows are
-                        // far apart in memory, so the block is fetched the other way round: lane = column,
+                        // far apart in memory (and TMA cannot step over places of a sampled R, a stride of the
+                        // innermost dimension), so the block is fetched the other way round: lane = column,
                         // one coalesced 128-byte read per row, parked in the warp's staging buffer (same
                         // swizzle as the Y block that follows it there) and read back a row per lane.
 #pragma unroll
@@ -401,18 +407,22 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         __syncwarp();
                         {
                             const int col = col0 + lane;
-                            long long coff = col;
+                            int pix = col, image = b;
                             if (p.y_split > 0) {
-                                const int grp = col / p.y_split;
-                                coff = (long long)grp * p.y_group + (col - grp * p.y_split);
+                                image = conv_fdiv(col, p.y_split, p.dv_split);
+                                pix = col - image * p.y_split;
                             }
-                            const float *rp = p.R + b * p.y_sb + (long long)row0 * p.y_ld + coff;
+                            if (p.r_q > 0) {
+                                const int pr = conv_fdiv(pix, p.r_q, p.dv_rq);
+                                pix = pr * p.r_row + (pix - pr * p.r_q) * p.r_col;
+                            }
+                            const float *rp = p.R + image * p.r_bs + (long long)row0 * p.r_ld + pix;
                             const int rows = min(32, p.M - row0);
                             float t[32];
 #pragma unroll
                             for (int r = 0; r < 32; ++r) {
                                 t[r] = (r < rows && col < p.N) ? __ldg(rp) : 0.f;
-                                rp += p.y_ld;
+                                rp += p.r_ld;
                             }
 #pragma unroll
                             for (int r = 0; r < 32; ++r)
@@ -470,6 +480,22 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                             tma_store_commit();
                         }
                         GP_MARK(5);
+                        if (!kC && p.Yr) {
+                            if (lane == 0) tma_store_wait_read<0>();
+                            __syncwarp();
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) {
+                                float4 *at = reinterpret_cast<float4 *>(buf + lane * 128 + ((c ^ (lane & 7)) << 4));
+                                const float4 val = *at;
+                                *at = make_float4(round_tf32(val.x), round_tf32(val.y), round_tf32(val.z), round_tf32(val.w));
+                            }
+                            fence_proxy_async_smem();
+                            __syncwarp();
+                            if (lane == 0) {
+                                tma_store_3d(&tmR, buf, col0, row0, b);
+                                tma_store_commit();
+                            }
+                        }
                     } else {
                         // Y rows cannot be described to TMA (row pitch not a multiple of 16 bytes): read the
                         // block back transposed, lanes along the columns, and store row by row (coalesced).
@@ -486,6 +512,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                             const float val = *reinterpret_cast<const float *>(
                                 buf + r * 128 + ((((lane >> 2) ^ (r & 7)) << 4) | ((lane & 3) << 2)));
                             if (col < p.N) *yp = val;
+                            if (!kC && p.Yr && col < p.N) p.Yr[yp - p.Y] = round_tf32(val);
                             yp += p.y_ld;
                         }
                         __syncwarp();
@@ -689,7 +716,12 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     const bool whole_c = g.C && g.c_si != 0 && g.c_sj != 0;
     p.R = whole_c ? g.C : g.C ? nullptr : g.residual;
     p.r_scale = whole_c ? g.beta : 1.f;
-    p.r_tma = p.R != nullptr && p.y_tma;
+    p.r_q = p.R ? g.r_q : 0; p.r_row = g.r_row; p.r_col = g.r_col; p.Yr = p.r_q ? g.Y_rounded : nullptr;
+    p.r_ld = p.r_q ? g.r_ld : g.y_ld;
+    p.r_bs = p.r_q ? g.r_bs : g.y_split > 0 ? g.y_group_stride : g.y_bs;
+    p.dv_rq = conv_divisor(std::max(p.r_q, 1));
+    p.dv_split = conv_divisor(std::max(g.y_split, 1));
+    p.r_tma = p.R != nullptr && p.y_tma && !p.r_q;
     // two blocks of R per epilogue warp when the operand ring keeps at least three stages beside them
     p.r_bufs = kResidualBufs;
     if ((kSmemLimit - 1024 - kBarrierBytes - kStagingBytes * (1 + kResidualBufs)) / (int)p.stage_bytes < 3) p.r_bufs = 1;
@@ -751,6 +783,12 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
         tmY = tmA;   // never dereferenced
     }
     tmR = tmY;
+    if (p.Yr && p.y_tma) {
+        uint64_t dims[3] = {(uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.batch};
+        uint64_t str[2] = {(uint64_t)g.y_ld * 4, g.batch > 1 ? (uint64_t)g.y_bs * 4 : (uint64_t)g.y_ld * 4 * g.M};
+        uint32_t box[3] = {32, 32, 1};
+        if (!make_tmap(&tmR, p.Yr, 3, dims, str, box, kTmapSwizzle128)) return (int)cudaErrorInvalidValue;
+    }
     if (p.r_tma) {
         // the addend has Y's shape and strides, so its view is Y's with another base
         uint64_t dims[3] = {(uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.batch};

@@ -53,6 +53,10 @@ struct SkParams {
     const float *C, *row_bias, *R;
     long long c_si, c_sj;
     int relu, vec;             // vec: four columns per access (rows of Y, R and C are 16-byte aligned)
+    int r_q, r_row, r_col;     // R sampled: see TcGemmProblem
+    float *Yr;
+    long long r_ld, r_bs;
+    ConvDivisor dv_rq;
     float *Y;
     long long y_ld, y_bs;
     int y_split;               // > 0: column j lies in group j / y_split, y_group elements further on
@@ -275,6 +279,13 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     if (gcol + e < p.N) add[e] = p.beta * __ldg(p.C + (long long)grow * p.c_si + (long long)(gcol + e) * p.c_sj);
+            } else if (p.R && p.r_q) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int j = gcol + e, im = p.y_split ? conv_fdiv(j, p.y_split, p.dv_split) : batch, pix = p.y_split ? j - im * p.y_split : j;
+                    const int pr = conv_fdiv(pix, p.r_q, p.dv_rq);
+                    if (j < p.N) add[e] = __ldg(p.R + im * p.r_bs + grow * p.r_ld + pr * p.r_row + (pix - pr * p.r_q) * p.r_col);
+                }
             } else if (p.R) {
                 if (p.vec) {
                     const float4 r = __ldg(reinterpret_cast<const float4 *>(p.R + yi[0]));
@@ -301,6 +312,11 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             if (p.relu) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) o[e] = fmaxf(o[e], 0.f);
+            }
+            if (p.Yr) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (gcol + e < p.N) p.Yr[yi[e]] = round_tf32(o[e]);
             }
             if (p.vec) {
                 *reinterpret_cast<float4 *>(p.Y + yi[0]) = make_float4(o[0], o[1], o[2], o[3]);
@@ -469,6 +485,9 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
     p.C = g.C; p.c_si = g.c_si; p.c_sj = g.c_sj;
     p.row_bias = g.row_bias;
     p.R = g.C ? nullptr : g.residual;
+    p.r_q = p.R ? g.r_q : 0; p.r_row = g.r_row; p.r_col = g.r_col; p.Yr = p.r_q ? g.Y_rounded : nullptr;
+    p.r_ld = g.r_ld; p.r_bs = g.r_bs;
+    p.dv_rq = conv_divisor(std::max(p.r_q, 1));
     p.relu = g.relu;
     p.Y = g.Y; p.y_ld = g.y_ld; p.y_bs = g.y_bs;
     p.y_split = g.y_split; p.y_group = g.y_group_stride;

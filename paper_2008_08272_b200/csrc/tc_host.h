@@ -23,6 +23,12 @@ struct TcGemmProblem {
     long long c_si, c_sj;
     const float *row_bias;
     const float *residual;   // optional addend with Y's own layout, added before Relu (ignored when C is given)
+    // A residual read at every r_col-th place of every so-many-th row of its own images instead (r_q > 0: pixels in a row of the
+    // output): planes r_ld elements apart, images r_bs, the rows that are read r_row, the places r_col.
+    int r_q;
+    long long r_ld, r_bs;
+    int r_row, r_col;
+    float *Y_rounded;        // (with r_q) a second output, laid out like Y: Y rounded to TF32; may be NULL
     int relu;
     int round_operands;      // A and B are raw fp32: the split-K form rounds them itself, the other form is given copies
     float *Y;

@@ -24,6 +24,7 @@ struct Abi {
     decltype(&onnx_conv2d_run) conv_run;
     decltype(&onnx_conv2d_add_run) conv_add_run;
     decltype(&onnx_conv2d_run_packed) conv_run_packed;
+    decltype(&onnx_conv2d_run_packed_sampled) conv_run_packed_sampled;
     decltype(&onnx_gemm_workspace_bytes) gemm_workspace_bytes;
     decltype(&onnx_gemm_run) gemm_run;
     decltype(&onnx_maxpool2d_shape) maxpool2d_shape;
@@ -115,6 +116,7 @@ PyObject *py_bind(PyObject *, PyObject *arg) {
     get(abi.conv_run, "onnx_conv2d_run");
     get(abi.conv_add_run, "onnx_conv2d_add_run");
     get(abi.conv_run_packed, "onnx_conv2d_run_packed");
+    get(abi.conv_run_packed_sampled, "onnx_conv2d_run_packed_sampled");
     get(abi.gemm_workspace_bytes, "onnx_gemm_workspace_bytes");
     get(abi.gemm_run, "onnx_gemm_run");
     get(abi.maxpool2d_shape, "onnx_maxpool2d_shape");
@@ -134,22 +136,41 @@ PyObject *py_plan(PyObject *, PyObject *args) {
     return PyCapsule_New(p, "onnxb.plan", plan_free);
 }
 
+// n integers of a tuple or list; None leaves the defaults
+inline bool ints(PyObject *o, int64_t *out, Py_ssize_t n) {
+    if (o == Py_None) return true;
+    PyObject *const *items;
+    if (PyTuple_CheckExact(o) && PyTuple_GET_SIZE(o) == n) items = &PyTuple_GET_ITEM(o, 0);
+    else if (PyList_CheckExact(o) && PyList_GET_SIZE(o) == n) items = &PyList_GET_ITEM(o, 0);
+    else return false;
+    for (Py_ssize_t i = 0; i < n; ++i) {
+        if (!PyLong_CheckExact(items[i])) return false;
+        out[i] = PyLong_AsLongLong(items[i]);
+    }
+    if (PyErr_Occurred()) { PyErr_Clear(); return false; }
+    return true;
+}
+
 // conv(plan, X, W, packed, B, R, Y, workspace, stream): run (packed and R None), run_add (R given) or
-// run_packed (packed given)
+// run_packed (packed given); with two more arguments R and packed are given, R is read at every such row and column,
+// and the last one, if any, gets Y rounded
 PyObject *py_conv(PyObject *, PyObject *const *a, Py_ssize_t n) {
-    if (n != 9) return slow_path();
+    if (n != 9 && n != 11) return slow_path();
     Plan *p = plan_of(a[0]);
     if (!p) { PyErr_Clear(); return slow_path(); }
     bool fine = true;
-    const at::Tensor *xt = nullptr;
+    const at::Tensor *xt = nullptr, *rt = nullptr;
     size_t packed_bytes, ws_bytes;
     const float *x = in_ptr(a[1], fine, &xt), *w = in_ptr(a[2], fine);
     const void *packed = ws_ptr(a[3], packed_bytes, fine);
-    const float *b = in_ptr(a[4], fine), *r = in_ptr(a[5], fine);
+    const float *b = in_ptr(a[4], fine), *r = in_ptr(a[5], fine, &rt);
     float *y = const_cast<float *>(in_ptr(a[6], fine));
     void *ws = ws_ptr(a[7], ws_bytes, fine), *st = stream_ptr(a[8], fine);
     if (!fine || !x || !w) return slow_path();
     const bool pre = a[3] != Py_None;
+    int64_t every[2];
+    float *y_rounded = n == 11 ? const_cast<float *>(in_ptr(a[10], fine)) : nullptr;
+    if (n == 11 && (!fine || !r || !pre || rt->dim() != 4 || a[9] == Py_None || !ints(a[9], every, 2))) return slow_path();
     at::Tensor ym, wm;
     if (!y) {
         ym = new_tensor(p->y, at::kFloat, xt->device(), a[8], st, true);
@@ -160,7 +181,9 @@ PyObject *py_conv(PyObject *, PyObject *const *a, Py_ssize_t n) {
         ws = wm.data_ptr();
         ws_bytes = p->workspace;
     }
-    const onnxb_status s = pre ? abi.conv_run_packed(p->desc, x, w, packed, packed_bytes, b, r, y, ws, ws_bytes, st)
+    const onnxb_status s = n == 11 ? abi.conv_run_packed_sampled(p->desc, x, w, packed, packed_bytes, b, r, rt->sizes().data() + 2, every,
+                                                                 y, y_rounded, ws, ws_bytes, st)
+                           : pre ? abi.conv_run_packed(p->desc, x, w, packed, packed_bytes, b, r, y, ws, ws_bytes, st)
                            : r ? abi.conv_add_run(p->desc, x, w, b, r, y, ws, ws_bytes, st)
                                : abi.conv_run(p->desc, x, w, b, y, ws, ws_bytes, st);
     return s == ONNXB_OK ? result(a[6], ym) : slow_path();
@@ -200,21 +223,6 @@ PyObject *py_gemm(PyObject *, PyObject *const *a, Py_ssize_t n) {
     const onnxb_status s = abi.gemm_run(ta, tb, (float)alpha, (float)beta, M, N, K, A, B, C, c_rank, C ? c_dims : nullptr,
                                         relu, y, ws, ws_bytes, st);
     return s == ONNXB_OK ? result(a[8], ym) : slow_path();
-}
-
-// n integers of a tuple or list; None leaves the defaults
-inline bool ints(PyObject *o, int64_t *out, Py_ssize_t n) {
-    if (o == Py_None) return true;
-    PyObject *const *items;
-    if (PyTuple_CheckExact(o) && PyTuple_GET_SIZE(o) == n) items = &PyTuple_GET_ITEM(o, 0);
-    else if (PyList_CheckExact(o) && PyList_GET_SIZE(o) == n) items = &PyList_GET_ITEM(o, 0);
-    else return false;
-    for (Py_ssize_t i = 0; i < n; ++i) {
-        if (!PyLong_CheckExact(items[i])) return false;
-        out[i] = PyLong_AsLongLong(items[i]);
-    }
-    if (PyErr_Occurred()) { PyErr_Clear(); return false; }
-    return true;
 }
 
 // maxpool(X, kernel_shape, pads, strides, Y, stream)
