@@ -209,6 +209,28 @@ onnxb_status onnx_conv2d_run_packed_sampled(onnxb_conv2d_desc_t desc, const floa
                                             const int64_t r_strides[2], float *Y, float *Y_rounded, void *workspace,
                                             size_t workspace_bytes, void *cuda_stream);
 
+/*
+ * onnx_conv2d_run_packed_rounded - onnx_conv2d_run_packed with Y rounded to TF32 (nearest) as well, for tensor-core layers to read
+ * that would truncate Y.  Descriptors of 1x1 convolutions, with an addend: into a tensor of its own, laid out like Y.  Descriptors
+ * of ONNXB_KERNEL_MMA_IMPLICIT with 16 input channels of a group and more, without: Y itself (Y_rounded == Y).  ERR_UNSUPPORTED for
+ * all else; other errors as for onnx_conv2d_run_packed.
+ */
+onnxb_status onnx_conv2d_run_packed_rounded(onnxb_conv2d_desc_t desc, const float *X, const float *W, const void *packed,
+                                            size_t packed_bytes, const float *B, const float *R, float *Y, float *Y_rounded,
+                                            void *workspace, size_t workspace_bytes, void *cuda_stream);
+
+/*
+ * onnx_conv2d_desc_layout - onnx_conv2d_desc for tensors between the layers of a model that are kept channel-major:
+ * [channel][image][row][column], a channel's pixels of all images one after the other, channels onnxb_channel_pitch(images, rows,
+ * columns) floats apart (whole 128-byte lines; what lies between is never read as a value).  x_channel_major: X;
+ * y_channel_major: Y, and R.  Every run call of the descriptor takes them so.  ERR_UNSUPPORTED where no kernel knows the layout:
+ * group-1, unpadded 1x1 convolutions of unit stride and 32 channels and more, and what ONNXB_KERNEL_MMA_IMPLICIT takes (16
+ * channels of a group and more where X is channel-major), do.
+ */
+onnxb_status onnx_conv2d_desc_layout(const onnxb_conv2d_attrs *attrs, int x_channel_major, int y_channel_major,
+                                     onnxb_conv2d_desc_t *out);
+size_t onnxb_channel_pitch(int64_t images, int64_t rows, int64_t columns);
+
 void onnx_conv2d_desc_destroy(onnxb_conv2d_desc_t desc);
 
 /*
@@ -307,12 +329,15 @@ onnxb_status onnx_maxpool2d_run(const int64_t x_dims[4], const int64_t kernel_sh
                                 const int64_t strides[2], const float *X, float *Y, void *cuda_stream);
 
 /*
+ * onnx_global_average_pool_channel_major_run - the same of a channel-major X (see onnx_conv2d_desc_layout).
+ *
  * onnx_global_average_pool_run - ONNX GlobalAveragePool (ResNet50's last pooling, Sec. 4.2):
  * Y[n,c,0,0] = mean over h, w of X[n,c,h,w].  x_dims = {N,C,H,W} (host); X device [N,C,H,W],
  * Y device [N,C,1,1]; fp32 accumulation (32 partial sums per plane, then a tree).  Enqueued on
  * cuda_stream; allocates and synchronises nothing.  Errors: ERR_NULL, ERR_SHAPE, ERR_UNSUPPORTED, ERR_CUDA.
  */
 onnxb_status onnx_global_average_pool_run(const int64_t x_dims[4], const float *X, float *Y, void *cuda_stream);
+onnxb_status onnx_global_average_pool_channel_major_run(const int64_t x_dims[4], const float *X, float *Y, void *cuda_stream);
 
 /* Human-readable name of a status code (static storage, never NULL). */
 const char *onnxb_status_string(onnxb_status status);

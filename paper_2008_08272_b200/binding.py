@@ -32,7 +32,8 @@ EXPORTS = [
     "onnxb_probe_tf32_mma_rate", "onnx_matmul_add_run",
     "onnx_maxpool2d_shape", "onnx_maxpool2d_run", "onnx_global_average_pool_run", "onnx_conv2d_add_run",
     "onnx_conv2d_prepack", "onnx_conv2d_run_prepacked", "onnx_conv2d_packed_bytes", "onnx_conv2d_run_packed",
-    "onnx_conv2d_run_packed_sampled",
+    "onnx_conv2d_run_packed_sampled", "onnx_conv2d_run_packed_rounded", "onnx_conv2d_desc_layout", "onnxb_channel_pitch",
+    "onnx_global_average_pool_channel_major_run",
     "onnxb_probe_wait_timeout",
 ]
 
@@ -123,6 +124,14 @@ def load(build_if_missing: bool = True):
     lib.onnx_conv2d_run_packed_sampled.restype = ctypes.c_int
     lib.onnx_conv2d_run_packed_sampled.argtypes = [vp, vp, vp, vp, sz, vp, vp, ctypes.POINTER(i64), ctypes.POINTER(i64),
                                                    vp, vp, vp, sz, vp]
+    lib.onnx_conv2d_run_packed_rounded.restype = ctypes.c_int
+    lib.onnx_conv2d_run_packed_rounded.argtypes = [vp, vp, vp, vp, sz, vp, vp, vp, vp, vp, sz, vp]
+    lib.onnx_conv2d_desc_layout.restype = ctypes.c_int
+    lib.onnx_conv2d_desc_layout.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.POINTER(vp)]
+    lib.onnxb_channel_pitch.restype = sz
+    lib.onnxb_channel_pitch.argtypes = [i64, i64, i64]
+    lib.onnx_global_average_pool_channel_major_run.restype = ctypes.c_int
+    lib.onnx_global_average_pool_channel_major_run.argtypes = [ctypes.POINTER(i64), vp, vp, vp]
     lib.onnx_conv2d_run_prepacked.restype = ctypes.c_int
     lib.onnx_conv2d_run_prepacked.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]
     lib.onnx_conv2d_run_static.restype = ctypes.c_int
@@ -246,19 +255,27 @@ def make_attrs(x_shape, w_shape, *, kernel_shape=None, pads=None, strides=None, 
     return a
 
 
+def channel_pitch(shape) -> int:
+    """Floats from one channel to the next of a channel-major tensor of the logical shape (images, channels, rows, columns)."""
+    return int(load().onnxb_channel_pitch(shape[0], shape[2], shape[3]))
+
+
 class Conv2dDesc:
     """Owns an ``onnxb_conv2d_desc_t`` (``onnx_conv2d_desc`` .. ``onnx_conv2d_desc_destroy``)."""
 
-    def __init__(self, x_shape, w_shape, **attrs):
+    def __init__(self, x_shape, w_shape, *, x_channel_major=False, y_channel_major=False, **attrs):
         self._lib = load()
         self._h = ctypes.c_void_p()
         self.attrs = make_attrs(x_shape, w_shape, **attrs)
-        _check(self._lib.onnx_conv2d_desc(ctypes.byref(self.attrs), ctypes.byref(self._h)), "onnx_conv2d_desc")
+        _check(self._lib.onnx_conv2d_desc_layout(ctypes.byref(self.attrs), int(x_channel_major), int(y_channel_major),
+                                                 ctypes.byref(self._h)), "onnx_conv2d_desc")
         y = (ctypes.c_int64 * 4)()
         p = (ctypes.c_int64 * 4)()
         ws = ctypes.c_size_t()
         _check(self._lib.onnx_conv2d_desc_query(self._h, y, p, ctypes.byref(ws)), "onnx_conv2d_desc_query")
         self.y_shape = tuple(int(v) for v in y)
+        # as it lies in memory: itself, or (channel, floats from one channel to the next)
+        self.y_storage = (self.y_shape[1], channel_pitch(self.y_shape), 1, 1) if y_channel_major else self.y_shape
         self.pads = tuple(int(v) for v in p)
         self.workspace_bytes = int(ws.value)
         self.kernel_family = KERNEL_FAMILIES[self._lib.onnx_conv2d_desc_query_kernel(self._h)]
@@ -271,7 +288,7 @@ class Conv2dDesc:
         if self._plan is None:
             if not self._h:
                 return None
-            self._plan = _fast().plan(self._h.value, self.y_shape, self.workspace_bytes, self.packed_bytes, self._packed_needs_ws)
+            self._plan = _fast().plan(self._h.value, self.y_storage, self.workspace_bytes, self.packed_bytes, self._packed_needs_ws)
         return _fast_mod.conv(self._plan, X, W, packed, B, R, Y, workspace, stream, *sampled)
 
     def run(self, X, W, B=None, Y=None, workspace=None, stream=None):
@@ -280,7 +297,7 @@ class Conv2dDesc:
         if y is not None:
             return y
         if Y is None:
-            Y = _new(self.y_shape, X.device, stream)
+            Y = _new(self.y_storage, X.device, stream)
         needs = workspace is None and self.workspace_bytes
         workspace, ws_ptr, ws_len, no_memory = _scratch(self.workspace_bytes, X.device, stream) if needs else _given(workspace)
         _check(self._lib.onnx_conv2d_run(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
@@ -295,7 +312,7 @@ class Conv2dDesc:
             if y is not None:
                 return y
         if Y is None:
-            Y = _new(self.y_shape, X.device, stream)
+            Y = _new(self.y_storage, X.device, stream)
         needs = workspace is None and self.workspace_bytes
         workspace, ws_ptr, ws_len, no_memory = _scratch(self.workspace_bytes, X.device, stream) if needs else _given(workspace)
         _check(self._lib.onnx_conv2d_add_run(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
@@ -324,7 +341,7 @@ class Conv2dDesc:
             if y is not None:
                 return y
         if Y is None:
-            Y = _new(self.y_shape, X.device, stream)
+            Y = _new(self.y_storage, X.device, stream)
         packed_len = packed.numel() * packed.element_size()
         needs = workspace is None and self.workspace_bytes and (self._packed_needs_ws or packed_len < self.packed_bytes)
         workspace, ws_ptr, ws_len, no_memory = _scratch(self.workspace_bytes, X.device, stream) if needs else _given(workspace)
@@ -335,24 +352,38 @@ class Conv2dDesc:
                "onnx_conv2d_run_packed", no_memory)
         return Y
 
-    def run_prepacked_sampled(self, X, W, packed, B, R, strides, Y=None, Y_rounded=None, workspace=None, stream=None):
+    def run_prepacked_sampled(self, X, W, packed, B, R, strides, Y=None, Y_rounded=None, r_dims=None, workspace=None, stream=None):
         """``onnx_conv2d_run_packed_sampled``: run_prepacked with the addend R[:, :, ::strides[0], ::strides[1]]; Y rounded to TF32
-        goes to ``Y_rounded`` where it is given."""
-        if R.dim() != 4 or tuple(R.shape[:2]) != self.y_shape[:2]:
-            raise OnnxB200Error(3, "run_prepacked_sampled: the addend's images and channels are not the output's")
-        y = self._native(X, W, packed, B, R, Y, workspace, stream, strides, Y_rounded)
+        goes to ``Y_rounded`` where it is given.  ``r_dims``: rows and columns of a channel-major R."""
+        if r_dims is None:
+            if R.dim() != 4 or tuple(R.shape[:2]) != self.y_shape[:2]:
+                raise OnnxB200Error(3, "run_prepacked_sampled: the addend's images and channels are not the output's")
+            r_dims = tuple(R.shape[2:])
+        y = self._native(X, W, packed, B, R, Y, workspace, stream, r_dims, strides, Y_rounded)
         if y is not None:
             return y
         if Y is None:
-            Y = _new(self.y_shape, X.device, stream)
+            Y = _new(self.y_storage, X.device, stream)
         needs = workspace is None and self.workspace_bytes and self._packed_needs_ws
         workspace, ws_ptr, ws_len, no_memory = _scratch(self.workspace_bytes, X.device, stream) if needs else _given(workspace)
         _check(self._lib.onnx_conv2d_run_packed_sampled(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
                                                         ctypes.c_void_p(packed.data_ptr()), packed.numel() * packed.element_size(),
                                                         _dev_ptr(B, "B", allow_none=True), _dev_ptr(R, "R"),
-                                                        _i64(R.shape[2:], 2), _i64(strides, 2), _dev_ptr(Y, "Y"),
+                                                        _i64(r_dims, 2), _i64(strides, 2), _dev_ptr(Y, "Y"),
                                                         _dev_ptr(Y_rounded, "Y_rounded", allow_none=True), ws_ptr, ws_len, _stream_ptr(stream)),
                "onnx_conv2d_run_packed_sampled", no_memory)
+        return Y
+
+    def run_prepacked_rounded(self, X, W, packed, B, R, Y, Y_rounded, stream=None):
+        """``onnx_conv2d_run_packed_rounded``: run_prepacked, and Y rounded to TF32 into ``Y_rounded`` (Y itself where it is that)."""
+        y = self._native(X, W, packed, B, R, Y, None, stream, None, None, Y_rounded)
+        if y is not None:
+            return y
+        _check(self._lib.onnx_conv2d_run_packed_rounded(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"), ctypes.c_void_p(packed.data_ptr()),
+                                                        packed.numel() * packed.element_size(), _dev_ptr(B, "B", allow_none=True),
+                                                        _dev_ptr(R, "R", allow_none=True), _dev_ptr(Y, "Y"),
+                                                        _dev_ptr(Y_rounded, "Y_rounded"), None, 0, _stream_ptr(stream)),
+               "onnx_conv2d_run_packed_rounded")
         return Y
 
     def run_static(self, X, W, B=None, Y=None, stream=None):
@@ -360,7 +391,7 @@ class Conv2dDesc:
         stands in for the workspace, so no device memory is allocated for scratch.  (Y is
         still allocated here with torch when the caller does not pass one.)"""
         if Y is None:
-            Y = _new(self.y_shape, X.device, stream)
+            Y = _new(self.y_storage, X.device, stream)
         _check(self._lib.onnx_conv2d_run_static(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"),
                                                 _dev_ptr(B, "B", allow_none=True), _dev_ptr(Y, "Y"),
                                                 _stream_ptr(stream)), "onnx_conv2d_run_static")
@@ -504,6 +535,13 @@ def onnx_maxpool2d(X, kernel_shape, *, pads=None, strides=None, Y=None, stream=N
         Y = _new(y_shape, X.device, stream)
     _check(load().onnx_maxpool2d_run(_i64(tuple(X.shape), 4), _i64(kernel_shape, 2), _i64(pads, 4), _i64(strides, 2),
                                      _dev_ptr(X, "X"), _dev_ptr(Y, "Y"), _stream_ptr(stream)), "onnx_maxpool2d_run")
+    return Y
+
+
+def global_average_pool_channel_major(X, x_shape, Y, stream=None):
+    """``onnx_global_average_pool_channel_major_run``: Y[n,c,0,0] = mean of X[n,c,:,:], X channel-major."""
+    _check(load().onnx_global_average_pool_channel_major_run(_i64(x_shape, 4), _dev_ptr(X, "X"), _dev_ptr(Y, "Y"), _stream_ptr(stream)),
+           "onnx_global_average_pool_channel_major_run")
     return Y
 
 

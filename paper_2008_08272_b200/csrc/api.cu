@@ -73,6 +73,15 @@ static TcGemmProblem conv1x1_as_gemm(const ConvGeom &g, const float *X, const fl
     t.alpha = 1.f; t.beta = 0.f; t.C = nullptr;
     t.row_bias = B; t.relu = g.relu; t.residual = R;
     t.Y = Y; t.y_ld = HW; t.y_bs = (long long)g.M * HW;
+    // Channel-major tensors hold a channel's pixels of all images one after the other: one wide GEMM
+    const long long pitch = channel_pitch(g.N, g.H, g.W);
+    if (g.x_cm) {
+        // (with what lies between two channels, where that has a place in Y, too: whole 16-byte pieces)
+        t.N = (int)(g.y_cm ? pitch : HW * g.N); t.batch = 1; t.b_batched = 0;
+        t.b_ld = pitch; t.b_bs = 0;
+        if (!g.y_cm) { t.y_bs = 0; t.y_split = (int)HW; t.y_group_stride = (long long)g.M * HW; }
+    }
+    if (g.y_cm) { t.y_ld = pitch; t.y_bs = g.x_cm ? 0 : HW; }
     return t;
 }
 
@@ -142,15 +151,19 @@ static inline bool misaligned(const void *p) { return (reinterpret_cast<uintptr_
 
 // An addend that is read at every sh-th row and sw-th column of images of H x W.
 struct SampledAddend {
-    int H, W, sh, sw;
+    int H, W, sh, sw;        // (H 0: the addend is laid out like Y, and read as it is)
     float *Y_rounded;
 };
 static TcGemmProblem sample(TcGemmProblem t, const ConvGeom &g, const SampledAddend *a) {
-    if (a) {
+    if (a) t.Y_rounded = a->Y_rounded;
+    if (a && a->H) {
+        const long long plane = (long long)a->H * a->W;
         t.r_q = g.Q;
-        t.r_ld = (long long)a->H * a->W; t.r_bs = t.r_ld * g.M;
+        t.r_split = t.batch == 1 ? g.P * g.Q : 0;
+        if (g.x_cm) t.N = g.P * g.Q * g.N;               // (no image of R's lies there)
+        t.r_ld = g.y_cm ? channel_pitch(g.N, a->H, a->W) : plane;
+        t.r_bs = g.y_cm ? plane : plane * g.M;
         t.r_row = a->sh * a->W; t.r_col = a->sw;
-        t.Y_rounded = a->Y_rounded;
     }
     return t;
 }
@@ -205,7 +218,9 @@ static onnxb_status conv2d_run_impl(onnxb_conv2d_desc_t d, const float *X, const
             break;
         }
         case ONNXB_KERNEL_MMA_IMPLICIT:
-            err = launch_tc_conv(d->plan, X, W, B, R, Y, workspace, cuda_stream, phase);
+            // (a second output in the first one's place: Y itself rounded)
+            if (sampled && sampled->Y_rounded && sampled->Y_rounded != Y) return ONNXB_ERR_UNSUPPORTED;
+            err = launch_tc_conv(d->plan, X, W, B, R, Y, workspace, cuda_stream, phase, sampled && sampled->Y_rounded);
             break;
         default:
             return ONNXB_ERR_UNSUPPORTED;
@@ -261,6 +276,17 @@ static onnxb_status run_packed(onnxb_conv2d_desc_t d, const float *X, const floa
                                static_cast<const float *>(packed), sampled);
     // the packed copy stands in for the workspace
     return conv2d_run_impl(d, X, W, B, R, Y, const_cast<void *>(packed), need, cuda_stream, kTcConvRunOnly, nullptr, sampled);
+}
+
+extern "C" onnxb_status onnx_conv2d_run_packed_rounded(onnxb_conv2d_desc_t d, const float *X, const float *W, const void *packed,
+                                                       size_t packed_bytes, const float *B, const float *R, float *Y, float *Y_rounded,
+                                                       void *workspace, size_t workspace_bytes, void *cuda_stream) {
+    if (!d || !Y_rounded) return ONNXB_ERR_NULL;
+    const bool gemm = d->family == ONNXB_KERNEL_MMA_GEMM || d->family == ONNXB_KERNEL_MMA_GATHER_GEMM;
+    if (gemm ? !R || Y_rounded == Y : d->family != ONNXB_KERNEL_MMA_IMPLICIT || R || Y_rounded != Y || d->plan.KB == 4) return ONNXB_ERR_UNSUPPORTED;
+    if (misaligned(Y_rounded)) return ONNXB_ERR_UNSUPPORTED;
+    const SampledAddend a{0, 0, 0, 0, Y_rounded};
+    return run_packed(d, X, W, packed, packed_bytes, B, R, Y, workspace, workspace_bytes, cuda_stream, &a);
 }
 
 extern "C" onnxb_status onnx_conv2d_run_packed(onnxb_conv2d_desc_t d, const float *X, const float *W, const void *packed,

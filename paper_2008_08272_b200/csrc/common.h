@@ -10,7 +10,11 @@
 namespace onnxb {
 
 // A convolution problem with every ONNX default and auto_pad already resolved.
+// Floats from one channel to the next in a channel-major tensor ([channel][image][row][column]), padded to whole 128-byte lines.
+inline long long channel_pitch(long long images, long long h, long long w) { return (images * h * w + 31) / 32 * 32; }
+
 struct ConvGeom {
+    int x_cm, y_cm;          // X, Y (and R) are channel-major
     int N, C, H, W;          // input
     int M, Cg, kH, kW;       // weights: M output channels, Cg = C/group input channels each
     int P, Q;                // output spatial size
@@ -70,7 +74,7 @@ size_t tc_conv_workspace_bytes(const TcConvPlan &plan);
 // phase: both steps (pack the weights into the workspace, then convolve), or one of them alone
 constexpr int kTcConvPackAndRun = 0, kTcConvPackOnly = 1, kTcConvRunOnly = 2;
 int launch_tc_conv(const TcConvPlan &plan, const float *X, const float *W, const float *B, const float *R, float *Y,
-                   void *workspace, void *stream, int phase = kTcConvPackAndRun);   // 1x1 stride-1 convolution expressible as a batched TMA GEMM
+                   void *workspace, void *stream, int phase = kTcConvPackAndRun, bool round_y = false);   // 1x1 stride-1 convolution expressible as a batched TMA GEMM
 
 struct GemmProblem {
     int M, N, K;

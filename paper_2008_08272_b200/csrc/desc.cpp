@@ -42,6 +42,12 @@ static bool mul_fits(int64_t a, int64_t b, int64_t c, int64_t d) {
 using namespace onnxb;
 
 extern "C" onnxb_status onnx_conv2d_desc(const onnxb_conv2d_attrs *a, onnxb_conv2d_desc_t *out) {
+    return onnx_conv2d_desc_layout(a, 0, 0, out);
+}
+
+extern "C" size_t onnxb_channel_pitch(int64_t images, int64_t h, int64_t w) { return (size_t)channel_pitch(images, h, w); }
+
+extern "C" onnxb_status onnx_conv2d_desc_layout(const onnxb_conv2d_attrs *a, int x_channel_major, int y_channel_major, onnxb_conv2d_desc_t *out) {
     if (!a || !out) return ONNXB_ERR_NULL;
     *out = nullptr;
     if (a->reserved != 0) return ONNXB_ERR_ATTR;
@@ -122,6 +128,7 @@ extern "C" onnxb_status onnx_conv2d_desc(const onnxb_conv2d_attrs *a, onnxb_conv
     g.sh = (int)st[0]; g.sw = (int)st[1]; g.dh = (int)di[0]; g.dw = (int)di[1];
     g.group = (int)group; g.Mg = (int)(M / group);
     g.has_bias = a->has_bias != 0; g.relu = a->fuse_relu != 0;
+    g.x_cm = x_channel_major != 0; g.y_cm = y_channel_major != 0;
     d->y_dims[0] = N; d->y_dims[1] = M; d->y_dims[2] = P; d->y_dims[3] = Q;
     for (int i = 0; i < 4; ++i) d->pads[i] = pads[i];
 
@@ -129,7 +136,13 @@ extern "C" onnxb_status onnx_conv2d_desc(const onnxb_conv2d_attrs *a, onnxb_conv
     // contractions run on the SIMT family.
     const int forced = kernel_override();
     int family = ONNXB_KERNEL_SIMT_DIRECT;
-    if (simt_depthwise_supports(g)) family = ONNXB_KERNEL_SIMT_DEPTHWISE;
+    if (g.x_cm || g.y_cm) {
+        // (two families know these layouts)
+        if (forced >= 0 || channel_pitch(N, H, W) * C > kMaxElems || channel_pitch(N, P, Q) * M > kMaxElems) { delete d; return ONNXB_ERR_UNSUPPORTED; }
+        if (conv_fits_mma_gemm(g)) family = ONNXB_KERNEL_MMA_GEMM;
+        else if (!conv_fits_mma_gather_gemm(g) && tc_conv_plan(g, d->plan)) family = ONNXB_KERNEL_MMA_IMPLICIT;
+        else { delete d; return ONNXB_ERR_UNSUPPORTED; }
+    } else if (simt_depthwise_supports(g)) family = ONNXB_KERNEL_SIMT_DEPTHWISE;
     else if (conv_fits_mma_gemm(g)) family = ONNXB_KERNEL_MMA_GEMM;
     else if (conv_fits_mma_gather_gemm(g)) family = ONNXB_KERNEL_MMA_GATHER_GEMM;
     else if (tc_conv_plan(g, d->plan)) family = ONNXB_KERNEL_MMA_IMPLICIT;

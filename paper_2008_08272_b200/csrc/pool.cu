@@ -126,11 +126,13 @@ maxpool_3x3s2_kernel(const float *__restrict__ X, float *__restrict__ Y, int H, 
 // partial sums in fp32, then a shuffle tree inside the group.
 template <int TPP>
 __global__ void __launch_bounds__(256)
-global_average_pool_kernel(const float *__restrict__ X, float *__restrict__ Y, unsigned planes, unsigned HW, float inv_hw) {
+global_average_pool_kernel(const float *__restrict__ X, float *__restrict__ Y, unsigned planes, unsigned HW, float inv_hw, unsigned C,
+                           size_t image, size_t channel, ConvDivisor dv_C) {
     const unsigned gid = (blockIdx.x * 256u + threadIdx.x) / TPP, sub = threadIdx.x % TPP;
     float acc = 0.f;
     if (gid < planes) {
-        const float *xp = X + (size_t)gid * HW;
+        const unsigned n = (unsigned)conv_fdiv((int)gid, (int)C, dv_C);
+        const float *xp = X + n * image + (gid - n * C) * channel;
         for (unsigned k = sub; k < HW; k += TPP) acc += __ldg(xp + k);
     }
 #pragma unroll
@@ -210,21 +212,30 @@ extern "C" onnxb_status onnx_maxpool2d_run(const int64_t x_dims[4], const int64_
     return cudaGetLastError() == cudaSuccess ? ONNXB_OK : ONNXB_ERR_CUDA;
 }
 
-extern "C" onnxb_status onnx_global_average_pool_run(const int64_t x_dims[4], const float *X, float *Y,
-                                                     void *cuda_stream) {
+static onnxb_status global_average_pool(const int64_t x_dims[4], bool channel_major, const float *X, float *Y, void *cuda_stream) {
     if (!x_dims || !X || !Y) return ONNXB_ERR_NULL;
     if (x_dims[0] < 1 || x_dims[1] < 1 || x_dims[2] < 1 || x_dims[3] < 1) return ONNXB_ERR_SHAPE;
     const int64_t planes = x_dims[0] * x_dims[1], hw = x_dims[2] * x_dims[3];
     if (planes > (1LL << 26) || hw > (1LL << 30) || planes * hw > 2147483647LL * 4) return ONNXB_ERR_UNSUPPORTED;
+    const size_t channel = channel_major ? (size_t)channel_pitch(x_dims[0], x_dims[2], x_dims[3]) : (size_t)hw;
+    const size_t image = (size_t)hw * (channel_major ? 1 : x_dims[1]);
+    const ConvDivisor dv_C = conv_divisor((int)x_dims[1]);
     if (hw <= 128) {
         const unsigned blocks = (unsigned)((planes * 8 + 255) / 256);
         global_average_pool_kernel<8><<<blocks, 256, 0, (cudaStream_t)cuda_stream>>>(X, Y, (unsigned)planes, (unsigned)hw,
-                                                                                   1.0f / (float)hw);
+                                                                                   1.0f / (float)hw, (unsigned)x_dims[1], image, channel, dv_C);
     } else {
         const unsigned blocks = (unsigned)((planes * 32 + 255) / 256);
         global_average_pool_kernel<32><<<blocks, 256, 0, (cudaStream_t)cuda_stream>>>(X, Y, (unsigned)planes, (unsigned)hw,
-                                                                                    1.0f / (float)hw);
+                                                                                    1.0f / (float)hw, (unsigned)x_dims[1], image, channel, dv_C);
     }
     count_launch();
     return cudaGetLastError() == cudaSuccess ? ONNXB_OK : ONNXB_ERR_CUDA;
+}
+
+extern "C" onnxb_status onnx_global_average_pool_run(const int64_t x_dims[4], const float *X, float *Y, void *cuda_stream) {
+    return global_average_pool(x_dims, false, X, Y, cuda_stream);
+}
+extern "C" onnxb_status onnx_global_average_pool_channel_major_run(const int64_t x_dims[4], const float *X, float *Y, void *cuda_stream) {
+    return global_average_pool(x_dims, true, X, Y, cuda_stream);
 }

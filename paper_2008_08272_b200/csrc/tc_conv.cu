@@ -67,7 +67,7 @@ constexpr int kSegBytes = 256;             // >= sizeof(TcConvSegs)
 constexpr int kBiasBytes = 8 * 128;        // 32 biases per epilogue warp
 static_assert(sizeof(TcConvSegs) <= kSegBytes, "segment table does not fit its slot");
 
-enum { kNoAddend, kAddendNear, kAddendFar };
+enum { kNoAddend, kAddendNear, kAddendFar, kRoundedY };       // kRoundedY: no addend, and Y is rounded to TF32 (a form of its own: three instructions per output)
 
 struct Bars {
     uint64_t raw_full[kMaxRawStages], raw_empty[kMaxRawStages], a_full[kMaxAStages], a_empty[kMaxAStages];
@@ -122,7 +122,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                const float *__restrict__ Wpk, const float *__restrict__ bias, const float *__restrict__ R,
                float *__restrict__ Y, unsigned int *err) {
     constexpr int kOwned = kThin ? kOwnedThin : kOwnedThick;
-    constexpr bool kAdd = kAddend != kNoAddend, kLinear = kThin && kAddend != kAddendNear;
+    constexpr bool kAdd = kAddend == kAddendNear || kAddend == kAddendFar, kLinear = kThin && kAddend != kAddendNear;
     // may stage rows (raw_mode 2): the thin ones; but the schedule that the compiler finds for those with an addend, whose epilogue has
     // no register to spare, is the better one with that code in place (64 -> 64 3x3 56x56 batch 32 23.8 against 25.3 us)
     constexpr bool kRows = kThin || kAdd;
@@ -260,8 +260,9 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                     if (g.raw_mode == 0) {
                         mbar_arrive_expect_tx(&bars->raw_full[rs], tile_bytes);
                         for (int i = 0; i < nseg; ++i) {
-                            const int plane0 = (segs->n_first + i) * g.C + c0;
-                            const int nbox = segs->nbox[i], f0 = segs->f0[i];
+                            // (channel-major: all of it in the first segment)
+                            const int plane0 = g.x_cm ? c0 : (segs->n_first + i) * g.C + c0;
+                            const int nbox = segs->nbox[i], f0 = segs->f0[i] + (g.x_cm ? segs->n_first * g.H * g.W : 0);
                             float *d = dst + segs->base[i];
                             for (int j = 0; j < nbox; ++j)
                                 tma_load_2d(d + j * box_floats, &tmX, &bars->raw_full[rs], f0 + j * g.BOXP, plane0);
@@ -664,7 +665,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             // eight warps: two per TMEM lane quarter, each taking half of the tile
             const int hf = ew >> 2, mt = two ? hf : 0;
             const int ch_lo = two ? 0 : hf ? (nch + 1) / 2 : 0, ch_hi = two || hf ? nch : (nch + 1) / 2;
-            const uint32_t PQ4 = (uint32_t)g.P * (uint32_t)g.Q * 4u;
+            const uint32_t PQ4 = g.y_chan4;
             bool valid = false;
             uint32_t off = 0;                          // bytes from Y (and R): the launch keeps them below 2^32
             if (it == 0) pdl_wait();
@@ -677,7 +678,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                     const int n = conv_fdiv((int)G, g.L, g.dv_L), u = (int)G - n * g.L;
                     const int p = conv_fdiv(u, g.Ws, g.dv_Ws), q = u - p * g.Ws;
                     valid = p < g.P && q < g.Q;
-                    off = (uint32_t)(n * g.M + grp * g.Mg + ct * g.BN + ch_lo * 32) * PQ4 + (uint32_t)(p * g.Q + q) * 4u;
+                    off = (uint32_t)n * g.y_image4 + (uint32_t)(grp * g.Mg + ct * g.BN + ch_lo * 32) * PQ4 + (uint32_t)(p * g.Q + q) * 4u;
                 }
             }
             const char *rb = reinterpret_cast<const char *>(R);
@@ -695,7 +696,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                         if (n >= g.N || p >= g.P) continue;
                         const char *at = rb + (uint32_t)(p * g.Q + min(w - p * g.Ws, g.Q - 1)) * 4u;
                         for (int c = m0 + ch_lo * 32 + lane; c < min(g.Mg, m0 + min(g.BN, ch_hi * 32)); c += 32)
-                            prefetch_l2(at + (uint32_t)(n * g.M + gr * g.Mg + c) * PQ4);
+                            prefetch_l2(at + ((uint32_t)n * g.y_image4 + (uint32_t)(gr * g.Mg + c) * PQ4));
                     }
                 }
             }
@@ -774,6 +775,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                                 float x = __uint_as_float(v[j0 + j + e]) + b[e];
                                 if (kAdd) x += r[(j0 >> 3) & 1][j + e];
                                 x = fmaxf(x, lowest);
+                                if (kAddend == kRoundedY) x = round_tf32(x);
                                 if (valid && j0 + j + e < cnt) *reinterpret_cast<float *>(yb + off) = x;
                                 off += PQ4;
                             }
@@ -805,10 +807,10 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
             const int p = conv_fdiv(u, g.Ws, g.dv_Ws), q = u - p * g.Ws;
             if (G < (uint32_t)g.total_slots && p < g.P && q < g.Q) {
                 pdl_wait();                     // long since satisfied
-                const long long PQ = (long long)g.P * g.Q;
+                const long long PQ = g.y_chan4 / 4;
                 for (int col = col_lo + (tid >> 7) * 4; col < col_hi; col += kGroups * 4) {
                     const int m = grp * g.Mg + ct * g.BN + col, cnt = tile_ch - col;          // channels that exist (above 4: all)
-                    const long long o = ((long long)n * g.M + m) * PQ + (long long)p * g.Q + q;
+                    const long long o = (long long)n * (g.y_image4 / 4) + m * PQ + (long long)p * g.Q + q;
                     float b[4], r[4];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
@@ -830,6 +832,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap tmX, const TcConvPlan g, cons
                         float y = f[e] + b[e];
                         if (kAdd) y += r[e];
                         if (g.relu) y = fmaxf(y, 0.f);
+                        if (kAddend == kRoundedY) y = round_tf32(y);
                         if (e < cnt) Y[o + e * PQ] = y;
                     }
                 }
@@ -978,7 +981,16 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     g.total_tiles = (long long)g.pix_tiles * g.ctiles * c.group;
     // raw staging mode
     const long long HW = (long long)c.H * c.W;
-    if (HW % 4 == 0) {
+    g.x_cm = c.x_cm;
+    const long long y_pitch = channel_pitch(c.N, c.P, c.Q);
+    if (c.y_cm && y_pitch * c.M >= (1LL << 30)) return false;         // (one launch: offsets in 32 bits of bytes)
+    if (c.x_cm && (!c.y_cm && (long long)c.N * c.M * c.P * c.Q >= (1LL << 30))) return false;
+    g.y_image4 = (uint32_t)((c.y_cm ? 1LL : (long long)c.M) * c.P * c.Q * 4);
+    g.y_chan4 = (uint32_t)((c.y_cm ? y_pitch : (long long)c.P * c.Q) * 4);
+    if (c.x_cm) {
+        if (g.KB == 4 || channel_pitch(c.N, c.H, c.W) >= (1LL << 30)) return false;
+        g.raw_mode = 0;
+    } else if (HW % 4 == 0) {
         // Blocks of 4 channels of images that a tile touches two of at most: a copy per channel (a box per 256 pixels is more
         // copies there, and its places cost the transform a shift and a mask per unit).
         g.raw_mode = g.KB == 4 && (g.SLOTS + L - 2) / L + 1 <= 2 ? 2 : 0;
@@ -997,8 +1009,10 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
     // slot row the last reaches furthest, and the first image has the most slots after it, so one start per slot
     // row covers all tiles.
     g.KBR = std::min(g.KB, c.Cg);
+    // (channel-major: where a range of pixels begins within 16 bytes goes by its image, too)
     auto for_each_start = [&](auto &&f) {
-        for (int r = 0; r < g.Hs; ++r) f(std::min<long long>((long long)r * g.Ws + g.Ws - 1, g.total_slots - 1));
+        for (int n = 0; n < (c.x_cm ? std::min(c.N, 4) : 1); ++n)
+            for (int r = 0; r < g.Hs; ++r) f(std::min<long long>(n * L + (long long)r * g.Ws + g.Ws - 1, g.total_slots - 1));
     };
     auto stage_floats = [&](int boxp, int &boxes) {
         g.BOXP = boxp;
@@ -1030,7 +1044,15 @@ bool fill_plan(const ConvGeom &c, int ctas, int MT, int BN, int KB, TcConvPlan &
         // multiple of 128.  (Smaller boxes stage less beyond what a tile needs, but cost more than that gains:
         // 64 -> 64 channels at 56x56 44.3 -> 46 us.)
         int widest = 4;
-        for_each_start([&](long long G0) {
+        if (c.x_cm) {
+            g.BOXP = 4;                            // (boxes of four: the range itself)
+            for_each_start([&](long long G0) {
+                TcConvSegs segs;
+                tc_conv_segments(g, G0, segs);
+                if (segs.nseg > 0) widest = std::max(widest, segs.nbox[0] * 4);
+            });
+        }
+        else for_each_start([&](long long G0) {
             const long long Gend = std::min<long long>(G0 + g.SLOTS, g.total_slots);
             for (long long n = 0; n * L < Gend; ++n) {
                 const long long lo = std::max<long long>(G0, n * L), hi = std::min<long long>(Gend, (n + 1) * L);
@@ -1155,7 +1177,7 @@ double tile_cost(const TcConvPlan &p) {
     const double t_w = std::max(w_bytes / std::min(31.5, 3620.0 / active),
                                 p.split > 1 && ring >= w_bytes * p.cb_per ? 0.0 : w_bytes * 2090.0 / ring);
     const double t_x = 1075.0 + 42.0 * owned * p.chunks_per_unit + (pair ? 615.0 : 0.0);
-    const double t_p = 342.0 + 327.0 * ((p.SLOTS - 1) / p.L + 2);
+    const double t_p = 342.0 + 327.0 * (p.x_cm ? 1 : (p.SLOTS - 1) / p.L + 2);
     const double per_cb = std::max({t_mma, t_smem, t_w, t_x, t_p});
     if (p.split > 1) return (double)waves * (p.cb_per * (per_cb + 896.0) + 28.0 * p.BN + 5190.0) + 7090.0;
     return (double)waves * (p.ncb * (per_cb + (p.na_stages == 3 ? 0.0 : 449.0)) + 1650.0) + 9530.0;
@@ -1277,10 +1299,10 @@ static int max_pairs() {
 size_t tc_conv_workspace_bytes(const TcConvPlan &plan) { return (size_t)plan.packed_floats * 4; }
 
 static int launch_images(const TcConvPlan &plan, const float *X, const float *B, const float *R, float *Y, const void *workspace,
-                         unsigned int *err, cudaStream_t st);
+                         unsigned int *err, cudaStream_t st, bool round_y);
 
 int launch_tc_conv(const TcConvPlan &plan, const float *X, const float *W, const float *B, const float *R, float *Y,
-                   void *workspace, void *stream, int phase) {
+                   void *workspace, void *stream, int phase, bool round_y) {
     using namespace tc_host;
     cudaStream_t st = (cudaStream_t)stream;
     unsigned int *err = device_status_ptr();
@@ -1305,19 +1327,20 @@ int launch_tc_conv(const TcConvPlan &plan, const float *X, const float *W, const
         part.pix_tiles = (int)((part.total_slots + part.ctas * part.MT * 128 - 1) / (part.ctas * part.MT * 128));
         part.total_tiles = (long long)part.pix_tiles * part.ctiles * part.group;
         const int e = launch_images(part, X + (long long)n0 * plan.C * plan.H * plan.W, B, R ? R + n0 * image : nullptr, Y + n0 * image,
-                                    workspace, err, st);
+                                    workspace, err, st, round_y);
         if (e != 0) return e;
     }
     return 0;
 }
 
 static int launch_images(const TcConvPlan &plan, const float *X, const float *B, const float *R, float *Y, const void *workspace,
-                         unsigned int *err, cudaStream_t st) {
+                         unsigned int *err, cudaStream_t st, bool round_y) {
     using namespace tc_host;
     CUtensorMap tmX;
     if (plan.raw_mode == 0) {
-        const uint64_t dims[2] = {(uint64_t)plan.H * plan.W, (uint64_t)plan.N * plan.C};
-        const uint64_t str[1] = {(uint64_t)plan.H * plan.W * 4};
+        const uint64_t HW = (uint64_t)plan.H * plan.W, N = (uint64_t)plan.N, C = (uint64_t)plan.C;
+        const uint64_t dims[2] = {plan.x_cm ? N * HW : HW, plan.x_cm ? C : N * C};
+        const uint64_t str[1] = {plan.x_cm ? (uint64_t)channel_pitch(plan.N, plan.H, plan.W) * 4 : HW * 4};
         const uint32_t box[2] = {(uint32_t)plan.BOXP, (uint32_t)plan.KBR};
         if (!make_tmap(&tmX, X, 2, dims, str, box, kTmapSwizzleNone)) return (int)cudaErrorInvalidValue;
     } else {
@@ -1330,13 +1353,15 @@ static int launch_images(const TcConvPlan &plan, const float *X, const float *B,
     const bool pair = plan.ctas == 2;
     const bool add = R != nullptr;
     const bool split = plan.split > 1;
+    if (round_y && (add || plan.KB == 4)) return (int)cudaErrorInvalidValue;
     const bool thin = plan.KB == 4;
     // Asking ahead for an addend is worth it where L2 is unlikely to hold it still (64 -> 64 channels 3x3 56x56 batch 32, 26 MB:
     // 23.9 -> 25.1 us with it) and the main loop is too short to hide the epilogue (64 -> 64 3x3 112x112 batch 32, 72 steps:
     // 97 -> 102; 32 -> 128, 36 steps of 128 columns: 132 -> 138; 32 -> 64, 36 of 64: 77 -> 69; thin layers:
     // 3 -> 256 7x7 64x64 batch 64 197 -> 173, 12 -> 64 5x5 112x112 batch 32 82 -> 72).
     const bool far = add && 4LL * plan.N * plan.M * plan.P * plan.Q >= (64LL << 20) && (thin || plan.ncb * plan.n_steps * plan.BN <= 2560);
-    auto kern = split  ? (add ? tc_conv_kernel<1, kAddendNear, false, true> : tc_conv_kernel<1, kNoAddend, false, true>)
+    auto kern = round_y ? (split ? tc_conv_kernel<1, kRoundedY, false, true> : pair ? tc_conv_kernel<2, kRoundedY, false, false> : tc_conv_kernel<1, kRoundedY, false, false>)
+                : split ? (add ? tc_conv_kernel<1, kAddendNear, false, true> : tc_conv_kernel<1, kNoAddend, false, true>)
                 : thin ? (far   ? (pair ? tc_conv_kernel<2, kAddendFar, true, false> : tc_conv_kernel<1, kAddendFar, true, false>)
                           : add ? (pair ? tc_conv_kernel<2, kAddendNear, true, false> : tc_conv_kernel<1, kAddendNear, true, false>)
                                 : (pair ? tc_conv_kernel<2, kNoAddend, true, false> : tc_conv_kernel<1, kNoAddend, true, false>))

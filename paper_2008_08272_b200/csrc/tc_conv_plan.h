@@ -61,6 +61,10 @@ struct TcConvPlan {
     // raw staging
     int raw_mode;                    // 0: tensor-map boxes [KB][BOXP] over X seen as (H*W, N*C); 1: whole-image slabs;
                                      // 2: one copy of rows per channel, [channel][BOXP]
+    // X is channel-major: raw_mode 0 over X seen as (images x H*W, C).  The images that a tile touches follow one another there,
+    // so its pixels are one range, and a few boxes bring several small images that slabs or boxes of each took a copy for.
+    int x_cm;
+    uint32_t y_image4, y_chan4;      // bytes from one image of Y (and R) to the next, and from one channel
     int BOXP;
     int KBR;                         // channels staged per block: KB, or all of a group's if it has fewer
     // shared memory carve-up (bytes)
@@ -222,6 +226,8 @@ ONNXB_HD inline void tc_conv_segments(const TcConvPlan &g, long long G0, TcConvS
     if (t.nseg > kConvMaxSeg) t.nseg = kConvMaxSeg;   // excluded by the planner
     t.one_image = t.nseg == 1 && Gend == G0 + g.SLOTS;
     int base = 0;
+    int first = -1, end = 0;         // channel-major: the tile's range of pixels, from image n_first's first
+    const int HW = g.H * g.W;
     for (int i = 0; i < t.nseg; ++i) {
         const long long n = t.n_first + i;
         const long long lo = G0 > n * g.L ? G0 : n * g.L;
@@ -233,7 +239,13 @@ ONNXB_HD inline void tc_conv_segments(const TcConvPlan &g, long long G0, TcConvS
         if (h_min < 0) h_min = 0;
         if (h_max > g.H - 1) h_max = g.H - 1;
         t.base[i] = base;
-        if (h_min > h_max) {
+        if (g.x_cm) {
+            t.nbox[i] = 0;
+            if (h_min <= h_max) {
+                if (first < 0) first = i * HW + h_min * g.W;
+                end = i * HW + (h_max + 1) * g.W;
+            }
+        } else if (h_min > h_max) {
             t.f0[i] = 0;
             t.nbox[i] = 0;
         } else if (g.raw_mode == 1) {
@@ -252,6 +264,13 @@ ONNXB_HD inline void tc_conv_segments(const TcConvPlan &g, long long G0, TcConvS
             t.nbox[i] = conv_fdiv(len + g.BOXP - 1, g.BOXP, g.dv_BOXP);
             base += t.nbox[i] * g.BOXP * g.KBR;
         }
+    }
+    if (g.x_cm && first >= 0) {
+        // (a copy starts on a 16-byte boundary: up to three pixels of what lies before)
+        const int start = (int)(((long long)t.n_first * HW + first) & ~3LL) - t.n_first * HW;
+        for (int i = 0; i < t.nseg; ++i) t.f0[i] = start - i * HW;
+        t.nbox[0] = conv_fdiv(end - start + g.BOXP - 1, g.BOXP, g.dv_BOXP);
+        base = t.nbox[0] * g.BOXP * g.KBR;
     }
     t.total_floats = base;
 }

@@ -69,8 +69,9 @@ struct Params {
     float r_scale;             // added before Relu
     int r_q;                   // R sampled: see TcGemmProblem
     int r_row, r_col;
-    float *Yr;                 // Y rounded to TF32, a second output (by tmR where Y is stored by TMA), or NULL
+    float *Yr;                 // Y rounded to TF32, a second output (by TMA where Y is), or NULL
     long long r_ld, r_bs;      // R's planes and images are that far apart
+    int r_split;
     ConvDivisor dv_rq, dv_split;
     int r_tma;                 // R is fetched by TMA (when Y is stored by TMA: same geometry), r_bufs blocks ahead
     int r_bufs;                // 1 or 2 blocks of R in flight per epilogue warp
@@ -102,7 +103,7 @@ template <int kCtas, int kKS, bool kC>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmBb, const __grid_constant__ CUtensorMap tmY,
-               const __grid_constant__ CUtensorMap tmR, const Params p) {
+               const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmYr, const Params p) {
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment by pointer arithmetic on the shared array itself, so that the compiler
     // keeps treating everything derived from it as shared memory (LDS/STS, not generic accesses)
@@ -408,9 +409,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         {
                             const int col = col0 + lane;
                             int pix = col, image = b;
-                            if (p.y_split > 0) {
-                                image = conv_fdiv(col, p.y_split, p.dv_split);
-                                pix = col - image * p.y_split;
+                            if (p.r_split > 0) {
+                                image = conv_fdiv(col, p.r_split, p.dv_split);
+                                pix = col - image * p.r_split;
                             }
                             if (p.r_q > 0) {
                                 const int pr = conv_fdiv(pix, p.r_q, p.dv_rq);
@@ -492,7 +493,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                             fence_proxy_async_smem();
                             __syncwarp();
                             if (lane == 0) {
-                                tma_store_3d(&tmR, buf, col0, row0, b);
+                                tma_store_3d(&tmYr, buf, col0, row0, b);
                                 tma_store_commit();
                             }
                         }
@@ -716,11 +717,12 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     const bool whole_c = g.C && g.c_si != 0 && g.c_sj != 0;
     p.R = whole_c ? g.C : g.C ? nullptr : g.residual;
     p.r_scale = whole_c ? g.beta : 1.f;
-    p.r_q = p.R ? g.r_q : 0; p.r_row = g.r_row; p.r_col = g.r_col; p.Yr = p.r_q ? g.Y_rounded : nullptr;
+    p.r_q = p.R ? g.r_q : 0; p.r_row = g.r_row; p.r_col = g.r_col; p.Yr = p.R ? g.Y_rounded : nullptr;
     p.r_ld = p.r_q ? g.r_ld : g.y_ld;
     p.r_bs = p.r_q ? g.r_bs : g.y_split > 0 ? g.y_group_stride : g.y_bs;
     p.dv_rq = conv_divisor(std::max(p.r_q, 1));
-    p.dv_split = conv_divisor(std::max(g.y_split, 1));
+    p.r_split = p.r_q ? g.r_split : g.y_split;
+    p.dv_split = conv_divisor(std::max(p.r_split, 1));
     p.r_tma = p.R != nullptr && p.y_tma && !p.r_q;
     // two blocks of R per epilogue warp when the operand ring keeps at least three stages beside them
     p.r_bufs = kResidualBufs;
@@ -742,7 +744,7 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     p.err = device_status_ptr();
     if (!p.err) return (int)cudaErrorUnknown;
 
-    CUtensorMap tmA, tmB, tmY, tmR;
+    CUtensorMap tmA, tmB, tmY, tmR, tmYr;
     // Operand maps.  K-major: (32 terms of a K block, row, K block, batch) where K is whole blocks, so that one box
     // carries a stage; else (term, row, batch, 1).  MN-major: (row, term, batch, 1).
     p.a_kbox = !p.a_mn && g.K % kBK == 0;
@@ -782,12 +784,12 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     } else {
         tmY = tmA;   // never dereferenced
     }
-    tmR = tmY;
+    tmR = tmYr = tmY;
     if (p.Yr && p.y_tma) {
         uint64_t dims[3] = {(uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.batch};
         uint64_t str[2] = {(uint64_t)g.y_ld * 4, g.batch > 1 ? (uint64_t)g.y_bs * 4 : (uint64_t)g.y_ld * 4 * g.M};
         uint32_t box[3] = {32, 32, 1};
-        if (!make_tmap(&tmR, p.Yr, 3, dims, str, box, kTmapSwizzle128)) return (int)cudaErrorInvalidValue;
+        if (!make_tmap(&tmYr, p.Yr, 3, dims, str, box, kTmapSwizzle128)) return (int)cudaErrorInvalidValue;
     }
     if (p.r_tma) {
         // the addend has Y's shape and strides, so its view is Y's with another base
@@ -812,9 +814,9 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     const int grid = (int)(total < units ? total : units) * p.ctas;
     const cudaError_t le =
         p.ctas == 2 ? launch_pdl_cluster(kern, 2, dim3(grid), dim3(kThreads), smem, (cudaStream_t)stream, tmA,
-                                         tmB, tmBb, tmY, tmR, p)
+                                         tmB, tmBb, tmY, tmR, tmYr, p)
                     : launch_pdl(kern, dim3(grid), dim3(kThreads), smem, (cudaStream_t)stream, tmA, tmB, tmBb,
-                                 tmY, tmR, p);
+                                 tmY, tmR, tmYr, p);
     count_launch();
     return (int)le;
 }

@@ -56,7 +56,8 @@ struct SkParams {
     int r_q, r_row, r_col;     // R sampled: see TcGemmProblem
     float *Yr;
     long long r_ld, r_bs;
-    ConvDivisor dv_rq;
+    int r_split;
+    ConvDivisor dv_rq, dv_rsplit;
     float *Y;
     long long y_ld, y_bs;
     int y_split;               // > 0: column j lies in group j / y_split, y_group elements further on
@@ -282,7 +283,7 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             } else if (p.R && p.r_q) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const int j = gcol + e, im = p.y_split ? conv_fdiv(j, p.y_split, p.dv_split) : batch, pix = p.y_split ? j - im * p.y_split : j;
+                    const int j = gcol + e, im = p.r_split ? conv_fdiv(j, p.r_split, p.dv_rsplit) : batch, pix = p.r_split ? j - im * p.r_split : j;
                     const int pr = conv_fdiv(pix, p.r_q, p.dv_rq);
                     if (j < p.N) add[e] = __ldg(p.R + im * p.r_bs + grow * p.r_ld + pr * p.r_row + (pix - pr * p.r_q) * p.r_col);
                 }
@@ -485,7 +486,9 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
     p.C = g.C; p.c_si = g.c_si; p.c_sj = g.c_sj;
     p.row_bias = g.row_bias;
     p.R = g.C ? nullptr : g.residual;
-    p.r_q = p.R ? g.r_q : 0; p.r_row = g.r_row; p.r_col = g.r_col; p.Yr = p.r_q ? g.Y_rounded : nullptr;
+    p.r_q = p.R ? g.r_q : 0; p.r_row = g.r_row; p.r_col = g.r_col; p.Yr = p.R ? g.Y_rounded : nullptr;
+    p.r_split = g.r_split;
+    p.dv_rsplit = conv_divisor(std::max(g.r_split, 1));
     p.r_ld = g.r_ld; p.r_bs = g.r_bs;
     p.dv_rq = conv_divisor(std::max(p.r_q, 1));
     p.relu = g.relu;

@@ -26,9 +26,10 @@ struct TcGemmProblem {
     // A residual read at every r_col-th place of every so-many-th row of its own images instead (r_q > 0: pixels in a row of the
     // output): planes r_ld elements apart, images r_bs, the rows that are read r_row, the places r_col.
     int r_q;
+    int r_split;             // columns are the pixels of images of so many (0: of one image, the batch's)
     long long r_ld, r_bs;
     int r_row, r_col;
-    float *Y_rounded;        // (with r_q) a second output, laid out like Y: Y rounded to TF32; may be NULL
+    float *Y_rounded;        // a second output of a layer with a residual, laid out like Y: Y rounded to TF32; may be NULL
     int relu;
     int round_operands;      // A and B are raw fp32: the split-K form rounds them itself, the other form is given copies
     float *Y;

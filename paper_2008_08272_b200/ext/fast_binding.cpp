@@ -25,6 +25,7 @@ struct Abi {
     decltype(&onnx_conv2d_add_run) conv_add_run;
     decltype(&onnx_conv2d_run_packed) conv_run_packed;
     decltype(&onnx_conv2d_run_packed_sampled) conv_run_packed_sampled;
+    decltype(&onnx_conv2d_run_packed_rounded) conv_run_packed_rounded;
     decltype(&onnx_gemm_workspace_bytes) gemm_workspace_bytes;
     decltype(&onnx_gemm_run) gemm_run;
     decltype(&onnx_maxpool2d_shape) maxpool2d_shape;
@@ -117,6 +118,7 @@ PyObject *py_bind(PyObject *, PyObject *arg) {
     get(abi.conv_add_run, "onnx_conv2d_add_run");
     get(abi.conv_run_packed, "onnx_conv2d_run_packed");
     get(abi.conv_run_packed_sampled, "onnx_conv2d_run_packed_sampled");
+    get(abi.conv_run_packed_rounded, "onnx_conv2d_run_packed_rounded");
     get(abi.gemm_workspace_bytes, "onnx_gemm_workspace_bytes");
     get(abi.gemm_run, "onnx_gemm_run");
     get(abi.maxpool2d_shape, "onnx_maxpool2d_shape");
@@ -152,25 +154,27 @@ inline bool ints(PyObject *o, int64_t *out, Py_ssize_t n) {
 }
 
 // conv(plan, X, W, packed, B, R, Y, workspace, stream): run (packed and R None), run_add (R given) or
-// run_packed (packed given); with two more arguments R and packed are given, R is read at every such row and column,
-// and the last one, if any, gets Y rounded
+// run_packed (packed given); with three more arguments (dims, strides, Y_rounded)
+// packed is given, R, of those rows and columns, is read at every such row and column, and Y_rounded, if any, gets Y rounded;
+// dims and strides None: R, if any, is read as it lies
 PyObject *py_conv(PyObject *, PyObject *const *a, Py_ssize_t n) {
-    if (n != 9 && n != 11) return slow_path();
+    if (n != 9 && n != 12) return slow_path();
     Plan *p = plan_of(a[0]);
     if (!p) { PyErr_Clear(); return slow_path(); }
     bool fine = true;
-    const at::Tensor *xt = nullptr, *rt = nullptr;
+    const at::Tensor *xt = nullptr;
     size_t packed_bytes, ws_bytes;
     const float *x = in_ptr(a[1], fine, &xt), *w = in_ptr(a[2], fine);
     const void *packed = ws_ptr(a[3], packed_bytes, fine);
-    const float *b = in_ptr(a[4], fine), *r = in_ptr(a[5], fine, &rt);
+    const float *b = in_ptr(a[4], fine), *r = in_ptr(a[5], fine);
     float *y = const_cast<float *>(in_ptr(a[6], fine));
     void *ws = ws_ptr(a[7], ws_bytes, fine), *st = stream_ptr(a[8], fine);
     if (!fine || !x || !w) return slow_path();
     const bool pre = a[3] != Py_None;
-    int64_t every[2];
-    float *y_rounded = n == 11 ? const_cast<float *>(in_ptr(a[10], fine)) : nullptr;
-    if (n == 11 && (!fine || !r || !pre || rt->dim() != 4 || a[9] == Py_None || !ints(a[9], every, 2))) return slow_path();
+    int64_t dims[2], every[2];
+    float *y_rounded = n == 12 ? const_cast<float *>(in_ptr(a[11], fine)) : nullptr;
+    const bool sampled = n == 12 && a[9] != Py_None;
+    if (!fine || (n == 12 && !pre) || (sampled && (!r || a[10] == Py_None || !ints(a[9], dims, 2) || !ints(a[10], every, 2)))) return slow_path();
     at::Tensor ym, wm;
     if (!y) {
         ym = new_tensor(p->y, at::kFloat, xt->device(), a[8], st, true);
@@ -181,8 +185,8 @@ PyObject *py_conv(PyObject *, PyObject *const *a, Py_ssize_t n) {
         ws = wm.data_ptr();
         ws_bytes = p->workspace;
     }
-    const onnxb_status s = n == 11 ? abi.conv_run_packed_sampled(p->desc, x, w, packed, packed_bytes, b, r, rt->sizes().data() + 2, every,
-                                                                 y, y_rounded, ws, ws_bytes, st)
+    const onnxb_status s = sampled   ? abi.conv_run_packed_sampled(p->desc, x, w, packed, packed_bytes, b, r, dims, every, y, y_rounded, ws, ws_bytes, st)
+                           : n == 12 ? abi.conv_run_packed_rounded(p->desc, x, w, packed, packed_bytes, b, r, y, y_rounded, ws, ws_bytes, st)
                            : pre ? abi.conv_run_packed(p->desc, x, w, packed, packed_bytes, b, r, y, ws, ws_bytes, st)
                            : r ? abi.conv_add_run(p->desc, x, w, b, r, y, ws, ws_bytes, st)
                                : abi.conv_run(p->desc, x, w, b, y, ws, ws_bytes, st);
