@@ -210,10 +210,12 @@ static onnxb_status conv2d_run_impl(onnxb_conv2d_desc_t d, const float *X, const
             float *ws = static_cast<float *>(workspace);
             const float *Wr = w_copy ? w_copy : ws;
             float *Xg = w_copy ? ws : ws + (size_t)d->g.M * d->g.C;
-            err = 0;
-            if (!w_copy) err = launch_round_tf32_copy(W, ws, (long long)d->g.M * d->g.C, nullptr, nullptr, 0, cuda_stream);
-            if (pack_only) break;
-            if (err == 0) err = launch_gather1x1(d->g, X, Xg, gather_pitch(d->g), gather_merged(d->g), cuda_stream);
+            const long long w_count = (long long)d->g.M * d->g.C;
+            if (pack_only) {
+                err = launch_round_tf32_copy(W, ws, w_count, nullptr, nullptr, 0, cuda_stream);
+                break;
+            }
+            err = launch_gather1x1(d->g, X, Xg, gather_pitch(d->g), gather_merged(d->g), w_copy ? nullptr : W, ws, w_count, cuda_stream);
             if (err == 0) err = launch_tc_gemm(sample(conv1x1_gathered_as_gemm(d->g, Xg, Wr, B, Y, R), d->g, sampled), cuda_stream);
             break;
         }

@@ -206,14 +206,29 @@ conv2d_depthwise_kernel(const ConvGeom g, const float *__restrict__ X, const flo
 // Both kernels below are bound by HBM (the pixels read once, the copy written once): one wave of eight blocks per SM, indices
 // by multiplication (256 channels 56x56 -> 28x28 at batch 32: some 20 -> 15 us).
 
+// Weights of the call, rounded to TF32 ahead of the pixels: a launch of its own for them in front took 3 us (256 -> 512 channels
+// 56x56/2 at batch 32 41.2 -> 39.8 us in all), most of it the launch.
+struct RoundedCopy {
+    const float4 *in;
+    float4 *out;
+    unsigned n4;
+};
+__device__ __forceinline__ void round_copy(const RoundedCopy &w) {
+    for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < w.n4; i += gridDim.x * 256u) {
+        const float4 v = __ldg(w.in + i);
+        w.out[i] = make_float4(tc::round_tf32(v.x), tc::round_tf32(v.y), tc::round_tf32(v.z), tc::round_tf32(v.w));
+    }
+}
+
 // Any layout whose pitch is a multiple of four (both layouts have one): four consecutive outputs per
 // thread, indices divided once and then stepped, four independent scalar loads, one 16-byte store.
 __global__ void __launch_bounds__(256)
 gather1x1_quad_kernel(const float *__restrict__ X, float4 *__restrict__ Xg4, unsigned total4, unsigned pitch,
                       unsigned NPQ, unsigned PQ, unsigned Q, unsigned C, unsigned HW, unsigned rowstep, unsigned sw,
-                      int merged, const ConvDivisor dv_pitch, const ConvDivisor dv_PQ, const ConvDivisor dv_Q) {
+                      int merged, const ConvDivisor dv_pitch, const ConvDivisor dv_PQ, const ConvDivisor dv_Q, const RoundedCopy w) {
     tc::pdl_launch_dependents();
     tc::pdl_wait();
+    round_copy(w);
     for (unsigned i4 = blockIdx.x * 256u + threadIdx.x; i4 < total4; i4 += gridDim.x * 256u) {
         const unsigned i = i4 * 4u;
         const unsigned row = (unsigned)conv_fdiv((int)i, (int)pitch, dv_pitch);   // merged: channel; per image: n*C + c
@@ -243,9 +258,10 @@ gather1x1_quad_kernel(const float *__restrict__ X, float4 *__restrict__ Xg4, uns
 template <int SW>
 __global__ void __launch_bounds__(256)
 gather1x1_vec_kernel(const float4 *__restrict__ X4, float4 *__restrict__ Xg4, unsigned total4, unsigned PQ4,
-                     unsigned Q4, unsigned HW4, unsigned rowstep4, const ConvDivisor dv_PQ4, const ConvDivisor dv_Q4) {
+                     unsigned Q4, unsigned HW4, unsigned rowstep4, const ConvDivisor dv_PQ4, const ConvDivisor dv_Q4, const RoundedCopy w) {
     tc::pdl_launch_dependents();
     tc::pdl_wait();
+    round_copy(w);
     for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < total4; i += gridDim.x * 256u) {
         const unsigned plane = (unsigned)conv_fdiv((int)i, (int)PQ4, dv_PQ4), r = i - plane * PQ4;
         const unsigned p = (unsigned)conv_fdiv((int)r, (int)Q4, dv_Q4), q4 = r - p * Q4;
@@ -681,7 +697,8 @@ bool simt_depthwise_supports(const ConvGeom &g) {
     return q_tiles * p_tiles * (long long)g.N * g.C <= 2147483647LL;
 }
 
-int launch_gather1x1(const ConvGeom &g, const float *X, float *Xg, long long pitch, bool merged, void *stream) {
+int launch_gather1x1(const ConvGeom &g, const float *X, float *Xg, long long pitch, bool merged, const float *W, float *Wr, long long w_count, void *stream) {
+    const RoundedCopy w{reinterpret_cast<const float4 *>(W), reinterpret_cast<float4 *>(Wr), W ? (unsigned)(w_count / 4) : 0u};
     const long long total = merged ? (long long)g.C * pitch : (long long)g.N * g.C * pitch;
     cudaStream_t st = (cudaStream_t)stream;
     const long long total4 = total / 4;                       // every pitch is a multiple of four
@@ -697,12 +714,12 @@ int launch_gather1x1(const ConvGeom &g, const float *X, float *Xg, long long pit
     if (!merged && g.Q % 4 == 0 && g.W % 4 == 0 && (g.sw == 1 || g.sw == 2) && g.Q * g.sw <= g.W) {
         const unsigned PQ4 = g.P * g.Q / 4, Q4 = g.Q / 4, HW4 = g.H * g.W / 4, rowstep4 = g.sh * g.W / 4;
         e = launch(g.sw == 1 ? gather1x1_vec_kernel<1> : gather1x1_vec_kernel<2>, reinterpret_cast<const float4 *>(X),
-                   reinterpret_cast<float4 *>(Xg), (unsigned)total4, PQ4, Q4, HW4, rowstep4, conv_divisor((int)PQ4), conv_divisor((int)Q4));
+                   reinterpret_cast<float4 *>(Xg), (unsigned)total4, PQ4, Q4, HW4, rowstep4, conv_divisor((int)PQ4), conv_divisor((int)Q4), w);
     } else {
         e = launch(gather1x1_quad_kernel, X, reinterpret_cast<float4 *>(Xg), (unsigned)total4, (unsigned)pitch,
                    (unsigned)(merged ? g.N * g.P * g.Q : g.P * g.Q), (unsigned)(g.P * g.Q), (unsigned)g.Q, (unsigned)g.C,
                    (unsigned)(g.H * g.W), (unsigned)(g.sh * g.W), (unsigned)g.sw, merged ? 1 : 0, conv_divisor((int)pitch),
-                   conv_divisor(g.P * g.Q), conv_divisor(g.Q));
+                   conv_divisor(g.P * g.Q), conv_divisor(g.Q), w);
     }
     count_launch();
     return (int)e;
