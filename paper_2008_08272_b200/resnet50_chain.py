@@ -10,6 +10,7 @@ operator runs in the library's kernels.
 """
 from __future__ import annotations
 
+import operator
 from dataclasses import dataclass, replace
 from typing import Dict, List, Optional
 
@@ -154,6 +155,7 @@ class Resnet50Chain:
             else:
                 self.store[op.dst] = self.buf[op.dst] = torch.empty(shape, dtype=torch.float32, device=device)
         self.flops = sum(op.case.flops for op in graph if op.case is not None) + 2 * batch * 2048 * 1000
+        self._capture()
 
     def _descriptors(self, ops: List[Op], channel_major: bool):
         """The convolutions' descriptors; None where one of them knows no channel-major tensors."""
@@ -183,10 +185,48 @@ class Resnet50Chain:
         d.close()
         return family == "mma_gather_gemm"
 
+    def _tensors(self):
+        """What the operators behind the first one read and write."""
+        return [t for k, t in self.store.items() if k != "input"] + list(self.rounded.values()) + list(self.packed.values()) + \
+            [t for pair in self.params.values() for t in pair] + [self.workspace, self.fc_workspace]
+
+    def _capture(self):
+        """The operators behind the first one, which alone reads the caller's tensor, as one CUDA graph."""
+        torch = self.torch
+        with torch.cuda.device(self.dev):
+            stream, before = torch.cuda.Stream(), binding.launch_count()
+            stream.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(stream):
+                self.store["input"] = torch.zeros((self.batch, 3, 224, 224), device=self.dev)
+                self._run(self.ops)                 # (what a first launch sets up is set up before the capture)
+                del self.store["input"]
+                self.launches = binding.launch_count() - before
+                # (begun and ended by hand: the context manager also collects garbage and empties the allocator's cache)
+                graph = torch.cuda.CUDAGraph()
+                graph.capture_begin(capture_error_mode="thread_local")
+                try:
+                    self._run(self.ops[1:])
+                finally:
+                    graph.capture_end()
+            torch.cuda.current_stream().wait_stream(stream)
+        self._graph, self._captured = graph, self._tensors()
+
     def forward(self, x):
         """Enqueue the whole model on the current stream; returns the logits buffer."""
         self.buf["input"] = self.store["input"] = x
-        for op in self.ops:
+        # All but the first operator in one launch in place of some fifty.  Made one by one where the call is itself being captured,
+        # or where a tensor of the graph's has been put in another's place.
+        now = self._tensors()
+        if self._graph is None or len(now) != len(self._captured) or not all(map(operator.is_, now, self._captured)) or \
+                self.torch.cuda.is_current_stream_capturing():
+            self._run(self.ops)
+        else:
+            self._run(self.ops[:1])
+            self._graph.replay()
+        return self.buf["logits"]
+
+    def _run(self, ops: List[Op]):
+        for op in ops:
             src, dst = self.store[op.src], self.store[op.dst]
             if op.kind in ("conv", "conv_add") and self.channel_major:
                 d, (W, B), packed = self.descs[op.name], self.params[op.name], self.packed[op.name]
@@ -221,9 +261,9 @@ class Resnet50Chain:
             else:
                 W, B = self.params["fc"]
                 binding.onnx_matmul_add(src.view(self.batch, 2048), W, B, Y=dst, workspace=self.fc_workspace)
-        return self.buf["logits"]
 
     def close(self):
+        self._graph = self._captured = None
         for d in self.descs.values():
             d.close()
         self.descs.clear()
