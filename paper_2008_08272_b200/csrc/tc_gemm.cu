@@ -99,7 +99,10 @@ struct Params {
 // of a 256 x 64 pair tile: 660 -> 390 cycles; Gemm 1024 x 1024 x 4096 48.6 -> 34.3 us, 4096^3 239 -> 223 us.
 // kC: with a broadcast addend, a form of its own, so that the others, which most launches are, carry none of its code (the
 // epilogue runs a few times per launch, mostly out of cold instruction memory: see its loop).
-template <int kCtas, int kKS, bool kC>
+// kS: with a sampled R, whose blocks' values are in flight in 32 registers a block ahead.  Read where they are used, as those of
+// an R laid out like Y are, each block waits for a trip to memory: 64 -> 256 channels at 28x28, batch 64, R of 56x56, 65 us against 61 (ncu);
+// asked into L2 a tile ahead by prefetches instead, 76.
+template <int kCtas, int kKS, bool kC, bool kS = false>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmBb, const __grid_constant__ CUtensorMap tmY,
@@ -355,6 +358,21 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 const int col = tn * p.BN + chunk * 32 + lane;
                 cv = chunk < c_hi && col < p.N ? __ldg(p.C + col) : 0.f;
             };
+            // the sampled R of a block: lane = column, a row per register
+            float rv[32];
+            auto fetch_sampled = [&](int chunk) {
+                const int col = tn * p.BN + chunk * 32 + lane, rows = min(32, p.M - row0);
+                const bool in = chunk < c_hi && col < p.N;
+                const int image = p.r_split > 0 ? conv_fdiv(col, p.r_split, p.dv_split) : b, pix = p.r_split > 0 ? col - image * p.r_split : col;
+                const int pr = conv_fdiv(pix, p.r_q, p.dv_rq);
+                const float *rp = p.R + image * p.r_bs + (long long)row0 * p.r_ld + pr * p.r_row + (pix - pr * p.r_q) * p.r_col;
+#pragma unroll
+                for (int r = 0; r < 32; ++r) {
+                    rv[r] = in && r < rows ? __ldg(rp) : 0.f;
+                    rp += p.r_ld;
+                }
+            };
+            if (kS && row0 < p.M) fetch_sampled(c_lo);
             if (kC) {
                 if (p.c_sj != 0) fetch_c(c_lo);
                 else if (row < p.M) cv = __ldg(p.C + (long long)row * p.c_si);
@@ -368,13 +386,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 auto finish = [&](const uint32_t (&v)[32], int chunk) {
                     const int col0 = tn * p.BN + chunk * 32;
                     float f[32];
-                    if (!kC && p.R == nullptr) {
+                    if (!kC && !kS && p.R == nullptr) {
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
                             const float x = fmaf(p.alpha, __uint_as_float(v[j]), rb);
                             f[j] = p.relu ? fmaxf(x, 0.f) : x;
                         }
-                    } else if (!kC && p.r_tma) {
+                    } else if (!kC && !kS && p.r_tma) {
                         // Residual addend by TMA: the block of R lands in the warp's ring with the same 128-byte
                         // swizzle as the Y staging block, so a lane reads its row back in eight 16-byte pieces;
                         // the slot is then refilled with the block two ahead.
@@ -408,26 +426,24 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         __syncwarp();
                         {
                             const int col = col0 + lane;
-                            int pix = col, image = b;
-                            if (p.r_split > 0) {
-                                image = conv_fdiv(col, p.r_split, p.dv_split);
-                                pix = col - image * p.r_split;
-                            }
-                            if (p.r_q > 0) {
-                                const int pr = conv_fdiv(pix, p.r_q, p.dv_rq);
-                                pix = pr * p.r_row + (pix - pr * p.r_q) * p.r_col;
-                            }
-                            const float *rp = p.R + image * p.r_bs + (long long)row0 * p.r_ld + pix;
-                            const int rows = min(32, p.M - row0);
-                            float t[32];
+                            if (!kS) {
+                                int pix = col, image = b;
+                                if (p.r_split > 0) {
+                                    image = conv_fdiv(col, p.r_split, p.dv_split);
+                                    pix = col - image * p.r_split;
+                                }
+                                const float *rp = p.R + image * p.r_bs + (long long)row0 * p.r_ld + pix;
+                                const int rows = min(32, p.M - row0);
 #pragma unroll
-                            for (int r = 0; r < 32; ++r) {
-                                t[r] = (r < rows && col < p.N) ? __ldg(rp) : 0.f;
-                                rp += p.r_ld;
+                                for (int r = 0; r < 32; ++r) {
+                                    rv[r] = (r < rows && col < p.N) ? __ldg(rp) : 0.f;
+                                    rp += p.r_ld;
+                                }
                             }
 #pragma unroll
                             for (int r = 0; r < 32; ++r)
-                                *reinterpret_cast<float *>(buf + r * 128 + ((((lane >> 2) ^ (r & 7)) << 4) | ((lane & 3) << 2))) = t[r];
+                                *reinterpret_cast<float *>(buf + r * 128 + ((((lane >> 2) ^ (r & 7)) << 4) | ((lane & 3) << 2))) = rv[r];
+                            if (kS) fetch_sampled(chunk + 1);
                         }
                         __syncwarp();
 #pragma unroll
@@ -804,7 +820,9 @@ int launch_tc_gemm(const TcGemmProblem &g, void *stream) {
     }
 
     const size_t smem = smem_with_tmem(1024 + (size_t)p.num_stages * p.stage_bytes + p.staging_bytes + kBarrierBytes, 512);
-    auto kern = p.C ? (p.ctas == 2 ? (ks == 2 ? tc_gemm_kernel<2, 2, true> : tc_gemm_kernel<2, 1, true>)
+    auto kern = p.r_q ? (p.ctas == 2 ? (ks == 2 ? tc_gemm_kernel<2, 2, false, true> : tc_gemm_kernel<2, 1, false, true>)
+                                     : (ks == 2 ? tc_gemm_kernel<1, 2, false, true> : tc_gemm_kernel<1, 1, false, true>))
+                : p.C ? (p.ctas == 2 ? (ks == 2 ? tc_gemm_kernel<2, 2, true> : tc_gemm_kernel<2, 1, true>)
                                    : (ks == 2 ? tc_gemm_kernel<1, 2, true> : tc_gemm_kernel<1, 1, true>))
                     : p.ctas == 2 ? (ks == 2 ? tc_gemm_kernel<2, 2, false> : tc_gemm_kernel<2, 1, false>)
                                   : (ks == 2 ? tc_gemm_kernel<1, 2, false> : tc_gemm_kernel<1, 1, false>);
