@@ -283,13 +283,22 @@ class Conv2dDesc:
         self._packed_needs_ws = self.workspace_bytes > self.packed_bytes
         self._plan = None
 
-    def _native(self, X, W, packed, B, R, Y, workspace, stream, *sampled):
+    def _native(self, X, W, packed, B, R, Y, workspace, stream):
         """The call through the native path; None when it declined."""
         if self._plan is None:
             if not self._h:
                 return None
             self._plan = _fast().plan(self._h.value, self.y_storage, self.workspace_bytes, self.packed_bytes, self._packed_needs_ws)
-        return _fast_mod.conv(self._plan, X, W, packed, B, R, Y, workspace, stream, *sampled)
+        return _fast_mod.conv(self._plan, X, W, packed, B, R, Y, workspace, stream)
+
+    def _native_rounded(self, X, W, packed, B, R, Y, workspace, stream, r_dims, strides, Y_rounded):
+        """The same with an addend that is sampled (r_dims not None), or Y rounded as well.  (A function of its own: arguments passed on
+        as a tuple would cost every call 0.1 us.)"""
+        if self._plan is None:
+            if not self._h:
+                return None
+            self._plan = _fast().plan(self._h.value, self.y_storage, self.workspace_bytes, self.packed_bytes, self._packed_needs_ws)
+        return _fast_mod.conv(self._plan, X, W, packed, B, R, Y, workspace, stream, r_dims, strides, Y_rounded)
 
     def run(self, X, W, B=None, Y=None, workspace=None, stream=None):
         """``onnx_conv2d_run``; allocates Y (and a workspace) with torch when not supplied."""
@@ -359,7 +368,7 @@ class Conv2dDesc:
             if R.dim() != 4 or tuple(R.shape[:2]) != self.y_shape[:2]:
                 raise OnnxB200Error(3, "run_prepacked_sampled: the addend's images and channels are not the output's")
             r_dims = tuple(R.shape[2:])
-        y = self._native(X, W, packed, B, R, Y, workspace, stream, r_dims, strides, Y_rounded)
+        y = self._native_rounded(X, W, packed, B, R, Y, workspace, stream, r_dims, strides, Y_rounded)
         if y is not None:
             return y
         if Y is None:
@@ -376,7 +385,7 @@ class Conv2dDesc:
 
     def run_prepacked_rounded(self, X, W, packed, B, R, Y, Y_rounded, stream=None):
         """``onnx_conv2d_run_packed_rounded``: run_prepacked, and Y rounded to TF32 into ``Y_rounded`` (Y itself where it is that)."""
-        y = self._native(X, W, packed, B, R, Y, None, stream, None, None, Y_rounded)
+        y = self._native_rounded(X, W, packed, B, R, Y, None, stream, None, None, Y_rounded)
         if y is not None:
             return y
         _check(self._lib.onnx_conv2d_run_packed_rounded(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"), ctypes.c_void_p(packed.data_ptr()),
