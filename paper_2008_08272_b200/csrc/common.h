@@ -22,6 +22,7 @@ struct ConvGeom {
     int sh, sw, dh, dw;
     int group, Mg;           // Mg = M/group
     int has_bias, relu;
+    int small_mb;            // output channels per block of the small-image kernel
 };
 
 struct Fp32GemmPlan {        // tile width, and CTAs that share a tile's reduction (tc_fp32.cu)
@@ -61,6 +62,7 @@ int simt_conv_on_tensor_cores(const ConvGeom &g, Fp32ConvPlan &plan, Fp32GemmPla
 int launch_simt_depthwise(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                           void *stream);
 double small_conv_cost(const ConvGeom &g);           // estimated SM cycles; negative: not for this problem
+int small_conv_channels(const ConvGeom &g);
 int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                       void *stream);
 bool simt_depthwise_supports(const ConvGeom &g);

@@ -26,7 +26,7 @@ template <int MB, int K>
 __global__ void __launch_bounds__(kSmallThreads)
 conv2d_small_kernel(const __grid_constant__ ConvGeom g, const float *__restrict__ X, const float *__restrict__ W,
                     const float *__restrict__ B, const float *__restrict__ R, float *__restrict__ Y, int Hp, int Wp, int taps4,
-                    const ConvDivisor dv_Wp, const ConvDivisor dv_HpWp, const ConvDivisor dv_Q, const ConvDivisor dv_taps) {
+                    const ConvDivisor dv_Hp, const ConvDivisor dv_Q, const ConvDivisor dv_taps) {
     extern __shared__ __align__(16) float sm[];
     const int taps = K > 0 ? K * K : g.kH * g.kW, kW = K > 0 ? K : g.kW;
     const int ptiles = (g.P * g.Q + kSmallThreads - 1) / kSmallThreads, mtiles = (g.Mg + MB - 1) / MB;
@@ -55,20 +55,22 @@ conv2d_small_kernel(const __grid_constant__ ConvGeom g, const float *__restrict_
         }
     }
     const float *xg = X + ((size_t)n * g.C + (size_t)grp * g.Cg) * g.H * g.W;
-    const int total = g.Cg * plane;
-    for (int i0 = threadIdx.x; i0 < total; i0 += 8 * kSmallThreads) {
-        float v[8];
+    // 8, 16 or 32 threads a row (a position divided by the row's width and the plane took three times the instructions)
+    const int rows = g.Cg * Hp, lanes = Wp <= 8 ? 8 : Wp <= 16 ? 16 : 32, step = kSmallThreads / lanes;
+    for (int wp = threadIdx.x & (lanes - 1); wp < Wp; wp += lanes) {
+        const int w = wp - g.pl;
+        const bool in = (unsigned)w < (unsigned)g.W;
+        for (int r0 = threadIdx.x / lanes; r0 < rows; r0 += 8 * step) {
+            float v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = i0 + u * kSmallThreads;
-            const int c = conv_fdiv(i, plane, dv_HpWp), r = i - c * plane;
-            const int hp = conv_fdiv(r, Wp, dv_Wp), h = hp - g.pt, w = r - hp * Wp - g.pl;
-            const bool ok = i < total && (unsigned)h < (unsigned)g.H && (unsigned)w < (unsigned)g.W;
-            v[u] = ok ? __ldg(xg + ((size_t)c * g.H + h) * g.W + w) : 0.f;
+            for (int u = 0; u < 8; ++u) {
+                const int r = r0 + u * step, c = conv_fdiv(r, Hp, dv_Hp), h = r - c * Hp - g.pt;
+                v[u] = in && r < rows && (unsigned)h < (unsigned)g.H ? __ldg(xg + ((size_t)c * g.H + h) * g.W + w) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (r0 + u * step < rows) xs[(r0 + u * step) * Wp + wp] = v[u];
         }
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (i0 + u * kSmallThreads < total) xs[i0 + u * kSmallThreads] = v[u];
     }
     __syncthreads();
 
@@ -637,29 +639,32 @@ void depthwise_window(const ConvGeom &g, int &rows, int &cols, int &pitch) {
 
 }  // namespace
 
-// Channels per block: as many as still leave every SM two blocks.
-static int small_mb(const ConvGeom &g) {
-    const long long ptiles = ((long long)g.P * g.Q + kSmallThreads - 1) / kSmallThreads;
-    for (int mb = 16; mb >= 4; mb /= 2)
-        if (g.Mg > mb / 2 && (long long)g.N * g.group * ((g.Mg + mb - 1) / mb) * ptiles >= 148 * 2) return mb;
-    return 1;
-}
 static size_t small_smem(const ConvGeom &g, int mb) {
     const long long Hp = (long long)(g.P - 1) * g.sh + (long long)(g.kH - 1) * g.dh + 1, Wp = (long long)(g.Q - 1) * g.sw + (long long)(g.kW - 1) * g.dw + 1;
     const long long taps = (long long)g.kH * g.kW;
     if (Hp * Wp > 16384 || taps > 4096 || g.Cg > 16384) return (size_t)-1;
     return (size_t)g.Cg * 4 * (Hp * Wp + (mb == 1 ? (taps + 3) / 4 * 4 : taps * mb));
 }
-// Estimated SM cycles, or a negative number where the kernel does not apply.
-double small_conv_cost(const ConvGeom &g) {
-    const int mb = small_mb(g);
-    const size_t smem = small_smem(g, mb);
-    if (smem > (size_t)kSmallSmem || (long long)g.P * g.Q > 4096) return -1;
+// Blocks of a problem with mb channels each, or a negative number where the kernel does not apply.
+static long long small_blocks(const ConvGeom &g, int mb) {
+    if (small_smem(g, mb) > (size_t)kSmallSmem || (long long)g.P * g.Q > 4096) return -1;
     const long long ptiles = ((long long)g.P * g.Q + kSmallThreads - 1) / kSmallThreads;
     const long long blocks = (long long)g.N * g.group * ((g.Mg + mb - 1) / mb) * ptiles;
-    if (blocks > 1000000) return -1;
+    return blocks > 1000000 ? -1 : blocks;
+}
+// Estimated SM cycles against the other kernels', or a negative number where the kernel does not apply: with as many channels per
+// block as still leave every SM two blocks.
+double small_conv_cost(const ConvGeom &g) {
+    const long long ptiles = ((long long)g.P * g.Q + kSmallThreads - 1) / kSmallThreads;
+    int mb = 16;
+    for (; mb >= 4; mb /= 2)
+        if (g.Mg > mb / 2 && (long long)g.N * g.group * ((g.Mg + mb - 1) / mb) * ptiles >= 148 * 2) break;
+    if (mb < 4) mb = 1;
+    const long long blocks = small_blocks(g, mb);
+    if (blocks < 0) return -1;
     // One wave of resident blocks: the loads come in batches of eight per thread, each a trip to L2, then the sum;
     // and no less than what an SM's blocks need in turn (measured: 100 cycles per element a thread brings in).
+    const size_t smem = small_smem(g, mb);
     const double kred = (double)g.Cg * g.kH * g.kW, per_sm = (double)((blocks + 147) / 148);
     const double unrolled = g.kH == g.kW && (g.kH == 3 || g.kH == 5) ? 1.0 : 2.5;
     const double fill = (double)smem / 4 / kSmallThreads;
@@ -668,9 +673,28 @@ double small_conv_cost(const ConvGeom &g) {
     const double issue = per_sm * (fill * 100.0 + kred * unrolled * (mb == 1 ? 3.0 : 1.5 + 2.2 * mb));
     return 5500.0 + std::max(latency, issue);
 }
+// Channels per block of a problem that comes here, fitted to MNIST's layers at batch 1 to 200: what a block takes by itself, and half of
+// that for every other block on its SM (0.4 with eight channels and more).  (By the rule above the second layer at batch 18, 576 blocks of one channel, brings every
+// image in sixteen times: 12.6 us, 5.8 with four channels; eight and more leave a warp alone with its latencies: 11.2 at batch 30.)
+int small_conv_channels(const ConvGeom &g) {
+    int best = 1;
+    double cost = -1;
+    const double kred = (double)g.Cg * g.kH * g.kW * (g.kH == g.kW && (g.kH == 3 || g.kH == 5) ? 1.0 : 2.5);
+    for (int mb : {1, 4, 8, 16}) {
+        const long long blocks = mb == 1 || g.Mg > mb / 2 ? small_blocks(g, mb) : -1;
+        if (blocks < 0) continue;
+        const double one = (double)small_smem(g, mb) / 4 / kSmallThreads / 8 * 900.0 + kred * (mb <= 4 ? 18.0 : 60.0);
+        const double c = one * (1.0 + (mb <= 4 ? 0.5 : 0.4) * (double)((blocks + 147) / 148 - 1));
+        if (cost < 0 || c < cost) {
+            cost = c;
+            best = mb;
+        }
+    }
+    return best;
+}
 
 int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y, void *stream) {
-    const int mb = small_mb(g), taps = g.kH * g.kW;
+    const int mb = g.small_mb, taps = g.kH * g.kW;
     const int Hp = (g.P - 1) * g.sh + (g.kH - 1) * g.dh + 1, Wp = (g.Q - 1) * g.sw + (g.kW - 1) * g.dw + 1;
     const long long ptiles = ((long long)g.P * g.Q + kSmallThreads - 1) / kSmallThreads;
     const long long blocks = (long long)g.N * g.group * ((g.Mg + mb - 1) / mb) * ptiles;
@@ -680,9 +704,17 @@ int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const f
                 : mb == 4 ? pick(conv2d_small_kernel<4, 3>, conv2d_small_kernel<4, 5>, conv2d_small_kernel<4, 0>)
                 : mb == 8 ? pick(conv2d_small_kernel<8, 3>, conv2d_small_kernel<8, 5>, conv2d_small_kernel<8, 0>)
                           : pick(conv2d_small_kernel<16, 3>, conv2d_small_kernel<16, 5>, conv2d_small_kernel<16, 0>);
-    const cudaError_t e = tc_host::launch_pdl(kern, dim3((unsigned)blocks), dim3(kSmallThreads), small_smem(g, mb), (cudaStream_t)stream,
-                                              g, X, W, B, R, Y, Hp, Wp, (taps + 3) / 4 * 4, conv_divisor(Wp),
-                                              conv_divisor(Hp * Wp), conv_divisor(g.Q), conv_divisor(taps));
+    // Blocks placed while the previous kernel still holds its SMs crowd on those that happen to have room: so much shared memory is
+    // asked for that no SM takes more than its share.  MNIST at batch 18 34.6 -> 19.6 us, at batch 39 36.7 -> 21.5 (with the channels per block above).
+    size_t smem = small_smem(g, mb);
+    const long long share = (blocks + 147) / 148;
+    if (blocks > 100 && share <= 8) {
+        smem = std::max(smem, (size_t)(228 * 1024 / share - 1024) / 128 * 128 - (share == 1 ? 1024 : 0));
+        const cudaError_t ae = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (ae != cudaSuccess) return (int)ae;
+    }
+    const cudaError_t e = tc_host::launch_pdl(kern, dim3((unsigned)blocks), dim3(kSmallThreads), smem, (cudaStream_t)stream, g, X, W, B, R, Y, Hp, Wp,
+                                              (taps + 3) / 4 * 4, conv_divisor(Hp), conv_divisor(g.Q), conv_divisor(taps));
     count_launch();
     return (int)e;
 }
