@@ -386,10 +386,15 @@ constexpr Shape kShape[kShapes] = {{128, 128, 256, 0.73}, {64, 128, 128, 0.68}, 
 template <int AM, int BMODE, int I, int BM, int BN, int TM, int TN>
 cudaError_t launch_shape(const SgemmArgs &a, int split, long long tiles, cudaStream_t st) {
     static_assert(kShape[I].bm == BM && kShape[I].bn == BN && kShape[I].threads == (BM / TM) * (BN / TN), "shape table");
-    constexpr size_t smem = sgemm_smem<BM, BN>();
+    // Blocks placed while the previous kernel still holds its SMs crowd on those that happen to have room: so much shared memory is
+    // asked for that no SM takes more than its share (clusters, which do not fit every GPC, one more).  Gemm 157 x 225 x 786 15.0 -> 9.6 us,
+    // 18 x 1543 x 181 10.0 -> 6.5, 1001 x 130 x 333 15.0 -> 13.2; 12 -> 40 channels 3x3 33x31 at batch 3 11.5 -> 9.9.
+    size_t smem = sgemm_smem<BM, BN>();
+    const long long ctas = tiles * split, share = (ctas + 147) / 148 + (split > 1 ? 1 : 0);
+    if (ctas > 100 && share <= 4) smem = std::max(smem, (size_t)(227 * 1024 / share - 1024) / 128 * 128);
     auto kern = sgemm_kernel<BM, BN, TM, TN, AM, BMODE>;
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) return e;
     }
     const dim3 grid((unsigned)(tiles * split)), block(kShape[I].threads);
