@@ -46,10 +46,10 @@ SAMPLE_TEXT = ("first 16 images of each of the 54 convolutions plus the full hea
 # DRAM traffic of the implicit-GEMM convolution kernel per benchmark step (its 17 launches), from the
 # ncu captures summarised in profiles/tc_conv_kernel_dram_traffic_per_layer_shape.md.  Valid only for
 # the kernel source those captures ran: the hash below is checked at run time.
-NCU_TRAFFIC = {"mma_implicit": {"bytes_per_step": 596.6e6,
+NCU_TRAFFIC = {"mma_implicit": {"bytes_per_step": 596.5e6,
                                 "sources": ["paper_2008_08272_b200/csrc/tc_conv.cu",
                                             "paper_2008_08272_b200/csrc/tc_conv_plan.h"],
-                                "sha1": "9c20d9df617b2ed45c55e5796fcb96036c4e019e"}}
+                                "sha1": "d636b8dbb166607bbc28444fd0930dc9b1256cf6"}}
 
 
 def ncu_traffic(family):
