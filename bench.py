@@ -648,7 +648,7 @@ def run_model(args):
     per_pass = int(net.launches)
     run = lambda: net.forward(x)
     if args.graph:
-        # the whole pass captured once into a CUDA graph and replayed: the 56 library calls per pass (argument
+        # the whole pass captured once into a CUDA graph and replayed: the library calls of a pass (argument
         # checks, tensor-map encoding, launches) then cost the host nothing, which is what bounds batch 1
         side = torch.cuda.Stream()
         side.wait_stream(torch.cuda.current_stream())
