@@ -22,7 +22,8 @@ struct ConvGeom {
     int sh, sw, dh, dw;
     int group, Mg;           // Mg = M/group
     int has_bias, relu;
-    int small_mb;            // output channels per block of the small-image kernel
+    int small_mb;            // output channels per block of the small-image kernel,
+    double small_cost;       // and its estimate (small_conv_cost)
 };
 
 struct Fp32GemmPlan {        // tile width, and CTAs that share a tile's reduction (tc_fp32.cu)

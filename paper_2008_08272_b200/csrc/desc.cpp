@@ -130,6 +130,7 @@ extern "C" onnxb_status onnx_conv2d_desc_layout(const onnxb_conv2d_attrs *a, int
     g.has_bias = a->has_bias != 0; g.relu = a->fuse_relu != 0;
     g.x_cm = x_channel_major != 0; g.y_cm = y_channel_major != 0;
     g.small_mb = small_conv_channels(g);
+    g.small_cost = small_conv_cost(g);
     d->y_dims[0] = N; d->y_dims[1] = M; d->y_dims[2] = P; d->y_dims[3] = Q;
     for (int i = 0; i < 4; ++i) d->pads[i] = pads[i];
 

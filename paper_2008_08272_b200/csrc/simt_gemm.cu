@@ -569,7 +569,7 @@ int launch_simt_conv(const ConvGeom &g, const float *X, const float *W, const fl
     a.dv_PQ = conv_divisor(a.PQ); a.dv_Q = conv_divisor(a.Q); a.dv_taps = conv_divisor(a.taps); a.dv_kW = conv_divisor(a.kW);
     const Choice ch = choose(a.M, a.N, a.K, g.group, true);
     const Pick pick = ch.pick;
-    const double small = small_conv_cost(g);
+    const double small = g.small_cost;
     const char *pin = getenv("ONNXB_FP32");              // "small" pins the small-image kernel
     if (small >= 0 && (pin ? pin[0] == 's' : 0.85 * small < ch.pick.cost))      // (the tiled estimate runs low here)
         return launch_small_conv(g, X, W, B, R, Y, stream);

@@ -67,7 +67,8 @@ struct SkParams {
 };
 
 // kKS: K blocks per stage (two wherever a CTA has two: see tc_gemm.cu for what a stage costs its issuing threads)
-template <int kKS>
+// kExt: with a sampled addend or a second, rounded output; a form of its own (the code, not executed, cost Gemm 2048 x 224 x 144 3 %)
+template <int kKS, bool kExt = false>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       const __grid_constant__ CUtensorMap tmBb, const __grid_constant__ SkParams p) {
@@ -280,7 +281,7 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     if (gcol + e < p.N) add[e] = p.beta * __ldg(p.C + (long long)grow * p.c_si + (long long)(gcol + e) * p.c_sj);
-            } else if (p.R && p.r_q) {
+            } else if (kExt && p.R && p.r_q) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int j = gcol + e, im = p.r_split ? conv_fdiv(j, p.r_split, p.dv_rsplit) : batch, pix = p.r_split ? j - im * p.r_split : j;
@@ -314,7 +315,7 @@ tc_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 #pragma unroll
                 for (int e = 0; e < 4; ++e) o[e] = fmaxf(o[e], 0.f);
             }
-            if (p.Yr) {
+            if (kExt && p.Yr) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     if (gcol + e < p.N) p.Yr[yi[e]] = round_tf32(o[e]);
@@ -530,7 +531,8 @@ int launch_tc_gemm_splitk(const TcGemmProblem &g, void *stream) {
     }
     p.recv_off = (uint32_t)p.num_stages * p.stage_bytes;
     const size_t smem = smem_with_tmem(2048 + p.recv_off + std::max(recv_bytes, (size_t)kABytes), kMaxBN);      // (at least what an MMA of the last stage reads)
-    auto kern = ks == 2 ? tc_gemm_splitk_kernel<2> : tc_gemm_splitk_kernel<1>;
+    auto kern = p.r_q || p.Yr ? (ks == 2 ? tc_gemm_splitk_kernel<2, true> : tc_gemm_splitk_kernel<1, true>)
+                              : (ks == 2 ? tc_gemm_splitk_kernel<2> : tc_gemm_splitk_kernel<1>);
     const cudaError_t ae = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (ae != cudaSuccess) return (int)ae;
     const dim3 grid((unsigned)((long long)p.tiles_m * p.tiles_n * g.batch * p.S)), block(kThreads);
