@@ -360,7 +360,14 @@ onnxb_status onnxb_last_device_status(void *cuda_stream);
  */
 void onnxb_set_kernel_override(int family);
 
-/* Number of kernels this library has launched since it was loaded (all streams). */
+/*
+ * onnxb_dispatch_state - a number that differs where what the calls choose their kernels by does: the override above, and the
+ * environment variables ONNXB_*, which pin shapes for A/B measurements and are read at every call.  For what keeps launches for
+ * later, as a CUDA graph does.
+ */
+uint64_t onnxb_dispatch_state(void);
+
+/* Number of kernels that calls of this library have launched since it was loaded (all streams). */
 uint64_t onnxb_launch_count(void);
 
 /*

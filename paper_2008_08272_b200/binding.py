@@ -33,7 +33,7 @@ EXPORTS = [
     "onnx_maxpool2d_shape", "onnx_maxpool2d_run", "onnx_global_average_pool_run", "onnx_conv2d_add_run",
     "onnx_conv2d_prepack", "onnx_conv2d_run_prepacked", "onnx_conv2d_packed_bytes", "onnx_conv2d_run_packed",
     "onnx_conv2d_run_packed_sampled", "onnx_conv2d_run_packed_rounded", "onnx_conv2d_desc_layout", "onnxb_channel_pitch",
-    "onnx_global_average_pool_channel_major_run",
+    "onnx_global_average_pool_channel_major_run", "onnxb_dispatch_state",
     "onnxb_probe_wait_timeout",
 ]
 
@@ -161,6 +161,8 @@ def load(build_if_missing: bool = True):
     lib.onnxb_last_device_status.argtypes = [vp]
     lib.onnxb_set_kernel_override.restype = None
     lib.onnxb_set_kernel_override.argtypes = [ctypes.c_int]
+    lib.onnxb_dispatch_state.restype = ctypes.c_uint64
+    lib.onnxb_dispatch_state.argtypes = []
     lib.onnxb_launch_count.restype = ctypes.c_uint64
     lib.onnxb_launch_count.argtypes = []
     lib.onnxb_probe_tf32_mma_rate.restype = ctypes.c_int
@@ -477,7 +479,14 @@ def set_kernel_override(family) -> None:
 
 
 def launch_count() -> int:
+    """``onnxb_launch_count``: kernels launched by operator calls (those of a replayed CUDA graph are launched by no call)."""
     return int(load().onnxb_launch_count())
+
+
+def call_state(tensors):
+    """Where the tensors lie and how (address, type, sizes, strides) and ``onnxb_dispatch_state``, as bytes to compare: calls on the same
+    tensors at the same state launch the same kernels on the same memory.  None without the native call path."""
+    return (_fast_mod or _fast()).state(tensors)
 
 
 def probe_tf32_mma_rate(n: int, instructions: int = 4096, stream=None) -> float:

@@ -5,6 +5,8 @@
 #include <cstring>
 #include <new>
 
+#include <unistd.h>
+
 #include "common.h"
 
 namespace onnxb {
@@ -190,6 +192,18 @@ extern "C" void onnx_conv2d_desc_destroy(onnxb_conv2d_desc_t d) { delete d; }
 extern "C" void onnxb_set_kernel_override(int family) {
     kernel_override();   // make sure the environment has been consumed first
     g_override.store(family < 0 ? -1 : family, std::memory_order_release);
+}
+
+// The sum of the entries' hashes (FNV-1a, of Fowler, Noll and Vo), whatever their order.
+extern "C" uint64_t onnxb_dispatch_state(void) {
+    uint64_t sum = (uint64_t)(uint32_t)kernel_override();
+    for (char **e = environ; e && *e; ++e) {
+        if (std::strncmp(*e, "ONNXB_", 6) != 0) continue;
+        uint64_t h = 14695981039346656037ull;
+        for (const char *c = *e; *c; ++c) h = (h ^ (unsigned char)*c) * 1099511628211ull;
+        sum += h;
+    }
+    return sum;
 }
 
 extern "C" uint64_t onnxb_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }

@@ -16,6 +16,8 @@
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <vector>
+
 #include "onnx_b200.h"
 
 namespace {
@@ -31,6 +33,7 @@ struct Abi {
     decltype(&onnx_maxpool2d_shape) maxpool2d_shape;
     decltype(&onnx_maxpool2d_run) maxpool2d_run;
     decltype(&onnx_global_average_pool_run) global_average_pool_run;
+    decltype(&onnxb_dispatch_state) dispatch_state;
 } abi;
 
 struct Plan {                    // what a convolution descriptor resolved to
@@ -124,6 +127,7 @@ PyObject *py_bind(PyObject *, PyObject *arg) {
     get(abi.maxpool2d_shape, "onnx_maxpool2d_shape");
     get(abi.maxpool2d_run, "onnx_maxpool2d_run");
     get(abi.global_average_pool_run, "onnx_global_average_pool_run");
+    get(abi.dispatch_state, "onnxb_dispatch_state");
     if (!ok) { PyErr_SetString(PyExc_OSError, "a symbol of the C ABI is missing"); return nullptr; }
     Py_RETURN_NONE;
 }
@@ -267,6 +271,25 @@ PyObject *py_gap(PyObject *, PyObject *const *a, Py_ssize_t n) {
     return abi.global_average_pool_run(xt->sizes().data(), x, y, stream) == ONNXB_OK ? result(a[1], ym) : slow_path();
 }
 
+// state(list of tensors): address, type, sizes and strides of each, and the library's dispatch state, as bytes
+PyObject *py_state(PyObject *, PyObject *const *a, Py_ssize_t n) {
+    if (n != 1 || !PyList_CheckExact(a[0])) return slow_path();
+    const Py_ssize_t count = PyList_GET_SIZE(a[0]);
+    std::vector<int64_t> out;
+    out.reserve(2 + 12 * (size_t)count);
+    out.push_back((int64_t)abi.dispatch_state());
+    for (Py_ssize_t i = 0; i < count; ++i) {
+        PyObject *o = PyList_GET_ITEM(a[0], i);
+        if (!THPVariable_CheckExact(o)) return slow_path();
+        const at::Tensor &x = THPVariable_Unpack(o);
+        out.push_back((int64_t)reinterpret_cast<uintptr_t>(x.data_ptr()));
+        out.push_back((int64_t)x.scalar_type() << 32 | x.dim());
+        out.insert(out.end(), x.sizes().begin(), x.sizes().end());
+        out.insert(out.end(), x.strides().begin(), x.strides().end());
+    }
+    return PyBytes_FromStringAndSize(reinterpret_cast<const char *>(out.data()), (Py_ssize_t)(out.size() * sizeof(int64_t)));
+}
+
 // a C++ exception (out of memory, no device) also leads to the checked path, which raises its own
 template <PyObject *(*F)(PyObject *, PyObject *const *, Py_ssize_t)>
 PyObject *guarded(PyObject *self, PyObject *const *a, Py_ssize_t n) {
@@ -284,6 +307,7 @@ PyMethodDef methods[] = {
     {"gemm", reinterpret_cast<PyCFunction>(&guarded<py_gemm>), METH_FASTCALL, nullptr},
     {"maxpool", reinterpret_cast<PyCFunction>(&guarded<py_maxpool>), METH_FASTCALL, nullptr},
     {"gap", reinterpret_cast<PyCFunction>(&guarded<py_gap>), METH_FASTCALL, nullptr},
+    {"state", reinterpret_cast<PyCFunction>(&guarded<py_state>), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_onnxb_fast", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

@@ -10,7 +10,6 @@ operator runs in the library's kernels.
 """
 from __future__ import annotations
 
-import operator
 from dataclasses import dataclass, replace
 from typing import Dict, List, Optional
 
@@ -90,8 +89,12 @@ def push_strides_up(ops: List[Op]) -> List[Op]:
 class Resnet50Chain:
     """The model with its buffers.  Between the layers tensors are channel-major: a channel's pixels of all images in one row, rows
     of whole 128-byte lines.  A 1x1 layer is then one wide GEMM whatever the images' size (7x7 planes are no whole 16-byte pieces,
-    14x14 ones no whole lines), and no layer's input is gathered: 64 images 1883 -> 1743 us, one image 402 -> 388.  ``buf`` shows
-    them as the ONNX tensors that they are."""
+    14x14 ones no whole lines), and no layer's input is gathered: 64 images 1883 -> 1743 us, one image 402 -> 388.
+
+    ``buf`` shows them as the ONNX tensors that they are, those that only strided 1x1 layers read at the places read
+    (``push_strides_up``).  A tensor put in another's place there is what the operator writes from then on.  Where it is not one of
+    the last two, ``pooled`` and ``logits``, the chain is laid out anew for it, as ONNX lays out the graph and every tensor (so from
+    the beginning with ``prepack`` off), and the other entries are new tensors, too; inside a capture that raises an error."""
 
     def __init__(self, batch: int, device, seed: int = wl.SEED_BASE + 9000, prepack: bool = True):
         import torch
@@ -100,19 +103,8 @@ class Resnet50Chain:
         graph = build_graph(batch)
         rng = np.random.default_rng(seed)
         self.prepack = prepack                  # weights are constants of the graph: pack them once (Sec. 3.4.4)
-        self.packed: Dict[str, object] = {}
         self.params: Dict[str, tuple] = {}
-        self.ops, self.descs, self.channel_major = graph, None, False
-        if prepack:
-            moved = push_strides_up(graph)
-            self.descs = self._descriptors(moved, True)
-            if self.descs is not None:
-                self.ops, self.channel_major = moved, True
-        if self.descs is None:                  # (a kernel family pinned by the override knows one layout)
-            self.descs = self._descriptors(graph, False)
-        # What a gather would round to TF32 for the tensor cores reaches them rounded, not truncated.
-        self._reads_rounded = {op.src for ops in (graph, self.ops) for op in ops if self._gathers(op)} if self.channel_major else set()
-        for op in self.ops:
+        for op in graph:
             if op.case is not None:
                 c = op.case
                 fan = c.w_shape[1] * c.w_shape[2] * c.w_shape[3]
@@ -121,41 +113,64 @@ class Resnet50Chain:
                     W *= np.float32(0.5)                   # keeps the activations of 16 stacked blocks in range
                 B = rng.standard_normal((c.w_shape[0],), dtype=np.float32) * np.float32(0.01)
                 self.params[op.name] = (torch.from_numpy(W).to(device), torch.from_numpy(B).to(device))
-                if prepack:
-                    self.packed[op.name] = self.descs[op.name].prepack(self.params[op.name][0])
         Wf = rng.standard_normal((2048, 1000), dtype=np.float32) * np.float32(np.sqrt(1.0 / 2048))
         Bf = rng.standard_normal((1000,), dtype=np.float32) * np.float32(0.01)
         self.params["fc"] = (torch.from_numpy(Wf).to(device), torch.from_numpy(Bf).to(device))
-        ws_bytes = max([16] + [d.workspace_bytes for d in self.descs.values()])
-        self.workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=device)
         self.fc_workspace = torch.empty(max(binding.gemm_workspace_bytes(False, False, batch, 1000, 2048), 16),
                                         dtype=torch.uint8, device=device)
+        self.buf: Dict[str, "torch.Tensor"] = {}
+        self._lay_out(prepack, {})
+        self.flops = sum(op.case.flops for op in graph if op.case is not None) + 2 * batch * 2048 * 1000
+        self._capture()
+
+    def _lay_out(self, channel_major: bool, given: Dict[str, "torch.Tensor"]):
+        """The operators, their descriptors, packed weights and buffers, on channel-major tensors where every layer knows them;
+        ``given``: tensors of ``buf`` to use as they are."""
+        torch = self.torch
+        graph = build_graph(self.batch)
+        self.ops, self.descs, self.channel_major = graph, None, False
+        if channel_major:
+            moved = push_strides_up(graph)
+            self.descs = self._descriptors(moved, True)
+            if self.descs is not None:
+                self.ops, self.channel_major = moved, True
+        if self.descs is None:                  # (a kernel family pinned by the override knows one layout)
+            self.descs = self._descriptors(graph, False)
+        # What a gather would round to TF32 for the tensor cores reaches them rounded, not truncated.
+        self._reads_rounded = {op.src for ops in (graph, self.ops) for op in ops if self._gathers(op)} if self.channel_major else set()
+        self.packed: Dict[str, object] = {}
+        if self.prepack:
+            self.packed = {name: d.prepack(self.params[name][0]) for name, d in self.descs.items()}
+        ws_bytes = max([16] + [d.workspace_bytes for d in self.descs.values()])
+        self.workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=self.dev)
         # one buffer per tensor of the graph, as it lies in memory and as the ONNX tensor it is; and the rounded second outputs
         self.store: Dict[str, "torch.Tensor"] = {}
-        self.buf: Dict[str, "torch.Tensor"] = {}
+        self.buf.clear()
         self.rounded: Dict[str, "torch.Tensor"] = {}
+        shapes: Dict[str, tuple] = {}
         for op in self.ops:
             if op.case is not None:
                 shape = self.descs[op.name].y_shape
                 if op.sampled:
                     self.buf[op.res] = self.buf[op.sampled][:, :, ::op.sample[0], ::op.sample[1]]
             elif op.kind == "maxpool":
-                shape = binding.maxpool2d_shape(tuple(self.buf[op.src].shape), (3, 3), (1, 1, 1, 1), (2, 2))
+                shape = binding.maxpool2d_shape(shapes[op.src], (3, 3), (1, 1, 1, 1), (2, 2))
             elif op.kind == "gap":
-                s = self.buf[op.src].shape
-                shape = (s[0], s[1], 1, 1)
+                shape = shapes[op.src][:2] + (1, 1)
             else:
-                shape = (batch, 1000)
+                shape = (self.batch, 1000)
+            shapes[op.dst] = shape
             if self.channel_major and op.kind in ("conv", "conv_add", "maxpool"):
                 n, c, h, w = shape
-                self.store[op.dst] = torch.empty((c, binding.channel_pitch(shape)), dtype=torch.float32, device=device)
+                self.store[op.dst] = torch.empty((c, binding.channel_pitch(shape)), dtype=torch.float32, device=self.dev)
                 self.buf[op.dst] = self.store[op.dst].as_strided(shape, (h * w, self.store[op.dst].shape[1], w, 1))
                 if op.kind == "conv_add" and op.dst in self._reads_rounded:
                     self.rounded[op.dst] = torch.empty_like(self.store[op.dst])
             else:
-                self.store[op.dst] = self.buf[op.dst] = torch.empty(shape, dtype=torch.float32, device=device)
-        self.flops = sum(op.case.flops for op in graph if op.case is not None) + 2 * batch * 2048 * 1000
-        self._capture()
+                t = given[op.dst] if op.dst in given else torch.empty(shape, dtype=torch.float32, device=self.dev)
+                self.store[op.dst] = self.buf[op.dst] = t
+        # where the views lie: an entry of buf that lies elsewhere is another tensor, put in a view's place
+        self._views = {name: self._place(t) for name, t in self.buf.items() if name in self.store and self.store[name] is not t}
 
     def _descriptors(self, ops: List[Op], channel_major: bool):
         """The convolutions' descriptors; None where one of them knows no channel-major tensors."""
@@ -185,15 +200,39 @@ class Resnet50Chain:
         d.close()
         return family == "mma_gather_gemm"
 
-    def _tensors(self):
-        """What the operators behind the first one read and write."""
-        return [t for k, t in self.store.items() if k != "input"] + list(self.rounded.values()) + list(self.packed.values()) + \
-            [t for pair in self.params.values() for t in pair] + [self.workspace, self.fc_workspace]
+    @staticmethod
+    def _place(t):
+        return t.data_ptr(), t.dtype, t.shape, t.stride()
+
+    def _state(self):
+        """Where all tensors but the input lie and how, and what the library chooses its kernels by (None without the native call
+        path): what the graph was captured with, and what a replay of it stands for."""
+        tensors = [t for k, t in self.store.items() if k != "input"] + [t for k, t in self.buf.items() if k != "input"] + \
+            list(self.rounded.values()) + list(self.packed.values()) + [t for pair in self.params.values() for t in pair] + \
+            [self.workspace, self.fc_workspace]
+        state = binding.call_state(tensors)
+        return None if state is None else (self.prepack, state)
+
+    def _follow_buf(self):
+        """Goes over to the tensors that ``buf`` holds now, and to ``prepack`` as it is now."""
+        if self.channel_major and (not self.prepack or any(self._place(self.buf[k]) != place for k, place in self._views.items())):
+            if self.torch.cuda.is_current_stream_capturing():
+                raise RuntimeError("Resnet50Chain: an entry of buf was replaced; its buffers are made anew by a pass outside a capture")
+            x, descs = self.buf["input"], self.descs
+            self._graph = self._captured = None
+            self._lay_out(False, {k: t for k, t in self.buf.items() if k not in self._views or self._place(t) != self._views[k]})
+            self.buf["input"] = self.store["input"] = x
+            for d in descs.values():
+                d.close()
+        for op in self.ops:
+            if op.dst not in self._views:
+                self.store[op.dst] = self.buf[op.dst]
 
     def _capture(self):
         """The operators behind the first one, which alone reads the caller's tensor, as one CUDA graph."""
         torch = self.torch
         with torch.cuda.device(self.dev):
+            self._device = torch.cuda.current_device()
             stream, before = torch.cuda.Stream(), binding.launch_count()
             stream.wait_stream(torch.cuda.current_stream())
             with torch.cuda.stream(stream):
@@ -209,16 +248,18 @@ class Resnet50Chain:
                 finally:
                     graph.capture_end()
             torch.cuda.current_stream().wait_stream(stream)
-        self._graph, self._captured = graph, self._tensors()
+        self._graph, self._captured = graph, self._state()
 
     def forward(self, x):
-        """Enqueue the whole model on the current stream; returns the logits buffer."""
+        """Enqueue the whole model on the current stream; returns the logits buffer.  (``binding.launch_count`` counts the one kernel
+        launched beside the graph; ``launches`` is how many a pass has.)"""
         self.buf["input"] = self.store["input"] = x
-        # All but the first operator in one launch in place of some fifty.  Made one by one where the call is itself being captured,
-        # or where a tensor of the graph's has been put in another's place.
-        now = self._tensors()
-        if self._graph is None or len(now) != len(self._captured) or not all(map(operator.is_, now, self._captured)) or \
-                self.torch.cuda.is_current_stream_capturing():
+        # All but the first operator in one launch in place of some fifty.  Made one by one where the call is itself being captured or
+        # on another device, or where anything differs from what the graph was captured with.
+        cuda = self.torch.cuda
+        state = None if self._graph is None or cuda.is_current_stream_capturing() or cuda.current_device() != self._device else self._state()
+        if state is None or state != self._captured:
+            self._follow_buf()
             self._run(self.ops)
         else:
             self._run(self.ops[:1])

@@ -72,3 +72,92 @@ def test_a_tensor_in_another_s_place(net):
     finally:
         net.params["fc"] = (W, B)
     assert torch.equal(net.forward(x), want)
+
+
+def test_another_tensor_for_the_logits(net):
+    x = _x(11)
+    want, own = net.forward(x).clone(), net.buf["logits"]
+    mine = torch.full_like(own, 7.0)
+    net.buf["logits"] = mine
+    try:
+        for _ in range(2):
+            mine.fill_(7.0)
+            assert net.forward(x) is mine and torch.equal(mine, want)
+    finally:
+        net.buf["logits"] = own
+    own.fill_(7.0)
+    for _ in range(2):
+        assert net.forward(x) is own and torch.equal(own, want)
+
+
+def test_a_parameter_with_other_memory():
+    x, net = _x(13), Resnet50Chain(2, torch.device("cuda:0"), seed=5)
+    W, B = net.params["fc"]
+    want = net.forward(x) - B
+    for value, rebind in ((1.0, lambda t: setattr(B, "data", t)), (2.0, lambda t: B.set_(t)), (3.0, lambda t: B.resize_(1 << 20).resize_(1000).copy_(t))):
+        rebind(torch.full((1 << 16,), value, device="cuda")[:1000])
+        assert torch.allclose(net.forward(x), want + value, rtol=1e-5, atol=1e-5)
+    net.close()
+
+
+def test_pins_set_after_the_chain_was_built(net, monkeypatch):
+    x = _x(15)
+    want = net.forward(x).clone()
+    binding.set_kernel_override("simt_direct")             # (the head's Gemm in fp32)
+    try:
+        got, one_by_one = net.forward(x).clone(), _one_by_one(net, x)
+    finally:
+        binding.set_kernel_override(None)
+    assert torch.equal(got, one_by_one) and not torch.equal(got, want)
+    monkeypatch.setenv("ONNXB_GEMM_SPLITK", "0")
+    launches = binding.launch_count()
+    net.forward(x)
+    assert binding.launch_count() - launches > 50
+    monkeypatch.delenv("ONNXB_GEMM_SPLITK")
+    launches = binding.launch_count()
+    assert torch.equal(net.forward(x), want) and binding.launch_count() - launches == 1
+
+
+def test_on_another_current_device(net, monkeypatch):
+    x = _x(17)
+    want, launches = net.forward(x).clone(), binding.launch_count()
+    monkeypatch.setattr(net, "_device", net._device + 1)
+    assert torch.equal(net.forward(x), want) and binding.launch_count() - launches == net.launches
+
+
+@pytest.mark.parametrize("prepack", [True, False])
+def test_another_tensor_inside_the_graph(prepack):
+    """The tensors that the operators write are the graph's as ONNX has it: whole ones also where the chain moved a stride up."""
+    x, given = _x(19), ("r50_08_s2b2_b", "r50_08_s2b2_out", "stem", "pooled")
+    other, net = (Resnet50Chain(2, torch.device("cuda:0"), seed=5, prepack=p) for p in (False, prepack))
+    want = other.forward(x)
+    assert set(given) <= set(other.buf)
+    near = net.forward(x).clone()
+    for name in given:
+        net.buf[name] = torch.full_like(other.buf[name], 7.0)
+    mine = {name: net.buf[name] for name in given}
+    if prepack:
+        with pytest.raises(RuntimeError, match="outside a capture"):
+            with torch.cuda.graph(torch.cuda.CUDAGraph()):
+                mine["stem"].zero_()                       # (a graph of nothing draws a warning)
+                net.forward(x)
+    for _ in range(2):
+        assert torch.equal(net.forward(x), want)
+    for op in other.ops:
+        assert torch.equal(net.buf[op.dst], other.buf[op.dst]), op.name
+    assert all(net.buf[name] is mine[name] for name in given) and torch.allclose(near, want, rtol=0, atol=2e-2 * float(want.std()))
+    net.close()
+    other.close()
+
+
+def test_prepack_switched_off():
+    x = _x(21)
+    other, net = (Resnet50Chain(2, torch.device("cuda:0"), seed=5, prepack=p) for p in (False, True))
+    net.forward(x)
+    net.prepack = False
+    for n in (other, net):
+        for W, _ in n.params.values():
+            W.mul_(0.9)
+    assert torch.equal(net.forward(x), other.forward(x))
+    net.close()
+    other.close()

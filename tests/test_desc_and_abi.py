@@ -171,3 +171,25 @@ def test_run_calls_reject_bad_arguments_before_any_launch():
     assert g(1 << 20, 1 << 20, 4) == 4
     assert g(4, 5, 6, Y=ctypes.c_void_p(0x1008)) == 4
     assert binding.launch_count() == before
+
+
+def test_dispatch_state(monkeypatch):
+    """Differs with the override and with every ONNXB_* variable, whatever their order, and with nothing else."""
+    state = binding.load().onnxb_dispatch_state
+    plain = state()
+    binding.set_kernel_override("simt_direct")
+    assert state() != plain
+    binding.set_kernel_override(None)
+    monkeypatch.setenv("ONNXB_GEMM_BN", "64")
+    one = state()
+    monkeypatch.setenv("ONNXB_GEMM_KS", "2")
+    both = state()
+    monkeypatch.setenv("ONNXB_GEMM_BN", "32")
+    assert len({plain, one, both, state()}) == 4
+    for name in ("ONNXB_GEMM_BN", "ONNXB_GEMM_KS"):
+        monkeypatch.delenv(name)
+    monkeypatch.setenv("ONNX_B", "1")
+    assert state() == plain
+    monkeypatch.setenv("ONNXB_GEMM_KS", "2")
+    monkeypatch.setenv("ONNXB_GEMM_BN", "64")
+    assert state() == both
