@@ -385,16 +385,18 @@ class Conv2dDesc:
                "onnx_conv2d_run_packed_sampled", no_memory)
         return Y
 
-    def run_prepacked_rounded(self, X, W, packed, B, R, Y, Y_rounded, stream=None):
+    def run_prepacked_rounded(self, X, W, packed, B, R, Y, Y_rounded, stream=None, workspace=None):
         """``onnx_conv2d_run_packed_rounded``: run_prepacked, and Y rounded to TF32 into ``Y_rounded`` (Y itself where it is that)."""
-        y = self._native_rounded(X, W, packed, B, R, Y, None, stream, None, None, Y_rounded)
+        y = self._native_rounded(X, W, packed, B, R, Y, workspace, stream, None, None, Y_rounded)
         if y is not None:
             return y
+        needs = workspace is None and self.workspace_bytes and self._packed_needs_ws
+        workspace, ws_ptr, ws_len, no_memory = _scratch(self.workspace_bytes, X.device, stream) if needs else _given(workspace)
         _check(self._lib.onnx_conv2d_run_packed_rounded(self._h, _dev_ptr(X, "X"), _dev_ptr(W, "W"), ctypes.c_void_p(packed.data_ptr()),
                                                         packed.numel() * packed.element_size(), _dev_ptr(B, "B", allow_none=True),
                                                         _dev_ptr(R, "R", allow_none=True), _dev_ptr(Y, "Y"),
-                                                        _dev_ptr(Y_rounded, "Y_rounded"), None, 0, _stream_ptr(stream)),
-               "onnx_conv2d_run_packed_rounded")
+                                                        _dev_ptr(Y_rounded, "Y_rounded"), ws_ptr, ws_len, _stream_ptr(stream)),
+               "onnx_conv2d_run_packed_rounded", no_memory)
         return Y
 
     def run_static(self, X, W, B=None, Y=None, stream=None):

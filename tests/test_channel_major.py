@@ -168,6 +168,27 @@ def test_rounded_outputs(x, w, kw):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("given", [True, False])
+@pytest.mark.parametrize("native", [True, False])
+@pytest.mark.parametrize("x,w,strides", [((3, 64, 28, 28), (96, 64, 1, 1), (2, 2)), ((5, 96, 7, 7), (80, 96, 1, 1), (1, 1))])
+def test_rounded_outputs_behind_a_gather(x, w, strides, native, given, monkeypatch):
+    """The copy of the pixels needs a workspace beside the packed weights, the caller's or one made for the call."""
+    import torch
+    if not native:
+        monkeypatch.setattr(binding, "_fast_mod", binding._Declined())
+    g = torch.Generator(device="cuda").manual_seed(3)
+    d = binding.Conv2dDesc(x, w, has_bias=True, strides=strides)
+    assert d.kernel_family == "mma_gather_gemm"
+    X, W, B, R = (torch.randn(s, generator=g, device="cuda") for s in (x, w, (w[0],), d.y_shape))
+    packed = d.prepack(W)
+    want = d.run_prepacked(X, W, packed, B, R)
+    y, yr = torch.empty_like(want), torch.empty_like(want)
+    d.run_prepacked_rounded(X, W, packed, B, R, y, yr, workspace=torch.empty(d.workspace_bytes, dtype=torch.uint8, device="cuda") if given else None)
+    assert binding.last_device_status() == 0 and torch.equal(y, want)
+    assert torch.equal(yr, ((want.view(torch.int32) + 0x1000) & ~0x1FFF).view(torch.float32))
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("native", [True, False])
 @pytest.mark.parametrize("batch,C,M,hw,strides", [(4, 64, 256, (56, 56), (2, 2)), (3, 128, 512, (27, 28), (2, 2)), (1, 256, 1024, (14, 14), (2, 2)),
                                                   (64, 64, 272, (13, 14), (2, 2))])
