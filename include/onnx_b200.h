@@ -202,7 +202,7 @@ onnxb_status onnx_conv2d_run_prepacked(onnxb_conv2d_desc_t desc, const float *X,
  * rounds it).
  * Errors: as onnx_conv2d_run_packed; ERR_NULL when R, r_dims or r_strides is; ERR_SHAPE when the places read are not
  * P x Q; ERR_UNSUPPORTED for descriptors other than of ONNXB_KERNEL_MMA_GEMM and ONNXB_KERNEL_MMA_GATHER_GEMM (those of
- * group-1, unpadded 1x1 convolutions of 32 channels and more), and for an R of 2^31 elements and more.
+ * group-1, unpadded 1x1 convolutions of 32 channels and more), for an R of 2^31 elements and more, and when Y_rounded is Y.
  */
 onnxb_status onnx_conv2d_run_packed_sampled(onnxb_conv2d_desc_t desc, const float *X, const float *W, const void *packed,
                                             size_t packed_bytes, const float *B, const float *R, const int64_t r_dims[2],

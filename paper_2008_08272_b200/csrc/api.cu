@@ -303,7 +303,8 @@ extern "C" onnxb_status onnx_conv2d_run_packed_sampled(onnxb_conv2d_desc_t d, co
                                                        const int64_t *r_dims, const int64_t *r_strides, float *Y, float *Y_rounded,
                                                        void *workspace, size_t workspace_bytes, void *cuda_stream) {
     if (!d || !R || !r_dims || !r_strides) return ONNXB_ERR_NULL;
-    if (d->family != ONNXB_KERNEL_MMA_GEMM && d->family != ONNXB_KERNEL_MMA_GATHER_GEMM) return ONNXB_ERR_UNSUPPORTED;
+    // (two outputs: the kernels store a block to both without an order between the stores)
+    if ((d->family != ONNXB_KERNEL_MMA_GEMM && d->family != ONNXB_KERNEL_MMA_GATHER_GEMM) || (Y && Y_rounded == Y)) return ONNXB_ERR_UNSUPPORTED;
     const int64_t out[2] = {d->g.P, d->g.Q};
     for (int i = 0; i < 2; ++i)
         if (r_dims[i] < 1 || r_strides[i] < 1 || r_dims[i] > 2147483647LL || (r_dims[i] - 1) / r_strides[i] + 1 != out[i]) return ONNXB_ERR_SHAPE;

@@ -109,3 +109,14 @@ def test_refused():
     assert call(d, two(1 << 20, 1 << 20), two((1 << 20) // 28 + 1, (1 << 20) // 28 + 1)) == 4
     assert call(binding.Conv2dDesc((2, 64, 28, 28), (128, 64, 3, 3), pads=(1,) * 4), two(56, 56), two(2, 2)) == 4
     assert binding.launch_count() == before
+
+
+def test_one_tensor_for_both_outputs_is_refused():
+    import ctypes
+    at, before = (lambda n: ctypes.c_void_p(n << 12)), binding.launch_count()
+    two = lambda *v: (ctypes.c_int64 * 2)(*v)
+    for x, w in (((2, 64, 28, 28), (128, 64, 1, 1)), ((2, 64, 7, 7), (128, 64, 1, 1))):
+        d = binding.Conv2dDesc(x, w)
+        assert binding.load().onnx_conv2d_run_packed_sampled(d._h, at(1), at(2), at(3), 1 << 30, None, at(4), two(2 * x[2], 2 * x[3]), two(2, 2),
+                                                             at(5), at(5), at(6), 1 << 30, None) == 4
+    assert binding.launch_count() == before
