@@ -369,8 +369,9 @@ class Conv2dDesc:
         if r_dims is None:
             if R.dim() != 4 or tuple(R.shape[:2]) != self.y_shape[:2]:
                 raise OnnxB200Error(3, "run_prepacked_sampled: the addend's images and channels are not the output's")
-            r_dims = tuple(R.shape[2:])
-        y = self._native_rounded(X, W, packed, B, R, Y, workspace, stream, r_dims, strides, Y_rounded)
+            r_dims = R.shape[2:]
+        # (tuples: of a torch.Size the native path knows nothing)
+        y = self._native_rounded(X, W, packed, B, R, Y, workspace, stream, tuple(r_dims), tuple(strides), Y_rounded)
         if y is not None:
             return y
         if Y is None:

@@ -120,3 +120,17 @@ def test_one_tensor_for_both_outputs_is_refused():
         assert binding.load().onnx_conv2d_run_packed_sampled(d._h, at(1), at(2), at(3), 1 << 30, None, at(4), two(2 * x[2], 2 * x[3]), two(2, 2),
                                                              at(5), at(5), at(6), 1 << 30, None) == 4
     assert binding.launch_count() == before
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["Size", "list"])
+def test_any_sequence_of_sizes_goes_the_native_way(kind, monkeypatch):
+    import torch
+    kind = torch.Size if kind == "Size" else list
+    R = torch.rand(2, 128, 56, 56, device="cuda")
+    X, W, d = torch.rand(2, 64, 28, 28, device="cuda"), torch.rand(128, 64, 1, 1, device="cuda"), binding.Conv2dDesc((2, 64, 28, 28), (128, 64, 1, 1))
+    packed = d.prepack(W)
+    want = d.run_prepacked_sampled(X, W, packed, None, R, (2, 2))
+    monkeypatch.setattr(binding, "_i64", None)             # (what the calls through ctypes convert sizes with)
+    got = d.run_prepacked_sampled(X, W, packed, None, R, kind((2, 2)), r_dims=kind((56, 56)))
+    assert torch.equal(got, want)
