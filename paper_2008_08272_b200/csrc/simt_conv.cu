@@ -208,8 +208,8 @@ conv2d_depthwise_kernel(const ConvGeom g, const float *__restrict__ X, const flo
 // Both kernels below are bound by HBM (the pixels read once, the copy written once): one wave of eight blocks per SM, indices
 // by multiplication (256 channels 56x56 -> 28x28 at batch 32: some 20 -> 15 us).
 
-// Weights of the call, rounded to TF32 ahead of the pixels: a launch of its own for them in front took 3 us (256 -> 512 channels
-// 56x56/2 at batch 32 41.2 -> 39.8 us in all), most of it the launch.
+// Weights of the call, rounded to TF32 ahead of the pixels: a launch of its own for them in front cost up to 2 us (256 -> 512
+// channels 56x56/2 at batch 32 41.2 -> 39.9 us in all, at batch 4 12.3 -> 10.3; with few pixels and many weights see launch_gather1x1).
 struct RoundedCopy {
     const float4 *in;
     float4 *out;
@@ -734,11 +734,16 @@ int launch_gather1x1(const ConvGeom &g, const float *X, float *Xg, long long pit
     const long long total = merged ? (long long)g.C * pitch : (long long)g.N * g.C * pitch;
     cudaStream_t st = (cudaStream_t)stream;
     const long long total4 = total / 4;                       // every pitch is a multiple of four
-    const unsigned blocks = (unsigned)std::min<long long>((total4 + 255) / 256, 148LL * 8);
+    // (for the weights of the call, too, which outnumber the pixels in wide layers on few of them: 52 blocks for the pixels of one image
+    // of 14x14 took 40 turns for 1024 -> 2048 channels' weights, 18.4 us in all; 9.3 by a turn's worth of blocks, 11.5 with a launch
+    // of its own for the weights; 512 -> 2048 on 7x7 15.8, 7.8, 8.6; 2048 -> 2048 7x7/2 35, 10.8, 12.1)
+    const long long for_pixels = (total4 + 255) / 256;
+    const unsigned blocks = (unsigned)std::min<long long>(std::max<long long>(for_pixels, (w.n4 + 255) / 256), 148LL * 8);
     // A small copy is set up beside the previous kernel's tail (one image, 7x7 to 28x28: 1.0-1.3 us less).  The blocks of a
-    // large one, placed while that kernel still holds its SMs, would crowd on some of them (batch 32: 15 -> 22 us).
+    // large one, placed while that kernel still holds its SMs, would crowd on some of them (batch 32: 15 -> 22 us); those of the
+    // weights, a turn or a few each, may (plainly launched 1024 -> 2048 14x14/2 at one to four images 10.3 to 14.4 us, early 9.3 to 12.6).
     auto launch = [&](auto kernel, auto... args) {
-        if (blocks <= 2 * 148) return tc_host::launch_pdl(kernel, dim3(blocks), dim3(256), 0, st, args...);
+        if (for_pixels <= 2 * 148) return tc_host::launch_pdl(kernel, dim3(blocks), dim3(256), 0, st, args...);
         kernel<<<blocks, 256, 0, st>>>(args...);
         return cudaGetLastError();
     };
