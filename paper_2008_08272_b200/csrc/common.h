@@ -63,7 +63,7 @@ int simt_conv_on_tensor_cores(const ConvGeom &g, Fp32ConvPlan &plan, Fp32GemmPla
 int launch_simt_depthwise(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                           void *stream);
 double small_conv_cost(const ConvGeom &g);           // estimated SM cycles; negative: not for this problem
-int small_conv_channels(const ConvGeom &g);
+int small_conv_channels(const ConvGeom &g);          // output channels per block, the descriptor's small_mb
 int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const float *B, const float *R, float *Y,
                       void *stream);
 bool simt_depthwise_supports(const ConvGeom &g);

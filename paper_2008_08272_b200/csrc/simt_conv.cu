@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdio>
+#include <cstdlib>
 
 #include "common.h"
 #include "tc_common.cuh"
@@ -677,11 +679,12 @@ double small_conv_cost(const ConvGeom &g) {
 // that for every other block on its SM (0.4 with eight channels and more).  (By the rule above the second layer at batch 18, 576 blocks of one channel, brings every
 // image in sixteen times: 12.6 us, 5.8 with four channels; eight and more leave a warp alone with its latencies: 11.2 at batch 30.)
 int small_conv_channels(const ConvGeom &g) {
-    int best = 1;
+    int best = 1, pinned = 0;                                // ONNXB_FP32 = "small,channels" pins them, too
     double cost = -1;
+    if (const char *pin = getenv("ONNXB_FP32")) sscanf(pin, "small,%d", &pinned);
     const double kred = (double)g.Cg * g.kH * g.kW * (g.kH == g.kW && (g.kH == 3 || g.kH == 5) ? 1.0 : 2.5);
     for (int mb : {1, 4, 8, 16}) {
-        const long long blocks = mb == 1 || g.Mg > mb / 2 ? small_blocks(g, mb) : -1;
+        const long long blocks = (pinned ? mb == pinned : mb == 1 || g.Mg > mb / 2) ? small_blocks(g, mb) : -1;
         if (blocks < 0) continue;
         const double one = (double)small_smem(g, mb) / 4 / kSmallThreads / 8 * 900.0 + kred * (mb <= 4 ? 18.0 : 60.0);
         const double c = one * (1.0 + (mb <= 4 ? 0.5 : 0.4) * (double)((blocks + 147) / 148 - 1));

@@ -1,5 +1,5 @@
 """The small-image convolution at the widths where its rows change their share of threads (8, 16, 32 lanes a row, and more than
-one turn), and for every number of channels per block; fp32 throughout."""
+one turn), and for every number of channels per block, pinned and as the rule picks them; fp32 throughout."""
 import numpy as np
 import pytest
 
@@ -21,8 +21,8 @@ CASES = [((n, c, h, wd), (m, c // kw.get("group", 1), k, k), kw) for n, c, h, wd
 
 @pytest.mark.parametrize("x,w,kw", CASES)
 @pytest.mark.parametrize("addend", [False, True])
-def test_small_conv(x, w, kw, addend, monkeypatch):
-    monkeypatch.setenv("ONNXB_FP32", "small")
+def test_small_conv(x, w, kw, addend, monkeypatch, pin="small"):
+    monkeypatch.setenv("ONNXB_FP32", pin)
     rng = np.random.default_rng(x[0] + w[0])
     X, W, B = rng.standard_normal(x, dtype=np.float32), rng.standard_normal(w, dtype=np.float32), rng.standard_normal(w[0], dtype=np.float32)
     binding.set_kernel_override("simt_direct")
@@ -39,3 +39,15 @@ def test_small_conv(x, w, kw, addend, monkeypatch):
     # one chain of fp32 additions of the window's terms, the bias and the addend
     bound = (W[0].size + 3) * 2.0 ** -24 * (S + np.abs(B).reshape(1, -1, 1, 1)) * 1.01
     assert binding.last_device_status() == 0 and np.all(np.abs(got.cpu().numpy() - want) <= bound)
+
+
+# a quotient and a remainder of channels at every number per block; 3x3, 5x5 and other filters; one block, and several per SM
+SIZES = [((n, c, h, wd), (m, c // kw.get("group", 1)) + k, kw) for n, c, h, wd, m, k, kw in (
+    (2, 3, 9, 17, 21, (3, 3), dict(pads=(1,) * 4)), (70, 2, 12, 15, 37, (3, 3), dict(pads=(1,) * 4)), (3, 5, 14, 14, 19, (5, 5), dict(pads=(2,) * 4)),
+    (80, 4, 10, 33, 34, (5, 5), dict(pads=(2,) * 4, group=2)), (2, 3, 11, 8, 18, (2, 4), {}), (90, 2, 13, 16, 23, (4, 3), dict(strides=(2, 1))))]
+
+
+@pytest.mark.parametrize("x,w,kw", SIZES)
+@pytest.mark.parametrize("channels", [1, 4, 8, 16])
+def test_every_number_of_channels_per_block(x, w, kw, channels, monkeypatch):
+    test_small_conv(x, w, kw, False, monkeypatch, "small,%d" % channels)
