@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
+#include <type_traits>
 
 #include "common.h"
 #include "tc_common.cuh"
@@ -21,14 +22,18 @@ namespace {
 // no bounds checks) and each thread then sums its pixel's MB outputs.  Filters lie as [c][tap, padded to 4]
 // (MB = 1: one 16-byte read serves four taps) or [c][tap][MB] (MB > 1: one read serves four channels).
 // K > 0: a K x K filter with unrolled taps; K = 0: any.  One 14x14 image, 8 -> 16 channels, 5x5: 6.8 -> 4 us.
+// The image is brought in position by position, no thread idle, stepping from one to the next without dividing; or (kRows) a warp a row,
+// which takes a third of the instructions, but idle lanes mean more trips to memory one behind the other: a 5x5 layer on one 14x14 image
+// 4.0 us by positions, 5.7 by rows, 3 -> 16 3x3 32x32 3.4, 5.9 (with two divisions a position both 4.6), 1 -> 8 5x5 28x28 (rows of 32) at
+// batch 200 10.1, 8.9.  So kRows where rows are all but whole warps and an SM has more than three blocks to issue.
 constexpr int kSmallThreads = 128;
 constexpr int kSmallSmem = 48 * 1024;
 
-template <int MB, int K>
+template <int MB, int K, bool kRows>
 __global__ void __launch_bounds__(kSmallThreads)
 conv2d_small_kernel(const __grid_constant__ ConvGeom g, const float *__restrict__ X, const float *__restrict__ W,
                     const float *__restrict__ B, const float *__restrict__ R, float *__restrict__ Y, int Hp, int Wp, int taps4,
-                    const ConvDivisor dv_Hp, const ConvDivisor dv_Q, const ConvDivisor dv_taps) {
+                    const ConvDivisor dv_Wp, const ConvDivisor dv_Hp, const ConvDivisor dv_Q, const ConvDivisor dv_taps) {
     extern __shared__ __align__(16) float sm[];
     const int taps = K > 0 ? K * K : g.kH * g.kW, kW = K > 0 ? K : g.kW;
     const int ptiles = (g.P * g.Q + kSmallThreads - 1) / kSmallThreads, mtiles = (g.Mg + MB - 1) / MB;
@@ -57,21 +62,44 @@ conv2d_small_kernel(const __grid_constant__ ConvGeom g, const float *__restrict_
         }
     }
     const float *xg = X + ((size_t)n * g.C + (size_t)grp * g.Cg) * g.H * g.W;
-    // 8, 16 or 32 threads a row (a position divided by the row's width and the plane took three times the instructions)
-    const int rows = g.Cg * Hp, lanes = Wp <= 8 ? 8 : Wp <= 16 ? 16 : 32, step = kSmallThreads / lanes;
-    for (int wp = threadIdx.x & (lanes - 1); wp < Wp; wp += lanes) {
-        const int w = wp - g.pl;
-        const bool in = (unsigned)w < (unsigned)g.W;
-        for (int r0 = threadIdx.x / lanes; r0 < rows; r0 += 8 * step) {
+    if (kRows) {
+        // a warp a row: a thread keeps its column
+        const int rows = g.Cg * Hp, step = kSmallThreads / 32;
+#pragma unroll 1
+        for (int wp = threadIdx.x & 31; wp < Wp; wp += 32) {
+            const int w = wp - g.pl;
+            const bool in = (unsigned)w < (unsigned)g.W;
+#pragma unroll 1
+            for (int r0 = threadIdx.x / 32; r0 < rows; r0 += 8 * step) {
+                float v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int r = r0 + u * step, c = conv_fdiv(r, Hp, dv_Hp), h = r - c * Hp - g.pt;
+                    v[u] = in && r < rows && (unsigned)h < (unsigned)g.H ? __ldg(xg + ((size_t)c * g.H + h) * g.W + w) : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (r0 + u * step < rows) xs[(r0 + u * step) * Wp + wp] = v[u];
+            }
+        }
+    } else {
+        // no thread idle, from one position to the next without dividing
+        const int total = g.Cg * plane, row = conv_fdiv(threadIdx.x, Wp, dv_Wp), dr = conv_fdiv(kSmallThreads, Wp, dv_Wp);
+        int c = conv_fdiv(row, Hp, dv_Hp), h = row - c * Hp, w = threadIdx.x - row * Wp;
+        const int dc = conv_fdiv(dr, Hp, dv_Hp), dh = dr - dc * Hp, dw = kSmallThreads - dr * Wp;
+        for (int i0 = threadIdx.x; i0 < total; i0 += 8 * kSmallThreads) {
             float v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int r = r0 + u * step, c = conv_fdiv(r, Hp, dv_Hp), h = r - c * Hp - g.pt;
-                v[u] = in && r < rows && (unsigned)h < (unsigned)g.H ? __ldg(xg + ((size_t)c * g.H + h) * g.W + w) : 0.f;
+                const bool in = i0 + u * kSmallThreads < total && (unsigned)(h - g.pt) < (unsigned)g.H && (unsigned)(w - g.pl) < (unsigned)g.W;
+                v[u] = in ? __ldg(xg + ((size_t)c * g.H + (h - g.pt)) * g.W + (w - g.pl)) : 0.f;
+                w += dw; h += dh; c += dc;
+                if (w >= Wp) { w -= Wp; ++h; }
+                if (h >= Hp) { h -= Hp; ++c; }
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if (r0 + u * step < rows) xs[(r0 + u * step) * Wp + wp] = v[u];
+                if (i0 + u * kSmallThreads < total) xs[i0 + u * kSmallThreads] = v[u];
         }
     }
     __syncthreads();
@@ -702,11 +730,16 @@ int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const f
     const long long ptiles = ((long long)g.P * g.Q + kSmallThreads - 1) / kSmallThreads;
     const long long blocks = (long long)g.N * g.group * ((g.Mg + mb - 1) / mb) * ptiles;
     const int k = g.kH == g.kW && (g.kH == 3 || g.kH == 5) ? g.kH : 0;
-    auto pick = [k](auto k3, auto k5, auto any) { return k == 3 ? k3 : k == 5 ? k5 : any; };
-    auto kern = mb == 1   ? pick(conv2d_small_kernel<1, 3>, conv2d_small_kernel<1, 5>, conv2d_small_kernel<1, 0>)
-                : mb == 4 ? pick(conv2d_small_kernel<4, 3>, conv2d_small_kernel<4, 5>, conv2d_small_kernel<4, 0>)
-                : mb == 8 ? pick(conv2d_small_kernel<8, 3>, conv2d_small_kernel<8, 5>, conv2d_small_kernel<8, 0>)
-                          : pick(conv2d_small_kernel<16, 3>, conv2d_small_kernel<16, 5>, conv2d_small_kernel<16, 0>);
+    const bool rows = (Wp + 3) % 32 < 4 && blocks > 3LL * tc_host::num_sms();
+    auto pick = [&](auto channels) {
+        constexpr int MB = decltype(channels)::value;
+        if (rows) return k == 3 ? conv2d_small_kernel<MB, 3, true> : k == 5 ? conv2d_small_kernel<MB, 5, true> : conv2d_small_kernel<MB, 0, true>;
+        return k == 3 ? conv2d_small_kernel<MB, 3, false> : k == 5 ? conv2d_small_kernel<MB, 5, false> : conv2d_small_kernel<MB, 0, false>;
+    };
+    auto kern = mb == 1   ? pick(std::integral_constant<int, 1>())
+                : mb == 4 ? pick(std::integral_constant<int, 4>())
+                : mb == 8 ? pick(std::integral_constant<int, 8>())
+                          : pick(std::integral_constant<int, 16>());
     // Blocks placed while the previous kernel still holds its SMs crowd on those that happen to have room: so much shared memory is
     // asked for that no SM takes more than its share.  MNIST at batch 18 34.6 -> 19.6 us, at batch 39 36.7 -> 21.5 (with the channels per block above).
     size_t smem = small_smem(g, mb);
@@ -717,7 +750,7 @@ int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const f
         if (ae != cudaSuccess) return (int)ae;
     }
     const cudaError_t e = tc_host::launch_pdl(kern, dim3((unsigned)blocks), dim3(kSmallThreads), smem, (cudaStream_t)stream, g, X, W, B, R, Y, Hp, Wp,
-                                              (taps + 3) / 4 * 4, conv_divisor(Hp), conv_divisor(g.Q), conv_divisor(taps));
+                                              (taps + 3) / 4 * 4, conv_divisor(Wp), conv_divisor(Hp), conv_divisor(g.Q), conv_divisor(taps));
     count_launch();
     return (int)e;
 }
