@@ -743,9 +743,9 @@ int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const f
     // Blocks placed while the previous kernel still holds its SMs crowd on those that happen to have room: so much shared memory is
     // asked for that no SM takes more than its share.  MNIST at batch 18 34.6 -> 19.6 us, at batch 39 36.7 -> 21.5 (with the channels per block above).
     size_t smem = small_smem(g, mb);
-    const long long share = (blocks + 147) / 148;
+    const long long sms = tc_host::num_sms(), share = (blocks + sms - 1) / sms;
     if (blocks > 100 && share <= 8) {
-        smem = std::max(smem, (size_t)(228 * 1024 / share - 1024) / 128 * 128 - (share == 1 ? 1024 : 0));
+        smem = std::max(smem, smem_for_share(share));
         const cudaError_t ae = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (ae != cudaSuccess) return (int)ae;
     }

@@ -390,8 +390,8 @@ cudaError_t launch_shape(const SgemmArgs &a, int split, long long tiles, cudaStr
     // asked for that no SM takes more than its share (clusters, which do not fit every GPC, one more).  Gemm 157 x 225 x 786 15.0 -> 9.6 us,
     // 18 x 1543 x 181 10.0 -> 6.5, 1001 x 130 x 333 15.0 -> 13.2; 12 -> 40 channels 3x3 33x31 at batch 3 11.5 -> 9.9.
     size_t smem = sgemm_smem<BM, BN>();
-    const long long ctas = tiles * split, share = (ctas + 147) / 148 + (split > 1 ? 1 : 0);
-    if (ctas > 100 && share <= 4) smem = std::max(smem, (size_t)(227 * 1024 / share - 1024) / 128 * 128);
+    const long long ctas = tiles * split, sms = tc_host::num_sms(), share = (ctas + sms - 1) / sms + (split > 1 ? 1 : 0);
+    if (ctas > 100 && share <= 4) smem = std::max(smem, smem_for_share(share));
     auto kern = sgemm_kernel<BM, BN, TM, TN, AM, BMODE>;
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
