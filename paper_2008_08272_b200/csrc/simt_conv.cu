@@ -23,19 +23,24 @@ namespace {
 // (MB = 1: one 16-byte read serves four taps) or [c][tap][MB] (MB > 1: one read serves four channels).
 // K > 0: a K x K filter with unrolled taps; K = 0: any.  One 14x14 image, 8 -> 16 channels, 5x5: 6.8 -> 4 us.
 // The image is brought in position by position, no thread idle, stepping from one to the next without dividing; or (kRows) a warp a row,
-// which takes a third of the instructions, but idle lanes mean more trips to memory one behind the other: a 5x5 layer on one 14x14 image
-// 4.0 us by positions, 5.7 by rows, 3 -> 16 3x3 32x32 3.4, 5.9 (with two divisions a position both 4.6), 1 -> 8 5x5 28x28 (rows of 32) at
-// batch 200 10.1, 8.9.  So kRows where rows are all but whole warps and an SM has more than three blocks to issue.
+// which takes a third of the instructions, but idle lanes mean more trips to memory one behind the other: 8 -> 16 5x5 on one 14x14 image
+// 3.9 us by positions, 4.5 by rows (4.6 by positions with two divisions each), 3 -> 16 3x3 32x32 3.3, 4.2 (4.6), 1 -> 6 5x5 32x32 at batch
+// 200 11.2, 14.5 (12.6); rows of 32 and 30: 1 -> 8 5x5 28x28 at batch 256 10.7, 10.1 (11.3), 1 -> 32 3x3 22.2, 21.1 (22.4).  So kRows where
+// rows are all but whole warps and an SM has more than three blocks to issue.
+// The arguments come to 224 bytes: a launch takes 0.3 us less of host time at 209 to 224 bytes of them (and 64 more) than at other sizes
+// (empty kernels of 168 to 288 bytes, 2.0 and 2.3 us); MNIST at one image, five calls one by one, 20.8 us at 228 bytes, 19.9 at 224.
+// Eight blocks per SM leave a thread 64 registers: with the 40 that the compiler takes by itself, for more blocks than shared memory has
+// room for, a window's pixels come from there piece by piece: 8 -> 16 5x5 14x14 at batch 18 4.9 us, 4.5 so; 1 -> 8 28x28 at 256 10.9, 10.1.
 constexpr int kSmallThreads = 128;
 constexpr int kSmallSmem = 48 * 1024;
 
 template <int MB, int K, bool kRows>
-__global__ void __launch_bounds__(kSmallThreads)
+__global__ void __launch_bounds__(kSmallThreads, 8)
 conv2d_small_kernel(const __grid_constant__ ConvGeom g, const float *__restrict__ X, const float *__restrict__ W,
-                    const float *__restrict__ B, const float *__restrict__ R, float *__restrict__ Y, int Hp, int Wp, int taps4,
+                    const float *__restrict__ B, const float *__restrict__ R, float *__restrict__ Y, int Hp, int Wp,
                     const ConvDivisor dv_Wp, const ConvDivisor dv_Hp, const ConvDivisor dv_Q, const ConvDivisor dv_taps) {
     extern __shared__ __align__(16) float sm[];
-    const int taps = K > 0 ? K * K : g.kH * g.kW, kW = K > 0 ? K : g.kW;
+    const int taps = K > 0 ? K * K : g.kH * g.kW, kW = K > 0 ? K : g.kW, taps4 = (taps + 3) / 4 * 4;
     const int ptiles = (g.P * g.Q + kSmallThreads - 1) / kSmallThreads, mtiles = (g.Mg + MB - 1) / MB;
     int b = blockIdx.x;
     const int pt = b % ptiles; b /= ptiles;
@@ -750,7 +755,7 @@ int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const f
         if (ae != cudaSuccess) return (int)ae;
     }
     const cudaError_t e = tc_host::launch_pdl(kern, dim3((unsigned)blocks), dim3(kSmallThreads), smem, (cudaStream_t)stream, g, X, W, B, R, Y, Hp, Wp,
-                                              (taps + 3) / 4 * 4, conv_divisor(Wp), conv_divisor(Hp), conv_divisor(g.Q), conv_divisor(taps));
+                                              conv_divisor(Wp), conv_divisor(Hp), conv_divisor(g.Q), conv_divisor(taps));
     count_launch();
     return (int)e;
 }
