@@ -65,7 +65,7 @@ SMALL_CONVS = [dict(x=(1, 1, 28, 28), w=(8, 1, 5, 5), pads=(2, 2, 2, 2)), dict(x
 
 @pytest.mark.parametrize("c", SMALL_CONVS, ids=lambda c: "x".join(map(str, c["x"] + c["w"])))
 def test_small_image_conv(binding, c, monkeypatch):
-    """The whole-image-in-shared-memory kernel at every channel count per block, ragged channels and pixels."""
+    """The whole-image-in-shared-memory kernel, ragged channels and pixels (every channel count per block: test_small_conv.py)."""
     monkeypatch.setenv("ONNXB_FP32", "small")
     rng = np.random.default_rng(17)
     X = rng.standard_normal(c["x"]).astype(np.float32)

@@ -1,5 +1,5 @@
-"""The small-image convolution at the widths where its rows change their share of threads (8, 16, 32 lanes a row, and more than
-one turn), and for every number of channels per block, pinned and as the rule picks them; fp32 throughout."""
+"""The small-image convolution at widths around a warp's share of lanes, images brought in by positions and (many blocks, rows of all
+but whole warps) by rows, and for every number of channels per block, pinned and as the rule picks them; fp32 throughout."""
 import numpy as np
 import pytest
 
@@ -44,7 +44,10 @@ def test_small_conv(x, w, kw, addend, monkeypatch, pin="small"):
 # a quotient and a remainder of channels at every number per block; 3x3, 5x5 and other filters; one block, and several per SM
 SIZES = [((n, c, h, wd), (m, c // kw.get("group", 1)) + k, kw) for n, c, h, wd, m, k, kw in (
     (2, 3, 9, 17, 21, (3, 3), dict(pads=(1,) * 4)), (70, 2, 12, 15, 37, (3, 3), dict(pads=(1,) * 4)), (3, 5, 14, 14, 19, (5, 5), dict(pads=(2,) * 4)),
-    (80, 4, 10, 33, 34, (5, 5), dict(pads=(2,) * 4, group=2)), (2, 3, 11, 8, 18, (2, 4), {}), (90, 2, 13, 16, 23, (4, 3), dict(strides=(2, 1))))]
+    (80, 4, 10, 33, 34, (5, 5), dict(pads=(2,) * 4, group=2)), (2, 3, 11, 8, 18, (2, 4), {}), (90, 2, 13, 16, 23, (4, 3), dict(strides=(2, 1))),
+    # by rows of 29, 32, 30 and 64, and by positions at 28 and 33 beside them
+    (120, 2, 10, 27, 21, (3, 3), dict(pads=(1,) * 4)), (130, 1, 9, 28, 19, (5, 5), dict(pads=(2,) * 4)), (120, 3, 9, 30, 18, (2, 4), {}),
+    (230, 1, 4, 64, 17, (3, 3), {}), (120, 2, 10, 26, 21, (3, 3), dict(pads=(1,) * 4)), (130, 1, 9, 29, 19, (5, 5), dict(pads=(2,) * 4)))]
 
 
 @pytest.mark.parametrize("x,w,kw", SIZES)
