@@ -86,6 +86,11 @@ def push_strides_up(ops: List[Op]) -> List[Op]:
     return ops
 
 
+def pass_flops(ops: List[Op]) -> int:
+    """Operations of the convolutions and the classifier of a graph, as its operators compute them."""
+    return sum(op.case.flops for op in ops if op.case is not None) + 2 * ops[0].case.x_shape[0] * 2048 * 1000
+
+
 class Resnet50Chain:
     """The model with its buffers.  Between the layers tensors are channel-major: a channel's pixels of all images in one row, rows
     of whole 128-byte lines.  A 1x1 layer is then one wide GEMM whatever the images' size (7x7 planes are no whole 16-byte pieces,
@@ -120,7 +125,7 @@ class Resnet50Chain:
                                         dtype=torch.uint8, device=device)
         self.buf: Dict[str, "torch.Tensor"] = {}
         self._lay_out(prepack, {})
-        self.flops = sum(op.case.flops for op in graph if op.case is not None) + 2 * batch * 2048 * 1000
+        self.flops = pass_flops(graph)          # the model's; of a pass as it is run: pass_flops(self.ops)
         self._capture()
 
     def _lay_out(self, channel_major: bool, given: Dict[str, "torch.Tensor"]):

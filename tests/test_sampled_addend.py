@@ -65,6 +65,17 @@ def test_moved_strides_leave_the_function_as_it_is():
         assert torch.allclose(v, w, rtol=1e-12, atol=1e-12), op.name
 
 
+def test_what_the_moved_graph_computes_is_counted():
+    """A rate is that of the operations made: three 3x3 layers and the three 1x1 layers behind them make a quarter of the model's."""
+    from paper_2008_08272_b200.resnet50_chain import build_graph, pass_flops, push_strides_up
+    graph = build_graph(2)
+    moved = push_strides_up(graph)
+    fewer = [g.case.flops for g, m in zip(graph, moved) if g.case is not None and g.case.y_shape != m.case.y_shape]
+    assert len(fewer) == 6 and pass_flops(graph) - pass_flops(moved) == sum(f * 3 // 4 for f in fewer)
+    convs = sum(2 * int(np.prod(o.case.y_shape)) * int(np.prod(o.case.w_shape[1:])) for o in moved if o.case is not None)
+    assert pass_flops(moved) == convs + 2 * 2 * 2048 * 1000
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("rounded", [False, True])
 @pytest.mark.parametrize("native", [True, False])
