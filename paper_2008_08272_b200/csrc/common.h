@@ -9,10 +9,10 @@
 
 namespace onnxb {
 
-// A convolution problem with every ONNX default and auto_pad already resolved.
 // Floats from one channel to the next in a channel-major tensor ([channel][image][row][column]), padded to whole 128-byte lines.
 inline long long channel_pitch(long long images, long long h, long long w) { return (images * h * w + 31) / 32 * 32; }
 
+// A convolution problem with every ONNX default and auto_pad already resolved.
 struct ConvGeom {
     int x_cm, y_cm;          // X, Y (and R) are channel-major
     int N, C, H, W;          // input

@@ -548,7 +548,7 @@ int simt_conv_on_tensor_cores(const ConvGeom &g, Fp32ConvPlan &plan, Fp32GemmPla
     const double tc = flat ? kGemmScale * tc_fp32_gemm_plan(g.M, (int)pixels, g.C, gemm) : tc_fp32_conv_plan(g, plan);
     if (tc < 0 || (flat && tc_fp32_gemm_workspace(g.M, (int)pixels, g.C, gemm) >= (1ull << 33))) return 0;
     if (!pin) {
-        const double small = small_conv_cost(g);
+        const double small = g.small_cost;
         const Pick fma = search_shape(g.Mg, (int)pixels, (int)K, g.group, true);
         if (tc >= fma.cost || (small >= 0 && 0.85 * small < tc) || !tc_is_as_exact(g.Mg, (int)pixels, K, g.group, true, fma)) return 0;
     }
