@@ -709,8 +709,10 @@ double small_conv_cost(const ConvGeom &g) {
     return 5500.0 + std::max(latency, issue);
 }
 // Channels per block of a problem that comes here, fitted to MNIST's layers at batch 1 to 200: what a block takes by itself, and half of
-// that for every other block on its SM (0.4 with eight channels and more).  (By the rule above the second layer at batch 18, 576 blocks of one channel, brings every
-// image in sixteen times: 12.6 us, 5.8 with four channels; eight and more leave a warp alone with its latencies: 11.2 at batch 30.)
+// that for every other block on its SM (0.4 with eight channels and more).  (By the rule above the second layer at batch 18, 576 blocks of
+// one channel, brings every image in sixteen times: 7.5 us, 4.5 with four channels, 6.3 with eight.)  Of 93 layers of other shapes (1 to
+// 12 channels, 3x3 to 7x7, images of 8x8 to 48x48, batch 1 to 256) it picks within 8 % of the best in 84 and 23 % off at most
+// (16 -> 32 channels 3x3 8x8 in two groups at batch 100: 5.0 us with four, 4.1 with eight).
 int small_conv_channels(const ConvGeom &g) {
     int best = 1, pinned = 0;                                // ONNXB_FP32 = "small,channels" pins them, too
     double cost = -1;
@@ -746,7 +748,9 @@ int launch_small_conv(const ConvGeom &g, const float *X, const float *W, const f
                 : mb == 8 ? pick(std::integral_constant<int, 8>())
                           : pick(std::integral_constant<int, 16>());
     // Blocks placed while the previous kernel still holds its SMs crowd on those that happen to have room: so much shared memory is
-    // asked for that no SM takes more than its share.  MNIST at batch 18 34.6 -> 19.6 us, at batch 39 36.7 -> 21.5 (with the channels per block above).
+    // asked for that no SM takes more than its share.  MNIST from a graph at batch 18 33.0 -> 11.4 us, at batch 39 43.1 -> 16.1 (with the
+    // channels per block above).  From 148 blocks on in place of 100, the second layer of four images and a 1x1 layer behind it took 12.4
+    // us for 8.1; from the first on nothing is gained, and two streams lose (5.6 -> 5.9 for a layer each); to 16 per SM: no difference.
     size_t smem = small_smem(g, mb);
     const long long sms = tc_host::num_sms(), share = (blocks + sms - 1) / sms;
     if (blocks > 100 && share <= 8) {

@@ -387,8 +387,11 @@ template <int AM, int BMODE, int I, int BM, int BN, int TM, int TN>
 cudaError_t launch_shape(const SgemmArgs &a, int split, long long tiles, cudaStream_t st) {
     static_assert(kShape[I].bm == BM && kShape[I].bn == BN && kShape[I].threads == (BM / TM) * (BN / TN), "shape table");
     // Blocks placed while the previous kernel still holds its SMs crowd on those that happen to have room: so much shared memory is
-    // asked for that no SM takes more than its share (clusters, which do not fit every GPC, one more).  Gemm 157 x 225 x 786 15.0 -> 9.6 us,
-    // 18 x 1543 x 181 10.0 -> 6.5, 1001 x 130 x 333 15.0 -> 13.2; 12 -> 40 channels 3x3 33x31 at batch 3 11.5 -> 9.9.
+    // asked for that no SM takes more than its share (clusters, which do not fit every GPC, one more).  From a graph Gemm 157 x 225 x 786
+    // 10.5 -> 8.6 us, 541 x 87 x 705 10.3 -> 6.7, 1001 x 130 x 333 13.8 -> 12.1; 12 -> 40 channels 3x3 33x31 at batch 3 10.6 -> 9.2; the one
+    // of 60 that lost, 885 x 63 x 115, 4.6 -> 4.8.  From 148 blocks on in place of 100: 355 x 49 x 571 10.0 us for 6.9; from the first on
+    // seven of 60 are 4 to 6 % shorter; to 8 per SM no difference; two more for clusters: 649 x 103 x 227 8.9 for 6.6.  Two streams with a
+    // Gemm each: 157 x 225 x 786 14.1 -> 11.8, 301 x 403 x 131 8.6 -> 9.3.
     size_t smem = sgemm_smem<BM, BN>();
     const long long ctas = tiles * split, sms = tc_host::num_sms(), share = (ctas + sms - 1) / sms + (split > 1 ? 1 : 0);
     if (ctas > 100 && share <= 4) smem = std::max(smem, smem_for_share(share));
