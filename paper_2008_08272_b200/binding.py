@@ -486,10 +486,11 @@ def launch_count() -> int:
     return int(load().onnxb_launch_count())
 
 
-def call_state(tensors):
-    """Where the tensors lie and how (address, type, sizes, strides) and ``onnxb_dispatch_state``, as bytes to compare: calls on the same
-    tensors at the same state launch the same kernels on the same memory.  None without the native call path."""
-    return (_fast_mod or _fast()).state(tensors)
+def call_state(*tensors):
+    """Where tensors lie and how (address, type, sizes, strides) and ``onnxb_dispatch_state``, as bytes to compare: calls on the same
+    tensors at the same state launch the same kernels on the same memory.  ``tensors``: tensors, tuples of them, and dicts of either,
+    whose entry "input" is left out.  None without the native call path."""
+    return (_fast_mod or _fast()).state(*tensors)
 
 
 def probe_tf32_mma_rate(n: int, instructions: int = 4096, stream=None) -> float:

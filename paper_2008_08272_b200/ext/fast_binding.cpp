@@ -271,22 +271,37 @@ PyObject *py_gap(PyObject *, PyObject *const *a, Py_ssize_t n) {
     return abi.global_average_pool_run(xt->sizes().data(), x, y, stream) == ONNXB_OK ? result(a[1], ym) : slow_path();
 }
 
-// state(list of tensors): address, type, sizes and strides of each, and the library's dispatch state, as bytes
-PyObject *py_state(PyObject *, PyObject *const *a, Py_ssize_t n) {
-    if (n != 1 || !PyList_CheckExact(a[0])) return slow_path();
-    const Py_ssize_t count = PyList_GET_SIZE(a[0]);
-    std::vector<int64_t> out;
-    out.reserve(2 + 12 * (size_t)count);
-    out.push_back((int64_t)abi.dispatch_state());
-    for (Py_ssize_t i = 0; i < count; ++i) {
-        PyObject *o = PyList_GET_ITEM(a[0], i);
-        if (!THPVariable_CheckExact(o)) return slow_path();
+// Address, type, sizes and strides of a tensor, or of those in a tuple or a dict (whose entry "input" is left out); false for anything else
+bool add_state(PyObject *o, std::vector<int64_t> &out) {
+    if (THPVariable_CheckExact(o)) {
         const at::Tensor &x = THPVariable_Unpack(o);
         out.push_back((int64_t)reinterpret_cast<uintptr_t>(x.data_ptr()));
         out.push_back((int64_t)x.scalar_type() << 32 | x.dim());
         out.insert(out.end(), x.sizes().begin(), x.sizes().end());
         out.insert(out.end(), x.strides().begin(), x.strides().end());
+        return true;
     }
+    if (PyTuple_CheckExact(o)) {
+        for (Py_ssize_t i = 0; i < PyTuple_GET_SIZE(o); ++i)
+            if (!add_state(PyTuple_GET_ITEM(o, i), out)) return false;
+        return true;
+    }
+    if (!PyDict_CheckExact(o)) return false;
+    PyObject *key, *value;
+    for (Py_ssize_t i = 0; PyDict_Next(o, &i, &key, &value);) {
+        if (!PyUnicode_Check(key)) return false;
+        if (PyUnicode_CompareWithASCIIString(key, "input") != 0 && !add_state(value, out)) return false;
+    }
+    return true;
+}
+
+// state(tensors, tuples, dicts...): that of all of them and the library's dispatch state, as bytes
+PyObject *py_state(PyObject *, PyObject *const *a, Py_ssize_t n) {
+    std::vector<int64_t> out;
+    out.reserve(4096);
+    out.push_back((int64_t)abi.dispatch_state());
+    for (Py_ssize_t i = 0; i < n; ++i)
+        if (!add_state(a[i], out)) return slow_path();
     return PyBytes_FromStringAndSize(reinterpret_cast<const char *>(out.data()), (Py_ssize_t)(out.size() * sizeof(int64_t)));
 }
 

@@ -212,10 +212,7 @@ class Resnet50Chain:
     def _state(self):
         """Where all tensors but the input lie and how, and what the library chooses its kernels by (None without the native call
         path): what the graph was captured with, and what a replay of it stands for."""
-        tensors = [t for k, t in self.store.items() if k != "input"] + [t for k, t in self.buf.items() if k != "input"] + \
-            list(self.rounded.values()) + list(self.packed.values()) + [t for pair in self.params.values() for t in pair] + \
-            [self.workspace, self.fc_workspace]
-        state = binding.call_state(tensors)
+        state = binding.call_state(self.store, self.buf, self.rounded, self.packed, self.params, self.workspace, self.fc_workspace)
         return None if state is None else (self.prepack, state)
 
     def _follow_buf(self):

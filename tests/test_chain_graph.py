@@ -161,3 +161,14 @@ def test_prepack_switched_off():
     assert torch.equal(net.forward(x), other.forward(x))
     net.close()
     other.close()
+
+
+def test_the_state_compared(monkeypatch):
+    a, b = torch.empty(6, 4, device="cuda"), torch.empty(6, 4, device="cuda")
+    plain = binding.call_state({"x": a, "input": b}, (a, b), b)
+    assert plain == binding.call_state({"x": a, "input": a}, (a, b), b) == binding.call_state({"x": a}, (a, b), b)
+    others = [binding.call_state({"x": t}, (a, u), b) for t, u in ((b, b), (a, a), (a.view(4, 6), b), (a[:, :2], b), (a.t(), b), (a.view(torch.int32), b))]
+    assert len({plain, *others, binding.call_state({"x": a}, (a, b)), binding.call_state({"x": a, "y": b}, (a, b), b)}) == 9
+    monkeypatch.setenv("ONNXB_GEMM_BN", "64")
+    assert plain != binding.call_state({"x": a}, (a, b), b)
+    assert binding.call_state([a]) is None and binding.call_state({"x": None}) is None
