@@ -220,6 +220,7 @@ class Resnet50Chain:
         if self.channel_major and (not self.prepack or any(self._place(self.buf[k]) != place for k, place in self._views.items())):
             if self.torch.cuda.is_current_stream_capturing():
                 raise RuntimeError("Resnet50Chain: an entry of buf was replaced; its buffers are made anew by a pass outside a capture")
+            self.torch.cuda.synchronize(self.dev)      # (a pass on another stream may still use what is let go here)
             x, descs = self.buf["input"], self.descs
             self._graph = self._captured = None
             self._lay_out(False, {k: t for k, t in self.buf.items() if k not in self._views or self._place(t) != self._views[k]})

@@ -172,3 +172,18 @@ def test_the_state_compared(monkeypatch):
     monkeypatch.setenv("ONNXB_GEMM_BN", "64")
     assert plain != binding.call_state({"x": a}, (a, b), b)
     assert binding.call_state([a]) is None and binding.call_state({"x": None}) is None
+
+
+def test_laid_out_anew_on_another_stream():
+    """While a pass on the first stream may still run, whose buffers go back to that stream's allocations."""
+    x, net = _x(23), Resnet50Chain(2, torch.device("cuda:0"), seed=5)
+    want, side = net.forward(x).clone(), torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    for _ in range(20):
+        net.forward(x)
+    net.buf["stem"] = torch.empty(2, 64, 112, 112, device="cuda")
+    with torch.cuda.stream(side):
+        got = net.forward(x)
+    torch.cuda.current_stream().wait_stream(side)
+    assert torch.allclose(got, want, rtol=0, atol=2e-2 * float(want.std())) and binding.last_device_status() == 0
+    net.close()
